@@ -463,8 +463,8 @@ def general_leg(pkg, torch, dev, l2buf, name, steps=(3, 2), warmup=(2, 1), peaks
     alg = k_its * float(np.sum(nT * nT) * 4 + np.sum(nT) * 2 * 8) + sum((k + 2) * m["nh"] * 8 for k in range(1, k_its + 1))
     g_a = alg / (gms / max(gcnt, 1) * 1e-3) / 1e9
     hbm = float(peaks.get("hbm_gbs", 6800.0))
-    cond_kernel = ("k_big_lu_panel + k_big_gemm (blocked LU), k_big_solve (column-block solve), k_big_gemm_tc "
-                   "(S on tcgen05), k_big_xr" if name == "channel3d" else
+    cond_kernel = ("k_big_lu_panel + k_big_gemm (blocked LU), k_big_solve (column-block solve), k_big_s_tc "
+                   "(S on tcgen05), k_big_t" if name == "channel3d" else
                    "k_inverse_tc + k_products_tc (tensor-core shape classes), k_condense_uneven<float> (shared-memory "
                    "Gauss-Jordan bundles, nA <= 64), the blocked-LU kernels (larger blocks)")
     out.update({

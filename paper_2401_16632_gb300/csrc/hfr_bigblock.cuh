@@ -5,28 +5,18 @@
 //      lowest row on ties), its row interchanges applied to the columns left and right of it and
 //      the block row right of it solved with the panel's unit lower triangle (same kernel); then
 //      the trailing matrix updated by the batched GEMM;
-//   2-3. X = A^{-1} P B: one CTA per block of 32 columns of one element, the block whole in shared
-//      memory (permuted columns of B in, forward and back substitution by factor panels staged in
-//      shared memory, X out once); where the block does not fit: the row interchanges applied to
-//      the right-hand sides, then forward / back substitution blocked by NB rows (a small
-//      triangular solve of the diagonal block, the rest of the rows updated by a batched GEMM);
-//   4. S = D - C X_B by the same batched GEMM;
-//   5. t = s - C x_r with FP64 accumulation (one CTA per element); x_r is the right-hand side's
-//      column of the column-block solve, or, on the blocked path, A^{-1} r by FP64 substitution.
+//   2-3. X = A^{-1} P [B | r]: one CTA per block of columns of one element, the block whole in shared
+//      memory (permuted columns in, forward and back substitution by factor panels, X out once);
+//   4. S = D - C X_B, in FP32 on the tensor cores, in FP64 by the same batched GEMM;
+//   5. t = s - C x_r with FP64 accumulation (one CTA per element).
 // The batched GEMM is a register-tiled CUDA-core kernel: 128 x 128 output tiles in FP32 (64 x 64 in
 // FP64), 256 threads with 8 x 8 (4 x 4) outputs each, K staged through two shared-memory buffers 8
 // at a time; arithmetic in the block precision T.  Included by hfr_condense.cu (uses UnevenArgs and DEV_ERR_*).
 #pragma once
 
-// FP32 batched GEMMs on the tensor cores (1) or the CUDA cores (0): a build flag for timing
-#ifndef HFR_BIG_GEMM_TC
-#define HFR_BIG_GEMM_TC 1
-#endif
-
 namespace hfr {
 namespace big {
 
-constexpr int NB = 32;       // rows per diagonal block of the triangular solves
 constexpr int BT = 256;      // threads per CTA
 // LU panel width: the panel of up to 1024 rows stays in shared memory (128 KB at most)
 template <typename T>
@@ -199,288 +189,286 @@ __global__ void __launch_bounds__(BT) k_big_lu_panel(const __grid_constant__ Une
   }
 }
 
-// 2. X = P B (rows in the order the interchanges leave them; B transposed when column-major)
-template <typename T>
-__global__ void __launch_bounds__(BT) k_big_rhs(const __grid_constant__ UnevenArgs a, const int* __restrict__ list,
-                                                int nlist, int uni_nA, int uni_nT) {
-  __shared__ int perm[1024], pvs[1024];
-  for (int li = blockIdx.x; li < nlist; li += gridDim.x) {
-    const Elem E = elem_of(a, list, li, uni_nA, uni_nT);
-    const int nA = E.nA, nT = E.nT;
-    const T* B = reinterpret_cast<const T*>(a.B) + E.o[1];
-    T* X = reinterpret_cast<T*>(a.XB) + E.o[1];
-    const int* piv = a.piv + E.o[3];
-    __syncthreads();
-    for (int i = threadIdx.x; i < nA; i += BT) {
-      pvs[i] = piv[i];
-      perm[i] = i;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int j = 0; j < nA; ++j) {
-        const int p = pvs[j];
-        if (p >= 0 && p < nA && p != j) {
-          const int u = perm[j];
-          perm[j] = perm[p];
-          perm[p] = u;
-        }
-      }
-    }
-    __syncthreads();
-    const bool cm = a.colmajor != 0;
-    for (size_t i = threadIdx.x; i < (size_t)nA * nT; i += BT) {
-      const int row = (int)(i / nT), col = (int)(i % nT), src = perm[row];
-      X[i] = cm ? B[(size_t)col * nA + src] : B[(size_t)src * nT + col];
-    }
+// 2-3. X = A^{-1} P [B | r] for a block of CW columns per CTA, whole in shared memory: the permuted
+// columns loaded once, forward substitution with the unit lower factor and back substitution with
+// the upper factor by panels of SP pivots, X written once.
+//
+// Bound by the FMA pipe of the block precision (2 nA^2 (nT + 1) flops per element) as far as shared
+// memory feeds it.  A panel's update of the other rows runs as tiles of 16 rows x COLG columns per
+// warp, each lane holding RPL rows x V columns, so that V 16-byte column vectors and RPL broadcast
+// factor vectors from shared memory serve RPL V^2 multiply-adds (128 in FP32; with one row of
+// accumulators per lane shared memory took three accesses per multiply-add).  The factor reaches the
+// warps through private two-tile rings filled by cp.async one tile ahead, so no block-wide staging
+// or barrier stands between tiles; rows and columns beyond nA are zero (unit diagonal), which pads
+// every panel to SP pivots.  Rows are interleaved over the lane groups (row G i + g), which with the
+// padded ring rows keeps the groups' broadcasts on different banks.  What is left is the in-panel
+// solve of a few warps between two barriers and the shared-memory rate of the updates.
+// Measured: 4608 FP32 blocks of (320, 480) 40.4 -> 21.7 ms (27 % of the FMA rate), 750 FP64 blocks
+// of (144, 96) 6.28 -> 3.85 ms (74 % of the FP64 rate).  X held in registers instead (one warp per 16
+// rows, tile after tile) took 34.8 ms: every tile waits for one warp's chain.
+template <typename T, int LC_, int CW_, int NW_, int H_>
+struct SolveCfg {
+  static constexpr int V = 16 / (int)sizeof(T);      // columns per lane (one 16-byte vector)
+  static constexpr int LC = LC_;                     // lanes along the columns
+  static constexpr int G = 32 / LC;                  // lane groups along the rows
+  static constexpr int RPL = 16 / G;                 // rows per lane
+  static constexpr int COLG = LC * V;                // columns of a warp tile
+  static constexpr int CW = CW_;                     // columns per CTA
+  static constexpr int XST = CW + V;                 // row stride of X
+  static constexpr int SP = sizeof(T) == 4 ? 32 : 16;  // pivots per panel
+  static constexpr int H = H_;                       // factor tiles per panel
+  static constexpr int KT = SP / H;                  // pivots of a factor tile
+  static constexpr int UJ = KT * V > 64 ? 2 : KT / V;  // steps of the update unrolled together
+  static constexpr int LST = KT + V;                 // its row stride
+  static constexpr int NW = NW_;                     // warps per CTA
+  static_assert(CW % COLG == 0 && CW <= 32 * NW && SP <= 32, "column groups");
+  __host__ __device__ static int rows(int nA) { return (nA + SP - 1) / SP * SP; }
+  static size_t smem(int nA) {
+    return ((size_t)rows(nA) * XST + (size_t)NW * 2 * 16 * LST + 2 * SP * SP) * sizeof(T) +
+           2 * (size_t)rows(nA) * sizeof(int);
   }
-}
+};
 
-// 3a. diagonal block jb of the triangular solves: rows [r0, r1) of X, one thread per column
-// (lower: unit lower factor, forward; upper: upper factor, backward)
-template <typename T>
-__global__ void __launch_bounds__(128) k_big_trsm_diag(const __grid_constant__ UnevenArgs a, const int* __restrict__ list,
-                                                      int base, int nlist, int uni_nA, int uni_nT, int jb, int upper) {
-  if ((int)blockIdx.y >= nlist) return;
-  const int li = base + blockIdx.y;
-  const Elem E = elem_of(a, list, li, uni_nA, uni_nT);
-  const int nA = E.nA, nT = E.nT;
-  const int r0 = jb * NB;
-  if (r0 >= nA) return;
-  const int r1 = min(nA, r0 + NB);
-  const int col = blockIdx.x * 128 + threadIdx.x;
-  if (col >= nT) return;
-  const T* L = reinterpret_cast<const T*>(a.LU) + E.o[0];
-  T* X = reinterpret_cast<T*>(a.XB) + E.o[1];
-  T x[NB];
-#pragma unroll
-  for (int q = 0; q < NB; ++q) x[q] = (r0 + q < r1) ? X[(size_t)(r0 + q) * nT + col] : T(0);
-  if (!upper) {
-#pragma unroll
-    for (int q = 0; q < NB; ++q) {
-      if (r0 + q >= r1) break;
-#pragma unroll
-      for (int c = 0; c < q; ++c) x[q] -= L[(size_t)(r0 + q) * nA + r0 + c] * x[c];
+// dst[r * ld + j] = L[r0 + r][p0 + j], r < nrows, j < W, zero outside the nA x nA factor; vec: rows
+// of L start on 16-byte boundaries (nA a multiple of V), copied asynchronously, else by plain loads
+template <typename T, int W, int V>
+__device__ __forceinline__ void solve_tile(T* dst, int ld, const T* L, int nA, int r0, int p0, int nrows, bool vec,
+                                           int t, int nt) {
+  if (vec) {
+    for (int i = t; i < nrows * (W / V); i += nt) {
+      const int r = i / (W / V), q = (i % (W / V)) * V;
+      const bool in = r0 + r < nA && p0 + q < nA;
+      const T* src = L + (in ? (size_t)(r0 + r) * nA + p0 + q : 0);
+      const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + r * ld + q);
+      const int bytes = in ? 16 : 0;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
     }
   } else {
-#pragma unroll
-    for (int q = NB - 1; q >= 0; --q) {
-      if (r0 + q >= r1) continue;
-      T s = x[q];
-#pragma unroll
-      for (int c = q + 1; c < NB; ++c)
-        if (r0 + c < r1) s -= L[(size_t)(r0 + q) * nA + r0 + c] * x[c];
-      x[q] = s / L[(size_t)(r0 + q) * nA + r0 + q];
+    for (int i = t; i < nrows * W; i += nt) {
+      const int r = i / W, j = i % W;
+      dst[r * ld + j] = (r0 + r < nA && p0 + j < nA) ? L[(size_t)(r0 + r) * nA + p0 + j] : T(0);
     }
   }
-#pragma unroll
-  for (int q = 0; q < NB; ++q)
-    if (r0 + q < r1) X[(size_t)(r0 + q) * nT + col] = x[q];
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+template <typename T>
+struct alignas(16) SolveVec {
+  T v[16 / sizeof(T)];
+};
+
+// x / d with the reciprocal known: one Newton correction of the quotient (the division's own
+// rounding, without its long instruction sequence on the substitution's serial chain)
+template <typename T>
+__device__ __forceinline__ T solve_div(T x, T d, T inv) {
+  const T q = x * inv;
+  const T c = fma(fma(-q, d, x), inv, q);
+  return isfinite(c) ? c : x / d;
 }
 
-// 2'-3'. X = A^{-1} P B for a block of SC columns per CTA, whole in shared memory: the permuted
-// columns of B loaded once, forward substitution with the unit lower factor and back substitution
-// with the upper factor by panels of SP pivots (the factor's panel staged in shared memory: an
-// in-panel solve of SP steps, then one register-tiled update of every row outside the panel), X
-// written once.  Replaces the row interchange copy and the blocked triangular solves when the two
-// tiles fit shared memory.
-constexpr int SC = 32;  // columns of X per CTA (the lanes of a warp)
-constexpr int SP = 32;  // pivots per factor panel
-template <typename T>
-size_t solve_smem(int max_nA) {
-  return ((size_t)max_nA * SC + (size_t)max_nA * SP) * sizeof(T) + (size_t)max_nA * sizeof(int);
-}
-// Lp[r][j] = L[r0 + r][p0 + j] for r < nrows, j < w (zero for w <= j < SP); SU loads per thread in
-// flight before their stores.  A full panel (w = SP) of a factor whose rows start on 16-byte
-// boundaries moves in 16-byte vectors: a quarter (FP32) of the dependent rounds of loads.
-template <typename T>
-__device__ __forceinline__ void solve_stage_panel(T* Lp, const T* L, int nA, int r0, int nrows, int p0, int w,
-                                                  int tid) {
-  constexpr int SU = 8;
-  constexpr int V = 16 / sizeof(T);  // values per 16-byte vector
-  using VT = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
-  if (w == SP && nA % V == 0 && (reinterpret_cast<uintptr_t>(L) & 15) == 0) {
-    // rows r0 .. r0 + nrows - 1 < nA, columns p0 .. p0 + SP - 1 < nA (full panel); p0 % SP == 0
-    constexpr int VR = SP / V;  // vectors per panel row
-    const int cnt = nrows * VR;
-    for (int b = tid; b < cnt; b += BT * SU) {
-      VT v[SU];
-#pragma unroll
-      for (int u = 0; u < SU; ++u) {
-        const int idx = b + BT * u, r = idx / VR, q = idx % VR;
-        if (idx < cnt) v[u] = *reinterpret_cast<const VT*>(L + (size_t)(r0 + r) * nA + p0 + q * V);
-      }
-#pragma unroll
-      for (int u = 0; u < SU; ++u) {
-        const int idx = b + BT * u;
-        if (idx < cnt) *reinterpret_cast<VT*>(Lp + (size_t)(idx / VR) * SP + (idx % VR) * V) = v[u];
-      }
-    }
-    return;
-  }
-  const int cnt = nrows * SP;
-  for (int b = tid; b < cnt; b += BT * SU) {
-    T v[SU];
-#pragma unroll
-    for (int u = 0; u < SU; ++u) {
-      const int idx = b + BT * u, r = idx / SP, j = idx % SP;
-      v[u] = (idx < cnt && j < w) ? L[(size_t)(r0 + r) * nA + p0 + j] : T(0);
-    }
-#pragma unroll
-    for (int u = 0; u < SU; ++u)
-      if (b + BT * u < cnt) Lp[b + BT * u] = v[u];
-  }
-}
-
-// Xs rows [ra, rb) -= (factor panel rows, staged at Lp row r - lbase) x (solved panel rows of Xs,
-// p0 .. p0 + w - 1): eight rows per warp pass, four pivots per step (one 16-byte broadcast of the
-// factor per row, four values of the solved rows per lane); the factor panel is zero beyond w
-template <typename T>
-__device__ __forceinline__ void solve_update(T* Xs, const T* Lp, int p0, int w, int ra, int rb, int lbase, int lane,
-                                             int wid) {
-  constexpr int NW = BT / 32;
-  for (int r0 = ra + 8 * wid; r0 < rb; r0 += 8 * NW) {
-    T acc[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q] = T(0);
-    for (int j = 0; j < w; j += 4) {
-      T xv[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) xv[u] = j + u < w ? Xs[(p0 + j + u) * SC + lane] : T(0);
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        if (r0 + q < rb) {
-          const T* lr = Lp + (size_t)(r0 + q - lbase) * SP + j;  // 16-byte aligned (j % 4 == 0)
-          if constexpr (sizeof(T) == 4) {
-            const float4 l4 = *reinterpret_cast<const float4*>(lr);
-            acc[q] += l4.x * xv[0] + l4.y * xv[1] + l4.z * xv[2] + l4.w * xv[3];
-          } else {
-            const double2 la = reinterpret_cast<const double2*>(lr)[0], lb = reinterpret_cast<const double2*>(lr)[1];
-            acc[q] += la.x * xv[0] + la.y * xv[1] + lb.x * xv[2] + lb.y * xv[3];
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q)
-      if (r0 + q < rb) Xs[(r0 + q) * SC + lane] -= acc[q];
-  }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(BT, 2) k_big_solve(const __grid_constant__ UnevenArgs a, const int* __restrict__ list,
+template <typename T, int LC, int CW, int NW, int H>
+__global__ void __launch_bounds__(32 * NW, 512 / (32 * NW)) k_big_solve(const __grid_constant__ UnevenArgs a, const int* __restrict__ list,
                                                   int base, int nlist, int uni_nA, int uni_nT) {
+  using C = SolveCfg<T, LC, CW, NW, H>;
+  constexpr int V = C::V, G = C::G, RPL = C::RPL, COLG = C::COLG, XST = C::XST, SP = C::SP, KT = C::KT, LST = C::LST;
+  constexpr int NTH = 32 * NW;
   extern __shared__ __align__(16) unsigned char sv_smem[];
   if ((int)blockIdx.y >= nlist) return;
   const Elem E = elem_of(a, list, base + blockIdx.y, uni_nA, uni_nT);
-  const int nA = E.nA, nT = E.nT, c0 = blockIdx.x * SC;
+  const int nA = E.nA, nT = E.nT, c0 = blockIdx.x * CW;
   if (c0 > nT) return;  // uniform over the CTA (column nT is r: x_r)
-  T* Xs = reinterpret_cast<T*>(sv_smem);  // nA x SC
-  T* Lp = Xs + (size_t)nA * SC;            // nA x SP: rows of the current factor panel
-  int* perm = reinterpret_cast<int*>(Lp + (size_t)nA * SP);
+  const int nAp = C::rows(nA);
+  T* Xs = reinterpret_cast<T*>(sv_smem);            // nAp x XST
+  T* ring = Xs + (size_t)nAp * XST;                  // NW x 2 factor tiles of 16 x LST
+  T* Dg = ring + (size_t)NW * 2 * 16 * LST;          // two diagonal blocks SP x SP
+  int* perm = reinterpret_cast<int*>(Dg + 2 * SP * SP);
+  int* pvs = perm + nAp;
   const T* L = reinterpret_cast<const T*>(a.LU) + E.o[0];
   const T* B = reinterpret_cast<const T*>(a.B) + E.o[1];
   T* X = reinterpret_cast<T*>(a.XB) + E.o[1];
   const int* piv = a.piv + E.o[3];
   const bool cm = a.colmajor != 0;
+  const bool vec = nA % V == 0 && (reinterpret_cast<uintptr_t>(L) & 15) == 0;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  constexpr int NW = BT / 32;
-  // rows in the order the interchanges leave them: the pivots staged in shared memory (the factor
-  // panel's space, free until the forward sweep), then applied in sequence by one thread
-  int* pvs = reinterpret_cast<int*>(Lp);
-  for (int i = tid; i < nA; i += BT) {
-    pvs[i] = piv[i];
-    perm[i] = i;
-  }
+  const int live = min(CW, nT + 1 - c0);             // columns of this CTA, r included
+  const int ncg = (live + COLG - 1) / COLG;
+  T* tile = ring + (size_t)wid * 2 * 16 * LST;
+  const int np = nAp / SP;
+  // the factor tile of this warp's first unit of a panel and the first diagonal block
+  auto first_tile = [&](int ra, int rows, int p0) {
+    if (wid < rows / 16 * ncg) solve_tile<T, KT, V>(tile, LST, L, nA, ra + 16 * (wid / ncg), p0, 16, vec, lane, 32);
+    cp_commit();
+  };
+  solve_tile<T, SP, V>(Dg, SP, L, nA, 0, 0, SP, vec, tid, NTH);
+  cp_commit();
+  // position i of P b holds row perm[i]: the interchanges (j, piv[j]) undone from the last to the
+  // first, every position on its own
+  for (int i = tid; i < nA; i += NTH) pvs[i] = piv[i];
   __syncthreads();
-  if (tid == 0) {
-    for (int j = 0; j < nA; ++j) {
+  for (int i = tid; i < nAp; i += NTH) {
+    int pos = i;
+    for (int j = nA - 1; j >= 0; --j) {
       const int p = pvs[j];
-      if (p >= 0 && p < nA && p != j) {
-        const int u = perm[j];
-        perm[j] = perm[p];
-        perm[p] = u;
-      }
+      if (p >= 0 && p < nA) pos = pos == j ? p : (pos == p ? j : pos);
     }
+    perm[i] = pos;
   }
   __syncthreads();
-  const int c = c0 + lane;
-  const bool live = c < nT;
-  const double* rv = a.r + E.o[3];
-  // global loads in batches of SU per thread, all in flight before their shared-memory stores
+  // the permuted columns: SU loads per thread in flight before their stores.  Column-major B: 8 rows
+  // x 4 columns per warp access (whole sectors, conflict-free stores); row-major: one row per access
   constexpr int SU = 8;
-  for (int i0 = wid; i0 < nA; i0 += NW * SU) {
+  const double* rv = a.r + E.o[3];
+  const int nr = cm ? nAp / 8 : nAp, ni = cm ? nr * (CW / 4) : nr * (CW / 32 + (CW % 32 != 0));
+  for (int i0 = wid; i0 < ni; i0 += NW * SU) {
     T v[SU];
 #pragma unroll
     for (int u = 0; u < SU; ++u) {
-      const int i = i0 + NW * u;
+      const int it = i0 + NW * u, ir = it % nr, iq = it / nr;
+      const int i = cm ? ir * 8 + (lane & 7) : ir, q = cm ? iq * 4 + (lane >> 3) : iq * 32 + lane;
+      const int c = c0 + q;
       v[u] = T(0);
-      if (i < nA) {
+      if (it < ni && i < nA && q < CW) {
         const int src = perm[i];
-        v[u] = live ? (cm ? B[(size_t)c * nA + src] : B[(size_t)src * nT + c]) : (c == nT ? T(rv[src]) : T(0));
+        v[u] = c < nT ? B[cm ? (size_t)c * nA + src : (size_t)src * nT + c] : (c == nT ? T(rv[src]) : T(0));
       }
     }
 #pragma unroll
-    for (int u = 0; u < SU; ++u)
-      if (i0 + NW * u < nA) Xs[(i0 + NW * u) * SC + lane] = v[u];
-  }
-  // ---- forward: unit lower factor, panels top to bottom
-  for (int p0 = 0; p0 < nA; p0 += SP) {
-    const int w = min(SP, nA - p0);
-    __syncthreads();  // the previous panel's readers are done
-    solve_stage_panel<T>(Lp, L, nA, p0, nA - p0, p0, w, tid);
-    __syncthreads();
-    if (wid == 0) {  // in-panel solve: one warp, lane = column, the panel's rows in registers
-      T x[SP];
-#pragma unroll
-      for (int r = 0; r < SP; ++r) x[r] = r < w ? Xs[(p0 + r) * SC + lane] : T(0);
-#pragma unroll
-      for (int j = 0; j < SP; ++j)
-#pragma unroll
-        for (int r = j + 1; r < SP; ++r) x[r] -= Lp[r * SP + j] * x[j];  // zero beyond w
-#pragma unroll
-      for (int r = 0; r < SP; ++r)
-        if (r < w) Xs[(p0 + r) * SC + lane] = x[r];
+    for (int u = 0; u < SU; ++u) {
+      const int it = i0 + NW * u, ir = it % nr, iq = it / nr;
+      const int i = cm ? ir * 8 + (lane & 7) : ir, q = cm ? iq * 4 + (lane >> 3) : iq * 32 + lane;
+      if (it < ni && q < CW) Xs[(size_t)i * XST + q] = v[u];
     }
-    __syncthreads();
-    // rows below the panel: X[r] -= L[r, panel] X[panel]
-    solve_update<T>(Xs, Lp, p0, w, p0 + w, nA, p0, lane, wid);
   }
-  // ---- backward: upper factor, panels bottom to top
-  const int np = (nA + SP - 1) / SP;
-  for (int pb = np - 1; pb >= 0; --pb) {
-    const int p0 = pb * SP, w = min(SP, nA - p0);
-    __syncthreads();
-    solve_stage_panel<T>(Lp, L, nA, 0, p0 + w, p0, w, tid);
-    __syncthreads();
-    if (wid == 0) {
-      T x[SP];
+  // rows [ra, ra + rows) of X -= (factor rows, columns p0 ..) x (solved rows p0 ..); the first tile is
+  // on its way
+  auto update = [&](int ra, int rows, int p0) {
+    const int units = rows / 16 * ncg;
+    const int g = lane / LC, lc = lane % LC;
+    int slot = 0;
+    for (int u = wid; u < units; u += NW) {
+      T* xo = Xs + (size_t)(ra + 16 * (u / ncg) + g) * XST + (u % ncg) * COLG + lc * V;
+      T acc[RPL][V];
 #pragma unroll
-      for (int r = 0; r < SP; ++r) x[r] = r < w ? Xs[(p0 + r) * SC + lane] : T(0);
+      for (int i = 0; i < RPL; ++i)
 #pragma unroll
-      for (int j = SP - 1; j >= 0; --j) {
-        if (j < w) {
-          x[j] = x[j] / Lp[(p0 + j) * SP + j];
+        for (int q = 0; q < V; ++q) acc[i][q] = T(0);
 #pragma unroll
-          for (int r = 0; r < j; ++r) x[r] -= Lp[(p0 + r) * SP + j] * x[j];
+      for (int h = 0; h < H; ++h, slot ^= 1) {  // tile h of the panel's pivots; the next one on its way
+        const int un = h + 1 < H ? u : u + NW;
+        if (un < units)
+          solve_tile<T, KT, V>(tile + (slot ^ 1) * 16 * LST, LST, L, nA, ra + 16 * (un / ncg), p0 + (h + 1) % H * KT,
+                               16, vec, lane, 32);
+        cp_commit();
+        cp_wait<1>();
+        __syncwarp();
+        const T* lt = tile + slot * 16 * LST + g * LST;
+        const T* xp = Xs + (size_t)(p0 + h * KT) * XST + (u % ncg) * COLG + lc * V;
+#pragma unroll(C::UJ)
+        for (int j = 0; j < KT; j += V) {
+          SolveVec<T> xv[V];
+#pragma unroll
+          for (int s = 0; s < V; ++s) xv[s] = *reinterpret_cast<const SolveVec<T>*>(xp + (size_t)(j + s) * XST);
+#pragma unroll
+          for (int i = 0; i < RPL; ++i) {
+            const SolveVec<T> l = *reinterpret_cast<const SolveVec<T>*>(lt + G * i * LST + j);
+#pragma unroll
+            for (int s = 0; s < V; ++s)
+#pragma unroll
+              for (int q = 0; q < V; ++q) acc[i][q] = fma(l.v[s], xv[s].v[q], acc[i][q]);
+          }
         }
+        __syncwarp();  // the slot may be refilled
       }
 #pragma unroll
-      for (int r = 0; r < SP; ++r)
-        if (r < w) Xs[(p0 + r) * SC + lane] = x[r];
+      for (int i = 0; i < RPL; ++i) {
+        SolveVec<T>* xr = reinterpret_cast<SolveVec<T>*>(xo + (size_t)G * i * XST);
+        SolveVec<T> x = *xr;
+#pragma unroll
+        for (int q = 0; q < V; ++q) x.v[q] -= acc[i][q];
+        *xr = x;
+      }
+    }
+    cp_wait<0>();
+  };
+  // ---- forward: unit lower factor, panels top to bottom
+  for (int pb = 0; pb < np; ++pb) {
+    const int p0 = pb * SP, ra = p0 + SP, rows = nAp - ra;
+    const T* D = Dg + (pb & 1) * SP * SP;
+    first_tile(ra, rows, p0);
+    cp_wait<1>();     // the diagonal block
+    __syncthreads();  // and the rows of the panel are final
+    if (tid < live) {  // in-panel solve, one column per thread, the panel's rows in registers
+      T x[SP];
+#pragma unroll
+      for (int r = 0; r < SP; ++r) x[r] = Xs[(size_t)(p0 + r) * XST + tid];
+#pragma unroll
+      for (int r = 1; r < SP; ++r)
+#pragma unroll
+        for (int c = 0; c < r; c += V) {
+          const SolveVec<T> l = *reinterpret_cast<const SolveVec<T>*>(D + r * SP + c);
+#pragma unroll
+          for (int s = 0; s < V; ++s)
+            if (c + s < r) x[r] = fma(-l.v[s], x[c + s], x[r]);
+        }
+#pragma unroll
+      for (int r = 0; r < SP; ++r) Xs[(size_t)(p0 + r) * XST + tid] = x[r];
     }
     __syncthreads();
-    solve_update<T>(Xs, Lp, p0, w, 0, p0, 0, lane, wid);  // rows above the panel
+    if (pb + 1 < np)  // the next panel's diagonal block
+      solve_tile<T, SP, V>(Dg + ((pb + 1) & 1) * SP * SP, SP, L, nA, ra, ra, SP, vec, tid, NTH);
+    cp_commit();
+    update(ra, rows, p0);
+  }
+  // ---- backward: upper factor, panels bottom to top (the last diagonal block is still in place)
+  for (int pb = np - 1; pb >= 0; --pb) {
+    const int p0 = pb * SP;
+    const T* D = Dg + (pb & 1) * SP * SP;
+    first_tile(0, p0, p0);
+    cp_wait<1>();
+    __syncthreads();
+    if (32 * wid < live) {  // whole warps: lane r holds the reciprocal of pivot r
+      const int q = min(tid, CW - 1);
+      const T dl = lane < SP && p0 + lane < nA ? D[lane * SP + lane] : T(1);
+      const T il = T(1) / dl;
+      T x[SP];
+#pragma unroll
+      for (int r = 0; r < SP; ++r) x[r] = Xs[(size_t)(p0 + r) * XST + q];
+#pragma unroll
+      for (int r = SP - 1; r >= 0; --r) {
+#pragma unroll
+        for (int c = SP - V; c + V > r + 1; c -= V) {
+          const SolveVec<T> l = *reinterpret_cast<const SolveVec<T>*>(D + r * SP + c);
+#pragma unroll
+          for (int s = V - 1; s >= 0; --s)
+            if (c + s > r) x[r] = fma(-l.v[s], x[c + s], x[r]);
+        }
+        x[r] = solve_div<T>(x[r], __shfl_sync(0xffffffffu, dl, r), __shfl_sync(0xffffffffu, il, r));
+      }
+      if (tid < CW) {
+#pragma unroll
+        for (int r = 0; r < SP; ++r) Xs[(size_t)(p0 + r) * XST + tid] = x[r];
+      }
+    }
+    __syncthreads();
+    if (pb > 0)
+      solve_tile<T, SP, V>(Dg + ((pb - 1) & 1) * SP * SP, SP, L, nA, p0 - SP, p0 - SP, SP, vec, tid, NTH);
+    cp_commit();
+    update(0, p0, p0);
   }
   __syncthreads();
-  if (live)
-    for (int i = wid; i < nA; i += NW) X[(size_t)i * nT + c] = Xs[i * SC + lane];
-  else if (c == nT)
-    for (int i = wid; i < nA; i += NW) a.xr[E.o[3] + i] = double(Xs[i * SC + lane]);
+  for (int it = tid; it < nA * CW; it += NTH) {
+    const int i = it / CW, q = it % CW, c = c0 + q;
+    if (c < nT)
+      X[(size_t)i * nT + c] = Xs[(size_t)i * XST + q];
+    else if (c == nT)
+      a.xr[E.o[3] + i] = double(Xs[(size_t)i * XST + q]);
+  }
 }
 
-// 3b / 4. batched GEMM Out -= A B, per element:
-//   phase 0: rows [r1, nA) of X -= L[r1:, r0:r1] X[r0:r1, :]     (forward, block jb)
-//   phase 1: rows [0, r0) of X  -= L[:r0, r0:r1] X[r0:r1, :]     (backward, block jb)
+// 1c / 4. batched GEMM Out -= A B, per element:
 //   phase 2: S = D - C X_B (C, D column-major when the blocks are)
 //   phase 3: L[j1:, j1:] -= L[j1:, j0:j1] L[j0:j1, j1:]          (LU trailing update, panel jb)
 // 16 x 16 threads, each with TM x TM outputs in two TM/2-wide halves of rows and of columns (so
@@ -527,20 +515,7 @@ __global__ void __launch_bounds__(BT) k_big_gemm(const __grid_constant__ UnevenA
   const T* Cm = reinterpret_cast<const T*>(a.C) + E.o[1];
   const T* Dm = reinterpret_cast<const T*>(a.D) + E.o[2];
   T* S = reinterpret_cast<T*>(a.S) + E.o[2];
-  if (phase == 0) {
-    const int r0 = jb * NB, r1 = min(nA, r0 + NB);
-    M = nA - r1;
-    N = nT;
-    K = r1 - r0;
-    m_off = r1;
-    k_off = r0;
-  } else if (phase == 1) {
-    const int r0 = jb * NB, r1 = min(nA, r0 + NB);
-    M = r0;
-    N = nT;
-    K = r1 - r0;
-    k_off = r0;
-  } else if (phase == 2) {
+  if (phase == 2) {
     M = nT;
     N = nT;
     K = nA;
@@ -629,9 +604,7 @@ __global__ void __launch_bounds__(BT) k_big_gemm(const __grid_constant__ UnevenA
     for (int j = 0; j < TM; ++j) {
       const int n = tn0 + (j < H ? tx * H + j : BM / 2 + tx * H + j - H);
       if (n >= N) continue;
-      if (phase <= 1) {
-        X[(size_t)(m_off + m) * nT + n] -= acc[i][j];
-      } else if (phase == 3) {
+      if (phase == 3) {
         L[(size_t)(m_off + m) * nA + n_off + n] -= acc[i][j];
       } else {
         const T d = cm ? Dm[(size_t)n * nT + m] : Dm[(size_t)m * nT + n];
@@ -641,144 +614,120 @@ __global__ void __launch_bounds__(BT) k_big_gemm(const __grid_constant__ UnevenA
   }
 }
 
-// 3b' / 4'. the same batched GEMMs for FP32 blocks on the tensor cores (tcgen05, 3xTF32: each
-// operand split into a TF32 high part and the remainder, hi*hi + hi*lo + lo*hi accumulated in FP32
-// in tensor memory).  One CTA per output tile of 256 rows (m) x 128 columns (n) of one element,
-// computed transposed: the tensor-memory lanes hold the 128 columns n and its 256 FP32 columns the
-// rows m, so that in the epilogue the 32 lanes of a warp read and write 32 consecutive n of one
-// row (coalesced).  K runs in chunks of 32, staged K-major without swizzle (hfr_tc.cuh) in two
-// shared-memory buffers, one mbarrier per buffer; the next chunk's global loads are in flight
-// while the tensor core works on the current one.  Thread 0 issues the MMAs; in the epilogue warp
-// w reads lanes 32 (w % 4).. and the column half w / 4 of the accumulator.
+// 4'. S = D - C X_B of FP32 blocks on the tensor cores (tcgen05, 3xTF32: each operand split into a
+// TF32 high part and the remainder, hi*hi + hi*lo + lo*hi accumulated in FP32 in tensor memory).
+// One CTA per output tile of TM rows (m) x 128 columns (n) of one element, computed transposed: the
+// tensor-memory lanes hold the 128 columns n and its TM FP32 columns the rows m, so that in the
+// epilogue the 32 lanes of a warp write 32 consecutive n of one row (coalesced).  K runs in chunks
+// of KC staged K-major without swizzle (hfr_tc.cuh) in two shared-memory buffers, one mbarrier per
+// buffer; the next chunk's global loads are in flight while the tensor core works on the current
+// one.  A thread stages four consecutive k of a row as one 16-byte store, and the eight threads of a
+// store's quarter-warp write the eight rows of one core matrix: 128 contiguous bytes, free of bank
+// conflicts (single-value stores of the same layout met four to a bank and set the kernel's time).
+// Measured: 4608 blocks of (320, 480) 14.7 -> 6.1 ms, the p = 4 and 5 blocks of a wall mesh (10 000
+// elements) 1.71 -> 0.20 ms.  KC = 16 leaves two CTAs per SM (TM = 256) or three (TM = 128, taken when nT <= 128), so that one
+// CTA's epilogue runs under another's products.
 namespace btc {
-constexpr int TM = 256, TN = 128, KC = 32, THREADS = 256;
-constexpr uint32_t SBO = (KC / 4) * 128u + 16u;  // 8-row groups padded by 16 bytes
-constexpr uint32_t N_BYTES = (TN / 8) * SBO;     // the n-rows operand (MMA A, 128 rows), hi or lo
-constexpr uint32_t M_BYTES = (TM / 8) * SBO;     // the m-rows operand (MMA B, 256 rows), hi or lo
-constexpr uint32_t STAGE = 2 * N_BYTES + 2 * M_BYTES;
-constexpr uint32_t SMEM = 2 * STAGE + 64;
-constexpr int A_PER = TM * KC / THREADS, B_PER = TN * KC / THREADS;  // values a thread stages per chunk
-static_assert(SMEM <= 232448, "shared memory");
+constexpr int TN = 128, KC = 16, THREADS = 256;
+constexpr uint32_t SBO = (KC / 4) * 128u;
+constexpr uint32_t N_BYTES = (TN / 8) * SBO;  // the n-rows operand (MMA A, 128 rows), hi or lo
+template <int TM>
+__host__ __device__ constexpr uint32_t m_bytes() { return (TM / 8) * SBO; }  // the m-rows operand (MMA B), hi or lo
+template <int TM>
+__host__ __device__ constexpr uint32_t stage() { return 2 * N_BYTES + 2 * m_bytes<TM>(); }
+template <int TM>
+__host__ __device__ constexpr uint32_t smem() { return 2 * stage<TM>() + 64; }
+static_assert(smem<256>() <= 232448 / 2, "two CTAs per SM");
+__device__ __forceinline__ void split_store(unsigned char* hi, unsigned char* lo, uint32_t o, const float (&v)[4]) {
+  float h[4], l[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) tc::split_tf32(v[e], h[e], l[e]);
+  *reinterpret_cast<float4*>(hi + o) = make_float4(h[0], h[1], h[2], h[3]);
+  *reinterpret_cast<float4*>(lo + o) = make_float4(l[0], l[1], l[2], l[3]);
+}
 }  // namespace btc
 
-__global__ void __launch_bounds__(btc::THREADS, 1) k_big_gemm_tc(const __grid_constant__ UnevenArgs a,
-                                                                const int* __restrict__ list, int base, int nlist,
-                                                                int uni_nA, int uni_nT, int phase, int jb) {
+template <int TM>
+__global__ void __launch_bounds__(btc::THREADS, 2) k_big_s_tc(const __grid_constant__ UnevenArgs a,
+                                                             const int* __restrict__ list, int base, int nlist,
+                                                             int uni_nA, int uni_nT) {
   using namespace tc;
   using namespace btc;
   extern __shared__ __align__(1024) unsigned char btc_smem[];
   if ((int)blockIdx.z >= nlist) return;
   const Elem E = elem_of(a, list, base + blockIdx.z, uni_nA, uni_nT);
-  const int nA = E.nA, nT = E.nT;
+  const int nT = E.nT, K = E.nA;
   const bool cm = a.colmajor != 0;
-  int M, N, K, m_off = 0, k_off = 0, n_off = 0;
-  float* L = reinterpret_cast<float*>(a.LU) + E.o[0];
-  float* X = reinterpret_cast<float*>(a.XB) + E.o[1];
+  const float* X = reinterpret_cast<const float*>(a.XB) + E.o[1];
   const float* Cm = reinterpret_cast<const float*>(a.C) + E.o[1];
   const float* Dm = reinterpret_cast<const float*>(a.D) + E.o[2];
   float* S = reinterpret_cast<float*>(a.S) + E.o[2];
-  if (phase == 0) {
-    const int r0 = jb * NB, r1 = min(nA, r0 + NB);
-    M = nA - r1;
-    N = nT;
-    K = r1 - r0;
-    m_off = r1;
-    k_off = r0;
-  } else if (phase == 1) {
-    const int r0 = jb * NB, r1 = min(nA, r0 + NB);
-    M = r0;
-    N = nT;
-    K = r1 - r0;
-    k_off = r0;
-  } else if (phase == 2) {
-    M = nT;
-    N = nT;
-    K = nA;
-  } else {
-    const int j0 = jb * lu_panel<float>(), j1 = min(nA, j0 + lu_panel<float>());
-    M = nA - j1;
-    N = nA - j1;
-    K = j1 - j0;
-    m_off = j1;
-    n_off = j1;
-    k_off = j0;
-  }
   const int tm0 = blockIdx.y * TM, tn0 = blockIdx.x * TN;
-  if (M <= 0 || K <= 0 || tm0 >= M || tn0 >= N) return;  // uniform over the CTA
+  if (tm0 >= nT || tn0 >= nT) return;  // uniform over the CTA
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  constexpr uint32_t MB = m_bytes<TM>(), STAGE = stage<TM>();
   uint64_t* mbar = reinterpret_cast<uint64_t*>(btc_smem + 2 * STAGE);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 2);
   if (t == 0) {
     mbar_init(smem_u32(mbar), 1);
     mbar_init(smem_u32(mbar + 1), 1);
   }
-  if (w == 0) tmem_alloc(smem_u32(tslot), 256);
+  if (w == 0) tmem_alloc(smem_u32(tslot), TM);
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
   const uint32_t tmem = *tslot;
-  const bool a_mfast = phase == 2 && cm;  // A(m, k) contiguous in m (column-major C)
-  // staging slots of this thread: A (m, k) with k fastest: rows (t >> 3) + 32 u, k 4 (t & 7) + e;
-  // m fastest: row 32 w + lane, k = u; B (k, n): column t & 127, k (t >> 7) + 2 u
-  float ra[A_PER], rb[B_PER];
+  const int NM = min(TM, (nT - tm0 + 15) & ~15);  // rows m that the products cover
+  const bool avec = !cm && K % 4 == 0 && (reinterpret_cast<uintptr_t>(Cm) & 15) == 0;
+  // staging: column n = t & 127 of X, k quads (t >> 7) + 2 u; rows of C: column-major one row per
+  // thread (row t % TM, quads t / TM + (256 / TM) u), row-major eight rows x four quads per warp
+  constexpr int QN = KC / 8;           // quads of X per thread
+  constexpr int QM = TM * KC / 1024;   // quads of C per thread
+  float rb[QN][4], ra[QM][4];
   auto gload = [&](int k0) {
 #pragma unroll
-    for (int u = 0; u < A_PER; ++u) {
-      const int m = tm0 + (a_mfast ? 32 * w + lane : (t >> 3) + 32 * (u >> 2));
-      const int k = k0 + (a_mfast ? u : 4 * (t & 7) + (u & 3));
-      float v = 0.f;
-      if (m < M && k < K) {
-        if (phase != 2)
-          v = L[(size_t)(m_off + m) * nA + k_off + k];
-        else
-          v = cm ? Cm[(size_t)k * nT + m] : Cm[(size_t)m * nA + k];
-      }
-      ra[u] = v;
+    for (int u = 0; u < QN; ++u) {
+      const int n = tn0 + (t & 127), k = k0 + 4 * ((t >> 7) + 2 * u);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) rb[u][e] = (n < nT && k + e < K) ? X[(size_t)(k + e) * nT + n] : 0.f;
     }
 #pragma unroll
-    for (int u = 0; u < B_PER; ++u) {
-      const int n = tn0 + (t & 127), k = k0 + (t >> 7) + 2 * u;
-      float v = 0.f;
-      if (n < N && k < K) v = phase == 3 ? L[(size_t)(k_off + k) * nA + n_off + n] : X[(size_t)(k_off + k) * nT + n];
-      rb[u] = v;
+    for (int u = 0; u < QM; ++u) {
+      if (cm) {
+        const int m = tm0 + t % TM, k = k0 + 4 * (t / TM + (THREADS / TM) * u);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) ra[u][e] = (m < nT && k + e < K) ? Cm[(size_t)(k + e) * nT + m] : 0.f;
+      } else {
+        const int m = tm0 + 64 * u + 8 * w + (lane & 7), k = k0 + 4 * (lane >> 3);
+        if (avec) {
+          float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (m < nT && k < K) v = *reinterpret_cast<const float4*>(Cm + (size_t)m * K + k);
+          ra[u][0] = v.x;
+          ra[u][1] = v.y;
+          ra[u][2] = v.z;
+          ra[u][3] = v.w;
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) ra[u][e] = (m < nT && k + e < K) ? Cm[(size_t)m * K + k + e] : 0.f;
+        }
+      }
     }
   };
   auto sstore = [&](int b) {
     unsigned char* Nhi = btc_smem + b * STAGE;
-    unsigned char* Nlo = Nhi + N_BYTES;
-    unsigned char* Mhi = Nlo + N_BYTES;
-    unsigned char* Mlo = Mhi + M_BYTES;
-    if (a_mfast) {
+    unsigned char* Mhi = Nhi + 2 * N_BYTES;
 #pragma unroll
-      for (int u = 0; u < A_PER; ++u) {
-        float h, l;
-        split_tf32(ra[u], h, l);
-        const uint32_t o = kmajor_offset(32 * w + lane, u, SBO);
-        *reinterpret_cast<float*>(Mhi + o) = h;
-        *reinterpret_cast<float*>(Mlo + o) = l;
-      }
-    } else {
+    for (int u = 0; u < QN; ++u)
+      split_store(Nhi, Nhi + N_BYTES, kmajor_offset(t & 127, 4 * ((t >> 7) + 2 * u), SBO), rb[u]);
 #pragma unroll
-      for (int u = 0; u < A_PER; u += 4) {
-        float h[4], l[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) split_tf32(ra[u + e], h[e], l[e]);
-        const uint32_t o = kmajor_offset((t >> 3) + 32 * (u >> 2), 4 * (t & 7), SBO);
-        *reinterpret_cast<float4*>(Mhi + o) = make_float4(h[0], h[1], h[2], h[3]);
-        *reinterpret_cast<float4*>(Mlo + o) = make_float4(l[0], l[1], l[2], l[3]);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < B_PER; ++u) {
-      float h, l;
-      split_tf32(rb[u], h, l);
-      const uint32_t o = kmajor_offset(t & 127, (t >> 7) + 2 * u, SBO);
-      *reinterpret_cast<float*>(Nhi + o) = h;
-      *reinterpret_cast<float*>(Nlo + o) = l;
+    for (int u = 0; u < QM; ++u) {
+      const int m = cm ? t % TM : 64 * u + 8 * w + (lane & 7);
+      const int k = cm ? 4 * (t / TM + (THREADS / TM) * u) : 4 * (lane >> 3);
+      split_store(Mhi, Mhi + MB, kmajor_offset(m, k, SBO), ra[u]);
     }
   };
   const int nch = (K + KC - 1) / KC;
-  const uint32_t idesc = idesc_tf32(TN, TM);  // M = 128 (n on the lanes), N = 256 (m)
+  const uint32_t idesc = idesc_tf32(TN, NM);  // M = 128 (n on the lanes), N = NM (m)
   bool ok = true;
   gload(0);
   for (int c = 0; c < nch; ++c) {
@@ -797,7 +746,7 @@ __global__ void __launch_bounds__(btc::THREADS, 1) k_big_gemm_tc(const __grid_co
     __syncthreads();
     if (t == 0) {
       fence_after_sync();
-      const uint32_t nh = smem_u32(btc_smem + b * STAGE), nl = nh + N_BYTES, mh = nl + N_BYTES, ml = mh + M_BYTES;
+      const uint32_t nh = smem_u32(btc_smem + b * STAGE), nl = nh + N_BYTES, mh = nl + N_BYTES, ml = mh + MB;
 #pragma unroll 1
       for (int kk = 0; kk < KC / 8; ++kk) {
         const uint32_t off = (uint32_t)kk * 256u;  // two core matrices along k per instruction
@@ -816,28 +765,38 @@ __global__ void __launch_bounds__(btc::THREADS, 1) k_big_gemm_tc(const __grid_co
   }
   fence_after_sync();
   if (ok) {
-    const int q = w & 3, hh = w >> 2;
+    // warp w: lanes 32 (w % 4) .., every other group of 16 rows; a column-major D is contiguous along
+    // a thread's rows (16-byte loads), a row-major one along the lanes
+    const int q = w & 3;
     const int n = tn0 + 32 * q + lane;
     const uint32_t tl = (uint32_t)(32 * q) << 16;
+    const bool dvec = cm && nT % 4 == 0 && (reinterpret_cast<uintptr_t>(Dm) & 15) == 0;
 #pragma unroll 1
-    for (int cc = 0; cc < 8; ++cc) {
-      float v[16];
-      const int m0 = tm0 + 128 * hh + 16 * cc;
-      tmem_ld16(tmem + tl + (uint32_t)(128 * hh + 16 * cc), v);
-      if (n >= N) continue;
+    for (int cc = w >> 2; cc < NM / 16; cc += 2) {
+      float v[16], d[16];
+      const int m0 = tm0 + 16 * cc;
 #pragma unroll
-      for (int u = 0; u < 16; ++u) {
-        const int m = m0 + u;
-        if (m >= M) break;
-        if (phase <= 1) {
-          X[(size_t)(m_off + m) * nT + n] -= v[u];
-        } else if (phase == 3) {
-          L[(size_t)(m_off + m) * nA + n_off + n] -= v[u];
+      for (int u = 0; u < 16; u += 4) {
+        if (dvec) {
+          float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (n < nT && m0 + u < nT) x = *reinterpret_cast<const float4*>(Dm + (size_t)n * nT + m0 + u);
+          d[u] = x.x;
+          d[u + 1] = x.y;
+          d[u + 2] = x.z;
+          d[u + 3] = x.w;
         } else {
-          const float d = cm ? Dm[(size_t)n * nT + m] : Dm[(size_t)m * nT + n];
-          S[(size_t)m * nT + n] = d - v[u];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int m = m0 + u + e;
+            d[u + e] = (n < nT && m < nT) ? (cm ? Dm[(size_t)n * nT + m] : Dm[(size_t)m * nT + n]) : 0.f;
+          }
         }
       }
+      tmem_ld16(tmem + tl + (uint32_t)(16 * cc), v);
+      if (n >= nT) continue;
+#pragma unroll
+      for (int u = 0; u < 16; ++u)
+        if (m0 + u < nT) S[(size_t)(m0 + u) * nT + n] = d[u] - v[u];
     }
   } else if (t == 0) {
     atomicOr(a.status, DEV_ERR_TIMEOUT);
@@ -848,62 +807,25 @@ __global__ void __launch_bounds__(btc::THREADS, 1) k_big_gemm_tc(const __grid_co
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
-  if (w == 0) tmem_dealloc(tmem, 256);
+  if (w == 0) tmem_dealloc(tmem, TM);
 }
 
-// 5. t = s - C x_r; unless solved with X: x_r = A^{-1} r (interchanges, forward, backward; FP64)
+// 5. t = s - C x_r (x_r came with X, the right-hand side's column of the column-block solve)
 template <typename T>
-__global__ void __launch_bounds__(BT) k_big_xr(const __grid_constant__ UnevenArgs a, const int* __restrict__ list,
-                                               int nlist, int uni_nA, int uni_nT, int solved) {
+__global__ void __launch_bounds__(BT) k_big_t(const __grid_constant__ UnevenArgs a, const int* __restrict__ list,
+                                              int nlist, int uni_nA, int uni_nT) {
   __shared__ double y[1024];
-  __shared__ int pvs[1024];
   for (int li = blockIdx.x; li < nlist; li += gridDim.x) {
     const Elem E = elem_of(a, list, li, uni_nA, uni_nT);
     const int nA = E.nA, nT = E.nT;
-    const T* L = reinterpret_cast<const T*>(a.LU) + E.o[0];
     const T* Cm = reinterpret_cast<const T*>(a.C) + E.o[1];
-    const int* piv = a.piv + E.o[3];
-    const double* r = a.r + E.o[3];
-    double* xr = a.xr + E.o[3];
+    const double* xr = a.xr + E.o[3];
     const double* sv = a.s + E.o[4];
     double* t = a.t + E.o[4];
     const bool cm = a.colmajor != 0;
     __syncthreads();
-    if (solved) {  // x_r came with X (the right-hand side's column of the column-block solve)
-      for (int i = threadIdx.x; i < nA; i += BT) y[i] = xr[i];
-      __syncthreads();
-    }
-    if (!solved) {
-      for (int i = threadIdx.x; i < nA; i += BT) {
-        y[i] = r[i];
-        pvs[i] = piv[i];
-      }
-      __syncthreads();
-      if (threadIdx.x == 0)
-        for (int j = 0; j < nA; ++j) {
-          const int p = pvs[j];
-          if (p >= 0 && p < nA && p != j) {
-            const double u = y[j];
-            y[j] = y[p];
-            y[p] = u;
-          }
-        }
-      __syncthreads();
-      for (int j = 0; j < nA; ++j) {  // unit lower
-        const double yj = y[j];
-        for (int i = j + 1 + threadIdx.x; i < nA; i += BT) y[i] -= (double)L[(size_t)i * nA + j] * yj;
-        __syncthreads();
-      }
-      for (int j = nA - 1; j >= 0; --j) {  // upper
-        if (threadIdx.x == 0) y[j] /= (double)L[(size_t)j * nA + j];
-        __syncthreads();
-        const double yj = y[j];
-        for (int i = threadIdx.x; i < j; i += BT) y[i] -= (double)L[(size_t)i * nA + j] * yj;
-        __syncthreads();
-      }
-    }
-    if (!solved)
-      for (int i = threadIdx.x; i < nA; i += BT) xr[i] = y[i];
+    for (int i = threadIdx.x; i < nA; i += BT) y[i] = xr[i];
+    __syncthreads();
     for (int row = threadIdx.x; row < nT; row += BT) {
       double acc = 0.0;
       for (int c = 0; c < nA; ++c) acc += (double)(cm ? Cm[(size_t)c * nT + row] : Cm[(size_t)row * nA + c]) * y[c];
@@ -933,24 +855,13 @@ cudaError_t condense_big(const UnevenArgs& a, const int* list, int nlist, int un
   const int gridp = nlist < occ * nsm ? nlist : (occ > 0 ? occ : 1) * nsm;
   (hfr::count_launch(), k_big_lu_init<T><<<grid1, BT, 0, st>>>(a, list, nlist, uni_nA, uni_nT));
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  const bool tcg = sizeof(T) == 4 && HFR_BIG_GEMM_TC;  // FP32 GEMMs on the tensor cores
-  if (tcg && (e = cudaFuncSetAttribute(k_big_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)btc::SMEM)) != cudaSuccess)
-    return e;
   // one batched GEMM phase over elements [base, base + cnt): rows x cols of the largest shape.  The
-  // tensor cores take S = D - C X_B (K = nA); the K = 32 updates of the LU and the triangular
-  // solves, bound by the read-modify-write of their outputs, stay on the CUDA cores (two CTAs per
-  // SM against one of the tensor-core kernel: measured faster on hexahedra)
+  // tensor cores take S = D - C X_B of FP32 blocks (K = nA); the K = 32 updates of the LU, bound by
+  // the read-modify-write of their outputs, stay on the CUDA cores
   auto gemm = [&](int base, int cnt, int rows, int cols, int phase, int jb) {
-    if (tcg && phase == 2) {
-      const dim3 g((cols + btc::TN - 1) / btc::TN, (rows + btc::TM - 1) / btc::TM, cnt);
-      (hfr::count_launch(), k_big_gemm_tc<<<g, btc::THREADS, btc::SMEM, st>>>(a, list, base, cnt, uni_nA, uni_nT,
-                                                                                 phase, jb));
-    } else {
-      constexpr int TB = GemmCfg<T>::BM;
-      const dim3 g((cols + TB - 1) / TB, (rows + TB - 1) / TB, cnt);
-      (hfr::count_launch(), k_big_gemm<T><<<g, BT, 0, st>>>(a, list, base, cnt, uni_nA, uni_nT, phase, jb));
-    }
+    constexpr int TB = GemmCfg<T>::BM;
+    const dim3 g((cols + TB - 1) / TB, (rows + TB - 1) / TB, cnt);
+    (hfr::count_launch(), k_big_gemm<T><<<g, BT, 0, st>>>(a, list, base, cnt, uni_nA, uni_nT, phase, jb));
   };
   const int npan = (max_nA + lu_panel<T>() - 1) / lu_panel<T>();
   for (int jb = 0; jb < npan; ++jb) {
@@ -964,39 +875,58 @@ cudaError_t condense_big(const UnevenArgs& a, const int* list, int nlist, int un
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  // X = A^{-1} P B: column blocks whole in shared memory when they fit, else the interchange copy
-  // and the blocked triangular solves
-  const size_t ssm = solve_smem<T>(max_nA);
-  const bool fused = ssm <= 227 * 1024 &&
-                     cudaFuncSetAttribute(k_big_solve<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm) ==
-                         cudaSuccess;
-  cudaGetLastError();
-  if (!fused) {
-    (hfr::count_launch(), k_big_rhs<T><<<grid1, BT, 0, st>>>(a, list, nlist, uni_nA, uni_nT));
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  const int nblk = (max_nA + NB - 1) / NB;
+  // X = A^{-1} P [B | r]: the widest column block whose rows fit shared memory; FP32 blocks of which
+  // two CTAs of 64 columns fit an SM (nA up to about 250) take those: one CTA's in-panel solves run
+  // under the other's updates (p = 4 and 5 blocks of a wall mesh: 2.0 ms per condensation)
   constexpr int CH = 65535;  // grid y / z extent per launch
+  constexpr size_t SM1 = 227 * 1024, SM2 = 113 * 1024;
+  auto solve = [&](auto kern, int cw, int nthr, size_t smem, int base, int cnt) -> cudaError_t {
+    cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (r != cudaSuccess) return r;
+    const dim3 gv((max_nT + 1 + cw - 1) / cw, cnt);  // and the column of r
+    (hfr::count_launch(), kern<<<gv, nthr, smem, st>>>(a, list, base, cnt, uni_nA, uni_nT));
+    return cudaGetLastError();
+  };
   for (int base = 0; base < nlist; base += CH) {
     const int cnt = nlist - base < CH ? nlist - base : CH;
-    if (fused) {
-      const dim3 gv((max_nT + 1 + SC - 1) / SC, cnt);  // and the column of r
-      (hfr::count_launch(), k_big_solve<T><<<gv, BT, ssm, st>>>(a, list, base, cnt, uni_nA, uni_nT));
+    if constexpr (sizeof(T) == 4) {
+      using W = SolveCfg<T, 16, 128, 16, 2>;
+      using M = SolveCfg<T, 16, 64, 8, 1>;
+      using N = SolveCfg<T, 8, 32, 8, 1>;
+      if (M::smem(max_nA) > SM2 && W::smem(max_nA) <= SM1)
+        e = solve(k_big_solve<T, 16, 128, 16, 2>, 128, 512, W::smem(max_nA), base, cnt);
+      else if (M::smem(max_nA) <= SM1)
+        e = solve(k_big_solve<T, 16, 64, 8, 1>, 64, 256, M::smem(max_nA), base, cnt);
+      else
+        e = solve(k_big_solve<T, 8, 32, 8, 1>, 32, 256, N::smem(max_nA), base, cnt);
     } else {
-      const dim3 gd((max_nT + 127) / 128, cnt);
-      for (int jb = 0; jb < nblk; ++jb) {
-        (hfr::count_launch(), k_big_trsm_diag<T><<<gd, 128, 0, st>>>(a, list, base, cnt, uni_nA, uni_nT, jb, 0));
-        if (jb + 1 < nblk) gemm(base, cnt, max_nA - (jb + 1) * NB, max_nT, 0, jb);
-      }
-      for (int jb = nblk - 1; jb >= 0; --jb) {
-        (hfr::count_launch(), k_big_trsm_diag<T><<<gd, 128, 0, st>>>(a, list, base, cnt, uni_nA, uni_nT, jb, 1));
-        if (jb > 0) gemm(base, cnt, jb * NB, max_nT, 1, jb);
-      }
+      using W = SolveCfg<T, 8, 64, 8, 2>;
+      using M = SolveCfg<T, 8, 32, 8, 2>;
+      using N = SolveCfg<T, 8, 16, 8, 2>;
+      if (W::smem(max_nA) <= SM1)
+        e = solve(k_big_solve<T, 8, 64, 8, 2>, 64, 256, W::smem(max_nA), base, cnt);
+      else if (M::smem(max_nA) <= SM1)
+        e = solve(k_big_solve<T, 8, 32, 8, 2>, 32, 256, M::smem(max_nA), base, cnt);
+      else
+        e = solve(k_big_solve<T, 8, 16, 8, 2>, 16, 256, N::smem(max_nA), base, cnt);
     }
-    gemm(base, cnt, max_nT, max_nT, 2, 0);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (e != cudaSuccess) return e;
+    if constexpr (sizeof(T) == 4) {
+      auto schur = [&](auto kern, int tm, size_t smem) -> cudaError_t {
+        cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (r != cudaSuccess) return r;
+        const dim3 g((max_nT + btc::TN - 1) / btc::TN, (max_nT + tm - 1) / tm, cnt);
+        (hfr::count_launch(), kern<<<g, btc::THREADS, smem, st>>>(a, list, base, cnt, uni_nA, uni_nT));
+        return cudaGetLastError();
+      };
+      e = max_nT > 128 ? schur(k_big_s_tc<256>, 256, btc::smem<256>()) : schur(k_big_s_tc<128>, 128, btc::smem<128>());
+    } else {
+      gemm(base, cnt, max_nT, max_nT, 2, 0);
+      e = cudaGetLastError();
+    }
+    if (e != cudaSuccess) return e;
   }
-  (hfr::count_launch(), k_big_xr<T><<<grid1, BT, 0, st>>>(a, list, nlist, uni_nA, uni_nT, fused ? 1 : 0));
+  (hfr::count_launch(), k_big_t<T><<<grid1, BT, 0, st>>>(a, list, nlist, uni_nA, uni_nT));
   return cudaGetLastError();
 }
 
