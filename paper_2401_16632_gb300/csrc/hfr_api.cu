@@ -79,7 +79,7 @@ struct fr_ctx {
   unsigned char* implicit = nullptr;
   int *sides_e = nullptr, *sides_c = nullptr, *imp_idx = nullptr, *tr_of_c = nullptr;
   // residual workspace
-  double *Uf_all = nullptr, *qf_all = nullptr, *Rw = nullptr, *gview = nullptr, *gw = nullptr;
+  double *Uf_all = nullptr, *qf_all = nullptr, *q_all = nullptr, *Rw = nullptr, *gview = nullptr, *gw = nullptr;
   double *dUw = nullptr, *dRw = nullptr, *dgview = nullptr;
   // Newton system
   double *r = nullptr, *s = nullptr, *xr = nullptr, *te = nullptr, *tg = nullptr, *Pinv = nullptr;
@@ -576,6 +576,7 @@ extern "C" int fr_ctx_create(const fr_mesh_desc* mesh, const fr_config* cfg, voi
   if (ctx->need_nbr) {
     ctx->Uf_all = dalloc<double>(ctx, (size_t)E * NF * nv, &rc);
     ctx->qf_all = dalloc<double>(ctx, (size_t)E * NF * 2 * nv, &rc);
+    ctx->q_all = dalloc<double>(ctx, (size_t)E * ns * 2 * nv, &rc);
   }
   ctx->Rw = dalloc<double>(ctx, (size_t)E * nA, &rc);
   ctx->gview = dalloc<double>(ctx, (size_t)E * NF * nv, &rc);
@@ -742,6 +743,7 @@ static ResArgs res_args(fr_ctx* ctx, const double* u, const double* uhat) {
   a.qf_all = ctx->qf_all;
   a.Uf_out = ctx->Uf_all;
   a.qf_out = ctx->qf_all;
+  a.q_out = ctx->q_all;
   a.ntrace = ctx->ntrace;
   return a;
 }

@@ -144,6 +144,19 @@ template <> struct Phys<0> {
   __device__ static S stab(const PhysConst<R>& pc, const S* u, R n0, R n1) {
     return wave<S, R>(pc, u, n0, n1) + pc.nu_lref;
   }
+  // normal components F.n of both fluxes and the wave speed, without the tangential components
+  template <typename S, typename R>
+  __device__ static void conv_n(const PhysConst<R>& pc, const S* u, R n0, R n1, S F[1], S& wave) {
+    const R bn = pc.beta0 * n0 + pc.beta1 * n1;
+    F[0] = bn * u[0];
+    wave = S(dabs(bn));
+  }
+  template <typename S, typename R>
+  __device__ static S stab_n(const PhysConst<R>& pc, const S*, const S& wave) { return wave + pc.nu_lref; }
+  template <typename S, typename R>
+  __device__ static void visc_n(const PhysConst<R>& pc, const S*, const S q[2][1], R n0, R n1, S F[1]) {
+    F[0] = pc.nu * (n0 * q[0][0] + n1 * q[1][0]);
+  }
 };
 
 template <> struct Phys<1> {
@@ -204,6 +217,42 @@ template <> struct Phys<1> {
   __device__ static S stab(const PhysConst<R>& pc, const S* u, R n0, R n1) {
     return wave<S, R>(pc, u, n0, n1) + pc.mu_lref / u[0];
   }
+  template <typename S, typename R>
+  __device__ static void conv_n(const PhysConst<R>& pc, const S* u, R n0, R n1, S F[4], S& wave) {
+    const S ir = R(1) / u[0];
+    const S mn = u[1] * n0 + u[2] * n1;
+    const S vn = mn * ir;
+    const S p = pc.gm1 * (u[3] - R(0.5) * (u[1] * u[1] + u[2] * u[2]) * ir);
+    F[0] = mn;
+    F[1] = u[1] * vn + p * n0;
+    F[2] = u[2] * vn + p * n1;
+    F[3] = (u[3] + p) * vn;
+    wave = dabs(vn) + dsqrt(pc.gamma * p * ir);
+  }
+  template <typename S, typename R>
+  __device__ static S stab_n(const PhysConst<R>& pc, const S* u, const S& wave) {
+    return wave + pc.mu_lref * (R(1) / u[0]);
+  }
+  template <typename S, typename R>
+  __device__ static void visc_n(const PhysConst<R>& pc, const S* u, const S q[2][4], R n0, R n1, S F[4]) {
+    const S ir = R(1) / u[0];
+    const S vx = u[1] * ir, vy = u[2] * ir, e = u[3] * ir;
+    S dvx[2], dvy[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      dvx[c] = (q[c][1] - vx * q[c][0]) * ir;
+      dvy[c] = (q[c][2] - vy * q[c][0]) * ir;
+    }
+    // n . grad T from the normal derivatives
+    const S q0n = n0 * q[0][0] + n1 * q[1][0], q3n = n0 * q[0][3] + n1 * q[1][3];
+    const S dTn = pc.gm1 * ((q3n - e * q0n) * ir - vx * (n0 * dvx[0] + n1 * dvx[1]) - vy * (n0 * dvy[0] + n1 * dvy[1]));
+    const S dil = R(2.0 / 3.0) * (dvx[0] + dvy[1]);
+    const S txx = pc.mu * (R(2) * dvx[0] - dil), tyy = pc.mu * (R(2) * dvy[1] - dil), txy = pc.mu * (dvx[1] + dvy[0]);
+    F[0] = S(R(0));
+    F[1] = n0 * txx + n1 * txy;
+    F[2] = n0 * txy + n1 * tyy;
+    F[3] = vx * F[1] + vy * F[2] + pc.kappa * dTn;
+  }
 };
 
 // EDAC (Appendix A): u = (P, v_x, v_y), F^c_i = (v_i (P + Theta), v_i v_x + P delta_ix,
@@ -238,6 +287,24 @@ template <> struct Phys<2> {
   __device__ static S stab(const PhysConst<R>& pc, const S* u, R n0, R n1) {
     const S v2 = u[1] * u[1] + u[2] * u[2];
     return R(1.5) * dsqrt(v2) + dsqrt(R(0.25) * v2 + u[0] + pc.theta) + pc.nu_lref;
+  }
+  template <typename S, typename R>
+  __device__ static void conv_n(const PhysConst<R>& pc, const S* u, R n0, R n1, S F[3], S& wave) {
+    const S vn = u[1] * n0 + u[2] * n1;
+    F[0] = vn * (u[0] + pc.theta);
+    F[1] = u[1] * vn + u[0] * n0;
+    F[2] = u[2] * vn + u[0] * n1;
+    wave = R(1.5) * dabs(vn) + dsqrt(R(0.25) * vn * vn + u[0] + pc.theta);
+  }
+  template <typename S, typename R>
+  __device__ static S stab_n(const PhysConst<R>& pc, const S* u, const S&) {
+    const S v2 = u[1] * u[1] + u[2] * u[2];
+    return R(1.5) * dsqrt(v2) + dsqrt(R(0.25) * v2 + u[0] + pc.theta) + pc.nu_lref;
+  }
+  template <typename S, typename R>
+  __device__ static void visc_n(const PhysConst<R>& pc, const S*, const S q[2][3], R n0, R n1, S F[3]) {
+#pragma unroll
+    for (int v = 0; v < 3; ++v) F[v] = pc.nu * (n0 * q[0][v] + n1 * q[1][v]);
   }
 };
 

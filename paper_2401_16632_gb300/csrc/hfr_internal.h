@@ -63,6 +63,7 @@ struct ResArgs {
   const double* qf_all;  // neighbour face gradients (read)
   double* Uf_out;        // MODE_UF output
   double* qf_out;        // MODE_QF output
+  double* q_out;         // MODE_QF output: gradients of the solution points (read by MODE_RESQ)
   double* R;             // nullable
   double* dR;            // nullable (JVP)
   double* gview;         // nullable: w_q J_f F^.n on trace faces
