@@ -239,7 +239,10 @@ int imex_refresh_jacobian(fr_ctx* ctx);
  * available for trace blocks (nT, n nv) = (64,16), (80,20), (48,12) on devices with cooperative
  * launch.  Each barrier wait is bounded (about 2 s); a wait that runs out ends the launch and
  * hfr_trace_gmres returns FR_ERR_TIMEOUT.  FR_GMRES_MULTI: one short kernel per step with the
- * Krylov state on the device (any shape).  Both compute the same iteration (classical
+ * Krylov state on the device (any shape).  Contexts without the fixed-shape cycle (other trace
+ * blocks, general meshes) report FR_GMRES_MULTI and until it is set explicitly run each restart
+ * cycle as one launch as well (FP64 basis; bounded barriers, or one thread-block cluster for
+ * systems of a few thousand values); setting it gives the short kernels.  Both compute the same iteration (classical
  * Gram-Schmidt with a conditional second pass); their results agree to rounding.
  * set: FR_ERR_UNSUPPORTED if FR_GMRES_FUSED is not available for the context.
  * get: the mode in effect, -1 for a null context.  This switch has no counterpart in the paper. */

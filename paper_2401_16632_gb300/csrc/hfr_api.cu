@@ -90,6 +90,9 @@ struct fr_ctx {
   // Krylov
   GmresBuffers gm;
   int gm_mode = 0;          // 0: multi-kernel cycle, 1: one cooperative launch per cycle
+  CyclePlan plan;           // shapes without a compiled cycle: the single launch of any layout (grid 0: none)
+  int short_kernels = 0;    // FR_GMRES_MULTI asked for: one kernel per step on those shapes too
+  double* yv = nullptr;     // its element view
   int jac_policy = 0;       // fr_jacobian_policy
   // condensation held for FR_JAC_KEEP: valid, for which a_ii dt, refresh asked by the caller
   int keep_valid = 0;
@@ -403,6 +406,35 @@ __global__ void k_initial_trace(int ntrace, int npf, int NF_npf, const int* __re
 
 static inline unsigned nblk(size_t n, int t = 256) { return (unsigned)((n + t - 1) / t); }
 
+// the single-launch GMRES cycle of any layout on this context
+static CycleArgs cycle_args(fr_ctx* ctx) {
+  CycleArgs a;
+  memset(static_cast<void*>(&a), 0, sizeof(a));
+  a.Eim = ctx->Eim;
+  a.ntrace = ctx->ntrace;
+  a.nv = ctx->nv;
+  a.uni_nT = ctx->nT;
+  a.uni_bs = ctx->n * ctx->nv;
+  a.tr_of_c = ctx->tr_of_c;
+  a.sides = ctx->sides_c;
+  a.sumTT = (long long)ctx->Eim * ctx->nT * ctx->nT;
+  a.bsmax = a.uni_bs;
+  a.S = ctx->S;
+  a.Pinv = ctx->Pinv;
+  a.t = ctx->tg;
+  a.x = ctx->duhat;
+  a.V = ctx->gm.V;
+  a.Z = ctx->gm.Z;
+  a.yv = ctx->yv;
+  a.partial = ctx->gm.partial;
+  a.bar = ctx->gm_bar;
+  a.st = ctx->gm.state;
+  a.n = ctx->gm.n;
+  a.m = ctx->restart;
+  a.x_zero = 1;
+  return a;
+}
+
 // ------------------------------------------------------------------------ context
 extern "C" int fr_ctx_create(const fr_mesh_desc* mesh, const fr_config* cfg, void* stream, fr_ctx** out) {
   FR_NVTX("fr_ctx_create");
@@ -618,6 +650,10 @@ extern "C" int fr_ctx_create(const fr_mesh_desc* mesh, const fr_config* cfg, voi
     const size_t np = std::max((size_t)GM_NBLK * (GM_MAXM + 1), fused_partial_doubles(std::max(nsm, 1)));
     ctx->gm.partial = dalloc<double>(ctx, np, &rc);
     ctx->gm_bar = dalloc<unsigned>(ctx, 64, &rc);
+    if (ctx->gm_fused_grid <= 0) {
+      ctx->yv = dalloc<double>(ctx, (size_t)Eim * nT, &rc);
+      ctx->plan = cycle_plan(ctx->prec_bytes, cycle_args(ctx));
+    }
   }
   ctx->gm.state = dalloc<GmresState>(ctx, 1, &rc);
   ctx->sdev = dalloc<StageDev>(ctx, 1, &rc);
@@ -1086,7 +1122,14 @@ static int gmres_impl(fr_ctx* ctx, double* duhat, double rtol, int maxit, int* i
     grc = run_gmres_fused(fa, ctx->prec_bytes, ctx->gm_fused_grid, rtol, ctx->restart, maxit, &res, &timed_out,
                           ctx->stream, cond_status ? ctx->status : nullptr, cond_status);
   } else {
-    grc = run_gmres(ops, ctx->gm, ctx->tg, duhat, rtol, ctx->restart, maxit, 4, &res, ctx->stream);
+    if (ctx->plan.grid > 0 && !ctx->short_kernels) {
+      CycleArgs a = cycle_args(ctx);
+      a.x = duhat;
+      grc = run_gmres_any(a, ctx->prec_bytes, ctx->plan, rtol, ctx->restart, maxit, true_res, &res, &timed_out,
+                          ctx->stream);
+    } else {
+      grc = run_gmres(ops, ctx->gm, ctx->tg, duhat, rtol, ctx->restart, maxit, 4, &res, ctx->stream);
+    }
     if (grc == 0 && cond_status) {
       CK(cudaMemcpyAsync(cond_status, ctx->status, 2 * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
       CK(cudaStreamSynchronize(ctx->stream));
@@ -1120,13 +1163,17 @@ extern "C" int imex_refresh_jacobian(fr_ctx* ctx) {
 }
 
 extern "C" int hfr_gmres_set_mode(fr_ctx* ctx, int mode) {
-  if (ctx && ctx->gen && mode == FR_GMRES_MULTI) return FR_OK;
+  if (ctx && ctx->gen && mode == FR_GMRES_MULTI) {
+    hfr::gen::set_short_kernels(ctx->gen);
+    return FR_OK;
+  }
   NOT_GENERAL(ctx, "hfr_gmres_set_mode (single-launch cycle)");
   if (!ctx || (mode != FR_GMRES_MULTI && mode != FR_GMRES_FUSED))
     return set_err(ctx, FR_ERR_INVALID_ARG, "hfr_gmres_set_mode: bad argument");
   if (mode == FR_GMRES_FUSED && ctx->gm_fused_grid <= 0)
     return set_err(ctx, FR_ERR_UNSUPPORTED, "hfr_gmres_set_mode: no single-launch cycle for this shape or device");
   ctx->gm_mode = mode;
+  if (mode == FR_GMRES_MULTI) ctx->short_kernels = 1;
   return FR_OK;
 }
 

@@ -1419,6 +1419,41 @@ void destroy(GenCtx* g) {
   delete g;
 }
 
+// the single-launch GMRES cycle's view of the context
+static CycleArgs cycle_args(GenCtx* g) {
+  CycleArgs a;
+  a.Eim = g->Eim;
+  a.ntrace = g->ntrace;
+  a.nv = g->nv;
+  a.nTk = g->nTk;
+  a.offD = g->offD;
+  a.offs = g->offs;
+  a.gmap = g->gmap;
+  a.vptr = g->vptr;
+  a.vidx = g->vidx;
+  a.tpts = g->tpts;
+  a.toff = g->toff;
+  a.poff = g->poff;
+  a.sumTT = (long long)g->sumTT;
+  a.bsmax = g->bsmax;
+  a.S = g->S;
+  a.Pinv = g->Pinv;
+  a.t = g->tg;
+  a.x = g->duhat;
+  a.V = g->gm.V;
+  a.Z = g->gm.Z;
+  a.yv = g->yv;
+  a.partial = g->gm.partial;
+  a.bar = g->gm_bar;
+  a.st = g->gm.state;
+  a.n = g->nh;
+  a.m = g->restart;
+  a.rtol = 0.0;
+  a.x_zero = 1;
+  a.true_res = 0;
+  return a;
+}
+
 int create(const fr_mesh_desc* mesh, const fr_config* cfg, cudaStream_t st, const Hooks& hooks, GenCtx** out) {
   *out = nullptr;
   const int E = mesh->nelem;
@@ -1838,6 +1873,7 @@ int create(const fr_mesh_desc* mesh, const fr_config* cfg, cudaStream_t st, cons
   g->gm.partial = galloc<double>(g, (size_t)GM_NBLK * (GM_MAXM + 1), &rc);
   g->gm.ticket = galloc<unsigned int>(g, 1, &rc);
   g->gm.state = galloc<GmresState>(g, 1, &rc);
+  g->gm_bar = galloc<unsigned>(g, 64, &rc);
   if (hex && Eim > 0) {
     g->jgrid = std::min(hex_jacobian_grid((int)pb), Eim);
     g->jscratch = galloc<unsigned char>(g, hex_jacobian_scratch_bytes((int)pb, g->jgrid), &rc);
@@ -1941,6 +1977,7 @@ int create(const fr_mesh_desc* mesh, const fr_config* cfg, cudaStream_t st, cons
   }
   g->h_uoff = uoff;
   g->h_toff = toff;
+  g->plan = cycle_plan(g->pb, cycle_args(g));
   *out = g;
   return FR_OK;
 }
@@ -2299,7 +2336,9 @@ static void cb_precond_g(void* c, const GmresState* st, int j, double* x, double
          j > 0 ? &st->inv_hn : nullptr, y32));
 }
 
-static int gmres_impl(GenCtx* g, double* duhat, double rtol, int maxit, int* iters, double* final_rel) {
+// true_res: report the true final residual (the Newton iteration does not need it)
+static int gmres_impl(GenCtx* g, double* duhat, double rtol, int maxit, int* iters, double* final_rel,
+                      bool true_res = true) {
   if (g->ntrace == 0) {
     if (iters) *iters = 0;
     if (final_rel) *final_rel = 0.0;
@@ -2313,8 +2352,17 @@ static int gmres_impl(GenCtx* g, double* duhat, double rtol, int maxit, int* ite
   GmresResult res;
   memset(&res, 0, sizeof(res));
   const int ph = pbeg(g, 4);
-  const int grc = run_gmres(ops, g->gm, g->tg, duhat, rtol, g->restart, maxit, 4, &res, g->st);
+  int grc = 0, timed_out = 0;
+  if (g->plan.grid > 0 && !g->short_kernels && maxit >= 1) {
+    CycleArgs a = cycle_args(g);
+    a.x = duhat;
+    grc = run_gmres_any(a, g->pb, g->plan, rtol, g->restart, maxit, true_res, &res, &timed_out, g->st);
+  } else {
+    grc = run_gmres(ops, g->gm, g->tg, duhat, rtol, g->restart, maxit, 4, &res, g->st);
+  }
   pend(g, ph);
+  if (timed_out)
+    return err(g, FR_ERR_TIMEOUT, "hfr_trace_gmres: grid barrier wait timed out", -1, res.iterations);
   if (grc != 0) return err(g, FR_ERR_CUDA, cudaGetErrorString(cudaGetLastError()));
   GCK(cudaGetLastError());
   if (iters) *iters = res.iterations;
@@ -2473,6 +2521,12 @@ __global__ void k_gs_gmres_done(GStageDev* sd, const GmresGraphDev* gd) {
   sd->gtot += gd->total;
   sd->cycles += gd->cycles;
   if (gd->nan) sd->err |= 2;
+  if (gd->timeout) sd->err |= 4;
+}
+
+void set_short_kernels(GenCtx* g) {
+  g->short_kernels = 1;
+  g->gvalid = false;
 }
 
 int set_graph(GenCtx* g, int on) {
@@ -2583,7 +2637,10 @@ static int stage_graph_capture(GenCtx* g, const GenCtx::GKey& key) {
     ops.precond = cb_precond_g;
     const cudaStream_t sc[2] = {g->cap[3], g->cap[4]};
     lg0 = launch_count();
-    SK(capture_gmres(ops, g->gm, g->tg, g->duhat, key.grtol, g->restart, key.gmax, gd, g->st, sc, &g->gl_gm));
+    if (g->plan.grid > 0 && !g->short_kernels && key.gmax >= 1)
+      SK(capture_gmres_any(cycle_args(g), g->pb, g->plan, key.grtol, g->restart, key.gmax, gd, g->st, sc[0], &g->gl_gm));
+    else
+      SK(capture_gmres(ops, g->gm, g->tg, g->duhat, key.grtol, g->restart, key.gmax, gd, g->st, sc, &g->gl_gm));
     lg1 = launch_count();
     (count_launch(), k_gs_gmres_done<<<1, 1, 0, g->st>>>(sd, gd));
     SK(cudaGetLastError());
@@ -2665,6 +2722,7 @@ static int stage_graph(GenCtx* g, const GenCtx::GKey& key, fr_stage_stats* stats
     GCK(cudaStreamSynchronize(st));
     return err(g, FR_ERR_SINGULAR, "imex_stage: zero pivot in condensation", h.sing >= 0 ? h.sing : -1, h.it);
   }
+  if (h.err & 4) return err(g, FR_ERR_TIMEOUT, "imex_stage: a bounded device wait timed out", -1, h.it);
   if (h.err & 1) return err(g, FR_ERR_DIVERGED, "imex_stage: non-finite Newton residual", -1, h.it);
   if (h.err & 2) return err(g, FR_ERR_DIVERGED, "imex_stage: non-finite GMRES residual", -1, h.it);
   if (!h.conv) return err(g, FR_ERR_NOT_CONVERGED, "imex_stage: Newton iteration limit", -1, h.it, h.norm);
@@ -2755,7 +2813,7 @@ int stage(GenCtx* g, int stage, double dt, const double* u_n, double* u_stage, d
     if (rc) return rc;
     int its = 0;
     double rel = 0.0;
-    rc = gmres_impl(g, g->duhat, gmres_rtol, gmres_maxit, &its, &rel);
+    rc = gmres_impl(g, g->duhat, gmres_rtol, gmres_maxit, &its, &rel, false);
     gtot += its;
     if (rc && rc != FR_ERR_NOT_CONVERGED) return rc;
     rc = backsolve_impl(g, g->duhat, g->du);

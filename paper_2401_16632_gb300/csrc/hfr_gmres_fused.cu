@@ -213,6 +213,70 @@ __host__ __device__ constexpr int pg_basis_width() {
   return BS % (16 / (int)sizeof(T)) == 0 ? 16 / (int)sizeof(T) : 1;
 }
 
+// The FP64 form of the dot pass below.  Every FP64 instruction of a warp occupies the SM's FP64 pipe
+// for about 19 cycles, whatever its lanes hold, so the pass spends them on products alone: one
+// multiply-add per value and basis vector (sixteen vectors at a time, their loads in flight
+// together), a lane reduction sized to the vectors left, and none in warps without entries.  The
+// paired form that FP32 uses cost half as many again in separate products, and as many lanes of the
+// last step (459 000 values, 16 vectors: 40 us against 25).  Entries are visited as the updates of this file do.
+__device__ __forceinline__ double pg_lane_sum16(double (&acc)[16], int cnt, int lane) {
+  // butterfly over the lane bits 4 .. 1 (each level halves the values a lane carries), then bit 0:
+  // lane l ends with the warp sum of value l >> 1; levels whose upper half is empty only add
+  double v8[8], v4[4], v2[2];
+  const bool u4 = lane & 16, u3 = lane & 8, u2 = lane & 4, u1 = lane & 2;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const double send = u4 ? acc[q] : acc[q + 8], keep = u4 ? acc[q + 8] : acc[q];
+    v8[q] = q < cnt ? keep + __shfl_xor_sync(0xffffffffu, send, 16) : 0.0;
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const double send = u3 ? v8[q] : v8[q + 4], keep = u3 ? v8[q + 4] : v8[q];
+    v4[q] = q < cnt ? keep + __shfl_xor_sync(0xffffffffu, send, 8) : 0.0;
+  }
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const double send = u2 ? v4[q] : v4[q + 2], keep = u2 ? v4[q + 2] : v4[q];
+    v2[q] = q < cnt ? keep + __shfl_xor_sync(0xffffffffu, send, 4) : 0.0;
+  }
+  const double send = u1 ? v2[0] : v2[1], keep = u1 ? v2[1] : v2[0];
+  const double r = keep + __shfl_xor_sync(0xffffffffu, send, 2);
+  return r + __shfl_xor_sync(0xffffffffu, r, 1);
+}
+__device__ void pg_block_dots64(PGShared<double>& sh, const double* V, size_t n, int nd, const double* w, size_t x0,
+                                size_t x1, double* partial) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const size_t nw = (x1 - x0 + 31) / 32;
+  const int active = nw < PG_WARPS ? (int)nw : PG_WARPS;  // warps with entries
+  if (wid < active) {
+    for (int c0 = 0; c0 < nd; c0 += 16) {
+      const int cnt = min(16, nd - c0);
+      double acc[16];
+#pragma unroll
+      for (int q = 0; q < 16; ++q) acc[q] = 0.0;
+      for (size_t x = x0 + threadIdx.x; x < x1; x += PG_THREADS) {
+        const double wx = w[x];
+        double v[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q)
+          if (q < cnt) v[q] = V[(size_t)(c0 + q) * n + x];
+#pragma unroll
+        for (int q = 0; q < 16; ++q)
+          if (q < cnt) acc[q] = fma(v[q], wx, acc[q]);
+      }
+      const double s = pg_lane_sum16(acc, cnt, lane);
+      const int vi = c0 + (lane >> 1);
+      if ((lane & 1) == 0 && vi < nd) sh.red[vi][wid] = s;
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < nd; i += PG_THREADS) {
+    double t = 0.0;
+    for (int k = 0; k < active; ++k) t += sh.red[i][k];
+    partial[(size_t)i * gridDim.x + blockIdx.x] = t;
+  }
+}
+
 // CTA partial of V_i . w over this CTA's entries [x0, x1), i < nd, written to
 // partial[i * gridDim.x + blockIdx.x].  Each thread visits the entries x0 + tid + PG_THREADS u,
 // the same ones the vector updates of this file give it, so it only re-reads its own writes.
@@ -224,7 +288,9 @@ template <typename T, int W = 1>
 __device__ void pg_block_dots(PGShared<T>& sh, const T* V, size_t n, int nd, const T* w, size_t x0, size_t x1,
                               T* partial) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if constexpr (W > 1) {
+  if constexpr (sizeof(T) == 8) {
+    pg_block_dots64(sh, V, n, nd, w, x0, x1, partial);
+  } else if constexpr (W > 1) {
     const size_t g0 = x0 / W, g1 = x1 / W, nW = n / W;
     for (int c0 = 0; c0 < nd; c0 += PG_VC) {
       T acc[8];
@@ -435,6 +501,24 @@ __device__ __forceinline__ PGVec<T, VW> pg_ld_cg(const T* ptr) {
   return r;
 }
 
+// VW consecutive values that are not written during the kernel (16-byte vectors)
+template <typename T, int VW>
+__device__ __forceinline__ PGVec<T, VW> pg_ld_stream(const T* ptr) {
+  PGVec<T, VW> r;
+  if constexpr (sizeof(T) == 4) {
+    const float4 q = __ldg(reinterpret_cast<const float4*>(ptr));
+    r.v[0] = q.x;
+    r.v[1] = q.y;
+    r.v[2] = q.z;
+    r.v[3] = q.w;
+  } else {
+    const double2 q = __ldg(reinterpret_cast<const double2*>(ptr));
+    r.v[0] = q.x;
+    r.v[1] = q.y;
+  }
+  return r;
+}
+
 // widest vector (16 bytes at most) that divides both the per-lane column count and the face block
 template <typename T, int NT, int BS>
 struct PGShape {
@@ -607,6 +691,24 @@ template <typename T>
 __device__ __forceinline__ void pg_axpy_multi(const T* V, size_t n, const T* c, int cnt, T* dst, T scale,
                                               size_t x0, size_t x1, int tid0, int nthreads) {
   const size_t st = (size_t)nthreads;
+  if constexpr (sizeof(T) == 8) {  // one multiply-add per value and vector (see the FP64 dot pass)
+    for (size_t x = x0 + tid0; x < x1; x += st) {
+      T s0 = T(0), s1 = T(0);
+      int i = 0;
+      for (; i + 8 <= cnt; i += 8) {
+        T v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = V[(size_t)(i + u) * n + x];
+#pragma unroll
+        for (int u = 0; u < 8; u += 2) {
+          s0 = fma(c[i + u], v[u], s0);
+          s1 = fma(c[i + u + 1], v[u + 1], s1);
+        }
+      }
+      for (; i < cnt; ++i) s0 = fma(c[i], V[(size_t)i * n + x], s0);
+      dst[x] = (dst[x] - (s0 + s1)) * scale;
+    }
+  } else {
   for (size_t xb = x0 + tid0; xb < x1; xb += 4 * st) {
     size_t xs[4];
     bool ok[4];
@@ -635,6 +737,7 @@ __device__ __forceinline__ void pg_axpy_multi(const T* V, size_t n, const T* c, 
 #pragma unroll
     for (int u = 0; u < 4; ++u)
       if (ok[u]) dst[xs[u]] = (dst[xs[u]] - sacc[u]) * scale;
+  }
   }
 }
 
@@ -878,6 +981,519 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_gmres_cycle(const __grid_cons
   }
 }
 
+// ------------------------------------------------------- the cycle on any trace layout
+// The same iteration with an FP64 basis, for trace units of any size and element blocks of any shape
+// (mixed degrees, hexahedra, EFR nodes, uniform shapes without a compiled cycle).  The operator runs
+// in the element view, which adds one barrier: (A) z = P^-1 v_j; (B) y_k = S_k z_k; (C) w = the sum of
+// the element entries, h = V^T w; (D) w' = w - V h, d = V^T w', ||w'||.  Z keeps P^-1 v_j, so x
+// moves by sum y_j z_j with the very vectors that the operator saw.
+//
+// What bounds it: the S blocks from HBM in (B), the FP64 pipe in (C), (D) and the deferred second
+// pass (4 (j + 1) n multiply-adds per iteration).  The S values are cut into equal runs of rows, one
+// per warp of the grid, whatever the element shapes.  As one kernel per step (seven launches per
+// iteration, two of them reductions that ended in one block reading every partial sum and updating
+// the rotations from global memory) an iteration cost 280 us on EFR nodes (128 x 128, p = 4), 290 us
+// on a wall mesh of 10 000 implicit elements and 70 us on 64 scalar elements; it takes 230, 155
+// and 22 us.
+// Systems of a few thousand values run on one cluster of eight CTAs, whose barrier is hardware.
+
+struct AnyShape {  // the layout of one element or trace unit, from the tables or the uniform sizes
+  const CycleArgs& a;
+  __device__ __forceinline__ int nT(int k) const { return a.uni_nT ? a.uni_nT : __ldg(a.nTk + k); }
+  __device__ __forceinline__ long long offD(int k) const {
+    return a.uni_nT ? (long long)k * a.uni_nT * a.uni_nT : __ldg(a.offD + k);
+  }
+  __device__ __forceinline__ long long offs(int k) const {
+    return a.uni_nT ? (long long)k * a.uni_nT : __ldg(a.offs + k);
+  }
+  // trace value of local unknown l of element k (its entries start at o), -1 off traces
+  __device__ __forceinline__ long long gmap(int k, long long o, int l) const {
+    if (!a.uni_nT) return __ldg(a.gmap + o + l);
+    const int f = l / a.uni_bs, t = __ldg(a.tr_of_c + 4 * k + f);
+    return t < 0 ? -1 : (long long)t * a.uni_bs + (l - f * a.uni_bs);
+  }
+  __device__ __forceinline__ int bs(int t) const { return a.uni_nT ? a.uni_bs : __ldg(a.tpts + t) * a.nv; }
+  __device__ __forceinline__ long long toff(int t) const {
+    return a.uni_nT ? (long long)t * a.uni_bs : __ldg(a.toff + t);
+  }
+  __device__ __forceinline__ long long poff(int t) const {
+    return a.uni_nT ? (long long)t * a.uni_bs * a.uni_bs : __ldg(a.poff + t);
+  }
+};
+
+// FP32 to FP64 by the integer pipes (exact; zeros, subnormals, infinities and NaN by the conversion
+// instruction, which shares the FP64 pipe)
+__device__ __forceinline__ double any_widen(float x) {
+  const unsigned u = __float_as_uint(x), e = (u >> 23) & 255u;
+  if (e == 0u || e == 255u) return (double)x;
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+__device__ __forceinline__ double any_widen(double x) { return x; }
+
+// out[d] = base[d] - (or, without base, +) the sum of the element-view entries of trace value d, over
+// [x0, x1); four values per thread in flight (their table entries, then the values themselves)
+template <typename T>
+__device__ void any_gather(const CycleArgs& a, const double* base, double* out, size_t x0, size_t x1) {
+  const T* yv = reinterpret_cast<const T*>(a.yv);
+  for (size_t xb = x0 + threadIdx.x; xb < x1; xb += 4 * PG_THREADS) {
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    if (a.uni_nT) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const size_t d = xb + (size_t)u * PG_THREADS;
+        if (d >= x1) break;
+        const int t = (int)(d / a.uni_bs), b = (int)(d % a.uni_bs);
+#pragma unroll
+        for (int sd = 0; sd < 2; ++sd) {
+          const int e = __ldg(a.sides + 4 * t + 2 * sd), f = __ldg(a.sides + 4 * t + 2 * sd + 1);
+          if (e >= 0) s[u] += any_widen(__ldcg(yv + (size_t)e * a.uni_nT + f * a.uni_bs + b));
+        }
+      }
+    } else {
+      long long c[4], c1[4];
+      int most = 0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const size_t d = xb + (size_t)u * PG_THREADS;
+        c[u] = d < x1 ? __ldg(a.vptr + d) : 0;
+        c1[u] = d < x1 ? __ldg(a.vptr + d + 1) : 0;
+        most = max(most, (int)(c1[u] - c[u]));
+      }
+      for (int i = 0; i < most; ++i) {
+        long long ix[4];
+        T v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) ix[u] = c[u] + i < c1[u] ? __ldg(a.vidx + c[u] + i) : -1;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = ix[u] >= 0 ? __ldcg(yv + ix[u]) : T(0);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (ix[u] >= 0) s[u] += any_widen(v[u]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const size_t d = xb + (size_t)u * PG_THREADS;
+      if (d < x1) out[d] = base ? __ldcg(base + d) - s[u] : s[u];
+    }
+  }
+}
+
+// y_k = S_k x_k over this warp's run of rows (X: T, the preconditioned vector, or double, x itself).
+// The element's trace values are staged in the warp's shared memory, those of the next element
+// loaded meanwhile; then 32 rows at a time, four lanes per row and four rows per lane, each lane
+// every fourth 16-byte vector of its rows (scalar where the rows do not start on vectors).  Short
+// FP64 rows go one per lane: their lane sums would cost the FP64 pipe more than the products.
+template <typename T, typename X>
+__device__ void any_matvec(const CycleArgs& a, const X* x, T* xs) {
+  constexpr int VW = 16 / (int)sizeof(T), PF = 4;  // PF: values per lane of a next element loaded ahead
+  struct alignas(16) Vec {
+    T v[VW];
+  };
+  const AnyShape sh{a};
+  const int lane = threadIdx.x & 31, r8 = lane >> 2, c4 = lane & 3;
+  const long long W = (long long)gridDim.x * PG_WARPS, w = (long long)blockIdx.x * PG_WARPS + (threadIdx.x >> 5);
+  const long long s0 = a.sumTT / W * w + a.sumTT % W * w / W, s1 = a.sumTT / W * (w + 1) + a.sumTT % W * (w + 1) / W;
+  if (s0 >= s1) return;
+  int lo = 0, hi = a.Eim - 1;  // the element that holds value s0
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (sh.offD(mid) <= s0) lo = mid;
+    else hi = mid - 1;
+  }
+  const T* S = reinterpret_cast<const T*>(a.S);
+  T* yv = reinterpret_cast<T*>(a.yv);
+  auto value = [&](int k, long long o, int l) -> T {
+    const long long g = sh.gmap(k, o, l);
+    return g >= 0 ? T(__ldcg(x + g)) : T(0);
+  };
+  T nx[PF];
+  bool have = false;  // nx holds the first 32 PF values of element k
+  for (int k = lo; k < a.Eim; ++k) {
+    const int nT = sh.nT(k);
+    const long long od = sh.offD(k), o = sh.offs(k);
+    if (od >= s1) break;
+    // rows whose first value lies in [s0, s1)
+    const int ra = od >= s0 ? 0 : (int)((s0 - od + nT - 1) / nT);
+    const int rb = (int)min((long long)nT, (s1 - od + nT - 1) / nT);
+    __syncwarp();
+    if (ra < rb) {
+#pragma unroll
+      for (int q = 0; q < PF; ++q)
+        if (lane + 32 * q < nT) xs[lane + 32 * q] = have ? nx[q] : value(k, o, lane + 32 * q);
+      for (int l = lane + 32 * PF; l < nT; l += 32) xs[l] = value(k, o, l);
+    }
+    have = k + 1 < a.Eim && od + (long long)nT * nT < s1;
+    if (have) {
+      const int nT1 = sh.nT(k + 1);
+      const long long o1 = sh.offs(k + 1);
+#pragma unroll
+      for (int q = 0; q < PF; ++q)
+        if (lane + 32 * q < nT1) nx[q] = value(k + 1, o1, lane + 32 * q);
+    }
+    if (ra >= rb) continue;
+    __syncwarp();
+    const T* Sk = S + od;
+    const bool vec = nT % VW == 0 && od % VW == 0;
+    if (sizeof(T) == 8 && nT <= 16) {
+      for (int r = ra + lane; r < rb; r += 32) {
+        T acc = T(0);
+        for (int c = 0; c < nT; ++c) acc = fma(__ldg(Sk + (size_t)r * nT + c), xs[c], acc);
+        yv[o + r] = acc;
+      }
+      continue;
+    }
+    for (int r0 = ra; r0 < rb; r0 += 32) {
+      T acc[4];
+      const T* row[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        acc[u] = T(0);
+        const int r = r0 + r8 + 8 * u;
+        row[u] = Sk + (size_t)(r < rb ? r : rb - 1) * nT;  // a row past the end repeats the last one
+      }
+      if (vec) {
+#pragma unroll 2
+        for (int c = c4 * VW; c < nT; c += 4 * VW) {
+          const Vec xv = *reinterpret_cast<const Vec*>(xs + c);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const PGVec<T, VW> sv = pg_ld_stream<T, VW>(row[u] + c);
+#pragma unroll
+            for (int q = 0; q < VW; ++q) acc[u] = fma(sv.v[q], xv.v[q], acc[u]);
+          }
+        }
+      } else {
+        for (int c = c4; c < nT; c += 4) {
+          const T xv = xs[c];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) acc[u] = fma(__ldg(row[u] + c), xv, acc[u]);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], 1);
+        acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], 2);
+        const int r = r0 + r8 + 8 * u;
+        if (c4 == 0 && r < rb) yv[o + r] = acc[u];
+      }
+    }
+  }
+}
+
+// z = P^-1 v over the trace units [t0, t1), in the block precision.  Units of up to 8 values one per
+// thread; up to 32 one per warp and lane a row, two units' rows in flight; larger ones one per warp
+// with a lane on every 32nd row.  tid0, nthr: the threads that take part
+template <typename T>
+__device__ void any_precond(const CycleArgs& a, const double* v, T* z, int t0, int t1, int tid0, int nthr) {
+  constexpr int VW = 16 / (int)sizeof(T);
+  const AnyShape sh{a};
+  const T* P = reinterpret_cast<const T*>(a.Pinv);
+  if (a.bsmax <= 8) {
+    for (int t = t0 + tid0; t < t1; t += nthr) {
+      const int bs = sh.bs(t);
+      const long long o = sh.toff(t);
+      const T* Pt = P + sh.poff(t);
+      T x[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) x[c] = c < bs ? T(v[o + c]) : T(0);
+      for (int r = 0; r < bs; ++r) {
+        T s = T(0);
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+          if (c < bs) s = fma(__ldg(Pt + r * bs + c), x[c], s);
+        z[o + r] = s;
+      }
+    }
+    return;
+  }
+  const int lane = threadIdx.x & 31, nw = nthr >> 5;
+  constexpr int RV = 24 / VW;  // vectors of a row held in registers
+  if (sizeof(T) == 4 && a.bsmax <= 24) {
+    for (int t = t0 + (tid0 >> 5); t < t1; t += 2 * nw) {
+      PGVec<T, VW> row[2][RV];
+      T x[2];
+      int bs[2];
+      long long o[2];
+      bool ok[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int tt = t + h * nw < t1 ? t + h * nw : t;
+        bs[h] = sh.bs(tt);
+        o[h] = sh.toff(tt);
+        const long long po = sh.poff(tt);
+        ok[h] = bs[h] % VW == 0 && po % VW == 0;
+        x[h] = lane < bs[h] ? T(v[o[h] + lane]) : T(0);
+        const T* pr = P + po + (size_t)(lane < bs[h] ? lane : 0) * bs[h];
+#pragma unroll
+        for (int c = 0; c < RV; ++c) {
+          if (ok[h] && c * VW < bs[h]) {
+            row[h][c] = pg_ld_stream<T, VW>(pr + c * VW);
+          } else {
+#pragma unroll
+            for (int e = 0; e < VW; ++e) row[h][c].v[e] = c * VW + e < bs[h] ? __ldg(pr + c * VW + e) : T(0);
+          }
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        T s = T(0);
+#pragma unroll
+        for (int c = 0; c < RV * VW; ++c)
+          if (c < bs[h]) s = fma(row[h][c / VW].v[c % VW], __shfl_sync(0xffffffffu, x[h], c), s);
+        if (lane < bs[h] && (h == 0 || t + nw < t1)) z[o[h] + lane] = s;
+      }
+    }
+    return;
+  }
+  for (int t = t0 + (tid0 >> 5); t < t1; t += nw) {
+    const int bs = sh.bs(t);
+    const long long o = sh.toff(t), po = sh.poff(t);
+    const bool vec = bs % VW == 0 && po % VW == 0;
+    T x[4], acc[4];
+    const T* row[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = lane + 32 * q;
+      x[q] = i < bs ? T(v[o + i]) : T(0);
+      acc[q] = T(0);
+      row[q] = P + po + (size_t)(i < bs ? i : 0) * bs;
+    }
+#pragma unroll
+    for (int qc = 0; qc < 4; ++qc) {
+      const int cn = min(32, bs - 32 * qc);
+      if (cn <= 0) break;
+      if (vec) {
+#pragma unroll 4
+        for (int c = 0; c < cn; c += VW) {
+          T xv[VW];
+#pragma unroll
+          for (int e = 0; e < VW; ++e) xv[e] = __shfl_sync(0xffffffffu, x[qc], c + e);
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (32 * q < bs) {
+              const PGVec<T, VW> pv = pg_ld_stream<T, VW>(row[q] + 32 * qc + c);
+#pragma unroll
+              for (int e = 0; e < VW; ++e) acc[q] = fma(pv.v[e], xv[e], acc[q]);
+            }
+        }
+      } else {
+        for (int c = 0; c < cn; ++c) {
+          const T xv = __shfl_sync(0xffffffffu, x[qc], c);
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (32 * q < bs) acc[q] = fma(__ldg(row[q] + 32 * qc + c), xv, acc[q]);
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (lane + 32 * q < bs) z[o + lane + 32 * q] = acc[q];
+  }
+}
+
+// x += sum_{i<k} y_i Z_i over [x0, x1) (FP64 sums of block-precision vectors)
+template <typename T>
+__device__ void any_update_x(const T* Z, size_t n, const double* y, int k, double* x, size_t x0, size_t x1) {
+  for (size_t i = x0 + threadIdx.x; i < x1; i += PG_THREADS) {
+    double s0 = 0.0, s1 = 0.0;
+    int j = 0;
+    for (; j + 8 <= k; j += 8) {
+      T v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = Z[(size_t)(j + u) * n + i];
+#pragma unroll
+      for (int u = 0; u < 8; u += 2) {
+        s0 = fma(y[j + u], any_widen(v[u]), s0);
+        s1 = fma(y[j + u + 1], any_widen(v[u + 1]), s1);
+      }
+    }
+    for (; j < k; ++j) s0 = fma(y[j], any_widen(Z[(size_t)j * n + i]), s0);
+    x[i] += s0 + s1;
+  }
+}
+
+constexpr int ANY_MAXT = 512;    // trace unknowns of an element
+constexpr int ANY_CLUSTER = 8;
+template <typename T>
+constexpr size_t any_smem() {
+  return (sizeof(PGShared<double>) + 15) / 16 * 16 + (size_t)PG_WARPS * ANY_MAXT * sizeof(T);
+}
+
+// CLUSTER: one cluster of ANY_CLUSTER CTAs instead of a cooperative grid
+template <typename T, bool CLUSTER>
+__global__ void __launch_bounds__(PG_THREADS, 1) k_gmres_cycle_any(const __grid_constant__ CycleArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  PGShared<double>& sh = *reinterpret_cast<PGShared<double>*>(smem_raw);
+  T* xs = reinterpret_cast<T*>(smem_raw + (sizeof(PGShared<double>) + 15) / 16 * 16) + (threadIdx.x >> 5) * ANY_MAXT;
+  const AnyShape lay{a};
+  const int tid = threadIdx.x;
+  const size_t n = a.n;
+  // trace units of this CTA: about n / gridDim.x values each
+  auto first_unit = [&](int b) -> int {
+    if (a.uni_nT) return (int)((long long)b * a.ntrace / gridDim.x);
+    const long long want = (long long)b * (long long)n / gridDim.x;
+    int lo = 0, hi = a.ntrace;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (__ldg(a.toff + mid) < want) lo = mid + 1;
+      else hi = mid;
+    }
+    return lo;
+  };
+  const int t0 = first_unit(blockIdx.x), t1 = blockIdx.x + 1 == gridDim.x ? a.ntrace : first_unit(blockIdx.x + 1);
+  const size_t x0 = (size_t)lay.toff(t0), x1 = t1 == a.ntrace ? n : (size_t)lay.toff(t1);
+  unsigned epoch = 0;
+  int par = 0;
+  const size_t pstride = (size_t)PG_ND * gridDim.x;
+  double *V = a.V, *partial = a.partial;
+  T* Z = reinterpret_cast<T*>(a.Z);
+  auto sync = [&]() -> bool {
+    if constexpr (CLUSTER) {
+      __syncthreads();
+      asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+      return true;
+    } else {
+      return pg_sync(sh, a.bar, epoch);
+    }
+  };
+  const int xz = a.dyn ? a.dyn[0] : a.x_zero;
+  const int mm = a.dyn ? a.dyn[1] : a.m;
+  // r0 = t - L x into V_0 (x = 0: r0 = t); beta = ||r0||, bnorm = ||t||
+  if (!xz) {
+    any_matvec<T, double>(a, a.x, xs);
+    if (!sync()) return;
+    any_gather<T>(a, a.t, V, x0, x1);
+  } else {
+    for (size_t x = x0 + tid; x < x1; x += PG_THREADS) V[x] = __ldcg(a.t + x);
+  }
+  __syncthreads();
+  pg_block_sq(sh, V, a.t, x0, x1, partial + par * pstride);
+  if (!sync()) return;
+  pg_reduce(sh, 2, partial + par * pstride);
+  par ^= 1;
+  if (tid == 0) {
+    const double beta = sqrt(sh.dot[0]);
+    sh.beta = beta;
+    sh.bnorm = sqrt(sh.dot[1]);
+    sh.g[0] = beta;
+    sh.res = beta;
+    sh.hn = beta;
+    sh.k = 0;
+    sh.conv = 0;
+    sh.nan = 0;
+    sh.done = 0;
+    sh.corr = 0;
+    sh.invT = beta > 0.0 ? 1.0 / beta : 0.0;
+    if (!(beta == beta)) {
+      sh.nan = 1;
+      sh.done = 1;
+    } else if (beta <= a.rtol * sh.bnorm || beta == 0.0) {
+      sh.conv = 1;
+      sh.done = 1;
+    }
+  }
+  __syncthreads();
+  if (!sh.done) {
+    for (int j = 0;; ++j) {
+      double* vj = V + (size_t)j * n;
+      double* w = V + (size_t)(j + 1) * n;
+      // (A) lane 0 of warp 0: Givens rotation of column j-1; warps 1..: finish v_j, z_j = P^-1 v_j
+      if (j > 0 && tid == 0) pg_givens(sh, j - 1, a.rtol, mm);
+      if (tid >= 32) {
+        pg_finish(V, n, sh.cf, sh.corr ? j : 0, sh.invT, vj, x0, x1);
+        pg_sync_workers();
+        any_precond<T>(a, vj, Z + (size_t)j * n, t0, t1, tid - 32, PG_THREADS - 32);
+      }
+      if (!sync()) return;
+      __syncthreads();
+      if (sh.done) break;
+      // (B) y_k = S_k z_k
+      any_matvec<T, T>(a, Z + (size_t)j * n, xs);
+      if (!sync()) return;
+      // (C) w = L z and h = V^T w
+      any_gather<T>(a, nullptr, w, x0, x1);
+      double* part = partial + par * pstride;
+      pg_block_dots<double>(sh, V, n, j + 1, w, x0, x1, part);
+      if (!sync()) return;
+      pg_reduce(sh, j + 1, part);
+      par ^= 1;
+      for (int i = tid; i <= j; i += PG_THREADS) {
+        sh.hc[i] = sh.dot[i];
+        sh.cf[i] = sh.dot[i];
+      }
+      __syncthreads();
+      // (D) w' = w - V h, then d = V^T w' and ||w'||^2
+      pg_subtract(V, n, sh.cf, j, w, x0, x1);
+      part = partial + par * pstride;
+      pg_block_dots<double>(sh, V, n, j + 2, w, x0, x1, part);
+      if (!sync()) return;
+      pg_reduce(sh, j + 2, part);
+      par ^= 1;
+      if (tid < 32) {
+        double dd = 0.0;
+        for (int i = tid; i <= j; i += 32) {
+          const double d = sh.dot[i];
+          dd += d * d;
+          sh.hc[i] += d;
+          sh.cf[i] = d;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) dd += __shfl_xor_sync(0xffffffffu, dd, o);
+        if (tid == 0) {
+          const double n1 = sh.dot[j + 1];
+          sh.corr = dd <= 0.25 * n1 ? 1 : 0;
+          if (sh.corr) sh.hc[j + 1] = sqrt(n1 - dd);
+        }
+      }
+      __syncthreads();
+      if (!sh.corr) {  // severe cancellation: form w'' = w' - V d now and sum its norm
+        pg_subtract(V, n, sh.cf, j, w, x0, x1);
+        part = partial + par * pstride;
+        pg_block_sq(sh, w, (const double*)nullptr, x0, x1, part);
+        if (!sync()) return;
+        pg_reduce(sh, 1, part);
+        par ^= 1;
+        if (tid == 0) sh.hc[j + 1] = sqrt(sh.dot[0]);
+      }
+      if (tid == 0) sh.invT = sh.hc[j + 1] != 0.0 ? 1.0 / sh.hc[j + 1] : 0.0;
+      __syncthreads();
+    }
+  }
+  // y = H^{-1} g, x += Z y
+  const int k = sh.k;
+  if (tid == 0) {
+    for (int i = k - 1; i >= 0; --i) {
+      double s = sh.g[i];
+      for (int c = i + 1; c < k; ++c) s -= sh.H[i * GM_MAXM + c] * sh.y[c];
+      sh.y[i] = s * sh.rdi[i];
+    }
+  }
+  __syncthreads();
+  if (k > 0) any_update_x<T>(Z, n, sh.y, k, a.x, x0, x1);
+  if (a.true_res) {  // ||t - L x|| (V_0 as scratch)
+    if (!sync()) return;
+    any_matvec<T, double>(a, a.x, xs);
+    if (!sync()) return;
+    any_gather<T>(a, a.t, V, x0, x1);
+    __syncthreads();
+    pg_block_sq(sh, V, (const double*)nullptr, x0, x1, partial + par * pstride);
+    if (!sync()) return;
+    pg_reduce(sh, 1, partial + par * pstride);
+  }
+  if (blockIdx.x == 0 && tid == 0) {
+    GmresState* st = a.st;
+    st->beta = a.true_res ? sqrt(sh.dot[0]) : sh.res;
+    st->bnorm = sh.bnorm;
+    st->res = sh.res;
+    st->hn = sh.hn;
+    st->k = k;
+    st->kdone = k;
+    st->converged = sh.conv;
+    st->nan = sh.nan;
+  }
+}
+
 template <typename T, int NT, int BS, bool SB>
 cudaError_t launch_cycle(const FusedArgs& a, int grid, cudaStream_t s) {
   const size_t smem = sizeof(PGShared<T>);
@@ -992,6 +1608,164 @@ cudaError_t launch_gmres_cycle(const FusedArgs& a, int prec_bytes, int grid, cud
   CycleFn fn = pick(prec_bytes, a.nT, bs, &occ, a.s_bf16 != 0);
   if (!fn || grid < 1) return cudaErrorInvalidValue;
   return fn(a, grid, s);
+}
+
+template <typename T, bool CLUSTER>
+static cudaError_t launch_any(const CycleArgs& a, const CyclePlan& p, cudaStream_t s) {
+  auto kern = k_gmres_cycle_any<T, CLUSTER>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)any_smem<T>());
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(p.grid);
+  cfg.blockDim = dim3(PG_THREADS);
+  cfg.dynamicSmemBytes = any_smem<T>();
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  if (CLUSTER) {
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = ANY_CLUSTER;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+  } else {
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  hfr::count_launch();
+  return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+cudaError_t launch_cycle_any(const CycleArgs& a, int prec_bytes, const CyclePlan& p, cudaStream_t s) {
+  if (p.grid < 1) return cudaErrorInvalidValue;
+  if (prec_bytes == 4) return p.cluster ? launch_any<float, true>(a, p, s) : launch_any<float, false>(a, p, s);
+  return p.cluster ? launch_any<double, true>(a, p, s) : launch_any<double, false>(a, p, s);
+}
+
+// The cluster form up to about 200 000 multiply-adds per iteration (S once, the FP64 vectors some
+// forty times): above that, eight SMs' FP64 pipes take longer than the grid barriers of the whole
+// device cost (four per iteration, about 2 us each).
+CyclePlan cycle_plan(int prec_bytes, const CycleArgs& a) {
+  CyclePlan p;
+  int dev = 0, coop = 0, nsm = 0, occ = 0;
+  if (a.ntrace <= 0 || a.Eim <= 0 || a.bsmax > 128) return p;
+  if (cudaGetDevice(&dev) != cudaSuccess) return p;
+  if (a.sumTT + 40 * (long long)a.n <= 200000) {
+    p.grid = ANY_CLUSTER;
+    p.cluster = 1;
+    return p;
+  }
+  if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) return p;
+  if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return p;
+  auto fits = [&](auto kern, size_t smem) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
+           cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, PG_THREADS, smem) == cudaSuccess && occ >= 1;
+  };
+  const bool ok = prec_bytes == 4 ? fits(k_gmres_cycle_any<float, false>, any_smem<float>())
+                                  : fits(k_gmres_cycle_any<double, false>, any_smem<double>());
+  if (ok) p.grid = nsm;  // one CTA per SM
+  return p;
+}
+
+int run_gmres_any(const CycleArgs& base, int prec_bytes, const CyclePlan& p, double rtol, int restart, int maxit,
+                  bool true_res, GmresResult* res, int* timed_out, cudaStream_t s) {
+  const int m = restart > GM_MAXM ? GM_MAXM : (restart < 1 ? 1 : restart);
+  CycleArgs a = base;
+  a.rtol = rtol;
+  a.true_res = true_res ? 1 : 0;
+  *timed_out = 0;
+  if (cudaMemsetAsync(a.x, 0, a.n * sizeof(double), s) != cudaSuccess) return -1;
+  int total = 0;
+  for (bool first = true;; first = false) {
+    a.m = m < maxit - total ? m : maxit - total;
+    a.x_zero = first ? 1 : 0;
+    if (total + a.m >= maxit) a.true_res = 1;  // the cycle that may end at the limit: its residual is reported
+    if (cudaMemsetAsync(a.bar, 0, 2 * sizeof(unsigned), s) != cudaSuccess) return -1;
+    if (launch_cycle_any(a, prec_bytes, p, s) != cudaSuccess) return -1;
+    GmresHead hs;
+    unsigned flags[2] = {0u, 0u};
+    if (cudaMemcpyAsync(&hs, a.st, sizeof(GmresHead), cudaMemcpyDeviceToHost, s) != cudaSuccess) return -1;
+    if (cudaMemcpyAsync(flags, a.bar, sizeof(flags), cudaMemcpyDeviceToHost, s) != cudaSuccess) return -1;
+    if (cudaStreamSynchronize(s) != cudaSuccess) return -1;
+    res->iterations = total;
+    res->nan = res->converged = 0;
+    if (flags[1] != 0u) {
+      *timed_out = 1;
+      return 0;
+    }
+    total += hs.k;
+    res->bnorm = hs.bnorm;
+    res->rel = hs.bnorm > 0.0 ? hs.beta / hs.bnorm : 0.0;
+    res->iterations = total;
+    res->nan = hs.nan;
+    res->converged = hs.converged;
+    if (hs.nan || hs.converged || total >= maxit || hs.k == 0) return 0;
+  }
+}
+
+// ------------------------------------------------------------ inside a captured graph
+__global__ void k_ga_begin(GmresGraphDev* d, int m, int maxit, cudaGraphConditionalHandle hw) {
+  d->total = 0;
+  d->cycles = 0;
+  d->nan = 0;
+  d->converged = 0;
+  d->timeout = 0;
+  d->dyn[0] = 1;
+  d->dyn[1] = m < maxit ? m : maxit;
+  cudaGraphSetConditional(hw, 1u);
+}
+__global__ void k_ga_after(GmresGraphDev* d, const GmresState* st, const unsigned* bar, int m, int maxit,
+                           cudaGraphConditionalHandle hw) {
+  int cont = 0;
+  d->cycles += 1;
+  if (bar[1] != 0u) {
+    d->timeout = 1;
+  } else {
+    d->total += st->k;
+    if (st->nan) d->nan = 1;
+    d->converged = st->converged;
+    cont = (st->nan || st->converged || d->total >= maxit || st->k == 0) ? 0 : 1;
+    const int rem = maxit - d->total;
+    d->dyn[0] = 0;
+    d->dyn[1] = m < rem ? m : rem;
+  }
+  cudaGraphSetConditional(hw, (unsigned)cont);
+}
+
+cudaError_t capture_gmres_any(CycleArgs a, int prec_bytes, const CyclePlan& p, double rtol, int restart, int maxit,
+                              GmresGraphDev* dev, cudaStream_t s, cudaStream_t sc, GmresGraphLaunches* counts) {
+  const int m = restart > GM_MAXM ? GM_MAXM : (restart < 1 ? 1 : restart);
+  a.rtol = rtol;
+  a.m = m;
+  a.x_zero = 1;
+  a.true_res = 0;
+  a.dyn = dev->dyn;
+  cudaError_t e;
+  const unsigned long long l0 = hfr::launch_count();
+  cudaGraphConditionalHandle hw;
+  if ((e = graph_conditional_handle(s, 0u, 0u, &hw)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(a.x, 0, a.n * sizeof(double), s)) != cudaSuccess) return e;
+  (hfr::count_launch(), k_ga_begin<<<1, 1, 0, s>>>(dev, m, maxit, hw));
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  cudaGraph_t body = nullptr;
+  if ((e = graph_add_conditional(s, hw, cudaGraphCondTypeWhile, &body)) != cudaSuccess) return e;
+  const unsigned long long l1 = hfr::launch_count();
+  if ((e = cudaStreamBeginCaptureToGraph(sc, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed)) != cudaSuccess)
+    return e;
+  e = cudaMemsetAsync(a.bar, 0, 2 * sizeof(unsigned), sc);
+  if (e == cudaSuccess) e = launch_cycle_any(a, prec_bytes, p, sc);
+  if (e == cudaSuccess) {
+    (hfr::count_launch(), k_ga_after<<<1, 1, 0, sc>>>(dev, a.st, a.bar, m, maxit, hw));
+    e = cudaGetLastError();
+  }
+  cudaGraph_t tmp = nullptr;
+  const cudaError_t e2 = cudaStreamEndCapture(sc, &tmp);
+  if (counts) {
+    counts->fixed = (int)(l1 - l0);
+    counts->cycle = (int)(hfr::launch_count() - l1);
+    counts->residual = 0;
+  }
+  return e != cudaSuccess ? e : e2;
 }
 
 // Host side of the barrier self-test (declared in hfr_krylov.h).

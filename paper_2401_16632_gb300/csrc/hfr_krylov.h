@@ -93,6 +93,45 @@ int run_gmres_fused(const FusedArgs& a, int prec_bytes, int grid, double rtol, i
 // one restart cycle (enqueue only; a.bar must be zeroed before it): cudaErrorInvalidValue when
 // the shape has no single-launch cycle
 cudaError_t launch_gmres_cycle(const FusedArgs& a, int prec_bytes, int grid, cudaStream_t s);
+// One restart cycle per launch for any trace layout (hfr_gmres_fused.cu, k_gmres_cycle_any), FP64
+// Krylov basis, the operator in the element view: y_k = S_k x_k, then the sum of the element entries
+// of every trace value.  General meshes give the tables; a uniform mesh (uni_nT > 0) its sizes.
+struct CycleArgs {
+  int Eim, ntrace, nv;
+  const int* nTk;                       // trace unknowns of each implicit element
+  const long long *offD, *offs;         // their S blocks and element-view entries (Eim + 1)
+  const int* gmap;                      // element-view entry -> trace value, -1 off traces
+  const long long *vptr, *vidx;         // trace value <- element-view entries (CSR)
+  const int* tpts;                      // points of each trace unit
+  const long long *toff, *poff;         // its values and its face-block inverse (ntrace + 1)
+  int uni_nT = 0, uni_bs = 0;           // uniform mesh: nT, values per trace face
+  const int *tr_of_c = nullptr, *sides = nullptr;
+  long long sumTT = 0;                  // values of all S blocks
+  int bsmax = 0;                        // values of the largest trace unit (at most 128)
+  const void *S, *Pinv;                 // block precision
+  const double* t;                      // right-hand side
+  double *x, *V, *partial;              // solution, basis, reductions
+  void *Z, *yv;                         // P^-1 basis and element view (block precision)
+  unsigned* bar;                        // 2 words: barrier arrivals, abort flag
+  GmresState* st;
+  size_t n;
+  int m;
+  double rtol;
+  int x_zero, true_res;
+  const int* dyn = nullptr;             // as in FusedArgs
+};
+// how the cycle is launched: grid 0 not available; cluster 1 = one cluster of 8 CTAs (small systems:
+// its hardware barrier), else a cooperative launch of one CTA per SM
+struct CyclePlan {
+  int grid = 0, cluster = 0;
+};
+CyclePlan cycle_plan(int prec_bytes, const CycleArgs& a);
+cudaError_t launch_cycle_any(const CycleArgs& a, int prec_bytes, const CyclePlan& p, cudaStream_t s);
+// whole solve; as run_gmres_fused.  The true final residual is computed when true_res is set and
+// for a solve that ends without meeting rtol
+int run_gmres_any(const CycleArgs& a, int prec_bytes, const CyclePlan& p, double rtol, int restart, int maxit,
+                  bool true_res, GmresResult* res, int* timed_out, cudaStream_t s);
+
 // Self-test of the bounded grid barrier used by the single-launch cycle (cooperative launch of
 // nblocks CTAs, `rounds` barriers; CTA `absent` never arrives when 0 <= absent < nblocks).
 // Returns 0 (timed_out set when the abort flag was raised), -1 on a CUDA error, -2 on arguments
@@ -110,6 +149,8 @@ int run_gmres(const GmresOps& ops, const GmresBuffers& b, const double* t, doubl
 // The iteration limit is checked per cycle.  dev: the solve's counters (device memory).
 struct GmresGraphDev {
   int first, total, cycles, nan, converged;
+  int timeout;  // a bounded barrier wait of the single-launch cycle ran out
+  int dyn[2];   // x_zero and length of its next cycle
 };
 struct GmresGraphLaunches {
   int fixed = 0;     // once per solve
@@ -119,5 +160,8 @@ struct GmresGraphLaunches {
 cudaError_t capture_gmres(const GmresOps& ops, const GmresBuffers& b, const double* t, double* x, double rtol,
                           int restart, int maxit, GmresGraphDev* dev, cudaStream_t s, const cudaStream_t sc[2],
                           GmresGraphLaunches* counts);
+// the same with the single-launch cycle as the body of the WHILE node
+cudaError_t capture_gmres_any(CycleArgs a, int prec_bytes, const CyclePlan& p, double rtol, int restart, int maxit,
+                              GmresGraphDev* dev, cudaStream_t s, cudaStream_t sc, GmresGraphLaunches* counts);
 
 }  // namespace hfr
