@@ -480,76 +480,133 @@ __global__ void k_gen_initial_trace(size_t npts, int nv, const long long* __rest
 }
 
 // ------------------------------------------------------------------------ element blocks
-// One CTA per implicit element.  Primal state, pointwise Jacobians of the volume flux (state and
-// reference gradient) and of the face flux and trace row (face state, trace, face gradient) by
-// dual numbers, then one warp per seed point (a solution point: NV columns of A and C; a trace
-// face point: NV columns of B and D) propagating the unit tangent through the linear chain of the
-// element operator: face nodes -> face points -> common values at the nodes -> corrected gradient
-// -> flux tangents at the solution points and the face points -> projection to the face nodes ->
-// divergence.  Columns are staged per seed point and written as rows of NV consecutive values.
+// One CTA per implicit element of N points per line (the elements of each degree in one launch).
+// Primal state, pointwise Jacobians of the volume flux (state and reference gradient) and of the
+// face flux (face state, trace, face gradient) by dual numbers, then one warp per seed point: a
+// solution point (NV columns of A and C) or a trace face point (NV columns of B and D).
+//
+// A unit seed of a solution point moves the reference gradient on the grid row and the grid column
+// through it alone: the common value at a face node is the trace's projection, and projecting what
+// was interpolated gives the node's own value back (P T = 1), so the seed leaves it unmoved on every
+// kind of face.  A seed of a trace point whose face carries the element's own points moves it on
+// one line; on faces of a higher neighbour degree and on EFR faces on every point, by the products
+// dg[a] P[b][q0].  So line seeds form the flux tangents on their lines and the line sums (as the
+// uniform kernel does), the others sum over the lines per output.  Lane (v, g): output variable v,
+// lane group g; a lane carries the NV seed variables of the point (16-byte loads and stores).
+//
+// What bounds it: instruction issue.  The dense form (every tangent of every point for each column,
+// line lengths known at run time only) took 5.77 ms on 16 384 EFR elements of p = 4 and 3.58 ms on
+// 10 000 wall elements of p = 2..5; this one 2.21 and 1.34 ms.
 
-template <int NV, typename T>
+template <int N, int NV, typename T>
 struct JWork {
-  T U[GNS][NV];
-  T Ufn[GF][NV], Ufp[GF][NV], ubp[GF][NV], ubn[GF][NV], un[GF][NV];
-  T q[GNS][2][NV];
-  T qfn[GF][2][NV], qfp[GF][2][NV];
-  T iJ[GNS], ciJ[GNS], Sm[GNS][2][2];
-  T fJ[GF], fnr[GF][2];
-  T M[GN][GN], lm[GN], lp[GN], dgL[GN], dgR[GN];
-  T Tf[4][GN][GN], Pf[4][GN][GN], wq[4][GN];
+  static constexpr int NS = N * N, NN = 4 * N;
+  static constexpr int PAD = NV == 4 ? 4 : 0;
+  static constexpr int LNS = 2 * NV * NV + PAD, RCS = NV * NV + PAD;
   // pointwise Jacobians, innermost index the input variable
-  T KU[GNS][2][NV][NV];
-  T KQ[GNS][2][2][NV][NV];
-  T GU[GF][NV][NV], GH[GF][NV][NV], GQ[GF][2][NV][NV];
-  T RU[GF][NV][NV], RH[GF][NV][NV], RQ[GF][2][NV][NV];
+  alignas(16) T KU[NS][2][NV][NV];
+  alignas(16) T KQ[NS][2][2][NV][NV];
+  alignas(16) T GU[GF][NV][NV], GH[GF][NV][NV], GQ[GF][2][NV][NV];
+  alignas(16) T RH[GF][NV][NV];  // boundary faces: trace row by the trace; far field: by the state RU 1
+  // per-warp tangents of one seed point, entries [v][v0] (v0 innermost)
   struct Col {
-    T dUfn[GF], dUfp[GF], dubp[GF], dubn[GF];
-    T dQ[GNS][2], dq[GNS][2];
-    T dqfn[GF][2], dqfp[GF][2];
-    T dFt[GNS][2][NV];
-    T dFnp[GF][NV], drow[GF][NV], dFnn[GF][NV];
+    alignas(16) T LN[2][N][LNS];  // flux tangents [r][v][v0] on the seed's row (0) / column (1)
+    alignas(16) T RC[2][N][RCS];  // their line sums
+    alignas(16) T FP[GF][RCS];    // face flux at the face points
+    alignas(16) T FN[NN][RCS];    // and projected to the face nodes (faces with other points)
+    T DQ[2][N][2];                // physical gradient tangents on the two lines
+    T qn[NN][2], qp[GF][2];       // at the face nodes and points
+    T du[GF];                     // face state at the face points
   } col[JW];
+  T U[NS][NV];
+  T Ufn[NN][NV], Ufp[GF][NV], ubp[GF][NV], ubn[NN][NV], un[GF][NV];
+  T q[NS][2][NV];
+  T qfn[NN][2][NV], qfp[GF][2][NV];
+  T iJ[NS], ciJ[NS], Sm[NS][2][2];
+  T fJ[GF], fnr[GF][2], RU[GF];
+  T M[N][N], lm[N], lp[N], dgL[N], dgR[N];
+  T Tf[4][GN][N], Pf[4][N][GN], wq[4][GN];
   T uinf[5];
-  int nf[4], kf[4], tr[4], lto[4];
+  int nf[4], kf[4], tr[4], lto[4], own[4];
+  int npt, pt[GF];  // the face points f GN + q in use
 };
 
-static_assert(sizeof(JWork<4, double>) <= 227 * 1024, "block kernel workspace exceeds shared memory");
+static_assert(sizeof(JWork<GN, 4, double>) <= 227 * 1024, "block kernel workspace exceeds shared memory");
 static_assert(sizeof(GWork<4>) * GEPB <= 227 * 1024, "residual workspace exceeds shared memory");
 
-template <int PHYS, typename T>
-__global__ void __launch_bounds__(JT, sizeof(T) == 4 ? 3 : 1) k_gen_jacobian(const __grid_constant__ PhysParams pp,
-                                                    const __grid_constant__ GArgs a,
-                                                    const __grid_constant__ JArgs j) {
-  constexpr int NV = Phys<PHYS>::NV;
+template <typename T, int NV>
+__device__ __forceinline__ void gldv(const T* p, T (&x)[NV]) {
+  if constexpr (NV == 4 && sizeof(T) == 4) {
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
+  } else if constexpr (NV == 4 && sizeof(T) == 8) {
+    const double2 q0 = reinterpret_cast<const double2*>(p)[0], q1 = reinterpret_cast<const double2*>(p)[1];
+    x[0] = q0.x; x[1] = q0.y; x[2] = q1.x; x[3] = q1.y;
+  } else {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) x[v] = p[v];
+  }
+}
+template <typename T, int NV>
+__device__ __forceinline__ void gstv(T* p, const T (&x)[NV]) {
+  if constexpr (NV == 4 && sizeof(T) == 4) {
+    *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
+  } else if constexpr (NV == 4 && sizeof(T) == 8) {
+    reinterpret_cast<double2*>(p)[0] = make_double2(x[0], x[1]);
+    reinterpret_cast<double2*>(p)[1] = make_double2(x[2], x[3]);
+  } else {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) p[v] = x[v];
+  }
+}
+// o += c * p[0 .. NV)
+template <typename T, int NV>
+__device__ __forceinline__ void gfma(T c, const T* p, T (&o)[NV]) {
+  T t[NV];
+  gldv<T, NV>(p, t);
+#pragma unroll
+  for (int x = 0; x < NV; ++x) o[x] += c * t[x];
+}
+
+template <int N, int PHYS, typename T>
+__global__ void __launch_bounds__(JT, sizeof(T) == 4 ? (N <= 5 ? 3 : 2) : 1) k_gen_jacobian(
+    const __grid_constant__ PhysParams pp, const __grid_constant__ GArgs a, const __grid_constant__ JArgs j,
+    const int* __restrict__ list) {
+  constexpr int NV = Phys<PHYS>::NV, NS = N * N, NN = 4 * N, nA = NS * NV;
+  using W = JWork<N, NV, T>;
   using DT = Dual<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  JWork<NV, T>& w = *reinterpret_cast<JWork<NV, T>*>(smem_raw);
-  const int k = blockIdx.x;
-  if (k >= j.Eim) return;
+  W& w = *reinterpret_cast<W*>(smem_raw);
+  const int k = list[blockIdx.x];
   const int e = j.imp_idx[k];
   const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
-  const int n = a.deg[e], ns = n * n;
-  const int nA = ns * NV;
   const GenRef& RF = *a.ref;
   const bool visc = phys_viscous(pp);
   const PhysConst<T> pc = phys_const<T>(pp);
   const double* gs = a.geo_sol + (size_t)a.goff[e] * 5;
-  for (int i = tid; i < n * n; i += JT) w.M[i / n][i % n] = T(RF.M[n][i / n][i % n]);
-  if (tid < n) {
-    w.lm[tid] = T(RF.lm[n][tid]);
-    w.lp[tid] = T(RF.lp[n][tid]);
-    w.dgL[tid] = T(RF.dgL[n][tid]);
-    w.dgR[tid] = T(RF.dgR[n][tid]);
+  for (int i = tid; i < N * N; i += JT) w.M[i / N][i % N] = T(RF.M[N][i / N][i % N]);
+  if (tid < N) {
+    w.lm[tid] = T(RF.lm[N][tid]);
+    w.lp[tid] = T(RF.lp[N][tid]);
+    w.dgL[tid] = T(RF.dgL[N][tid]);
+    w.dgR[tid] = T(RF.dgR[N][tid]);
   }
   if (tid < 4) {
-    w.nf[tid] = a.nfp[4 * e + tid];
+    const int m = a.nfp[4 * e + tid];
+    w.nf[tid] = m;
     w.kf[tid] = a.kind[4 * e + tid];
     w.tr[tid] = a.tr_of[4 * e + tid];
     w.lto[tid] = j.lto[4 * k + tid];
+    w.own[tid] = (m == N && a.fset[4 * e + tid] == 0) ? 1 : 0;  // the element's own Gauss points
   }
   if (tid < 5) w.uinf[tid] = T(a.uinf[tid]);
-  for (int i = tid; i < ns; i += JT) {
+  if (tid == 0) {
+    int c = 0;
+    for (int f = 0; f < 4; ++f)
+      for (int q = 0; q < a.nfp[4 * e + f]; ++q) w.pt[c++] = f * GN + q;
+    w.npt = c;
+  }
+  for (int i = tid; i < NS; i += JT) {
     w.iJ[i] = T(gs[i * 5]);
     w.ciJ[i] = T(j.a_dt * gs[i * 5]);
     w.Sm[i][0][0] = T(gs[i * 5 + 1]);
@@ -559,97 +616,100 @@ __global__ void __launch_bounds__(JT, sizeof(T) == 4 ? 3 : 1) k_gen_jacobian(con
   }
   const double* Ue = a.U + a.uoff[e];
   for (int i = tid; i < nA; i += JT) w.U[i / NV][i % NV] = T(Ue[i]);
+  // the warps' tangent buffers: a line that a seed does not have is read with a zero factor
+  for (int i = tid; i < (int)(sizeof(w.col) / sizeof(T)); i += JT) reinterpret_cast<T*>(w.col)[i] = T(0);
   __syncthreads();
-  for (int i = tid; i < 4 * GN * GN; i += JT) {
-    const int f = i / (GN * GN), x = (i / GN) % GN, y = i % GN, m = w.nf[f];
+  for (int i = tid; i < 4 * GN * N; i += JT) {
+    const int f = i / (GN * N), x = (i / N) % GN, y = i % N, m = w.nf[f];
     const bool gll = a.fset[4 * e + f] != 0;
-    w.Tf[f][x][y] = (x < m && y < n) ? T(gll ? RF.TL[n][x][y] : RF.T[n][m][x][y]) : T(0);
-    w.Pf[f][x][y] = (x < n && y < m) ? T(gll ? RF.PL[n][x][y] : RF.P[n][m][x][y]) : T(0);
+    w.Tf[f][x][y] = x < m ? T(gll ? RF.TL[N][x][y] : RF.T[N][m][x][y]) : T(0);
+    w.Pf[f][y][x] = x < m ? T(gll ? RF.PL[N][y][x] : RF.P[N][m][y][x]) : T(0);
   }
   for (int jj = tid; jj < GF; jj += JT) {
     const int f = jj / GN, q = jj % GN;
-    w.wq[f][q] = q < w.nf[f] ? T(a.fset[4 * e + f] ? RF.wl[n][q] : RF.w[w.nf[f]][q]) : T(0);
+    w.wq[f][q] = q < w.nf[f] ? T(a.fset[4 * e + f] ? RF.wl[N][q] : RF.w[w.nf[f]][q]) : T(0);
     const double* G = a.geo_face + ((size_t)(4 * e + f) * GN + q) * 3;
     w.fJ[jj] = q < w.nf[f] ? T(G[0]) : T(0);
     w.fnr[jj][0] = q < w.nf[f] ? T(G[1]) : T(0);
     w.fnr[jj][1] = q < w.nf[f] ? T(G[2]) : T(0);
+    w.RU[jj] = T(0);
   }
-  for (int it = tid; it < 4 * n * NV; it += JT) {
-    const int f = it / (n * NV), b = (it / NV) % n, v = it % NV, r = f >> 1;
+  for (int it = tid; it < NN * NV; it += JT) {
+    const int f = it / (N * NV), b = (it / NV) % N, v = it % NV, r = f >> 1;
     const T* l = (f & 1) ? w.lp : w.lm;
     T s = T(0);
-    for (int c = 0; c < n; ++c) s += l[c] * w.U[gline(r, b, c, n)][v];
-    w.Ufn[f * GN + b][v] = s;
+#pragma unroll
+    for (int c = 0; c < N; ++c) s += l[c] * w.U[gline(r, b, c, N)][v];
+    w.Ufn[f * N + b][v] = s;
   }
   __syncthreads();
-  for (int it = tid; it < GF * NV; it += JT) {
-    const int f = it / (GN * NV), q = (it / NV) % GN, v = it % NV;
-    T s = T(0), ub = T(0), un = T(0);
-    if (q < w.nf[f]) {
-      for (int b = 0; b < n; ++b) s += w.Tf[f][q][b] * w.Ufn[f * GN + b][v];
-      const int t = w.tr[f];
-      if (t >= 0) {
-        ub = T(a.uhat[(size_t)FR_IDX(a.fnode[(4 * e + f) * GN + q], a.npts, 4) * NV + v]);
-        un = s;
-      } else {  // interface face of an implicit element: the explicit neighbour's state
-        const int nb = (int)FR_IDX(a.nbr[4 * e + f], a.E, 2), fn = (int)FR_IDX(a.nbr_face[4 * e + f], 4, 3);
-        un = T(a.Uf_all[((size_t)(4 * nb + fn) * GN + q) * NV + v]);
-        ub = un;
-      }
+  for (int it = tid; it < w.npt * NV; it += JT) {
+    const int jj = w.pt[it / NV], v = it % NV, f = jj / GN, q = jj % GN;
+    T s = T(0), ub, un;
+#pragma unroll
+    for (int b = 0; b < N; ++b) s += w.Tf[f][q][b] * w.Ufn[f * N + b][v];
+    if (w.tr[f] >= 0) {
+      ub = T(a.uhat[(size_t)FR_IDX(a.fnode[(4 * e + f) * GN + q], a.npts, 4) * NV + v]);
+      un = s;
+    } else {  // interface face of an implicit element: the explicit neighbour's state
+      const int nb = (int)FR_IDX(a.nbr[4 * e + f], a.E, 2), fn = (int)FR_IDX(a.nbr_face[4 * e + f], 4, 3);
+      un = T(a.Uf_all[((size_t)(4 * nb + fn) * GN + q) * NV + v]);
+      ub = un;
     }
-    w.Ufp[f * GN + q][v] = s;
-    w.ubp[f * GN + q][v] = ub;
-    w.un[f * GN + q][v] = un;
+    w.Ufp[jj][v] = s;
+    w.ubp[jj][v] = ub;
+    w.un[jj][v] = un;
   }
   __syncthreads();
-  for (int it = tid; it < 4 * GN * NV; it += JT) {
-    const int f = it / (GN * NV), b = (it / NV) % GN, v = it % NV;
-    T s = T(0);
-    if (b < n) {
-      s = w.Ufn[f * GN + b][v];
-      for (int q = 0; q < w.nf[f]; ++q) s += w.Pf[f][b][q] * (w.ubp[f * GN + q][v] - w.Ufp[f * GN + q][v]);
-    }
-    w.ubn[f * GN + b][v] = s;
+  for (int it = tid; it < NN * NV; it += JT) {
+    const int f = it / (N * NV), b = (it / NV) % N, v = it % NV;
+    T s = w.Ufn[f * N + b][v];
+    for (int q = 0; q < w.nf[f]; ++q) s += w.Pf[f][b][q] * (w.ubp[f * GN + q][v] - w.Ufp[f * GN + q][v]);
+    w.ubn[f * N + b][v] = s;
   }
   __syncthreads();
   if (visc) {
-    for (int it = tid; it < ns * NV; it += JT) {
-      const int i = it / NV, v = it % NV, ai = i % n, bi = i / n;
-      T q0 = w.dgL[ai] * w.ubn[0 * GN + bi][v] + w.dgR[ai] * w.ubn[1 * GN + bi][v];
-      T q1 = w.dgL[bi] * w.ubn[2 * GN + ai][v] + w.dgR[bi] * w.ubn[3 * GN + ai][v];
-      for (int c = 0; c < n; ++c) {
-        q0 += w.M[ai][c] * w.U[c + n * bi][v];
-        q1 += w.M[bi][c] * w.U[ai + n * c][v];
+    for (int it = tid; it < NS * NV; it += JT) {
+      const int i = it / NV, v = it % NV, ai = i % N, bi = i / N;
+      T q0 = w.dgL[ai] * w.ubn[0 * N + bi][v] + w.dgR[ai] * w.ubn[1 * N + bi][v];
+      T q1 = w.dgL[bi] * w.ubn[2 * N + ai][v] + w.dgR[bi] * w.ubn[3 * N + ai][v];
+#pragma unroll
+      for (int c = 0; c < N; ++c) {
+        q0 += w.M[ai][c] * w.U[c + N * bi][v];
+        q1 += w.M[bi][c] * w.U[ai + N * c][v];
       }
       w.q[i][0][v] = w.iJ[i] * (w.Sm[i][0][0] * q0 + w.Sm[i][1][0] * q1);
       w.q[i][1][v] = w.iJ[i] * (w.Sm[i][0][1] * q0 + w.Sm[i][1][1] * q1);
     }
     __syncthreads();
-    for (int it = tid; it < 4 * n * 2 * NV; it += JT) {
-      const int f = it / (n * 2 * NV), b = (it / (2 * NV)) % n, c2 = (it / NV) % 2, v = it % NV, r = f >> 1;
+    for (int it = tid; it < NN * 2 * NV; it += JT) {
+      const int f = it / (N * 2 * NV), b = (it / (2 * NV)) % N, c2 = (it / NV) % 2, v = it % NV, r = f >> 1;
       const T* l = (f & 1) ? w.lp : w.lm;
       T s = T(0);
-      for (int c = 0; c < n; ++c) s += l[c] * w.q[gline(r, b, c, n)][c2][v];
-      w.qfn[f * GN + b][c2][v] = s;
+#pragma unroll
+      for (int c = 0; c < N; ++c) s += l[c] * w.q[gline(r, b, c, N)][c2][v];
+      w.qfn[f * N + b][c2][v] = s;
     }
     __syncthreads();
-    for (int it = tid; it < GF * 2 * NV; it += JT) {
-      const int f = it / (GN * 2 * NV), q = (it / (2 * NV)) % GN, c2 = (it / NV) % 2, v = it % NV;
+    for (int it = tid; it < w.npt * 2 * NV; it += JT) {
+      const int jj = w.pt[it / (2 * NV)], c2 = (it / NV) % 2, v = it % NV, f = jj / GN, q = jj % GN;
       T s = T(0);
-      if (q < w.nf[f])
-        for (int b = 0; b < n; ++b) s += w.Tf[f][q][b] * w.qfn[f * GN + b][c2][v];
-      w.qfp[f * GN + q][c2][v] = s;
+#pragma unroll
+      for (int b = 0; b < N; ++b) s += w.Tf[f][q][b] * w.qfn[f * N + b][c2][v];
+      w.qfp[jj][c2][v] = s;
     }
   } else {
-    for (int i = tid; i < GNS * 2 * NV; i += JT) (&w.q[0][0][0])[i] = T(0);
+    for (int i = tid; i < NS * 2 * NV; i += JT) (&w.q[0][0][0])[i] = T(0);
     for (int i = tid; i < GF * 2 * NV; i += JT) (&w.qfp[0][0][0])[i] = T(0);
   }
   __syncthreads();
 
   // -------------------------------------------------- pointwise Jacobians
-  for (int it = tid; it < 2 * ns * NV; it += JT) {
-    const bool isq = it >= ns * NV;
-    const int idx = isq ? it - ns * NV : it;
+  constexpr int NI = (NS * NV + 31) / 32 * 32;  // state and gradient seeds in separate whole warps
+  for (int it = tid; it < 2 * NI; it += JT) {
+    const bool isq = it >= NI;
+    const int idx = isq ? it - NI : it;
+    if (idx >= NS * NV) continue;
     const int i = idx / NV, vp = idx % NV;
     DT u[NV], qd[2][NV], F[2][NV];
 #pragma unroll
@@ -704,10 +764,9 @@ __global__ void __launch_bounds__(JT, sizeof(T) == 4 ? 3 : 1) k_gen_jacobian(con
           for (int v = 0; v < NV; ++v) w.KQ[i][r][r2][v][vp] = acc[r][r2][v];
     }
   }
-  for (int it = tid; it < GF * 4 * NV; it += JT) {
-    const int jj = it / (4 * NV), dir = it % (4 * NV), grp = dir / NV, vp = dir % NV;
-    const int f = jj / GN, q = jj % GN;
-    const bool live = q < w.nf[f];
+  for (int it = tid; it < w.npt * 4 * NV; it += JT) {
+    const int jj = w.pt[it / (4 * NV)], dir = it % (4 * NV), grp = dir / NV, vp = dir % NV;
+    const int f = jj / GN;
     const int kf = w.kf[f];
     const bool traced = w.tr[f] >= 0;
     DT uf[NV], ub[NV], un[NV], qf[2][NV], qn[2][NV], Fn[NV], row[NV];
@@ -720,32 +779,28 @@ __global__ void __launch_bounds__(JT, sizeof(T) == 4 ? 3 : 1) k_gen_jacobian(con
       qf[1][v] = DT(w.qfp[jj][1][v], (grp == 3 && v == vp) ? T(1) : T(0));
       qn[0][v] = qn[1][v] = DT(T(0));
     }
-    const bool zero = !live || (grp >= 2 && !visc) || (grp == 1 && !traced);
+    const bool zero = (grp >= 2 && !visc) || (grp == 1 && !traced);
     if (!zero)
       gface_flux<PHYS, DT, T, NV>(pc, visc, kf, traced, true, uf, ub, qf, un, qn, w.fJ[jj], w.fnr[jj][0],
                                   w.fnr[jj][1], w.uinf, Fn, row);
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       const T d = zero ? T(0) : Fn[v].d;
-      const T dr = (zero || !traced) ? T(0) : row[v].d;
       if (grp == 0) {
         w.GU[jj][v][vp] = d;
-        w.RU[jj][v][vp] = dr;
+        // a far-field row moves with the state as J_f s 1
+        if (kf == FK_FAR && traced && v == 0 && vp == 0) w.RU[jj] = row[0].d;
       } else if (grp == 1) {
         w.GH[jj][v][vp] = d;
-        w.RH[jj][v][vp] = dr;
+        w.RH[jj][v][vp] = zero ? T(0) : row[v].d;
       } else {
         w.GQ[jj][grp - 2][v][vp] = d;
-        w.RQ[jj][grp - 2][v][vp] = dr;
       }
     }
   }
   __syncthreads();
 
   // -------------------------------------------------- columns, one seed point per warp
-  int nseed_tr = 0;
-  for (int f = 0; f < 4; ++f)
-    if (w.tr[f] >= 0) nseed_tr += w.nf[f];
   int nT = 0;
   for (int f = 0; f < 4; ++f) nT += w.nf[f] * NV;
   T* Ab = reinterpret_cast<T*>(j.A) + j.offA[k];
@@ -764,152 +819,200 @@ __global__ void __launch_bounds__(JT, sizeof(T) == 4 ? 3 : 1) k_gen_jacobian(con
         Db[(size_t)(rrow - nA) * nT + c] = T(0);
     }
   }
-  typename JWork<NV, T>::Col& cw = w.col[wp];
-  for (int sp = wp; sp < ns + nseed_tr; sp += JW) {
-    const bool vol = sp < ns;
-    int a0 = 0, b0 = 0, f0 = -1, q0 = -1;
-    if (vol) {
-      a0 = sp % n;
-      b0 = sp / n;
-    } else {
-      int rem = sp - ns;
-      for (int f = 0; f < 4; ++f) {
-        if (w.tr[f] < 0) continue;
-        if (rem < w.nf[f]) {
-          f0 = f;
-          q0 = rem;
-          break;
-        }
-        rem -= w.nf[f];
+  constexpr int G = 32 / NV;
+  const int vv = lane % NV, g = lane / NV;
+  typename W::Col& cw = w.col[wp];
+  const int npt = w.npt;
+  for (int sp = wp; sp < NS + npt; sp += JW) {
+    const bool vol = sp < NS;
+    const int j0 = vol ? -1 : w.pt[sp - NS];
+    const int f0 = vol ? 0 : j0 / GN, q0 = vol ? 0 : j0 % GN;
+    if (!vol && w.tr[f0] < 0) continue;
+    const bool line_seed = vol || w.own[f0];  // moves the gradient on its lines only
+    const bool has_row = vol || (line_seed && (f0 >> 1) == 0), has_col = vol || (line_seed && (f0 >> 1) == 1);
+    const int a0 = vol ? sp % N : q0, b0 = vol ? sp / N : q0;
+    const T* dgs = (f0 & 1) ? w.dgR : w.dgL;  // weights of a trace seed along the normal
+    const int r0 = f0 >> 1;
+    // reference-gradient tangents (dQ_xi, dQ_eta) at point c of line 0 (row b0) or 1 (column a0)
+    auto seed_dq = [&](int line, int c, T& dQ0, T& dQ1) {
+      if (line == 0) {
+        dQ0 = vol ? w.M[c][a0] : dgs[c];
+        dQ1 = (vol && c == a0) ? w.M[b0][b0] : T(0);
+      } else {
+        dQ1 = vol ? w.M[c][b0] : dgs[c];
+        dQ0 = (vol && c == b0) ? w.M[a0][a0] : T(0);
       }
-    }
-    // the tangents of the linear chain (face values, common values, gradients) depend on the seed
-    // point only: formed once for its NV columns
-    // face node and face point tangents of the state, trace tangent
-    for (int jj = lane; jj < GF; jj += 32) {
-      const int f = jj / GN, b = jj % GN, r = f >> 1;
-      T d = T(0);
-      if (vol && b < n) {
-        const T* l = (f & 1) ? w.lp : w.lm;
-        if (r == 0 && b == b0) d = l[a0];
-        if (r == 1 && b == a0) d = l[b0];
+    };
+    // dQ along r0 at point (ai, bi) of a trace seed that moves every point
+    auto dense_dq = [&](int ai, int bi) -> T {
+      return r0 == 0 ? dgs[ai] * w.Pf[f0][bi][q0] : dgs[bi] * w.Pf[f0][ai][q0];
+    };
+    if (line_seed && lane < 4 * N) {
+      const int line = lane / (2 * N), c = (lane >> 1) % N, c2 = lane & 1;
+      if (line == 0 ? has_row : has_col) {
+        const int pt = line == 0 ? c + N * b0 : a0 + N * c;
+        T d0, d1;
+        seed_dq(line, c, d0, d1);
+        cw.DQ[line][c][c2] = w.iJ[pt] * (w.Sm[pt][0][c2] * d0 + w.Sm[pt][1][c2] * d1);
       }
-      cw.dUfn[jj] = d;
-      cw.dubp[jj] = (!vol && f == f0 && b == q0) ? T(1) : T(0);
     }
     __syncwarp();
-    for (int jj = lane; jj < GF; jj += 32) {
-      const int f = jj / GN, q = jj % GN;
+    // gradient tangents at the face nodes; face state tangents at the face points
+    for (int it = lane; it < 2 * NN; it += 32) {
+      const int jn = it >> 1, c2 = it & 1, f = jn / N, b = jn % N, r = f >> 1;
+      const T* l = (f & 1) ? w.lp : w.lm;
       T s = T(0);
-      if (q < w.nf[f])
-        for (int b = 0; b < n; ++b) s += w.Tf[f][q][b] * cw.dUfn[f * GN + b];
-      cw.dUfp[jj] = s;
+      if (line_seed) {
+        const bool along = r == 0 ? (has_row && b == b0) : (has_col && b == a0);
+        if (along) {
+#pragma unroll
+          for (int c = 0; c < N; ++c) s += l[c] * cw.DQ[r][c][c2];
+        } else if (r == 0 ? has_col : has_row) {
+          s = r == 0 ? l[a0] * cw.DQ[1][b][c2] : l[b0] * cw.DQ[0][b][c2];
+        }
+      } else {
+#pragma unroll
+        for (int c = 0; c < N; ++c) {
+          const int pt = gline(r, b, c, N);
+          s += l[c] * (w.iJ[pt] * w.Sm[pt][r0][c2] * dense_dq(pt % N, pt / N));
+        }
+      }
+      cw.qn[jn][c2] = s;
+    }
+    for (int it = lane; it < npt; it += 32) {
+      const int jj = w.pt[it], f = jj / GN, q = jj % GN;
+      const T* l = (f & 1) ? w.lp : w.lm;
+      cw.du[jj] = !vol ? T(0) : ((f >> 1) == 0 ? w.Tf[f][q][b0] * l[a0] : w.Tf[f][q][a0] * l[b0]);
     }
     __syncwarp();
-    if (visc) {
-      for (int jj = lane; jj < GF; jj += 32) {
-        const int f = jj / GN, b = jj % GN;
-        T s = T(0);
-        if (b < n) {
-          s = cw.dUfn[jj];
-          for (int q = 0; q < w.nf[f]; ++q) s += w.Pf[f][b][q] * (cw.dubp[f * GN + q] - cw.dUfp[f * GN + q]);
+    for (int it = lane; it < 2 * npt; it += 32) {
+      const int jj = w.pt[it >> 1], c2 = it & 1, f = jj / GN, q = jj % GN;
+      T s;
+      if (w.own[f]) {
+        s = cw.qn[f * N + q][c2];
+      } else {
+        s = T(0);
+#pragma unroll
+        for (int b = 0; b < N; ++b) s += w.Tf[f][q][b] * cw.qn[f * N + b][c2];
+      }
+      cw.qp[jj][c2] = s;
+    }
+    __syncwarp();
+    // flux tangents on the lines and at the face points
+    for (int it = line_seed ? g : g + 2 * N; it < 2 * N + npt && g < G; it += G) {
+      if (it < 2 * N) {
+        const int line = it / N, c = it % N;
+        if (!(line == 0 ? has_row : has_col)) continue;
+        const int pt = line == 0 ? c + N * b0 : a0 + N * c;
+        T d0, d1;
+        seed_dq(line, c, d0, d1);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          T o[NV];
+#pragma unroll
+          for (int x = 0; x < NV; ++x) o[x] = T(0);
+          gfma<T, NV>(d0, &w.KQ[pt][r][0][vv][0], o);
+          gfma<T, NV>(d1, &w.KQ[pt][r][1][vv][0], o);
+          if (vol && pt == sp) gfma<T, NV>(T(1), &w.KU[pt][r][vv][0], o);
+          gstv<T, NV>(&cw.LN[line][c][(r * NV + vv) * NV], o);
         }
-        cw.dubn[jj] = s;
-      }
-      __syncwarp();
-      for (int i = lane; i < ns; i += 32) {
-        const int ai = i % n, bi = i / n;
-        T q0v = w.dgL[ai] * cw.dubn[0 * GN + bi] + w.dgR[ai] * cw.dubn[1 * GN + bi];
-        T q1v = w.dgL[bi] * cw.dubn[2 * GN + ai] + w.dgR[bi] * cw.dubn[3 * GN + ai];
-        if (vol && bi == b0) q0v += w.M[ai][a0];
-        if (vol && ai == a0) q1v += w.M[bi][b0];
-        cw.dQ[i][0] = q0v;
-        cw.dQ[i][1] = q1v;
-        cw.dq[i][0] = w.iJ[i] * (w.Sm[i][0][0] * q0v + w.Sm[i][1][0] * q1v);
-        cw.dq[i][1] = w.iJ[i] * (w.Sm[i][0][1] * q0v + w.Sm[i][1][1] * q1v);
-      }
-      __syncwarp();
-      for (int it = lane; it < GF * 2; it += 32) {
-        const int jj = it >> 1, c2 = it & 1, f = jj / GN, b = jj % GN, r = f >> 1;
-        T s = T(0);
-        if (b < n) {
-          const T* l = (f & 1) ? w.lp : w.lm;
-          for (int c = 0; c < n; ++c) s += l[c] * cw.dq[gline(r, b, c, n)][c2];
-        }
-        cw.dqfn[jj][c2] = s;
-      }
-      __syncwarp();
-      for (int it = lane; it < GF * 2; it += 32) {
-        const int jj = it >> 1, c2 = it & 1, f = jj / GN, q = jj % GN;
-        T s = T(0);
-        if (q < w.nf[f])
-          for (int b = 0; b < n; ++b) s += w.Tf[f][q][b] * cw.dqfn[f * GN + b][c2];
-        cw.dqfp[jj][c2] = s;
+      } else {
+        const int jj = w.pt[it - 2 * N];
+        T o[NV];
+#pragma unroll
+        for (int x = 0; x < NV; ++x) o[x] = T(0);
+        gfma<T, NV>(cw.qp[jj][0], &w.GQ[jj][0][vv][0], o);
+        gfma<T, NV>(cw.qp[jj][1], &w.GQ[jj][1][vv][0], o);
+        if (vol) gfma<T, NV>(cw.du[jj], &w.GU[jj][vv][0], o);
+        if (jj == j0) gfma<T, NV>(T(1), &w.GH[jj][vv][0], o);
+        gstv<T, NV>(&cw.FP[jj][vv * NV], o);
       }
     }
     __syncwarp();
-    // the seed point's NV columns, written column by column (the writes of one seed point's
-    // columns meet in the same sectors in L2)
+    // line sums, and the face fluxes projected to the nodes of faces with other points
+    for (int it = line_seed ? g : g + 2 * N; it < 2 * N + NN && g < G; it += G) {
+      T o[NV];
+#pragma unroll
+      for (int x = 0; x < NV; ++x) o[x] = T(0);
+      if (it < 2 * N) {
+        const int line = it / N, i = it % N;
+        if (!(line == 0 ? has_row : has_col)) continue;
+#pragma unroll
+        for (int c = 0; c < N; ++c) gfma<T, NV>(w.M[i][c], &cw.LN[line][c][(line * NV + vv) * NV], o);
+        gstv<T, NV>(&cw.RC[line][i][vv * NV], o);
+      } else {
+        const int jn = it - 2 * N, f = jn / N, b = jn % N;
+        if (w.own[f]) continue;
+        for (int q = 0; q < w.nf[f]; ++q) gfma<T, NV>(w.Pf[f][b][q], &cw.FP[f * GN + q][vv * NV], o);
+        gstv<T, NV>(&cw.FN[jn][vv * NV], o);
+      }
+    }
+    __syncwarp();
     const int col0 = vol ? sp * NV : w.lto[f0] + q0 * NV;
     const int ncol = vol ? nA : nT;
     T* top = vol ? Ab : Bb;
     T* bot = vol ? Cb : Db;
-    for (int v0 = 0; v0 < NV; ++v0) {
-      // flux tangents at the solution points
-      for (int it = lane; it < ns * 2 * NV; it += 32) {
-        const int i = it / (2 * NV), r = (it / NV) % 2, v = it % NV;
-        T s = T(0);
-        if (visc) s = w.KQ[i][r][0][v][v0] * cw.dQ[i][0] + w.KQ[i][r][1][v][v0] * cw.dQ[i][1];
-        if (vol && i == sp) s += w.KU[i][r][v][v0];
-        cw.dFt[i][r][v] = s;
-      }
-      // face-point flux and trace-row tangents
-      for (int it = lane; it < GF * NV; it += 32) {
-        const int jj = it / NV, v = it % NV, f = jj / GN, q = jj % GN;
-        T s = T(0), sr = T(0);
-        if (q < w.nf[f]) {
-          const T du = cw.dUfp[jj], dh = cw.dubp[jj];
-          s = w.GU[jj][v][v0] * du + w.GH[jj][v][v0] * dh;
-          sr = w.RU[jj][v][v0] * du + w.RH[jj][v][v0] * dh;
-          if (visc) {
-            s += w.GQ[jj][0][v][v0] * cw.dqfp[jj][0] + w.GQ[jj][1][v][v0] * cw.dqfp[jj][1];
-            sr += w.RQ[jj][0][v][v0] * cw.dqfp[jj][0] + w.RQ[jj][1][v][v0] * cw.dqfp[jj][1];
+    auto fnode = [&](int f, int b) -> const T* {
+      return w.own[f] ? &cw.FP[f * GN + b][vv * NV] : &cw.FN[f * N + b][vv * NV];
+    };
+    for (int it = g; it < NS + npt && g < G; it += G) {
+      T o[NV];
+#pragma unroll
+      for (int x = 0; x < NV; ++x) o[x] = T(0);
+      if (it < NS) {
+        // A / B rows: a dt / J times the divergence tangent (plus the identity of A)
+        const int ai = it % N, bi = it / N;
+        if (line_seed) {
+          const bool xrow = has_row && bi == b0, ycol = has_col && ai == a0;
+          const T cx = xrow ? T(1) : (has_col ? w.M[ai][a0] : T(0));
+          const T cy = ycol ? T(1) : (has_row ? w.M[bi][b0] : T(0));
+          gfma<T, NV>(cx, xrow ? &cw.RC[0][ai][vv * NV] : &cw.LN[1][bi][vv * NV], o);
+          gfma<T, NV>(cy, ycol ? &cw.RC[1][bi][vv * NV] : &cw.LN[0][ai][(NV + vv) * NV], o);
+        } else {
+#pragma unroll
+          for (int c = 0; c < N; ++c) {
+            gfma<T, NV>(w.M[ai][c] * dense_dq(c, bi), &w.KQ[c + N * bi][0][r0][vv][0], o);
+            gfma<T, NV>(w.M[bi][c] * dense_dq(ai, c), &w.KQ[ai + N * c][1][r0][vv][0], o);
           }
         }
-        cw.dFnp[jj][v] = s;
-        cw.drow[jj][v] = sr;
-      }
-      __syncwarp();
-      for (int it = lane; it < GF * NV; it += 32) {
-        const int jj = it / NV, v = it % NV, f = jj / GN, b = jj % GN;
-        T s = T(0);
-        if (b < n)
-          for (int q = 0; q < w.nf[f]; ++q) s += w.Pf[f][b][q] * cw.dFnp[f * GN + q][v];
-        cw.dFnn[jj][v] = s;
-      }
-      __syncwarp();
-      // A / B column: a dt / J times the divergence tangent (plus the identity of A)
-      for (int it = lane; it < nA; it += 32) {
-        const int i = it / NV, v = it % NV, ai = i % n, bi = i / n;
-        T d = -w.dgL[ai] * cw.dFnn[0 * GN + bi][v] + w.dgR[ai] * cw.dFnn[1 * GN + bi][v] -
-              w.dgL[bi] * cw.dFnn[2 * GN + ai][v] + w.dgR[bi] * cw.dFnn[3 * GN + ai][v];
-        for (int c = 0; c < n; ++c) d += w.M[ai][c] * cw.dFt[c + n * bi][0][v] + w.M[bi][c] * cw.dFt[ai + n * c][1][v];
-        T o = w.ciJ[i] * d;
-        if (vol && i == sp && v == v0) o += T(1);
-        top[(size_t)it * ncol + col0 + v0] = o;
-      }
-      // C / D column: the element's trace rows w_q (row tangent), zero off traces
-      for (int it = lane; it < nT; it += 32) {
-        int f = 0, rem = it;
-        while (rem >= w.nf[f] * NV) {
-          rem -= w.nf[f] * NV;
-          ++f;
+        gfma<T, NV>(-w.dgL[ai], fnode(0, bi), o);
+        gfma<T, NV>(w.dgR[ai], fnode(1, bi), o);
+        gfma<T, NV>(-w.dgL[bi], fnode(2, ai), o);
+        gfma<T, NV>(w.dgR[bi], fnode(3, ai), o);
+        const T cj = w.ciJ[it];
+#pragma unroll
+        for (int x = 0; x < NV; ++x) o[x] *= cj;
+        if (vol && it == sp) {
+#pragma unroll
+          for (int x = 0; x < NV; ++x)
+            if (x == vv) o[x] += T(1);
         }
-        const int q = rem / NV, v = rem % NV;
-        bot[(size_t)it * ncol + col0 + v0] = w.tr[f] >= 0 ? w.wq[f][q] * cw.drow[f * GN + q][v] : T(0);
+        gstv<T, NV>(top + (size_t)(it * NV + vv) * ncol + col0, o);
+      } else {
+        // C / D rows: w_q times the trace row's tangent, zero off traces.  Interior rows are the
+        // face flux; a wall keeps it in mass and energy and has rows of the trace alone in momentum;
+        // far-field rows are J_f s (u_f - u^) and the trace's own part
+        const int jj = w.pt[it - NS], f = jj / GN, q = jj % GN, kf = w.kf[f];
+        if (w.tr[f] >= 0) {
+          const bool wall = kf == FK_WALL && vv != 0 && vv != NV - 1;
+          if (!wall && kf != FK_FAR) {
+            gfma<T, NV>(T(1), &cw.FP[jj][vv * NV], o);
+          } else {
+            if (jj == j0) gfma<T, NV>(T(1), &w.RH[jj][vv][0], o);
+            if (kf == FK_FAR) {
+#pragma unroll
+              for (int x = 0; x < NV; ++x)
+                if (x == vv) o[x] += w.RU[jj] * cw.du[jj];
+            }
+          }
+          const T wm = w.wq[f][q];
+#pragma unroll
+          for (int x = 0; x < NV; ++x) o[x] *= wm;
+        }
+        gstv<T, NV>(bot + (size_t)(w.lto[f] + q * NV + vv) * ncol + col0, o);
       }
-      __syncwarp();
     }
+    __syncwarp();  // the next seed point rewrites this warp's buffers
   }
 }
 
@@ -1797,6 +1900,13 @@ int create(const fr_mesh_desc* mesh, const fr_config* cfg, cudaStream_t st, cons
     destroy(g);
     return FR_ERR_INVALID_ARG;
   }
+  // implicit elements by degree (points per line n: jl_off[n] .. jl_off[n + 1])
+  std::vector<int> jlist;
+  for (int n = 0; n <= GN + 1; ++n) {
+    g->jl_off[n] = (int)jlist.size();
+    for (int k = 0; k < Eim && n >= 2; ++k)
+      if (deg[imp_idx[k]] == n) jlist.push_back(k);
+  }
   // device memory
   int rc = FR_OK;
   const size_t pb = g->pb;
@@ -1821,6 +1931,7 @@ int create(const fr_mesh_desc* mesh, const fr_config* cfg, cudaStream_t st, cons
   g->imp_idx = galloc<int>(g, std::max(Eim, 1), &rc);
   g->exp_list = galloc<int>(g, std::max(g->Eex, 1), &rc);
   g->lto = galloc<int>(g, lto.size(), &rc);
+  g->jlist = galloc<int>(g, std::max(Eim, 1), &rc);
   g->nAk = galloc<int>(g, nAk.size(), &rc);
   g->nTk = galloc<int>(g, nTk.size(), &rc);
   g->gmap = galloc<int>(g, gmap.size(), &rc);
@@ -1907,6 +2018,7 @@ int create(const fr_mesh_desc* mesh, const fr_config* cfg, cudaStream_t st, cons
   GUP(g->poff, poff.data(), poff.size());
   GUP(g->imp_idx, imp_idx.data(), imp_idx.size());
   if (!exp_idx.empty()) GUP(g->exp_list, exp_idx.data(), exp_idx.size());
+  if (!jlist.empty()) GUP(g->jlist, jlist.data(), jlist.size());
   GUP(g->lto, lto.data(), lto.size());
   GUP(g->nAk, nAk.data(), nAk.size());
   GUP(g->nTk, nTk.data(), nTk.size());
@@ -2163,16 +2275,27 @@ int initial_trace(GenCtx* g, const double* u, double* uhat) {
   return FR_OK;
 }
 
+template <int N, int PHYS, typename T>
+static cudaError_t launch_gen_jac_n(GenCtx* g, const GArgs& a, const JArgs& j) {
+  const int n = g->jl_off[N + 1] - g->jl_off[N];
+  if (n == 0) return cudaSuccess;
+  const size_t smem = sizeof(JWork<N, Phys<PHYS>::NV, T>);
+  auto kern = k_gen_jacobian<N, PHYS, T>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  if (e != cudaSuccess) return e;
+  (count_launch(), kern<<<n, JT, smem, g->st>>>(g->pp, a, j, g->jlist + g->jl_off[N]));
+  return cudaGetLastError();
+}
+// the elements of each degree in a launch of their own, the largest first
 template <int PHYS, typename T>
 static cudaError_t launch_gen_jac(GenCtx* g, const GArgs& a, const JArgs& j) {
-  constexpr int NV = Phys<PHYS>::NV;
-  const size_t smem = sizeof(JWork<NV, T>);
-  auto kern = k_gen_jacobian<PHYS, T>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  if (j.Eim == 0) return cudaSuccess;
-  (count_launch(), kern<<<j.Eim, JT, smem, g->st>>>(g->pp, a, j));
-  return cudaGetLastError();
+  cudaError_t e = launch_gen_jac_n<6, PHYS, T>(g, a, j);
+  if (e == cudaSuccess) e = launch_gen_jac_n<5, PHYS, T>(g, a, j);
+  if (e == cudaSuccess) e = launch_gen_jac_n<4, PHYS, T>(g, a, j);
+  if (e == cudaSuccess) e = launch_gen_jac_n<3, PHYS, T>(g, a, j);
+  if (e == cudaSuccess) e = launch_gen_jac_n<2, PHYS, T>(g, a, j);
+  return e;
 }
 
 static int jacobian_blocks(GenCtx* g, const double* u, const double* uhat, double a_dt) {

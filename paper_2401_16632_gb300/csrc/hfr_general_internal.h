@@ -115,6 +115,8 @@ struct GenCtx {
   int* piv = nullptr;
   int* status = nullptr;
   int* exp_list = nullptr;  // the explicit elements (Eex)
+  int* jlist = nullptr;     // the implicit elements by degree: points per line n at jl_off[n] ..
+  int jl_off[GN + 2] = {};
   int Eex = 0;
   UnevenDev udev;
   // FP32 quadrilaterals: shape classes with the fixed-shape tensor-core condensation, condensed
