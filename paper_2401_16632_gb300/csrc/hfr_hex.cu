@@ -15,10 +15,8 @@
 // point met by the point's r-line.  Face kinds, common fluxes, trace rows and the viscous readings
 // are those of the quadrilateral path (one degree: face points are the element's face nodes).
 //
-// Element blocks are formed column by column (one warp per seed point, dense tangents through the
-// linear chain of the operator) and stored column-major, so that a warp writes its column as one
-// contiguous run; the pointwise Jacobians of a CTA's element live in a global slab of that CTA
-// (43 200 values for p = 3: too large for shared memory next to the column buffers).
+// Element blocks are formed column by column (one warp per seed point, tangents along the seed's
+// grid lines) and stored column-major, so that a warp writes its columns as contiguous runs.
 #include <math.h>
 #include <string.h>
 
@@ -33,7 +31,6 @@ constexpr int HNF = HN * HN;           // points per face
 constexpr int HFP = 6 * HNF;           // face points per element
 constexpr int HNV = 5;
 constexpr int HT = 128;                // threads of the residual kernel (one CTA per element)
-constexpr int HJT = 256, HJW = HJT / 32;  // block kernel
 
 // Navier-Stokes in three dimensions (ideal gas, R = 1, constant mu, Stokes hypothesis,
 // kappa = mu gamma / ((gamma - 1) Pr)); F[c][v], q[c][v] = du_v / dx_c
@@ -341,69 +338,97 @@ cudaError_t hex_elem_pass(GenCtx* g, const GArgs& a, int mode) {
 }
 
 // ------------------------------------------------------------------------ element blocks
-template <typename T>
+// One CTA per implicit element at a time.  Primal state, pointwise Jacobians by dual numbers, then
+// one warp per seed point (a solution point or a trace face point: HNV columns).  A seed moves the
+// reference gradient on the three grid lines through its point (a trace seed on the one line normal
+// to its face), so
+//   * the line through an output point along axis r meets them in one point at most, unless it is
+//     itself one of them: one product M dQ KQ per axis, or a line sum RC formed once per seed;
+//   * the face fluxes move at the 2N - 1 points of a face whose normal lines meet the seed's lines;
+//   * every other entry of the columns is zero (27 of 64 points and 54 of 96 face points at N = 4).
+// Lane = output row (coalesced column-major stores), HNV seed variables per lane.
+//
+// The pointwise Jacobians of an FP32 element (33 600 values at N = 4) stay in shared memory; in a
+// global slab per CTA, with every tangent of every point formed for each of the 800 columns, the
+// kernel took 21.8 ms on 4608 elements of N = 4; it takes 6.6 ms, bound by instruction issue (11.8 GB
+// of blocks are 1.7 ms of HBM).  FP64 keeps the slab (268 KB).
+template <typename T, int N>
+struct HJac {  // innermost index the input variable
+  static constexpr int NS = N * N * N, FP = 6 * N * N;
+  T KU[NS][3][HNV][HNV];
+  T KQ[NS][3][3][HNV][HNV];
+  T GU[FP][HNV][HNV], GH[FP][HNV][HNV], GQ[FP][3][HNV][HNV];
+  T RH[FP][HNV][HNV];  // boundary faces: the trace row by the trace
+};
+template <typename T, int N>
 struct HJWork {
-  T U[HNS][HNV];
-  T Uf[HFP][HNV], ub[HFP][HNV], un[HFP][HNV];
-  T q[HNS][3][HNV];
-  T qf[HFP][3][HNV];
-  T iJ[HNS], ciJ[HNS], Sm[HNS][3][3];
-  T fJ[HFP], fnr[HFP][3], wq[HNF];
-  T M[HN][HN], lm[HN], lp[HN], dgL[HN], dgR[HN];
-  T uinf[5];
-  struct Col {
-    T dQ[HNS][3], dq[HNS][3];
-    T dqf[HFP][3];
-    T dFt[HNS][3][HNV];
-    T dFn[HFP][HNV], drow[HFP][HNV];
-  } col[HJW];
+  static constexpr int NS = N * N * N, NF = N * N, FP = 6 * NF;
+  static constexpr int NW = sizeof(T) == 4 ? 12 : 8;  // warps of the CTA
+  T iJ[NS], ciJ[NS], Sm[NS][3][3], RU[FP];  // RU: far field, the row by the state (RU 1)
+  T M[N][N], lm[N], lp[N], dgL[N], dgR[N], wq[NF], uinf[5];
   int kf[6], tr[6];
+  struct Primal {
+    T U[NS][HNV];
+    T Uf[FP][HNV], ub[FP][HNV], un[FP][HNV];
+    T q[NS][3][HNV];
+    T qf[FP][3][HNV];
+    T fJ[FP], fnr[FP][3];
+  };
+  struct Col {  // tangents of one seed point, entries [v][v0]
+    T RC[3][N][HNV][HNV];       // line sums sum_s M[i][s] dF_r
+    T FN[6][2 * N][HNV][HNV];   // face fluxes at the active points (slots of hslot)
+    T SD[3][HNV][HNV];          // dF_r at the seed point itself
+    T DQ[3][N][3];              // physical gradient tangents on the lines
+    T qf[6][2 * N][3];          // gradient tangents at the active face points
+  };
+  union {
+    Primal pr;
+    Col col[NW];
+  };
 };
-static_assert(sizeof(HJWork<double>) <= 227 * 1024, "hexahedral block workspace exceeds shared memory");
+template <typename T, int N>
+constexpr size_t hex_jac_smem() {
+  return sizeof(HJWork<T, N>) + (sizeof(T) == 4 ? sizeof(HJac<T, N>) : 0);
+}
+static_assert(hex_jac_smem<float, HN>() <= 227 * 1024 && hex_jac_smem<double, HN>() <= 227 * 1024,
+              "hexahedral block workspace exceeds shared memory");
 
-// pointwise Jacobians of one element (global slab of the CTA), innermost index the input variable
-template <typename T>
-struct HJac {
-  T KU[HNS][3][HNV][HNV];
-  T KQ[HNS][3][3][HNV][HNV];
-  T GU[HFP][HNV][HNV], GH[HFP][HNV][HNV], GQ[HFP][3][HNV][HNV];
-  T RU[HFP][HNV][HNV], RH[HFP][HNV][HNV], RQ[HFP][3][HNV][HNV];
-};
-
-// NC: points per line as a compile-time constant (the index arithmetic of the lines folds), or 0
-// for the element's own degree at run time
-template <typename T, int NC>
-__global__ void __launch_bounds__(HJT, sizeof(T) == 4 ? 2 : 1) k_hex_jacobian(const __grid_constant__ PhysParams pp,
-                                                        const __grid_constant__ GArgs a,
-                                                        const __grid_constant__ JArgs j) {
+template <typename T, int N>
+__global__ void __launch_bounds__(32 * HJWork<T, N>::NW, 1) k_hex_jacobian(const __grid_constant__ PhysParams pp,
+                                                                         const __grid_constant__ GArgs a,
+                                                                         const __grid_constant__ JArgs j) {
   using DT = Dual<T>;
+  using W = HJWork<T, N>;
+  constexpr int ns = W::NS, nf = W::NF, NW = W::NW, NT = 32 * NW;
+  constexpr int nA = ns * HNV, nT = 6 * nf * HNV;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  HJWork<T>& w = *reinterpret_cast<HJWork<T>*>(smem_raw);
-  HJac<T>& J = reinterpret_cast<HJac<T>*>(j.scratch)[blockIdx.x];
+  W& w = *reinterpret_cast<W*>(smem_raw);
+  HJac<T, N>& J = sizeof(T) == 4 ? *reinterpret_cast<HJac<T, N>*>(smem_raw + sizeof(W))
+                                 : reinterpret_cast<HJac<T, N>*>(j.scratch)[blockIdx.x];
+  typename W::Primal& pr = w.pr;
   const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
   const bool visc = phys_viscous(pp);
   const PhysConst<T> pc = phys_const<T>(pp);
   const GenRef& RF = *a.ref;
+  const int FS = a.fs;
   for (int k = blockIdx.x; k < j.Eim; k += gridDim.x) {
     const int e = j.imp_idx[k];
-    const int n = NC > 0 ? NC : a.deg[e], ns = n * n * n, nf = n * n, FS = a.fs;
-    const int nA = ns * HNV, nT = 6 * nf * HNV;
     const double* gs = a.geo_sol + (size_t)a.goff[e] * 10;
     __syncthreads();  // the previous element's buffers are free
-    for (int i = tid; i < n * n; i += HJT) w.M[i / n][i % n] = T(RF.M[n][i / n][i % n]);
-    if (tid < n) {
-      w.lm[tid] = T(RF.lm[n][tid]);
-      w.lp[tid] = T(RF.lp[n][tid]);
-      w.dgL[tid] = T(RF.dgL[n][tid]);
-      w.dgR[tid] = T(RF.dgR[n][tid]);
+    for (int i = tid; i < N * N; i += NT) w.M[i / N][i % N] = T(RF.M[N][i / N][i % N]);
+    if (tid < N) {
+      w.lm[tid] = T(RF.lm[N][tid]);
+      w.lp[tid] = T(RF.lp[N][tid]);
+      w.dgL[tid] = T(RF.dgL[N][tid]);
+      w.dgR[tid] = T(RF.dgR[N][tid]);
     }
-    if (tid < nf) w.wq[tid] = T(RF.w[n][tid % n] * RF.w[n][tid / n]);
+    if (tid < nf) w.wq[tid] = T(RF.w[N][tid % N] * RF.w[N][tid / N]);
     if (tid < 6) {
       w.kf[tid] = a.kind[6 * e + tid];
       w.tr[tid] = a.tr_of[6 * e + tid];
     }
     if (tid < 5) w.uinf[tid] = T(a.uinf[tid]);
-    for (int i = tid; i < ns; i += HJT) {
+    for (int i = tid; i < ns; i += NT) {
       w.iJ[i] = T(gs[i * 10]);
       w.ciJ[i] = T(j.a_dt * gs[i * 10]);
 #pragma unroll
@@ -411,72 +436,76 @@ __global__ void __launch_bounds__(HJT, sizeof(T) == 4 ? 2 : 1) k_hex_jacobian(co
 #pragma unroll
         for (int c = 0; c < 3; ++c) w.Sm[i][r][c] = T(gs[i * 10 + 1 + 3 * r + c]);
     }
-    for (int jj = tid; jj < 6 * nf; jj += HJT) {
+    for (int jj = tid; jj < 6 * nf; jj += NT) {
       const double* G = a.geo_face + ((size_t)(6 * e + jj / nf) * FS + jj % nf) * 4;
-      w.fJ[jj] = T(G[0]);
-      w.fnr[jj][0] = T(G[1]);
-      w.fnr[jj][1] = T(G[2]);
-      w.fnr[jj][2] = T(G[3]);
+      pr.fJ[jj] = T(G[0]);
+      pr.fnr[jj][0] = T(G[1]);
+      pr.fnr[jj][1] = T(G[2]);
+      pr.fnr[jj][2] = T(G[3]);
+      w.RU[jj] = T(0);
     }
     const double* Ue = a.U + a.uoff[e];
-    for (int i = tid; i < nA; i += HJT) w.U[i / HNV][i % HNV] = T(Ue[i]);
+    for (int i = tid; i < nA; i += NT) pr.U[i / HNV][i % HNV] = T(Ue[i]);
     __syncthreads();
-    for (int it = tid; it < 6 * nf * HNV; it += HJT) {
+    for (int it = tid; it < 6 * nf * HNV; it += NT) {
       const int f = it / (nf * HNV), m = (it / HNV) % nf, v = it % HNV, r = f >> 1;
       const T* l = (f & 1) ? w.lp : w.lm;
       T s = T(0);
-      for (int c = 0; c < n; ++c) s += l[c] * w.U[hline(r, m, c, n)][v];
-      w.Uf[f * nf + m][v] = s;
+#pragma unroll
+      for (int c = 0; c < N; ++c) s += l[c] * pr.U[hline(r, m, c, N)][v];
+      pr.Uf[f * nf + m][v] = s;
       const int t = w.tr[f];
       if (t >= 0) {
-        w.ub[f * nf + m][v] = T(a.uhat[(size_t)FR_IDX(a.fnode[(6 * e + f) * FS + m], a.npts, 10) * HNV + v]);
-        w.un[f * nf + m][v] = s;
+        pr.ub[f * nf + m][v] = T(a.uhat[(size_t)FR_IDX(a.fnode[(6 * e + f) * FS + m], a.npts, 10) * HNV + v]);
+        pr.un[f * nf + m][v] = s;
       } else {  // interface face: the explicit neighbour's state
         const int nb = (int)FR_IDX(a.nbr[6 * e + f], a.E, 11), fn = (int)FR_IDX(a.nbr_face[6 * e + f], 6, 12);
         const T un = T(a.Uf_all[((size_t)(6 * nb + fn) * FS + m) * HNV + v]);
-        w.un[f * nf + m][v] = un;
-        w.ub[f * nf + m][v] = un;
+        pr.un[f * nf + m][v] = un;
+        pr.ub[f * nf + m][v] = un;
       }
     }
     __syncthreads();
     if (visc) {
-      for (int it = tid; it < ns * HNV; it += HJT) {
+      for (int it = tid; it < ns * HNV; it += NT) {
         const int i = it / HNV, v = it % HNV;
         T Q[3];
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
-          const int ar = hcoord(i, r, n), m = hfacept(i, r, n);
-          T s = w.dgL[ar] * w.ub[(2 * r) * nf + m][v] + w.dgR[ar] * w.ub[(2 * r + 1) * nf + m][v];
-          for (int c = 0; c < n; ++c) s += w.M[ar][c] * w.U[hline(r, m, c, n)][v];
+          const int ar = hcoord(i, r, N), m = hfacept(i, r, N);
+          T s = w.dgL[ar] * pr.ub[(2 * r) * nf + m][v] + w.dgR[ar] * pr.ub[(2 * r + 1) * nf + m][v];
+#pragma unroll
+          for (int c = 0; c < N; ++c) s += w.M[ar][c] * pr.U[hline(r, m, c, N)][v];
           Q[r] = s;
         }
 #pragma unroll
-        for (int c = 0; c < 3; ++c) w.q[i][c][v] = w.iJ[i] * (w.Sm[i][0][c] * Q[0] + w.Sm[i][1][c] * Q[1] + w.Sm[i][2][c] * Q[2]);
+        for (int c = 0; c < 3; ++c) pr.q[i][c][v] = w.iJ[i] * (w.Sm[i][0][c] * Q[0] + w.Sm[i][1][c] * Q[1] + w.Sm[i][2][c] * Q[2]);
       }
       __syncthreads();
-      for (int it = tid; it < 6 * nf * 3 * HNV; it += HJT) {
+      for (int it = tid; it < 6 * nf * 3 * HNV; it += NT) {
         const int f = it / (nf * 3 * HNV), m = (it / (3 * HNV)) % nf, c2 = (it / HNV) % 3, v = it % HNV, r = f >> 1;
         const T* l = (f & 1) ? w.lp : w.lm;
         T s = T(0);
-        for (int c = 0; c < n; ++c) s += l[c] * w.q[hline(r, m, c, n)][c2][v];
-        w.qf[f * nf + m][c2][v] = s;
+#pragma unroll
+        for (int c = 0; c < N; ++c) s += l[c] * pr.q[hline(r, m, c, N)][c2][v];
+        pr.qf[f * nf + m][c2][v] = s;
       }
     } else {
-      for (int i = tid; i < HNS * 3 * HNV; i += HJT) (&w.q[0][0][0])[i] = T(0);
-      for (int i = tid; i < HFP * 3 * HNV; i += HJT) (&w.qf[0][0][0])[i] = T(0);
+      for (int i = tid; i < ns * 3 * HNV; i += NT) (&pr.q[0][0][0])[i] = T(0);
+      for (int i = tid; i < 6 * nf * 3 * HNV; i += NT) (&pr.qf[0][0][0])[i] = T(0);
     }
     __syncthreads();
-    // pointwise Jacobians (dual numbers) into the CTA's slab
-    for (int it = tid; it < 2 * ns * HNV; it += HJT) {
+    // ---- pointwise Jacobians (dual numbers)
+    for (int it = tid; it < 2 * ns * HNV; it += NT) {
       const bool isq = it >= ns * HNV;
       const int idx = isq ? it - ns * HNV : it;
       const int i = idx / HNV, vp = idx % HNV;
       DT u[HNV], qd[3][HNV], F[3][HNV];
 #pragma unroll
       for (int v = 0; v < HNV; ++v) {
-        u[v] = DT(w.U[i][v], (!isq && v == vp) ? T(1) : T(0));
+        u[v] = DT(pr.U[i][v], (!isq && v == vp) ? T(1) : T(0));
 #pragma unroll
-        for (int c = 0; c < 3; ++c) qd[c][v] = DT(w.q[i][c][v]);
+        for (int c = 0; c < 3; ++c) qd[c][v] = DT(pr.q[i][c][v]);
       }
       if (!isq) {
         NS3::conv<DT, T>(pc, u, F);
@@ -525,7 +554,7 @@ __global__ void __launch_bounds__(HJT, sizeof(T) == 4 ? 2 : 1) k_hex_jacobian(co
             for (int v = 0; v < HNV; ++v) J.KQ[i][r][r2][v][vp] = acc[r][r2][v];
       }
     }
-    for (int it = tid; it < 6 * nf * 5 * HNV; it += HJT) {
+    for (int it = tid; it < 6 * nf * 5 * HNV; it += NT) {
       const int jj = it / (5 * HNV), dir = it % (5 * HNV), grp = dir / HNV, vp = dir % HNV;
       const int f = jj / nf;
       const int kf = w.kf[f];
@@ -533,38 +562,36 @@ __global__ void __launch_bounds__(HJT, sizeof(T) == 4 ? 2 : 1) k_hex_jacobian(co
       DT uf[HNV], ub[HNV], un[HNV], qf[3][HNV], qn[3][HNV], Fn[HNV], row[HNV];
 #pragma unroll
       for (int v = 0; v < HNV; ++v) {
-        uf[v] = DT(w.Uf[jj][v], (grp == 0 && v == vp) ? T(1) : T(0));
-        ub[v] = DT(w.ub[jj][v], (grp == 1 && v == vp) ? T(1) : T(0));
-        un[v] = DT(w.un[jj][v]);
+        uf[v] = DT(pr.Uf[jj][v], (grp == 0 && v == vp) ? T(1) : T(0));
+        ub[v] = DT(pr.ub[jj][v], (grp == 1 && v == vp) ? T(1) : T(0));
+        un[v] = DT(pr.un[jj][v]);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          qf[c][v] = DT(w.qf[jj][c][v], (grp == 2 + c && v == vp) ? T(1) : T(0));
+          qf[c][v] = DT(pr.qf[jj][c][v], (grp == 2 + c && v == vp) ? T(1) : T(0));
           qn[c][v] = DT(T(0));
         }
       }
       const bool zero = (grp >= 2 && !visc) || (grp == 1 && !traced);
       if (!zero) {
-        const T nr[3] = {w.fnr[jj][0], w.fnr[jj][1], w.fnr[jj][2]};
-        hface_flux<DT, T>(pc, visc, kf, traced, true, uf, ub, qf, un, qn, w.fJ[jj], nr, w.uinf, Fn, row);
+        const T nr[3] = {pr.fnr[jj][0], pr.fnr[jj][1], pr.fnr[jj][2]};
+        hface_flux<DT, T>(pc, visc, kf, traced, true, uf, ub, qf, un, qn, pr.fJ[jj], nr, w.uinf, Fn, row);
       }
 #pragma unroll
       for (int v = 0; v < HNV; ++v) {
         const T d = zero ? T(0) : Fn[v].d;
-        const T dr = (zero || !traced) ? T(0) : row[v].d;
         if (grp == 0) {
           J.GU[jj][v][vp] = d;
-          J.RU[jj][v][vp] = dr;
+          if (kf == FK_FAR && traced && v == 0 && vp == 0) w.RU[jj] = row[0].d;  // J_f s
         } else if (grp == 1) {
           J.GH[jj][v][vp] = d;
-          J.RH[jj][v][vp] = dr;
+          J.RH[jj][v][vp] = zero ? T(0) : row[v].d;
         } else {
           J.GQ[jj][grp - 2][v][vp] = d;
-          J.RQ[jj][grp - 2][v][vp] = dr;
         }
       }
     }
-    __syncthreads();
-    // columns, one seed point per warp (column-major blocks: one contiguous run per column)
+    __syncthreads();  // the primal arrays give way to the column buffers
+    // ---- columns, one seed point per warp (column-major blocks: one contiguous run per column)
     T* AT = reinterpret_cast<T*>(j.A) + j.offA[k];
     T* BT = reinterpret_cast<T*>(j.B) + j.offB[k];
     T* CT = reinterpret_cast<T*>(j.C) + j.offB[k];
@@ -572,7 +599,7 @@ __global__ void __launch_bounds__(HJT, sizeof(T) == 4 ? 2 : 1) k_hex_jacobian(co
     // trace unknowns of faces without a trace: zero columns of B and D
     for (int f = 0; f < 6; ++f) {
       if (w.tr[f] >= 0) continue;
-      for (int it = tid; it < nf * HNV * (nA + nT); it += HJT) {
+      for (int it = tid; it < nf * HNV * (nA + nT); it += NT) {
         const int col = f * nf * HNV + it / (nA + nT), rr = it % (nA + nT);
         if (rr < nA)
           BT[(size_t)col * nA + rr] = T(0);
@@ -580,165 +607,230 @@ __global__ void __launch_bounds__(HJT, sizeof(T) == 4 ? 2 : 1) k_hex_jacobian(co
           DTm[(size_t)col * nT + rr - nA] = T(0);
       }
     }
-    typename HJWork<T>::Col& cw = w.col[wp];
-    int nseed_tr = 0;
-    for (int f = 0; f < 6; ++f)
-      if (w.tr[f] >= 0) nseed_tr += nf;
-    for (int sp = wp; sp < ns + nseed_tr; sp += HJW) {
+    typename W::Col& cw = w.col[wp];
+    for (int sp = wp; sp < ns + 6 * nf; sp += NW) {
       const bool vol = sp < ns;
-      int f0 = -1, m0 = -1;
-      if (!vol) {
-        int rem = sp - ns;
-        for (int f = 0; f < 6; ++f) {
-          if (w.tr[f] < 0) continue;
-          if (rem < nf) {
-            f0 = f;
-            m0 = rem;
-            break;
-          }
-          rem -= nf;
-        }
-      }
+      const int f0 = vol ? -1 : (sp - ns) / nf, m0 = vol ? 0 : (sp - ns) % nf;
+      if (!vol && w.tr[f0] < 0) continue;
       const int r0 = vol ? -1 : f0 >> 1;
-      // the gradient tangents depend on the seed point only: formed once for its HNV columns
-      // reference and physical gradient tangents (the seed's lines only)
-      if (visc) {
-        for (int i = lane; i < ns; i += 32) {
-          T Q[3];
+      // seed coordinates; along the normal of a trace seed none (-1): its line runs there
+      const int sx = vol ? hcoord(sp, 0, N) : (r0 == 0 ? -1 : m0 % N);
+      const int sy = vol ? hcoord(sp, 1, N) : (r0 == 1 ? -1 : (r0 == 0 ? m0 % N : m0 / N));
+      const int sz = vol ? hcoord(sp, 2, N) : (r0 == 2 ? -1 : m0 / N);
+      const T* dg = (f0 & 1) ? w.dgR : w.dgL;  // a trace seed's weights along its line (f0 >= 0)
+      auto sc = [&](int r) { return r == 0 ? sx : (r == 1 ? sy : sz); };
+      // reference-gradient tangent along axis r at coordinate s of the seed's line along r
+      auto line_dq = [&](int r, int s) -> T { return vol ? w.M[s][sc(r)] : dg[s]; };
+      // the lines through face point (i, j) of axis r along its two tangential axes
+      auto match = [&](int r, int i, int jx, bool& A, bool& B) -> bool {
+        A = i == (r == 0 ? sy : sx);
+        B = jx == (r == 2 ? sy : sz);
+        return r == r0 ? (A && B) : (A || B);
+      };
+      // physical gradient tangents on the seed's lines (line r: the points that vary along r)
+      for (int it = lane; it < 9 * N; it += 32) {
+        const int r = it / (3 * N), s = (it / 3) % N, c = it % 3;
+        if (!vol && r != r0) continue;
+        const int m = vol ? hfacept(sp, r, N) : m0, pt = hline(r, m, s, N);
+        T d = line_dq(r, s) * w.Sm[pt][r][c];
+        if (vol && s == sc(r)) {
 #pragma unroll
-          for (int r = 0; r < 3; ++r) {
-            T s = T(0);
-            if (vol) {  // on sp's r-line: M[a_r(i)][a_r(sp)]
-              if (hfacept(i, r, n) == hfacept(sp, r, n)) s = w.M[hcoord(i, r, n)][hcoord(sp, r, n)];
-            } else if (r == r0 && hfacept(i, r, n) == m0) {
-              s = (f0 & 1) ? w.dgR[hcoord(i, r, n)] : w.dgL[hcoord(i, r, n)];
-            }
-            Q[r] = s;
-            cw.dQ[i][r] = s;
-          }
-#pragma unroll
-          for (int c = 0; c < 3; ++c)
-            cw.dq[i][c] = w.iJ[i] * (w.Sm[i][0][c] * Q[0] + w.Sm[i][1][c] * Q[1] + w.Sm[i][2][c] * Q[2]);
+          for (int r2 = 0; r2 < 3; ++r2)
+            if (r2 != r) d += w.M[sc(r2)][sc(r2)] * w.Sm[pt][r2][c];
         }
-        __syncwarp();
-        for (int it = lane; it < 6 * nf * 3; it += 32) {
-          const int jj = it / 3, c2 = it % 3, f = jj / nf, m = jj % nf, r = f >> 1;
-          const T* l = (f & 1) ? w.lp : w.lm;
-          T s = T(0);
-          for (int c = 0; c < n; ++c) s += l[c] * cw.dq[hline(r, m, c, n)][c2];
-          cw.dqf[jj][c2] = s;
+        cw.DQ[r][s][c] = w.iJ[pt] * d;
+      }
+      if (vol) {  // flux tangents at the seed point
+        for (int it = lane; it < 3 * HNV; it += 32) {
+          const int r = it / HNV, v = it % HNV;
+#pragma unroll
+          for (int x = 0; x < HNV; ++x) {
+            T o = J.KU[sp][r][v][x];
+#pragma unroll
+            for (int r2 = 0; r2 < 3; ++r2) o += J.KQ[sp][r][r2][v][x] * w.M[sc(r2)][sc(r2)];
+            cw.SD[r][v][x] = o;
+          }
         }
       }
       __syncwarp();
-      for (int v0 = 0; v0 < HNV; ++v0) {
-        // flux tangents at the solution points (the gradient tangent vanishes off the seed's lines:
-        // the pointwise Jacobians are read only where a tangent is nonzero)
-        for (int it = lane; it < ns * 3 * HNV; it += 32) {
-          const int i = it / (3 * HNV), r = (it / HNV) % 3, v = it % HNV;
-          T s = T(0);
-          if (visc) {
-            const T q0 = cw.dQ[i][0], q1 = cw.dQ[i][1], q2 = cw.dQ[i][2];
-            if (q0 != T(0) || q1 != T(0) || q2 != T(0))
-              s = J.KQ[i][r][0][v][v0] * q0 + J.KQ[i][r][1][v][v0] * q1 + J.KQ[i][r][2][v][v0] * q2;
-          }
-          if (vol && i == sp) s += J.KU[i][r][v][v0];
-          cw.dFt[i][r][v] = s;
-        }
-        // face flux and trace-row tangents
-        for (int it = lane; it < 6 * nf * HNV; it += 32) {
-          const int jj = it / HNV, v = it % HNV, f = jj / nf, m = jj % nf, r = f >> 1;
-          T du = T(0);  // face state tangent: l_sigma[a_r(sp)] on the face point of sp's r-line
-          if (vol && hfacept(sp, r, n) == m) du = ((f & 1) ? w.lp : w.lm)[hcoord(sp, r, n)];
-          const T dh = (!vol && f == f0 && m == m0) ? T(1) : T(0);
-          T s = T(0), sr = T(0);
-          if (du != T(0)) {
-            s += J.GU[jj][v][v0] * du;
-            sr += J.RU[jj][v][v0] * du;
-          }
-          if (dh != T(0)) {
-            s += J.GH[jj][v][v0] * dh;
-            sr += J.RH[jj][v][v0] * dh;
-          }
-          if (visc) {
+      // gradient tangents at the active face points: slot a (first tangential coordinate that of the
+      // seed) at the second coordinate, slot N + b (second that of the seed) at the first
+      for (int it = lane; it < 6 * 2 * N * 3; it += 32) {
+        const int f = it / (6 * N), sl = (it / 3) % (2 * N), c = it % 3, r = f >> 1;
+        const int t0 = r == 0 ? 1 : 0, t1 = r == 2 ? 1 : 2;
+        const int i = sl < N ? sc(t0) : sl - N, jx = sl < N ? sl : sc(t1);
+        if (i < 0 || jx < 0) continue;
+        bool A, B;
+        if (!match(r, i, jx, A, B)) continue;
+        const T* l = (f & 1) ? w.lp : w.lm;
+        T s = T(0);
+        if (A && B) {  // the normal line is the seed's own
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              const T dq = cw.dqf[jj][c];
-              if (dq != T(0)) {
-                s += J.GQ[jj][c][v][v0] * dq;
-                sr += J.RQ[jj][c][v][v0] * dq;
-              }
+          for (int c1 = 0; c1 < N; ++c1) s += l[c1] * cw.DQ[r][c1][c];
+        } else {  // it meets the seed's line along t1 (A) or t0 (B) in one point
+          s = l[sc(r)] * (A ? cw.DQ[t1][jx][c] : cw.DQ[t0][i][c]);
+        }
+        cw.qf[f][sl][c] = s;
+      }
+      // line sums
+      for (int it = lane; it < 3 * N * HNV; it += 32) {
+        const int r = it / (N * HNV), i = (it / HNV) % N, v = it % HNV;
+        if (!vol && r != r0) continue;
+        const int m = vol ? hfacept(sp, r, N) : m0;
+        T o[HNV];
+#pragma unroll
+        for (int x = 0; x < HNV; ++x) o[x] = T(0);
+#pragma unroll
+        for (int s = 0; s < N; ++s) {
+          if (vol && s == sc(r)) {
+#pragma unroll
+            for (int x = 0; x < HNV; ++x) o[x] += w.M[i][s] * cw.SD[r][v][x];
+          } else {
+            const T cf = w.M[i][s] * line_dq(r, s);
+            const T* kq = &J.KQ[hline(r, m, s, N)][r][r][v][0];
+#pragma unroll
+            for (int x = 0; x < HNV; ++x) o[x] += cf * kq[x];
+          }
+        }
+#pragma unroll
+        for (int x = 0; x < HNV; ++x) cw.RC[r][i][v][x] = o[x];
+      }
+      __syncwarp();
+      // face flux tangents at the active points
+      for (int it = lane; it < 6 * 2 * N * HNV; it += 32) {
+        const int f = it / (2 * N * HNV), sl = (it / HNV) % (2 * N), v = it % HNV, r = f >> 1;
+        const int t0 = r == 0 ? 1 : 0, t1 = r == 2 ? 1 : 2;
+        const int i = sl < N ? sc(t0) : sl - N, jx = sl < N ? sl : sc(t1);
+        if (i < 0 || jx < 0) continue;
+        bool A, B;
+        if (!match(r, i, jx, A, B)) continue;
+        const int jj = f * nf + i + N * jx;
+        const T q0 = cw.qf[f][sl][0], q1 = cw.qf[f][sl][1], q2 = cw.qf[f][sl][2];
+        T o[HNV];
+#pragma unroll
+        for (int x = 0; x < HNV; ++x)
+          o[x] = J.GQ[jj][0][v][x] * q0 + J.GQ[jj][1][v][x] * q1 + J.GQ[jj][2][v][x] * q2;
+        if (vol && A && B) {  // the face state on the seed's own normal line
+          const T du = ((f & 1) ? w.lp : w.lm)[sc(r)];
+#pragma unroll
+          for (int x = 0; x < HNV; ++x) o[x] += J.GU[jj][v][x] * du;
+        }
+        if (f == f0 && A && B) {
+#pragma unroll
+          for (int x = 0; x < HNV; ++x) o[x] += J.GH[jj][v][x];
+        }
+#pragma unroll
+        for (int x = 0; x < HNV; ++x) cw.FN[f][sl][v][x] = o[x];
+      }
+      __syncwarp();
+      const int col = vol ? sp * HNV : (f0 * nf + m0) * HNV;
+      T* top = (vol ? AT : BT) + (size_t)col * nA;
+      T* bot = (vol ? CT : DTm) + (size_t)col * nT;
+      // A / B columns: a dt / J times the divergence tangent (plus the identity of A)
+      for (int it = lane; it < nA; it += 32) {
+        const int pt = it / HNV, v = it % HNV;
+        T o[HNV];
+#pragma unroll
+        for (int x = 0; x < HNV; ++x) o[x] = T(0);
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+          const int t0 = r == 0 ? 1 : 0, t1 = r == 2 ? 1 : 2;
+          const int ar = hcoord(pt, r, N), i = hcoord(pt, t0, N), jx = hcoord(pt, t1, N);
+          bool A, B;
+          if (!match(r, i, jx, A, B)) continue;
+          if (A && B) {
+#pragma unroll
+            for (int x = 0; x < HNV; ++x) o[x] += cw.RC[r][ar][v][x];
+          } else {  // (sc(r) >= 0: a trace seed along r has A and B together)
+            const int tl = A ? t1 : t0, s = A ? jx : i;
+            const T cf = w.M[ar][sc(r)] * line_dq(tl, s);
+            const T* kq = &J.KQ[hline(r, i + N * jx, sc(r), N)][r][tl][v][0];
+#pragma unroll
+            for (int x = 0; x < HNV; ++x) o[x] += cf * kq[x];
+          }
+          const int sl = A ? jx : N + i;
+          const T gl = -w.dgL[ar], gr = w.dgR[ar];
+          const T* fl = &cw.FN[2 * r][sl][v][0];
+          const T* fr = &cw.FN[2 * r + 1][sl][v][0];
+#pragma unroll
+          for (int x = 0; x < HNV; ++x) o[x] += gl * fl[x] + gr * fr[x];
+        }
+        const T cj = w.ciJ[pt];
+#pragma unroll
+        for (int x = 0; x < HNV; ++x) {
+          T y = cj * o[x];
+          if (vol && it == col + x) y += T(1);
+          top[(size_t)x * nA + it] = y;
+        }
+      }
+      // C / D columns: w_q times the trace row's tangent (walls: momentum rows of the trace alone;
+      // far field: J_f s (u_f - u^) and the trace's own part)
+      for (int it = lane; it < nT; it += 32) {
+        const int jj = it / HNV, v = it % HNV, f = jj / nf, m = jj % nf, r = f >> 1, kf = w.kf[f];
+        T o[HNV];
+#pragma unroll
+        for (int x = 0; x < HNV; ++x) o[x] = T(0);
+        bool A, B;
+        if (w.tr[f] >= 0 && match(r, m % N, m / N, A, B)) {
+          const bool wall = kf == FK_WALL && v != 0 && v != HNV - 1;
+          if (!wall && kf != FK_FAR) {
+            const T* fn = &cw.FN[f][A ? m / N : N + m % N][v][0];
+#pragma unroll
+            for (int x = 0; x < HNV; ++x) o[x] = fn[x];
+          } else {
+            if (f == f0 && m == m0) {
+#pragma unroll
+              for (int x = 0; x < HNV; ++x) o[x] = J.RH[jj][v][x];
+            }
+            if (kf == FK_FAR && vol && A && B) {
+              const T du = w.RU[jj] * ((f & 1) ? w.lp : w.lm)[sc(r)];
+#pragma unroll
+              for (int x = 0; x < HNV; ++x)
+                if (x == v) o[x] += du;
             }
           }
-          cw.dFn[jj][v] = s;
-          cw.drow[jj][v] = sr;
-        }
-        __syncwarp();
-        const int col = vol ? sp * HNV + v0 : (f0 * nf + m0) * HNV + v0;
-        T* top = (vol ? AT : BT) + (size_t)col * nA;
-        T* bot = (vol ? CT : DTm) + (size_t)col * nT;
-        for (int it = lane; it < nA; it += 32) {
-          const int i = it / HNV, v = it % HNV;
-          T d = T(0);
+          const T wm = w.wq[m];
 #pragma unroll
-          for (int r = 0; r < 3; ++r) {
-            const int ar = hcoord(i, r, n), m = hfacept(i, r, n);
-            d += -w.dgL[ar] * cw.dFn[(2 * r) * nf + m][v] + w.dgR[ar] * cw.dFn[(2 * r + 1) * nf + m][v];
-            for (int c = 0; c < n; ++c) d += w.M[ar][c] * cw.dFt[hline(r, m, c, n)][r][v];
-          }
-          T o = w.ciJ[i] * d;
-          if (vol && it == col) o += T(1);
-          top[it] = o;
+          for (int x = 0; x < HNV; ++x) o[x] *= wm;
         }
-        for (int it = lane; it < nT; it += 32) {
-          const int jj = it / HNV, v = it % HNV, f = jj / nf, m = jj % nf;
-          bot[it] = w.tr[f] >= 0 ? w.wq[m] * cw.drow[jj][v] : T(0);
-        }
-        __syncwarp();
+#pragma unroll
+        for (int x = 0; x < HNV; ++x) bot[(size_t)x * nT + it] = o[x];
       }
+      __syncwarp();
     }
   }
 }
 
-// the kernel for a mesh whose elements all have n points per line (hexahedral meshes carry one
-// degree), the run-time form otherwise
-template <typename T>
-static auto hex_jac_kernel(int n) -> decltype(&k_hex_jacobian<T, 0>) {
-  switch (n) {
-    case 2: return &k_hex_jacobian<T, 2>;
-    case 3: return &k_hex_jacobian<T, 3>;
-    case 4: return &k_hex_jacobian<T, 4>;
-    default: return &k_hex_jacobian<T, 0>;
-  }
-}
-
 int hex_jacobian_grid(int prec_bytes) {
+  (void)prec_bytes;
   int dev = 0, nsm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  return nsm * (prec_bytes == 8 ? 1 : 2);
+  return nsm;
 }
 
 size_t hex_jacobian_scratch_bytes(int prec_bytes, int grid) {
-  return (size_t)grid * (prec_bytes == 8 ? sizeof(HJac<double>) : sizeof(HJac<float>));
+  return prec_bytes == 8 ? (size_t)grid * sizeof(HJac<double, HN>) : 0;  // FP32 keeps them in shared memory
 }
 
-cudaError_t hex_jacobian(GenCtx* g, const GArgs& a, const JArgs& j) {
-  cudaError_t e;
-  if (j.Eim == 0) return cudaSuccess;
-  if (g->pb == 8) {
-    const size_t smem = sizeof(HJWork<double>);
-    auto kern = hex_jac_kernel<double>(g->h_deg.empty() ? 0 : g->h_deg[0]);
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-      return e;
-    (count_launch(), kern<<<g->jgrid, HJT, smem, g->st>>>(g->pp, a, j));
-  } else {
-    const size_t smem = sizeof(HJWork<float>);
-    auto kern = hex_jac_kernel<float>(g->h_deg.empty() ? 0 : g->h_deg[0]);
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-      return e;
-    (count_launch(), kern<<<g->jgrid, HJT, smem, g->st>>>(g->pp, a, j));
-  }
+template <typename T, int N>
+static cudaError_t hex_jac_launch(GenCtx* g, const GArgs& a, const JArgs& j) {
+  const size_t smem = hex_jac_smem<T, N>();
+  auto kern = k_hex_jacobian<T, N>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  (count_launch(), kern<<<g->jgrid, 32 * HJWork<T, N>::NW, smem, g->st>>>(g->pp, a, j));
   return cudaGetLastError();
+}
+cudaError_t hex_jacobian(GenCtx* g, const GArgs& a, const JArgs& j) {
+  if (j.Eim == 0) return cudaSuccess;
+  const bool f64 = g->pb == 8;
+  switch (g->h_deg.empty() ? 0 : g->h_deg[0]) {  // hexahedral meshes carry one degree
+    case 2: return f64 ? hex_jac_launch<double, 2>(g, a, j) : hex_jac_launch<float, 2>(g, a, j);
+    case 3: return f64 ? hex_jac_launch<double, 3>(g, a, j) : hex_jac_launch<float, 3>(g, a, j);
+    case 4: return f64 ? hex_jac_launch<double, 4>(g, a, j) : hex_jac_launch<float, 4>(g, a, j);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 // ------------------------------------------------------------------------ geometry (host)
