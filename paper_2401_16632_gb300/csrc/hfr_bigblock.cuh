@@ -9,8 +9,8 @@
 //      memory (permuted columns in, forward and back substitution by factor panels, X out once);
 //   4. S = D - C X_B, in FP32 on the tensor cores, in FP64 by the same batched GEMM;
 //   5. t = s - C x_r with FP64 accumulation (one CTA per element).
-// The batched GEMM is a register-tiled CUDA-core kernel: 128 x 128 output tiles in FP32 (64 x 64 in
-// FP64), 256 threads with 8 x 8 (4 x 4) outputs each, K staged through two shared-memory buffers 8
+// The batched GEMM is a register-tiled CUDA-core kernel: 128 x 128 output tiles in FP32 (32 x 32 in
+// FP64), 256 threads with 8 x 8 (2 x 2) outputs each, K staged through two shared-memory buffers 8
 // at a time; arithmetic in the block precision T.  Included by hfr_condense.cu (uses UnevenArgs and DEV_ERR_*).
 #pragma once
 
@@ -77,7 +77,9 @@ __global__ void __launch_bounds__(BT) k_big_lu_panel(const __grid_constant__ Une
   constexpr int LB = lu_panel<T>(), PS = LB + 1;
   extern __shared__ __align__(16) unsigned char lu_smem[];
   T* P = reinterpret_cast<T*>(lu_smem);
-  __shared__ T rkey_v[BT / 32];
+  using Key = decltype(abs_key(T(0)));
+  __shared__ Key rkey_v[BT / 32];
+  __shared__ T s_inv;
   __shared__ int rkey_i[BT / 32];
   __shared__ int spiv[LB];
   __shared__ int s_bad;
@@ -97,18 +99,18 @@ __global__ void __launch_bounds__(BT) k_big_lu_panel(const __grid_constant__ Une
     if (tid == 0) s_bad = 0;
     __syncthreads();
     for (int c = 0; c < w; ++c) {
-      T bv = T(-1);
+      Key bv = -1;
       int bi = 0x7fffffff;
       for (int r = c + tid; r < R; r += BT) {
-        const T v = fabs(P[r * PS + c]);
-        if (v > bv || (v == bv && r < bi)) {
+        const Key v = abs_key(P[r * PS + c]);
+        if (v > bv || (v == bv && v >= 0 && r < bi)) {
           bv = v;
           bi = r;
         }
       }
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) {
-        const T ov = __shfl_xor_sync(0xffffffffu, bv, off);
+        const Key ov = __shfl_xor_sync(0xffffffffu, bv, off);
         const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
         if (ov > bv || (ov == bv && oi < bi)) {
           bv = ov;
@@ -121,7 +123,7 @@ __global__ void __launch_bounds__(BT) k_big_lu_panel(const __grid_constant__ Une
       }
       __syncthreads();
       if (tid == 0) {
-        T v = rkey_v[0];
+        Key v = rkey_v[0];
         int ii = rkey_i[0];
         for (int q = 1; q < BT / 32; ++q)
           if (rkey_v[q] > v || (rkey_v[q] == v && rkey_i[q] < ii)) {
@@ -129,7 +131,10 @@ __global__ void __launch_bounds__(BT) k_big_lu_panel(const __grid_constant__ Une
             ii = rkey_i[q];
           }
         spiv[c] = ii;
-        if (!(v > T(0))) s_bad = 1;
+        if (!(v > 0))
+          s_bad = 1;
+        else
+          s_inv = T(1) / P[ii * PS + c];  // once: a division by every warp held the FP64 pipe longest
       }
       __syncthreads();
       if (s_bad) break;
@@ -141,7 +146,7 @@ __global__ void __launch_bounds__(BT) k_big_lu_panel(const __grid_constant__ Une
           P[pr * PS + x] = u;
         }
       __syncthreads();
-      const T inv = T(1) / P[c * PS + c];
+      const T inv = s_inv;
       for (int r = c + 1 + tid; r < R; r += BT) {
         const T l = P[r * PS + c] * inv;
         P[r * PS + c] = l;
@@ -476,8 +481,11 @@ __global__ void __launch_bounds__(32 * NW, 512 / (32 * NW)) k_big_solve(const __
 // shared-memory stages with the next stage's global values held in registers meanwhile.
 template <typename T>
 struct GemmCfg {
-  static constexpr int TM = sizeof(T) == 8 ? 4 : 8;  // outputs per thread and dimension
-  static constexpr int H = TM / 2;                   // one 16-byte vector
+  // outputs per thread and dimension.  FP64: 32 x 32 tiles, so that blocks of 96 to 144 leave few idle
+  // lanes (64 x 64 tiles computed 16 384 outputs for the 9 216 of a 96 x 96 block); the FP64 pipe, not
+  // the shared memory that a larger tile saves, is the limit
+  static constexpr int TM = sizeof(T) == 8 ? 2 : 8;
+  static constexpr int H = TM / 2;                   // FP32: one 16-byte vector
   static constexpr int BM = 16 * TM;                 // output tile (rows = columns)
   static constexpr int GKK = 8;                      // k per stage
   static constexpr int PAD = 16 / sizeof(T);
@@ -486,9 +494,7 @@ struct GemmCfg {
 template <typename T>
 __device__ __forceinline__ void gemm_vec_ld(const T* p, T (&v)[GemmCfg<T>::H]) {
   if constexpr (sizeof(T) == 8) {
-    const double2 x = *reinterpret_cast<const double2*>(p);
-    v[0] = x.x;
-    v[1] = x.y;
+    v[0] = *p;
   } else {
     const float4 x = *reinterpret_cast<const float4*>(p);
     v[0] = x.x;

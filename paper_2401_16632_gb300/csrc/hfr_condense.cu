@@ -23,6 +23,16 @@ namespace hfr {
 
 template <typename T>
 __device__ __forceinline__ T tabs(T x) { return x < T(0) ? -x : x; }
+// |x| as an integer that orders as |x| does, -1 for NaN: pivot searches compare these on the integer
+// pipes (an FP64 comparison occupies the FP64 pipe as long as a multiply-add of a whole warp)
+__device__ __forceinline__ long long abs_key(double x) {
+  const long long k = __double_as_longlong(x) & 0x7fffffffffffffffll;
+  return k > 0x7ff0000000000000ll ? -1 : k;
+}
+__device__ __forceinline__ int abs_key(float x) {
+  const int k = __float_as_int(x) & 0x7fffffff;
+  return k > 0x7f800000 ? -1 : k;
+}
 
 // ------------------------------------------------------------------ register-tiled kernel
 // 256 threads = 16 row groups x 16 column groups; thread (rg, cg) owns physical rows
@@ -1852,6 +1862,9 @@ __device__ void condense_smem_elem(const CondElem<T>& e, unsigned char* smem_raw
   int* sflag = lpiv + nA;  // [0] pivot row of the step, [1] zero pivot seen
   unsigned char* used = reinterpret_cast<unsigned char*>(sflag + 2);
   const int lane = tid & 31, wid = tid >> 5, nw = nth >> 5;
+  __shared__ T s_invs[1 + 8];  // the step's reciprocal pivot, one per thread group (its barrier id)
+  T& s_inv = s_invs[bar];
+  using Key = decltype(abs_key(T(0)));
   int& s_p = sflag[0];
   int& s_bad = sflag[1];
   for (int i = tid; i < nA * nc; i += nth) {
@@ -1863,16 +1876,16 @@ __device__ void condense_smem_elem(const CondElem<T>& e, unsigned char* smem_raw
   grp_sync(bar, nth);
   for (int c = 0; c < nA; ++c) {
     if (tid < 32) {
-      T best = T(-1);
+      Key best = -1;
       int bi = 0x7fffffff;
       for (int r = tid; r < nA; r += 32) {
         if (used[r]) continue;
-        const T v = tabs(M[(size_t)r * nc + c]);
-        if (v > best || (v == best && r < bi)) { best = v; bi = r; }
+        const Key v = abs_key(M[(size_t)r * nc + c]);
+        if (v > best || (v == best && v >= 0 && r < bi)) { best = v; bi = r; }
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
-        const T ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const Key ob = __shfl_xor_sync(0xffffffffu, best, o);
         const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
         if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
       }
@@ -1883,13 +1896,15 @@ __device__ void condense_smem_elem(const CondElem<T>& e, unsigned char* smem_raw
         ipiv[bi] = c;
         lpiv[c] = bi;
         e.piv[c] = bi;
-        if (!(best > T(0))) s_bad = 1;
+        if (!(best > 0)) s_bad = 1;
+        // once per step: a division by every warp took a third of the FP64 pipe at nA = 100
+        const T pv = M[(size_t)bi * nc + c];
+        s_inv = pv != T(0) ? T(1) / pv : T(0);
       }
     }
     grp_sync(bar, nth);
     const int p = s_p;
-    const T pv = M[(size_t)p * nc + c];
-    const T inv = pv != T(0) ? T(1) / pv : T(0);
+    const T inv = s_inv;
     for (int j = tid; j < nc; j += nth) pr[j] = j == c ? inv : M[(size_t)p * nc + j] * inv;
     for (int r = tid; r < nA; r += nth) cb[r] = M[(size_t)r * nc + c];
     grp_sync(bar, nth);
@@ -2458,7 +2473,10 @@ __global__ void k_inv_apply(int Eim, int nA, const T* __restrict__ AinvT, const 
 // ---------------------------------------------------------------- LU kernel (FP64 path)
 // LU with partial pivoting (full-row interchanges) of A applied to [B | r] in shared memory,
 // then back substitution: X = A^{-1}[B | r] with nA^3/3 + nA^2 (nT+1) multiply-adds, ~25 % fewer
-// than Gauss-Jordan, which is what counts where the FP64 pipe is the roof.  Keeps LU + piv.
+// than Gauss-Jordan, which is what counts where the FP64 pipe is the roof.  Keeps LU + piv.  The
+// pivot searches compare integers and each reciprocal is formed once: comparisons on the FP64 pipe
+// and a division by each of the eight warps took a quarter of it (4096 blocks of 64 / 64: 7.15 ->
+// 5.55 ms; the products alone are 4.8 ms at the measured FP64 rate).
 constexpr int LU_THREADS = 256;
 
 template <typename T>
@@ -2470,6 +2488,8 @@ __global__ void __launch_bounds__(LU_THREADS) k_condense_lu(const __grid_constan
   const int rows2 = nA > nT ? nA : nT;
   T* sA = reinterpret_cast<T*>(smem_raw);  // rows2 x nA (A, later C)
   T* sX = sA + (size_t)rows2 * nA;          // nA x (nT + 1)
+  T* sI = sX + (size_t)nA * ldx;            // nA reciprocal pivots
+  using Key = decltype(abs_key(T(0)));
   __shared__ int s_piv;
   __shared__ int s_bad;
   const T* gA = reinterpret_cast<const T*>(a.A) + (size_t)k * nA * nA;
@@ -2486,22 +2506,24 @@ __global__ void __launch_bounds__(LU_THREADS) k_condense_lu(const __grid_constan
   int* piv = a.piv + (size_t)k * nA;
   for (int c = 0; c < nA; ++c) {
     if (tid < 32) {
-      T best = T(-1);
+      Key best = -1;
       int bi = c;
       for (int i = c + tid; i < nA; i += 32) {
-        T v = tabs(sA[i * nA + c]);
+        const Key v = abs_key(sA[i * nA + c]);
         if (v > best) { best = v; bi = i; }
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
-        T ov = __shfl_xor_sync(0xffffffffu, best, o);
+        const Key ov = __shfl_xor_sync(0xffffffffu, best, o);
         int oi = __shfl_xor_sync(0xffffffffu, bi, o);
         if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
       }
       if (tid == 0) {
         s_piv = bi;
         piv[c] = bi;
-        if (!(best > T(0)) || best != best) s_bad = 1;
+        if (!(best > 0)) s_bad = 1;
+        const T pv = sA[bi * nA + c];
+        sI[c] = pv != T(0) ? T(1) / pv : T(0);
       }
     }
     __syncthreads();
@@ -2519,8 +2541,7 @@ __global__ void __launch_bounds__(LU_THREADS) k_condense_lu(const __grid_constan
       }
     }
     __syncthreads();
-    const T pv = sA[c * nA + c];
-    const T inv = pv != T(0) ? T(1) / pv : T(0);
+    const T inv = sI[c];
     for (int i = c + 1 + tid; i < nA; i += LU_THREADS) sA[i * nA + c] *= inv;
     __syncthreads();
     const int nr = nA - c - 1;
@@ -2542,8 +2563,7 @@ __global__ void __launch_bounds__(LU_THREADS) k_condense_lu(const __grid_constan
   }
   // back substitution with U
   for (int c = nA - 1; c >= 0; --c) {
-    const T pv = sA[c * nA + c];
-    const T inv = pv != T(0) ? T(1) / pv : T(0);
+    const T inv = sI[c];
     for (int j = tid; j < ldx; j += LU_THREADS) sX[c * ldx + j] *= inv;
     __syncthreads();
     for (int it = tid; it < c * ldx; it += LU_THREADS) {
@@ -2711,7 +2731,7 @@ static cudaError_t cond_dispatch(const CondArgs& a, cudaStream_t st, int part) {
 template <typename T>
 static cudaError_t cond_lu(const CondArgs& a, cudaStream_t st) {
   const int rows2 = a.nA > a.nT ? a.nA : a.nT;
-  size_t smem = sizeof(T) * ((size_t)rows2 * a.nA + (size_t)a.nA * (a.nT + 1));
+  size_t smem = sizeof(T) * ((size_t)rows2 * a.nA + (size_t)a.nA * (a.nT + 1) + a.nA);
   if (smem > 227 * 1024) return cond_dispatch<T>(a, st, 0);
   cudaError_t err = cudaFuncSetAttribute(k_condense_lu<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
@@ -2727,7 +2747,7 @@ int condense_tc_available(int prec_bytes, int nA, int nT) {
 
 static bool lu_fits_smem(int prec_bytes, int nA, int nT) {
   const int rows2 = nA > nT ? nA : nT;
-  return prec_bytes == 8 && sizeof(double) * ((size_t)rows2 * nA + (size_t)nA * (nT + 1)) <= 227 * 1024;
+  return prec_bytes == 8 && sizeof(double) * ((size_t)rows2 * nA + (size_t)nA * (nT + 1) + nA) <= 227 * 1024;
 }
 static bool reg_shape(int nA, int nT) {
   return (nA == 9 && nT == 12) || (nA == 16 && nT == 16) || (nA == 36 && nT == 48) || (nA == 64 && nT == 64) ||
