@@ -711,14 +711,14 @@ __global__ void __launch_bounds__(JT, sizeof(T) == 4 ? (N <= 5 ? 3 : 2) : 1) k_g
     const int idx = isq ? it - NI : it;
     if (idx >= NS * NV) continue;
     const int i = idx / NV, vp = idx % NV;
-    DT u[NV], qd[2][NV], F[2][NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      u[v] = DT(w.U[i][v], (!isq && v == vp) ? T(1) : T(0));
-      qd[0][v] = DT(w.q[i][0][v]);
-      qd[1][v] = DT(w.q[i][1][v]);
-    }
     if (!isq) {
+      DT u[NV], qd[2][NV], F[2][NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        u[v] = DT(w.U[i][v], v == vp ? T(1) : T(0));
+        qd[0][v] = DT(w.q[i][0][v]);
+        qd[1][v] = DT(w.q[i][1][v]);
+      }
       Phys<PHYS>::template conv<DT, T>(pc, u, F);
       if (visc) {
         DT Fv[2][NV];
@@ -733,6 +733,7 @@ __global__ void __launch_bounds__(JT, sizeof(T) == 4 ? (N <= 5 ? 3 : 2) : 1) k_g
 #pragma unroll
         for (int v = 0; v < NV; ++v) w.KU[i][r][v][vp] = w.Sm[i][r][0] * F[0][v].d + w.Sm[i][r][1] * F[1][v].d;
     } else {
+      // only the viscous flux depends on the gradient, and linearly: its value at a unit gradient
       T acc[2][2][NV];
 #pragma unroll
       for (int r = 0; r < 2; ++r)
@@ -741,16 +742,25 @@ __global__ void __launch_bounds__(JT, sizeof(T) == 4 ? (N <= 5 ? 3 : 2) : 1) k_g
 #pragma unroll
           for (int v = 0; v < NV; ++v) acc[r][r2][v] = T(0);
       if (visc) {
+        T u[NV], qe[2][NV], F[2][NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          u[v] = w.U[i][v];
+          qe[0][v] = qe[1][v] = T(0);
+        }
 #pragma unroll
         for (int c2 = 0; c2 < 2; ++c2) {
-          qd[c2][vp].d = T(1);
-          Phys<PHYS>::template visc<DT, T>(pc, u, qd, F);
-          qd[c2][vp].d = T(0);
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            qe[c2][v] = v == vp ? T(1) : T(0);
+            qe[1 - c2][v] = T(0);
+          }
+          Phys<PHYS>::template visc<T, T>(pc, u, qe, F);
 #pragma unroll
           for (int r = 0; r < 2; ++r)
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
-              const T dFr = -(w.Sm[i][r][0] * F[0][v].d + w.Sm[i][r][1] * F[1][v].d);
+              const T dFr = -(w.Sm[i][r][0] * F[0][v] + w.Sm[i][r][1] * F[1][v]);  // d F~_r / d q_{c2}
 #pragma unroll
               for (int r2 = 0; r2 < 2; ++r2) acc[r][r2][v] += dFr * w.iJ[i] * w.Sm[i][r2][c2];
             }
@@ -764,37 +774,67 @@ __global__ void __launch_bounds__(JT, sizeof(T) == 4 ? (N <= 5 ? 3 : 2) : 1) k_g
           for (int v = 0; v < NV; ++v) w.KQ[i][r][r2][v][vp] = acc[r][r2][v];
     }
   }
-  for (int it = tid; it < w.npt * 4 * NV; it += JT) {
-    const int jj = w.pt[it / (4 * NV)], dir = it % (4 * NV), grp = dir / NV, vp = dir % NV;
-    const int f = jj / GN;
+  // face: items (face point, input variable), each kind of input in whole warps: 0 the trace (dual
+  // numbers), 1 the face state (on a traced face the flux moves with it as J_f s 1; interface faces
+  // by dual numbers), 2 and 3 the gradient (linear: the viscous flux at a unit gradient)
+  const int FI = (w.npt * NV + 31) / 32 * 32;
+  for (int it = tid; it < 4 * FI; it += JT) {
+    const int grp = it / FI, idx = it % FI;
+    if (idx >= w.npt * NV) continue;
+    const int jj = w.pt[idx / NV], vp = idx % NV, f = jj / GN;
     const int kf = w.kf[f];
     const bool traced = w.tr[f] >= 0;
-    DT uf[NV], ub[NV], un[NV], qf[2][NV], qn[2][NV], Fn[NV], row[NV];
+    const T n0 = w.fnr[jj][0], n1 = w.fnr[jj][1], Jf = w.fJ[jj];
+    T d[NV], dr[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      uf[v] = DT(w.Ufp[jj][v], (grp == 0 && v == vp) ? T(1) : T(0));
-      ub[v] = DT(w.ubp[jj][v], (grp == 1 && v == vp) ? T(1) : T(0));
-      un[v] = DT(w.un[jj][v]);
-      qf[0][v] = DT(w.qfp[jj][0][v], (grp == 2 && v == vp) ? T(1) : T(0));
-      qf[1][v] = DT(w.qfp[jj][1][v], (grp == 3 && v == vp) ? T(1) : T(0));
-      qn[0][v] = qn[1][v] = DT(T(0));
+    for (int v = 0; v < NV; ++v) d[v] = dr[v] = T(0);
+    if (grp >= 2) {
+      if (visc) {
+        T u[NV], qe[2][NV], F[2][NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          u[v] = traced ? w.ubp[jj][v] : w.Ufp[jj][v];
+          qe[0][v] = (grp == 2 && v == vp) ? T(1) : T(0);
+          qe[1][v] = (grp == 3 && v == vp) ? T(1) : T(0);
+        }
+        // faces without a trace between solved elements average both sides' viscous fluxes
+        const T Ja = (!traced && (kf == FK_FR || kf == FK_FAR)) ? T(0.5) * Jf : Jf;
+        Phys<PHYS>::template visc<T, T>(pc, u, qe, F);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) d[v] = -Ja * (n0 * F[0][v] + n1 * F[1][v]);
+      }
+    } else if (grp == 1 && traced) {
+      const T s = Jf * Phys<PHYS>::template stab<T, T>(pc, w.ubp[jj], n0, n1);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) d[v] = v == vp ? s : T(0);
+      if (kf == FK_FAR && vp == 0) w.RU[jj] = s;  // a far-field row moves with the state as J_f s 1
+    } else if (grp == 1 || traced) {
+      DT uf[NV], ub[NV], un[NV], qf[2][NV], qn[2][NV], Fn[NV], row[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        uf[v] = DT(w.Ufp[jj][v], (grp == 1 && v == vp) ? T(1) : T(0));
+        ub[v] = DT(w.ubp[jj][v], (grp == 0 && v == vp) ? T(1) : T(0));
+        un[v] = DT(w.un[jj][v]);
+        qf[0][v] = DT(w.qfp[jj][0][v]);
+        qf[1][v] = DT(w.qfp[jj][1][v]);
+        qn[0][v] = qn[1][v] = DT(T(0));
+      }
+      gface_flux<PHYS, DT, T, NV>(pc, visc, kf, traced, true, uf, ub, qf, un, qn, Jf, n0, n1, w.uinf, Fn, row);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        d[v] = Fn[v].d;
+        dr[v] = row[v].d;
+      }
     }
-    const bool zero = (grp >= 2 && !visc) || (grp == 1 && !traced);
-    if (!zero)
-      gface_flux<PHYS, DT, T, NV>(pc, visc, kf, traced, true, uf, ub, qf, un, qn, w.fJ[jj], w.fnr[jj][0],
-                                  w.fnr[jj][1], w.uinf, Fn, row);
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      const T d = zero ? T(0) : Fn[v].d;
       if (grp == 0) {
-        w.GU[jj][v][vp] = d;
-        // a far-field row moves with the state as J_f s 1
-        if (kf == FK_FAR && traced && v == 0 && vp == 0) w.RU[jj] = row[0].d;
+        w.GH[jj][v][vp] = d[v];
+        w.RH[jj][v][vp] = dr[v];
       } else if (grp == 1) {
-        w.GH[jj][v][vp] = d;
-        w.RH[jj][v][vp] = zero ? T(0) : row[v].d;
+        w.GU[jj][v][vp] = d[v];
       } else {
-        w.GQ[jj][grp - 2][v][vp] = d;
+        w.GQ[jj][grp - 2][v][vp] = d[v];
       }
     }
   }

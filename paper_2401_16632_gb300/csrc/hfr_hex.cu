@@ -496,18 +496,21 @@ __global__ void __launch_bounds__(32 * HJWork<T, N>::NW, 1) k_hex_jacobian(const
     }
     __syncthreads();
     // ---- pointwise Jacobians (dual numbers)
-    for (int it = tid; it < 2 * ns * HNV; it += NT) {
-      const bool isq = it >= ns * HNV;
-      const int idx = isq ? it - ns * HNV : it;
+    // volume: state and gradient seeds in separate whole warps
+    constexpr int NI = (ns * HNV + 31) / 32 * 32, FI = (6 * nf * HNV + 31) / 32 * 32;
+    for (int it = tid; it < 2 * NI; it += NT) {
+      const bool isq = it >= NI;
+      const int idx = isq ? it - NI : it;
+      if (idx >= ns * HNV) continue;
       const int i = idx / HNV, vp = idx % HNV;
-      DT u[HNV], qd[3][HNV], F[3][HNV];
-#pragma unroll
-      for (int v = 0; v < HNV; ++v) {
-        u[v] = DT(pr.U[i][v], (!isq && v == vp) ? T(1) : T(0));
-#pragma unroll
-        for (int c = 0; c < 3; ++c) qd[c][v] = DT(pr.q[i][c][v]);
-      }
       if (!isq) {
+        DT u[HNV], qd[3][HNV], F[3][HNV];
+#pragma unroll
+        for (int v = 0; v < HNV; ++v) {
+          u[v] = DT(pr.U[i][v], v == vp ? T(1) : T(0));
+#pragma unroll
+          for (int c = 0; c < 3; ++c) qd[c][v] = DT(pr.q[i][c][v]);
+        }
         NS3::conv<DT, T>(pc, u, F);
         if (visc) {
           DT Fv[3][HNV];
@@ -522,7 +525,7 @@ __global__ void __launch_bounds__(32 * HJWork<T, N>::NW, 1) k_hex_jacobian(const
 #pragma unroll
           for (int v = 0; v < HNV; ++v)
             J.KU[i][r][v][vp] = w.Sm[i][r][0] * F[0][v].d + w.Sm[i][r][1] * F[1][v].d + w.Sm[i][r][2] * F[2][v].d;
-      } else {
+      } else {  // the viscous flux is linear in the gradient: its value at a unit gradient
         T acc[3][3][HNV];
 #pragma unroll
         for (int r = 0; r < 3; ++r)
@@ -531,16 +534,21 @@ __global__ void __launch_bounds__(32 * HJWork<T, N>::NW, 1) k_hex_jacobian(const
 #pragma unroll
             for (int v = 0; v < HNV; ++v) acc[r][r2][v] = T(0);
         if (visc) {
+          T u[HNV], qe[3][HNV], F[3][HNV];
+#pragma unroll
+          for (int v = 0; v < HNV; ++v) u[v] = pr.U[i][v];
 #pragma unroll
           for (int c2 = 0; c2 < 3; ++c2) {
-            qd[c2][vp].d = T(1);
-            NS3::visc<DT, T>(pc, u, qd, F);
-            qd[c2][vp].d = T(0);
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+#pragma unroll
+              for (int v = 0; v < HNV; ++v) qe[c][v] = (c == c2 && v == vp) ? T(1) : T(0);
+            NS3::visc<T, T>(pc, u, qe, F);
 #pragma unroll
             for (int r = 0; r < 3; ++r)
 #pragma unroll
               for (int v = 0; v < HNV; ++v) {
-                const T dFr = -(w.Sm[i][r][0] * F[0][v].d + w.Sm[i][r][1] * F[1][v].d + w.Sm[i][r][2] * F[2][v].d);
+                const T dFr = -(w.Sm[i][r][0] * F[0][v] + w.Sm[i][r][1] * F[1][v] + w.Sm[i][r][2] * F[2][v]);
 #pragma unroll
                 for (int r2 = 0; r2 < 3; ++r2) acc[r][r2][v] += dFr * w.iJ[i] * w.Sm[i][r2][c2];
               }
@@ -554,39 +562,67 @@ __global__ void __launch_bounds__(32 * HJWork<T, N>::NW, 1) k_hex_jacobian(const
             for (int v = 0; v < HNV; ++v) J.KQ[i][r][r2][v][vp] = acc[r][r2][v];
       }
     }
-    for (int it = tid; it < 6 * nf * 5 * HNV; it += NT) {
-      const int jj = it / (5 * HNV), dir = it % (5 * HNV), grp = dir / HNV, vp = dir % HNV;
-      const int f = jj / nf;
+    // face: 0 the trace (dual numbers), 1 the face state (traced faces J_f s 1, interface faces by dual
+    // numbers), 2.. the gradient (the viscous flux at a unit gradient)
+    for (int it = tid; it < 5 * FI; it += NT) {
+      const int grp = it / FI, idx = it % FI;
+      if (idx >= 6 * nf * HNV) continue;
+      const int jj = idx / HNV, vp = idx % HNV, f = jj / nf;
       const int kf = w.kf[f];
       const bool traced = w.tr[f] >= 0;
-      DT uf[HNV], ub[HNV], un[HNV], qf[3][HNV], qn[3][HNV], Fn[HNV], row[HNV];
+      const T nr[3] = {pr.fnr[jj][0], pr.fnr[jj][1], pr.fnr[jj][2]}, Jf = pr.fJ[jj];
+      T d[HNV], dr[HNV];
 #pragma unroll
-      for (int v = 0; v < HNV; ++v) {
-        uf[v] = DT(pr.Uf[jj][v], (grp == 0 && v == vp) ? T(1) : T(0));
-        ub[v] = DT(pr.ub[jj][v], (grp == 1 && v == vp) ? T(1) : T(0));
-        un[v] = DT(pr.un[jj][v]);
+      for (int v = 0; v < HNV; ++v) d[v] = dr[v] = T(0);
+      if (grp >= 2) {
+        if (visc) {
+          T u[HNV], qe[3][HNV], F[3][HNV];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          qf[c][v] = DT(pr.qf[jj][c][v], (grp == 2 + c && v == vp) ? T(1) : T(0));
-          qn[c][v] = DT(T(0));
+          for (int v = 0; v < HNV; ++v) {
+            u[v] = traced ? pr.ub[jj][v] : pr.Uf[jj][v];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) qe[c][v] = (grp == 2 + c && v == vp) ? T(1) : T(0);
+          }
+          // faces without a trace between solved elements average both sides' viscous fluxes
+          const T Ja = (!traced && (kf == FK_FR || kf == FK_FAR)) ? T(0.5) * Jf : Jf;
+          NS3::visc<T, T>(pc, u, qe, F);
+#pragma unroll
+          for (int v = 0; v < HNV; ++v) d[v] = -Ja * (nr[0] * F[0][v] + nr[1] * F[1][v] + nr[2] * F[2][v]);
+        }
+      } else if (grp == 1 && traced) {
+        const T s = Jf * NS3::stab<T, T>(pc, pr.ub[jj], nr);
+#pragma unroll
+        for (int v = 0; v < HNV; ++v) d[v] = v == vp ? s : T(0);
+        if (kf == FK_FAR && vp == 0) w.RU[jj] = s;
+      } else if (grp == 1 || traced) {
+        DT uf[HNV], ub[HNV], un[HNV], qf[3][HNV], qn[3][HNV], Fn[HNV], row[HNV];
+#pragma unroll
+        for (int v = 0; v < HNV; ++v) {
+          uf[v] = DT(pr.Uf[jj][v], (grp == 1 && v == vp) ? T(1) : T(0));
+          ub[v] = DT(pr.ub[jj][v], (grp == 0 && v == vp) ? T(1) : T(0));
+          un[v] = DT(pr.un[jj][v]);
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            qf[c][v] = DT(pr.qf[jj][c][v]);
+            qn[c][v] = DT(T(0));
+          }
+        }
+        hface_flux<DT, T>(pc, visc, kf, traced, true, uf, ub, qf, un, qn, Jf, nr, w.uinf, Fn, row);
+#pragma unroll
+        for (int v = 0; v < HNV; ++v) {
+          d[v] = Fn[v].d;
+          dr[v] = row[v].d;
         }
       }
-      const bool zero = (grp >= 2 && !visc) || (grp == 1 && !traced);
-      if (!zero) {
-        const T nr[3] = {pr.fnr[jj][0], pr.fnr[jj][1], pr.fnr[jj][2]};
-        hface_flux<DT, T>(pc, visc, kf, traced, true, uf, ub, qf, un, qn, pr.fJ[jj], nr, w.uinf, Fn, row);
-      }
 #pragma unroll
       for (int v = 0; v < HNV; ++v) {
-        const T d = zero ? T(0) : Fn[v].d;
         if (grp == 0) {
-          J.GU[jj][v][vp] = d;
-          if (kf == FK_FAR && traced && v == 0 && vp == 0) w.RU[jj] = row[0].d;  // J_f s
+          J.GH[jj][v][vp] = d[v];
+          J.RH[jj][v][vp] = dr[v];
         } else if (grp == 1) {
-          J.GH[jj][v][vp] = d;
-          J.RH[jj][v][vp] = zero ? T(0) : row[v].d;
+          J.GU[jj][v][vp] = d[v];
         } else {
-          J.GQ[jj][grp - 2][v][vp] = d;
+          J.GQ[jj][grp - 2][v][vp] = d[v];
         }
       }
     }
