@@ -7,25 +7,25 @@
 // the tensor-product operators instead of differentiating the whole element residual:
 //   1. exact pointwise Jacobians of the volume flux (w.r.t. the state and the reference
 //      gradient) and of the common face flux (w.r.t. face state, trace, face gradient), by
-//      forward-mode dual numbers, one tangent per thread;
-//   2. per seed point (NV columns of the blocks), the tangent of the corrected gradient is
-//      nonzero only on the two grid lines through the seeded point (or on the one line normal
-//      to the seeded trace point), so the flux tangents are formed only there, by one warp;
-//   3. the output columns follow from the 1D operators M, dgL, dgR along the lines: a full
-//      line sum on the seed's row and column, one term elsewhere.
+//      forward-mode dual numbers where the flux is nonlinear in the input;
+//   2. a seed (a solution point or a trace point) moves the corrected gradient only on the two grid
+//      lines through it, and off its own line in proportion to one reference weight, so the bracket
+//      of every output along a line is an entry of a small table: full line sums for seeds on the
+//      line, single terms for seeds off it;
+//   3. every entry of the blocks is one or two table entries times reference weights, written in
+//      row order.
 // Work per element is O((nA + nT)^2), not the O((nA + nT) x residual) of a dense sweep.
 // T = double (plain path) or float (mixed path; blocks stored in FP32).
 #include "hfr_internal.h"
 
 namespace hfr {
 
-// resident CTAs per SM asked of the compiler for the FP32 p = 4 kernel (register cap 65536 /
-// (256 x blocks)); a build flag, for timing the register / occupancy trade
-#ifndef HFR_JAC_P4_BLOCKS
-#define HFR_JAC_P4_BLOCKS 4
-#endif
 constexpr int JAC_THREADS = 256;
-constexpr int JAC_WARPS = JAC_THREADS / 32;
+// resident CTAs per SM asked of the compiler: what the tables of JacWork leave room for
+template <typename T>
+constexpr int jac_blocks(int p) {
+  return sizeof(T) == 4 ? (p <= 3 ? 4 : (p == 4 ? 3 : 2)) : (p <= 3 ? 2 : 1);
+}
 
 template <int P, int PHYS, typename T>
 struct JacWork {
@@ -46,14 +46,13 @@ struct JacWork {
   alignas(16) T GH[NF][NV][NV];
   alignas(16) T GQ[NF][2][NV][NV];
   T ciJ[NS];  // a dt / J at each solution point
-  // per-warp tangents of one seed point, entries [v][v0] (NV seed columns innermost), rows
-  // padded by 16 bytes so that lane groups reading different points hit different banks
-  static constexpr int PAD = NV == 4 ? 4 : 0;
-  static constexpr int LNS = 2 * NV * NV + PAD, RCS = NV * NV + PAD;
-  alignas(16) T LN[JAC_WARPS][2][N][LNS];  // flux tangents [r][v][v0] on the seed's row (0) / column (1)
-  alignas(16) T RC[JAC_WARPS][2][N][RCS];  // row sums sum_c M[a][c] dFx(c, b0), column sums sum_c M[b][c] dFy(a0, c)
-  alignas(16) T FN[JAC_WARPS][NF][RCS];    // common face flux tangents
-  T DQ[JAC_WARPS][2][N][2];                // physical gradient tangents on the two lines
+  // direction d = 0: the xi line (grid row) m, 1: the eta line (grid column) m; position p along it;
+  // seed s along it, N and N + 1 the traces at its two ends; entries [v][seed][v0]
+  alignas(16) T XT[2][N][N][NV][N][NV];      // flux divergence of a seed off the line, per unit of its weight
+  alignas(16) T XF[2][N][N][NV][N + 2][NV];  // ... of a seed on the line
+  alignas(16) T HX[4][N][NV][N][NV];         // common face flux of a seed off the line, per unit of its weight
+  alignas(16) T FL[4][N][NV][N + 2][NV];     // ... of a seed on the line
+  T QO[4][N][N][2], QL[4][N][N + 2][2];      // the face gradients of the same seeds
   T rM[N][N], rdgL[N], rdgR[N], rlm[N], rlp[N], rw[N];  // reference operators in T
   int kf[4];
 };
@@ -82,6 +81,25 @@ __device__ __forceinline__ void stv(T* p, const T (&x)[NV]) {
   } else {
 #pragma unroll
     for (int v = 0; v < NV; ++v) p[v] = x[v];
+  }
+}
+
+// VW consecutive values: 16 bytes, or one value
+template <typename T, int VW>
+__device__ __forceinline__ void ldw(const T* p, T (&x)[VW]) {
+  if constexpr (VW == 2) {
+    const double2 q = *reinterpret_cast<const double2*>(p);
+    x[0] = q.x; x[1] = q.y;
+  } else {
+    ldv<T, VW>(p, x);
+  }
+}
+template <typename T, int VW>
+__device__ __forceinline__ void stw(T* p, const T (&x)[VW]) {
+  if constexpr (VW == 2) {
+    *reinterpret_cast<double2*>(p) = make_double2(x[0], x[1]);
+  } else {
+    stv<T, VW>(p, x);
   }
 }
 
@@ -133,7 +151,7 @@ __device__ __forceinline__ void imp_face_flux(const PhysConst<R>& pp, bool visc,
 }
 
 template <int P, int PHYS, typename T>
-__global__ void __launch_bounds__(JAC_THREADS, sizeof(T) == 4 ? (P <= 3 ? 4 : (P == 4 ? HFR_JAC_P4_BLOCKS : 2)) : 1) k_jacobian(const __grid_constant__ RefOps ref,
+__global__ void __launch_bounds__(JAC_THREADS, jac_blocks<T>(P)) k_jacobian(const __grid_constant__ RefOps ref,
                                                           const __grid_constant__ PhysParams pp,
                                                           const __grid_constant__ JacArgs a) {
   using W = JacWork<P, PHYS, T>;
@@ -167,9 +185,6 @@ __global__ void __launch_bounds__(JAC_THREADS, sizeof(T) == 4 ? (P <= 3 ? 4 : (P
     w.fn[j][1] = T(gf[j * 3 + 2]);
   }
   if (tid < 4) w.kf[tid] = a.kind[e * 4 + tid];
-  for (int i = tid; i < (int)(sizeof(w.LN) / sizeof(T)); i += JAC_THREADS) (&w.LN[0][0][0][0])[i] = T(0);
-  for (int i = tid; i < (int)(sizeof(w.RC) / sizeof(T)); i += JAC_THREADS) (&w.RC[0][0][0][0])[i] = T(0);
-  for (int i = tid; i < (int)(sizeof(w.FN) / sizeof(T)); i += JAC_THREADS) (&w.FN[0][0][0])[i] = T(0);
   for (int i = tid; i < N * N; i += JAC_THREADS) w.rM[i / N][i % N] = T(ref.M[i / N][i % N]);
   if (tid < N) {
     w.rdgL[tid] = T(ref.dgL[tid]);
@@ -230,7 +245,39 @@ __global__ void __launch_bounds__(JAC_THREADS, sizeof(T) == 4 ? (P <= 3 ? 4 : (P
   }
   __syncthreads();
 
-  // -------------------------------------------------- 1. pointwise Jacobians (dual numbers)
+  // the point of position c on line m of direction d
+  auto lpt = [](int d, int m, int c) -> int { return d == 0 ? c + N * m : m + N * c; };
+  // face gradients: of a unit move of the reference gradient across the line at its point s (QO), of
+  // a unit seed s on the line (QL)
+  for (int it = tid; it < 4 * N * (2 * N + 2); it += JAC_THREADS) {
+    const int s2 = it % (2 * N + 2), m = it / (2 * N + 2) % N, f = it / ((2 * N + 2) * N), d = f >> 1;
+    const T* l = (f & 1) ? w.rlp : w.rlm;
+    if (s2 < N) {
+      const int pt = lpt(d, m, s2);
+      const T c = l[s2] * w.iJ[pt];
+      w.QO[f][m][s2][0] = c * w.Sm[pt][1 - d][0];
+      w.QO[f][m][s2][1] = c * w.Sm[pt][1 - d][1];
+    } else {
+      const int sd = s2 - N;
+      T q0 = T(0), q1 = T(0);
+#pragma unroll
+      for (int c = 0; c < N; ++c) {
+        const int pt = lpt(d, m, c);
+        const T wl = l[c] * w.iJ[pt];
+        const T wd = wl * (sd < N ? w.rM[c][sd] : (sd == N ? w.rdgL[c] : w.rdgR[c]));
+        q0 += wd * w.Sm[pt][d][0];
+        q1 += wd * w.Sm[pt][d][1];
+        if (c == sd) {
+          q0 += wl * w.rM[m][m] * w.Sm[pt][1 - d][0];
+          q1 += wl * w.rM[m][m] * w.Sm[pt][1 - d][1];
+        }
+      }
+      w.QL[f][m][sd][0] = q0;
+      w.QL[f][m][sd][1] = q1;
+    }
+  }
+
+  // -------------------------------------------------- 1. pointwise Jacobians
   // volume: items (point, input variable) for the state, then the same for the gradient, each
   // range padded to whole warps so that a warp takes one branch.  Dual numbers only where the flux is
   // nonlinear in the input: the viscous flux is linear in the gradient and the stabilisation in the
@@ -351,217 +398,182 @@ __global__ void __launch_bounds__(JAC_THREADS, sizeof(T) == 4 ? (P <= 3 ? 4 : (P
   }
   __syncthreads();
 
-  // ------------------------------------------------ 2-3. columns, one seed point per warp
-  // A seed point is a solution point P0 = (a0, b0) (NV columns of A and C) or a flux point j0
-  // of a trace face (NV columns of B and D).  Its unit seeds move the reference gradient only on
-  // the grid row b0 (dQ_xi) and the grid column a0 (dQ_eta) through P0, or on the one line of
-  // points normal to the seeded face, so the flux tangents are formed on those lines alone and
-  // every output follows from them and the face tangents:
-  //   dR(ai, bi) = -1/J [ sum_c M[ai][c] dFx(c, bi) + M[bi][c] dFy(ai, c)
-  //                       - dgL[ai] dFn(xi-, bi) + dgR[ai] dFn(xi+, bi)
-  //                       - dgL[bi] dFn(eta-, ai) + dgR[bi] dFn(eta+, ai) ]
-  //   dg^k(f, m) = w_m dFn(f, m)   (trace faces)
-  // dFx(., bi) vanishes off the row b0 except at c = a0 and dFy(ai, .) off the column a0 except
-  // at c = b0, so with the line sums RC formed once per seed point every output is two
-  // one-term products and the four face terms.  Lane (v, g): output variable v, lane group g;
-  // each lane carries the NV seed variables v0 of the point (NV-wide loads and stores).  The
-  // warp's buffers are its own: no block barrier between seed points.
-  constexpr int G = 32 / NV, LNS = W::LNS, RCS = W::RCS;
-  const int lane = tid & 31, wp = tid >> 5;
-  const int vv = lane % NV, g = lane / NV;
-  T(*LN)[N][LNS] = w.LN[wp];
-  T(*RC)[N][RCS] = w.RC[wp];
-  T(*FN)[RCS] = w.FN[wp];
-  T(*DQ)[N][2] = w.DQ[wp];
+  // ------------------------------------------------ 2. tables of the lines
+  // A unit seed at the solution point (a0, b0) or on a trace moves the reference gradient only on its
+  // grid row and column:
+  //   dR(ai, bi) = -1/J [ sum_c M[ai][c] dFx(c, bi) - dgL[ai] dFn(xi-, bi) + dgR[ai] dFn(xi+, bi)
+  //                     + the same along eta ]
+  // On the row bi = b0 the xi bracket is a full line sum (XF[0][b0][ai][a0]).  On any other row only
+  // the point (a0, bi) moves, by its eta reference gradient M[bi][b0], and the two face points of
+  // that row with it: the bracket is M[bi][b0] times a table without b0 (XT[0][bi][ai][a0]).  The eta
+  // bracket likewise, with the columns; a trace seed replaces M[.][a0] by dgL or dgR.  So every
+  // output of A, B, C and D is a table entry times a reference weight, or the sum of two.
+  // Bound by the stores of the blocks, 130 KB per element at p = 4.  One seed point per warp with
+  // the tangents of its two lines, six vector reads of shared memory per output vector, kept the
+  // shared-memory pipe at 89 %: 368 us for 4096 elements, p = 4, FP32 (the blocks alone take 79 us
+  // at the copy rate); 175 us by the tables.  FP64, p = 3: 1.65 ms, 1.0 ms now.
+  constexpr int CI = N * NV * (2 * N + 2);
+  for (int it = tid; it < 4 * CI; it += JAC_THREADS) {
+    const int f = it / CI, s2 = it % (2 * N + 2), v = it / (2 * N + 2) % NV, m = it / ((2 * N + 2) * NV) % N;
+    const int j = f * N + m;
+    T g0[NV], g1[NV], o[NV];
+    ldv<T, NV>(&w.GQ[j][0][v][0], g0);
+    ldv<T, NV>(&w.GQ[j][1][v][0], g1);
+    const T q0 = s2 < N ? w.QO[f][m][s2][0] : w.QL[f][m][s2 - N][0];
+    const T q1 = s2 < N ? w.QO[f][m][s2][1] : w.QL[f][m][s2 - N][1];
+#pragma unroll
+    for (int x = 0; x < NV; ++x) o[x] = g0[x] * q0 + g1[x] * q1;
+    if (s2 < N) {
+      stv<T, NV>(&w.HX[f][m][v][s2][0], o);
+    } else {
+      const int sd = s2 - N;
+      if (sd < N) {
+        const T l = (f & 1) ? w.rlp[sd] : w.rlm[sd];
+        ldv<T, NV>(&w.GU[j][v][0], g0);
+#pragma unroll
+        for (int x = 0; x < NV; ++x) o[x] += g0[x] * l;
+      } else if (w.kf[(f & 2) + sd - N] != FK_TRACE) {
+#pragma unroll
+        for (int x = 0; x < NV; ++x) o[x] = T(0);
+      } else if (sd - N == (f & 1)) {
+        ldv<T, NV>(&w.GH[j][v][0], g0);
+#pragma unroll
+        for (int x = 0; x < NV; ++x) o[x] += g0[x];
+      }
+      stv<T, NV>(&w.FL[f][m][v][sd][0], o);
+    }
+  }
+  __syncthreads();
+  // XF items (line, v, seed), then XT items, each kind in whole warps; all positions p of the line
+  constexpr int FI2 = (2 * N * NV * (N + 2) + 31) / 32 * 32;
+  for (int it = tid; it < FI2 + 2 * N * NV * N; it += JAC_THREADS) {
+    const bool full = it < FI2;
+    const int idx = full ? it : it - FI2;
+    if (full && idx >= 2 * N * NV * (N + 2)) continue;
+    const int S1 = full ? N + 2 : N;
+    const int sd = idx % S1, v = idx / S1 % NV, m = idx / (S1 * NV) % N, d = idx / (S1 * NV * N);
+    T h0[NV], h1[NV], e[NV], t[N][NV];
+    if (full) {
+      ldv<T, NV>(&w.FL[2 * d][m][v][sd][0], h0);
+      ldv<T, NV>(&w.FL[2 * d + 1][m][v][sd][0], h1);
+    } else {
+      ldv<T, NV>(&w.HX[2 * d][m][v][sd][0], h0);
+      ldv<T, NV>(&w.HX[2 * d + 1][m][v][sd][0], h1);
+    }
+    if (sd < N) {
+      const int pt = lpt(d, m, sd);
+      ldv<T, NV>(&w.KQ[pt][d][1 - d][v][0], e);
+      if (full) {
+        T ku[NV];
+        ldv<T, NV>(&w.KU[pt][d][v][0], ku);
+        const T mm = w.rM[m][m];
+#pragma unroll
+        for (int x = 0; x < NV; ++x) e[x] = mm * e[x] + ku[x];
+      }
+    } else {
+#pragma unroll
+      for (int x = 0; x < NV; ++x) e[x] = T(0);
+    }
+    if (full) {
+      const bool on = sd < N || w.kf[2 * d + sd - N] == FK_TRACE;
+#pragma unroll
+      for (int c = 0; c < N; ++c) {
+        ldv<T, NV>(&w.KQ[lpt(d, m, c)][d][d][v][0], t[c]);
+        const T wc = sd < N ? w.rM[c][sd] : (on ? (sd == N ? w.rdgL[c] : w.rdgR[c]) : T(0));
+#pragma unroll
+        for (int x = 0; x < NV; ++x) t[c][x] *= wc;
+      }
+    }
+#pragma unroll 1
+    for (int p = 0; p < N; ++p) {
+      T o[NV];
+      const T me = sd < N ? w.rM[p][sd] : T(0), gl = w.rdgL[p], gr = w.rdgR[p], cj = w.ciJ[lpt(d, m, p)];
+#pragma unroll
+      for (int x = 0; x < NV; ++x) o[x] = me * e[x] - gl * h0[x] + gr * h1[x];
+      if (full) {
+#pragma unroll
+        for (int c = 0; c < N; ++c) {
+          const T mc = w.rM[p][c];
+#pragma unroll
+          for (int x = 0; x < NV; ++x) o[x] += mc * t[c][x];
+        }
+      }
+#pragma unroll
+      for (int x = 0; x < NV; ++x) o[x] *= cj;  // A = I - a dt dR, B = -a dt dR
+      stv<T, NV>(full ? &w.XF[d][m][p][v][sd][0] : &w.XT[d][m][p][v][sd][0], o);
+    }
+  }
+  __syncthreads();
+
+  // ------------------------------------------------ 3. outputs
+  // A thread keeps its column group (VW seed variables of one seed) and steps through the rows:
+  // consecutive threads write consecutive 16-byte groups.
+  constexpr int VW = NV % (16 / (int)sizeof(T)) == 0 ? 16 / (int)sizeof(T) : 1;
+  constexpr int CA = nA / VW, CB = nT / VW, RA = JAC_THREADS / CA, RB = JAC_THREADS / CB;
   T* A = reinterpret_cast<T*>(a.A) + (size_t)k * nA * nA;
   T* B = reinterpret_cast<T*>(a.B) + (size_t)k * nA * nT;
   T* C = reinterpret_cast<T*>(a.C) + (size_t)k * nT * nA;
   T* Dm = reinterpret_cast<T*>(a.D) + (size_t)k * nT * nT;
-  for (int sp = wp; sp < NS + NF; sp += JAC_WARPS) {
-    const bool vol = sp < NS;
-    int a0, b0;
-    bool has_row, has_col, active;
-    const T* dgs = w.rdgL;  // weights of a trace seed along its line
-    if (vol) {
-      a0 = sp % N;
-      b0 = sp / N;
-      has_row = has_col = active = true;
-    } else {
-      const int f0 = (sp - NS) / N, m0 = (sp - NS) % N;
-      active = w.kf[f0] == FK_TRACE;
-      has_row = (f0 >> 1) == 0;  // xi faces move dQ_xi on the grid row m0
-      has_col = !has_row;        // eta faces move dQ_eta on the grid column m0
-      a0 = b0 = m0;
-      if (f0 & 1) dgs = w.rdgR;
+  if (tid < RA * CA) {  // seeds: solution points
+    const int cg = tid % CA, sp = cg * VW / NV, v0 = cg * VW % NV, a0 = sp % N, b0 = sp / N;
+    for (int i = tid / CA; i < nA; i += RA) {
+      const int pt = i / NV, v = i % NV, ai = pt % N, bi = pt / N;
+      const bool xrow = bi == b0, ycol = ai == a0;
+      const T fx = xrow ? T(1) : w.rM[bi][b0], fy = ycol ? T(1) : w.rM[ai][a0];
+      T x[VW], y[VW];
+      ldw<T, VW>(xrow ? &w.XF[0][bi][ai][v][a0][v0] : &w.XT[0][bi][ai][v][a0][v0], x);
+      ldw<T, VW>(ycol ? &w.XF[1][ai][bi][v][b0][v0] : &w.XT[1][ai][bi][v][b0][v0], y);
+#pragma unroll
+      for (int u = 0; u < VW; ++u) {
+        x[u] = fx * x[u] + fy * y[u];
+        if (pt == sp && v == v0 + u) x[u] += T(1);
+      }
+      stw<T, VW>(A + (size_t)i * nA + cg * VW, x);
     }
-    // reference-gradient tangents (dQ_xi, dQ_eta) at point c of line 0 (row b0) or 1 (column a0)
-    auto seed_dq = [&](int line, int c, T& dQ0, T& dQ1) {
-      if (line == 0) {
-        dQ0 = vol ? w.rM[c][a0] : dgs[c];
-        dQ1 = (vol && c == a0) ? w.rM[b0][b0] : T(0);
-      } else {
-        dQ1 = vol ? w.rM[c][b0] : dgs[c];
-        dQ0 = (vol && c == b0) ? w.rM[a0][a0] : T(0);
-      }
-    };
-    if (active) {
-      // physical gradient tangents on the lines (independent of v0)
-      if (lane < 4 * N) {
-        const int line = lane / (2 * N), c = (lane >> 1) % N, c2 = lane & 1;
-        if (line == 0 ? has_row : has_col) {
-          const int pt = line == 0 ? c + N * b0 : a0 + N * c;
-          T dQ0, dQ1;
-          seed_dq(line, c, dQ0, dQ1);
-          DQ[line][c][c2] = w.iJ[pt] * (w.Sm[pt][0][c2] * dQ0 + w.Sm[pt][1][c2] * dQ1);
-        }
-      }
-      __syncwarp();
-      // flux tangents on the lines, then the common face flux tangents
-      for (int it = g; it < 2 * N + NF && g < G; it += G) {
-        if (it < 2 * N) {
-          const int line = it / N, c = it % N;
-          if (!(line == 0 ? has_row : has_col)) continue;
-          const int pt = line == 0 ? c + N * b0 : a0 + N * c;
-          T dQ0, dQ1;
-          seed_dq(line, c, dQ0, dQ1);
-          const bool self = vol && pt == sp;
+    for (int i = tid / CA; i < nT; i += RA) {
+      const int j = i / NV, v = i % NV, m = j % N, f = j / N;
+      const bool tr = w.kf[f] == FK_TRACE, eta = f >= 2;
+      const int sl = eta ? b0 : a0, so = eta ? a0 : b0;  // the seed's place along the line, its line
+      const bool on = m == so;
+      T x[VW];
+      ldw<T, VW>(on ? &w.FL[f][m][v][sl][v0] : &w.HX[f][m][v][sl][v0], x);
+      const T c = on ? w.rw[m] : w.rw[m] * w.rM[m][so];
 #pragma unroll
-          for (int r = 0; r < 2; ++r) {
-            T k0[NV], k1[NV], o[NV];
-            ldv<T, NV>(&w.KQ[pt][r][0][vv][0], k0);
-            ldv<T, NV>(&w.KQ[pt][r][1][vv][0], k1);
-#pragma unroll
-            for (int x = 0; x < NV; ++x) o[x] = k0[x] * dQ0 + k1[x] * dQ1;
-            if (self) {
-              ldv<T, NV>(&w.KU[pt][r][vv][0], k0);
-#pragma unroll
-              for (int x = 0; x < NV; ++x) o[x] += k0[x];
-            }
-            stv<T, NV>(&LN[line][c][(r * NV + vv) * NV], o);
-          }
-        } else {
-          const int j = it - 2 * N, f = j / N, m = j % N;
-          const T* l = (f & 1) ? w.rlp : w.rlm;
-          T dUf = T(0), q0 = T(0), q1 = T(0);
-          if ((f >> 1) == 0) {  // xi face: flux points along the grid row m
-            if (has_row && m == b0) {
-#pragma unroll
-              for (int c = 0; c < N; ++c) {
-                q0 += l[c] * DQ[0][c][0];
-                q1 += l[c] * DQ[0][c][1];
-              }
-            } else if (has_col) {
-              q0 = l[a0] * DQ[1][m][0];
-              q1 = l[a0] * DQ[1][m][1];
-            }
-            if (vol && m == b0) dUf = l[a0];
-          } else {  // eta face: flux points along the grid column m
-            if (has_col && m == a0) {
-#pragma unroll
-              for (int c = 0; c < N; ++c) {
-                q0 += l[c] * DQ[1][c][0];
-                q1 += l[c] * DQ[1][c][1];
-              }
-            } else if (has_row) {
-              q0 = l[b0] * DQ[0][m][0];
-              q1 = l[b0] * DQ[0][m][1];
-            }
-            if (vol && m == a0) dUf = l[b0];
-          }
-          T gu[NV], g0[NV], g1[NV], o[NV];
-          ldv<T, NV>(&w.GU[j][vv][0], gu);
-          ldv<T, NV>(&w.GQ[j][0][vv][0], g0);
-          ldv<T, NV>(&w.GQ[j][1][vv][0], g1);
-#pragma unroll
-          for (int x = 0; x < NV; ++x) o[x] = gu[x] * dUf + g0[x] * q0 + g1[x] * q1;
-          if (!vol && j == sp - NS) {
-            ldv<T, NV>(&w.GH[j][vv][0], gu);
-#pragma unroll
-            for (int x = 0; x < NV; ++x) o[x] += gu[x];
-          }
-          stv<T, NV>(&FN[j][vv * NV], o);
-        }
-      }
-      __syncwarp();
-      // line sums: RC[0][ai] = sum_c M[ai][c] dFx(c, b0), RC[1][bi] = sum_c M[bi][c] dFy(a0, c)
-      for (int it = g; it < 2 * N && g < G; it += G) {
-        const int line = it / N, e = it % N;
-        if (!(line == 0 ? has_row : has_col)) continue;
-        T o[NV], t[NV];
-#pragma unroll
-        for (int x = 0; x < NV; ++x) o[x] = T(0);
-#pragma unroll
-        for (int c = 0; c < N; ++c) {
-          ldv<T, NV>(&LN[line][c][(line * NV + vv) * NV], t);
-          const T mc = w.rM[e][c];
-#pragma unroll
-          for (int x = 0; x < NV; ++x) o[x] += mc * t[x];
-        }
-        stv<T, NV>(&RC[line][e][vv * NV], o);
-      }
-      __syncwarp();
+      for (int u = 0; u < VW; ++u) x[u] = tr ? c * x[u] : T(0);
+      stw<T, VW>(C + (size_t)i * nA + cg * VW, x);
     }
-    // outputs (the buffers are zeroed at entry, so a line the seed does not have reads finite
-    // values that are multiplied by zero)
-    for (int it = g; it < NS + NF && g < G; it += G) {
-      T o[NV];
-      T* dst;
-      if (it < NS) {
-        const int ai = it % N, bi = it / N;
+  }
+  if (tid < RB * CB) {  // seeds: trace points
+    const int cg = tid % CB, j0 = cg * VW / NV, v0 = cg * VW % NV, f0 = j0 / N, m0 = j0 % N;
+    const int d0 = f0 >> 1, sd = N + (f0 & 1);
+    const bool act = w.kf[f0] == FK_TRACE;
+    const T* dgs = (f0 & 1) ? w.rdgR : w.rdgL;
+    for (int i = tid / CB; i < nA; i += RB) {
+      const int pt = i / NV, v = i % NV, ai = pt % N, bi = pt / N;
+      const int p = d0 ? bi : ai, m = d0 ? ai : bi;  // the point on the lines along the seed's direction
+      T x[VW], y[VW];
+      ldw<T, VW>(&w.XT[1 - d0][p][m][v][m0][v0], y);
+      const T fy = act ? dgs[p] : T(0);
 #pragma unroll
-        for (int x = 0; x < NV; ++x) o[x] = T(0);
-        if (active) {
-          T t[NV];
-          const bool xrow = has_row && bi == b0, ycol = has_col && ai == a0;
-          const T cx = xrow ? T(1) : (has_col ? w.rM[ai][a0] : T(0));
-          const T cy = ycol ? T(1) : (has_row ? w.rM[bi][b0] : T(0));
-          ldv<T, NV>(xrow ? &RC[0][ai][vv * NV] : &LN[1][bi][vv * NV], t);
+      for (int u = 0; u < VW; ++u) x[u] = act ? fy * y[u] : T(0);
+      if (act && m == m0) {
+        ldw<T, VW>(&w.XF[d0][m][p][v][sd][v0], y);
 #pragma unroll
-          for (int x = 0; x < NV; ++x) o[x] = cx * t[x];
-          ldv<T, NV>(ycol ? &RC[1][bi][vv * NV] : &LN[0][ai][(NV + vv) * NV], t);
-#pragma unroll
-          for (int x = 0; x < NV; ++x) o[x] += cy * t[x];
-          const T cxm = -w.rdgL[ai], cxp = w.rdgR[ai], cym = -w.rdgL[bi], cyp = w.rdgR[bi];
-          ldv<T, NV>(&FN[bi][vv * NV], t);
-#pragma unroll
-          for (int x = 0; x < NV; ++x) o[x] += cxm * t[x];
-          ldv<T, NV>(&FN[N + bi][vv * NV], t);
-#pragma unroll
-          for (int x = 0; x < NV; ++x) o[x] += cxp * t[x];
-          ldv<T, NV>(&FN[2 * N + ai][vv * NV], t);
-#pragma unroll
-          for (int x = 0; x < NV; ++x) o[x] += cym * t[x];
-          ldv<T, NV>(&FN[3 * N + ai][vv * NV], t);
-#pragma unroll
-          for (int x = 0; x < NV; ++x) o[x] += cyp * t[x];
-          const T cj = w.ciJ[it];
-#pragma unroll
-          for (int x = 0; x < NV; ++x) o[x] *= cj;  // A = I - a dt dR, B = -a dt dR
-        }
-        if (vol && it == sp) {
-#pragma unroll
-          for (int x = 0; x < NV; ++x)
-            if (x == vv) o[x] += T(1);
-        }
-        const int i = it * NV + vv;
-        dst = vol ? A + (size_t)i * nA + sp * NV : B + (size_t)i * nT + (sp - NS) * NV;
-      } else {
-        const int j = it - NS, m = j % N;
-        if (active && w.kf[j / N] == FK_TRACE) {
-          ldv<T, NV>(&FN[j][vv * NV], o);
-          const T wm = w.rw[m];
-#pragma unroll
-          for (int x = 0; x < NV; ++x) o[x] *= wm;
-        } else {
-#pragma unroll
-          for (int x = 0; x < NV; ++x) o[x] = T(0);
-        }
-        const int lr = j * NV + vv;
-        dst = vol ? C + (size_t)lr * nA + sp * NV : Dm + (size_t)lr * nT + (sp - NS) * NV;
+        for (int u = 0; u < VW; ++u) x[u] += y[u];
       }
-      stv<T, NV>(dst, o);
+      stw<T, VW>(B + (size_t)i * nT + cg * VW, x);
     }
-    __syncwarp();  // the next seed point rewrites this warp's buffers
+    for (int i = tid / CB; i < nT; i += RB) {
+      const int j = i / NV, v = i % NV, m = j % N, f = j / N;
+      const bool same = (f >> 1) == d0;
+      const bool nz = act && w.kf[f] == FK_TRACE && (!same || m == m0);
+      T x[VW];
+      ldw<T, VW>(same ? &w.FL[f][m][v][sd][v0] : &w.HX[f][m][v][m0][v0], x);
+      const T c = same ? w.rw[m] : w.rw[m] * dgs[m];
+#pragma unroll
+      for (int u = 0; u < VW; ++u) x[u] = nz ? c * x[u] : T(0);
+      stw<T, VW>(Dm + (size_t)i * nT + cg * VW, x);
+    }
   }
 }
 
