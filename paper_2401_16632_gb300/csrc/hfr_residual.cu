@@ -326,12 +326,13 @@ static cudaError_t launch_elem_n(const RefOps& ref, const PhysParams& pp, const 
   return cudaGetLastError();
 }
 // elements per CTA: as many as fill whole warps with points (p = 2: 144 points of 160 lanes; p = 3
-// and 5: all lanes; p = 4: 200 of 224), fewer where that would leave SMs without a CTA: there the
-// passes last a few microseconds and a phase's latency counts, not its lanes
+// and 5: all lanes; p = 4: 200 of 224), fewer where that would leave less than two CTAs per SM:
+// there the passes last a few microseconds and a phase's latency counts, not its lanes (an IMEX step of
+// 2867 elements, p = 2: 2.40 ms with 16 elements per CTA, 2.29 ms with 4)
 template <int P, int PHYS, typename S, int MODE>
 static cudaError_t launch_elem(const RefOps& ref, const PhysParams& pp, const ResArgs& a, cudaStream_t st) {
   constexpr int EPB = P <= 2 ? 16 : 8, NT = P <= 3 ? 128 : 256;
-  if (a.E >= 152 * EPB) return launch_elem_n<P, PHYS, S, MODE, EPB, NT>(ref, pp, a, st);
+  if (a.E >= 304 * EPB) return launch_elem_n<P, PHYS, S, MODE, EPB, NT>(ref, pp, a, st);
   return launch_elem_n<P, PHYS, S, MODE, 4, 128>(ref, pp, a, st);
 }
 
