@@ -745,7 +745,7 @@ struct InvTcShape {
   static constexpr uint32_t OFF_RB = 2 * W_BYTES + 2 * P_BYTES;
   static constexpr int NQ = (NC + 31) / 32;     // 32-column groups (tensor-memory loads, output)
   static constexpr uint32_t OFF_CAND = OFF_RB + 32u * RB * 4u;
-  static constexpr uint32_t OFF_KEY = OFF_CAND + 2u * 4u * 16u * 4u;
+  static constexpr uint32_t OFF_KEY = OFF_CAND + 2u * 4u * 20u * 4u;  // 16 values, the reciprocal
   static constexpr uint32_t OFF_MBAR = OFF_KEY + 2u * 4u * 4u;
   static constexpr uint32_t NEED = OFF_MBAR + 16u;
   // requested so that at most four CTAs share an SM: each holds 128 of its 512 tensor-memory columns
@@ -765,7 +765,7 @@ __global__ void __launch_bounds__(128, 4) k_inverse_tc(const __grid_constant__ C
   unsigned char* Phi = iv_smem + Sh::OFF_PHI;
   unsigned char* Plo = iv_smem + Sh::OFF_PLO;
   float* rowbuf = reinterpret_cast<float*>(iv_smem + Sh::OFF_RB);
-  float* cand = reinterpret_cast<float*>(iv_smem + Sh::OFF_CAND);  // [2][4][16]
+  float* cand = reinterpret_cast<float*>(iv_smem + Sh::OFF_CAND);  // [2][4][20]
   unsigned* s_key = reinterpret_cast<unsigned*>(iv_smem + Sh::OFF_KEY);  // [2][4]
   uint64_t* mbar = reinterpret_cast<uint64_t*>(iv_smem + Sh::OFF_MBAR);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 1);
@@ -786,12 +786,12 @@ __global__ void __launch_bounds__(128, 4) k_inverse_tc(const __grid_constant__ C
     if (t == 0 && k + (int)gridDim.x < a.Eim)
       asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(gA + (size_t)gridDim.x * NA * NA),
                    "r"((unsigned)(NA * NA * 4)) : "memory");
-    // two 16-column chunks per round: eight 16-byte loads of the row in flight
+    // four 16-column chunks per round: sixteen 16-byte loads of the row in flight
 #pragma unroll 1
-    for (int cc = 0; cc < NP; cc += 2) {
-      float v[2][16];
+    for (int cc = 0; cc < NP; cc += 4) {
+      float v[4][16];
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
+      for (int h = 0; h < 4; ++h)
 #pragma unroll
         for (int u = 0; u < 16; u += 4) {
           const int c = 16 * (cc + h) + u;
@@ -799,8 +799,9 @@ __global__ void __launch_bounds__(128, 4) k_inverse_tc(const __grid_constant__ C
           if (row < NA && c < NA) x = __ldg(reinterpret_cast<const float4*>(gA + (size_t)row * NA + c));
           v[h][u] = x.x; v[h][u + 1] = x.y; v[h][u + 2] = x.z; v[h][u + 3] = x.w;
         }
-      tmem_st16(tl + (uint32_t)(16 * cc), v[0]);
-      if (cc + 1 < NP) tmem_st16(tl + (uint32_t)(16 * (cc + 1)), v[1]);
+#pragma unroll
+      for (int h = 0; h < 4; ++h)
+        if (cc + h < NP) tmem_st16(tl + (uint32_t)(16 * (cc + h)), v[h]);
     }
     tmem_st_wait();
     bool used = row >= NA;
@@ -814,17 +815,26 @@ __global__ void __launch_bounds__(128, 4) k_inverse_tc(const __grid_constant__ C
       __syncthreads();
       fence_after_sync();
       tmem_ld16(tl + (uint32_t)(16 * p), v);
-      // pivot candidates of column 0 of the panel
-      {
-        const unsigned key = used ? 0u : ((__float_as_uint(fabsf(v[0])) & ~MASK) | (MASK - (unsigned)row));
+      // A step's chain: barrier, keys, pivot row, one multiply-add, key of the next column, warp
+      // maximum, barrier.  So the candidate's reciprocal is formed before the barrier, beside the
+      // maximum, and pivot rows stay unscaled until the end of the panel (scaling commutes with the
+      // steps): every row takes the same multiply-adds, with factor 0 on the pivot row itself.
+      // 4096 blocks of nA = 100: 349 -> 336 us (the steps are about 55 % of it).
+      auto publish = [&](const float (&x)[16], int s, int b) {
+        const unsigned key = used ? 0u : ((__float_as_uint(fabsf(x[s])) & ~MASK) | (MASK - (unsigned)row));
+        const float inv = x[s] != 0.f ? rcp_approx(x[s]) : 0.f;  // 1-ulp hardware reciprocal
         const unsigned wk = __reduce_max_sync(0xffffffffu, key);
         if (key == wk && wk != 0u) {
+          float* c = cand + (b * 4 + w) * 20;
 #pragma unroll
           for (int u = 0; u < 16; u += 4)
-            *reinterpret_cast<float4*>(cand + (0 * 4 + w) * 16 + u) = make_float4(v[u], v[u + 1], v[u + 2], v[u + 3]);
+            *reinterpret_cast<float4*>(c + u) = make_float4(x[u], x[u + 1], x[u + 2], x[u + 3]);
+          c[16] = inv;
         }
-        if (lane == 0) s_key[0 * 4 + w] = wk;
-      }
+        if (lane == 0) s_key[b * 4 + w] = wk;
+      };
+      float myinv = 1.f;
+      publish(v, 0, 0);
       __syncthreads();
 #pragma unroll
       for (int s = 0; s < 16; ++s) {
@@ -833,42 +843,35 @@ __global__ void __launch_bounds__(128, 4) k_inverse_tc(const __grid_constant__ C
           const uint4 kq = *reinterpret_cast<const uint4*>(s_key + b * 4);
           const unsigned km = max(max(kq.x, kq.y), max(kq.z, kq.w));
           const int r = (int)(MASK - (km & MASK));
-          const int wb = r >> 5;                      // the warp that holds row r
           if ((km & 0x7F800000u) == 0u) bad = true;  // |pivot| below FLT_MIN (or no pivot left)
+          const float* c = cand + (b * 4 + (r >> 5)) * 20;  // of the warp that holds row r
           float prow[16];
+          const float pinv = c[16];
 #pragma unroll
           for (int u = 0; u < 16; u += 4) {
-            const float4 x = *reinterpret_cast<const float4*>(cand + (b * 4 + wb) * 16 + u);
+            const float4 x = *reinterpret_cast<const float4*>(c + u);
             prow[u] = x.x; prow[u + 1] = x.y; prow[u + 2] = x.z; prow[u + 3] = x.w;
           }
-          const float pv = prow[s];
-          const float pinv = pv != 0.f ? rcp_approx(pv) : 0.f;  // 1-ulp hardware reciprocal
-          if (row == r) {
+          const bool me = row == r;
+          const float g = me ? 0.f : v[s] * pinv;
+          if (s + 1 < 16) v[s + 1] -= g * prow[s + 1];
 #pragma unroll
-            for (int u = 0; u < 16; ++u) v[u] = prow[u] * pinv;
-            v[s] = pinv;
+          for (int u = 0; u < 16; ++u)
+            if (u != s && u != s + 1) v[u] -= g * prow[u];
+          v[s] = me ? 1.f : -g;
+          if (me) {
             used = true;
             mystep = 16 * p + s;
-          } else {
-            const float g = v[s] * pinv;
-#pragma unroll
-            for (int u = 0; u < 16; ++u) v[u] -= g * prow[u];
-            v[s] = -g;
+            myinv = pinv;
           }
           if (s + 1 < ns) {
-            const unsigned key = used ? 0u : ((__float_as_uint(fabsf(v[s + 1])) & ~MASK) | (MASK - (unsigned)row));
-            const unsigned wk = __reduce_max_sync(0xffffffffu, key);
-            if (key == wk && wk != 0u) {
-#pragma unroll
-              for (int u = 0; u < 16; u += 4)
-                *reinterpret_cast<float4*>(cand + ((b ^ 1) * 4 + w) * 16 + u) =
-                    make_float4(v[u], v[u + 1], v[u + 2], v[u + 3]);
-            }
-            if (lane == 0) s_key[(b ^ 1) * 4 + w] = wk;
+            publish(v, s + 1, b ^ 1);
             __syncthreads();
           }
         }
       }
+#pragma unroll
+      for (int u = 0; u < 16; ++u) v[u] *= myinv;
       // ---- W = E - I on the pivot columns (rows: all), 3xTF32 split, K-major 16-byte chunks
 #pragma unroll
       for (int sc = 0; sc < 4; ++sc) {
