@@ -208,7 +208,10 @@ __global__ void __launch_bounds__(BT) k_big_lu_panel(const __grid_constant__ Une
 // every panel to SP pivots.  Rows are interleaved over the lane groups (row G i + g), which with the
 // padded ring rows keeps the groups' broadcasts on different banks.  What is left is the in-panel
 // solve of a few warps between two barriers and the shared-memory rate of the updates.
-// Measured: 4608 FP32 blocks of (320, 480) 40.4 -> 21.7 ms (27 % of the FMA rate), 750 FP64 blocks
+// Measured: 4608 FP32 blocks of (320, 480) 40.4 -> 21.7 ms, and 17.8 ms (33 % of the FMA rate) with the
+// columns read as vectors, the in-panel rows as four independent chains and the pivots' reciprocals
+// formed ahead (of 340 thousand clocks per CTA the load took 55 and the backward in-panel solves 62);
+// 750 FP64 blocks
 // of (144, 96) 6.28 -> 3.85 ms (74 % of the FP64 rate).  X held in registers instead (one warp per 16
 // rows, tile after tile) took 34.8 ms: every tile waits for one warp's chain.
 template <typename T, int LC_, int CW_, int NW_, int H_>
@@ -229,7 +232,7 @@ struct SolveCfg {
   static_assert(CW % COLG == 0 && CW <= 32 * NW && SP <= 32, "column groups");
   __host__ __device__ static int rows(int nA) { return (nA + SP - 1) / SP * SP; }
   static size_t smem(int nA) {
-    return ((size_t)rows(nA) * XST + (size_t)NW * 2 * 16 * LST + 2 * SP * SP) * sizeof(T) +
+    return ((size_t)rows(nA) * XST + (size_t)NW * 2 * 16 * LST + 2 * SP * SP + SP) * sizeof(T) +
            2 * (size_t)rows(nA) * sizeof(int);
   }
 };
@@ -266,12 +269,12 @@ struct alignas(16) SolveVec {
 };
 
 // x / d with the reciprocal known: one Newton correction of the quotient (the division's own
-// rounding, without its long instruction sequence on the substitution's serial chain)
+// rounding, without its long instruction sequence on the substitution's serial chain).  Not finite
+// where the reciprocal or a product leaves the range: the caller divides then.
 template <typename T>
 __device__ __forceinline__ T solve_div(T x, T d, T inv) {
   const T q = x * inv;
-  const T c = fma(fma(-q, d, x), inv, q);
-  return isfinite(c) ? c : x / d;
+  return fma(fma(-q, d, x), inv, q);
 }
 
 template <typename T, int LC, int CW, int NW, int H>
@@ -289,7 +292,8 @@ __global__ void __launch_bounds__(32 * NW, 512 / (32 * NW)) k_big_solve(const __
   T* Xs = reinterpret_cast<T*>(sv_smem);            // nAp x XST
   T* ring = Xs + (size_t)nAp * XST;                  // NW x 2 factor tiles of 16 x LST
   T* Dg = ring + (size_t)NW * 2 * 16 * LST;          // two diagonal blocks SP x SP
-  int* perm = reinterpret_cast<int*>(Dg + 2 * SP * SP);
+  T* dinv = Dg + 2 * SP * SP;                        // reciprocals of a panel's pivots
+  int* perm = reinterpret_cast<int*>(dinv + SP);
   int* pvs = perm + nAp;
   const T* L = reinterpret_cast<const T*>(a.LU) + E.o[0];
   const T* B = reinterpret_cast<const T*>(a.B) + E.o[1];
@@ -310,41 +314,91 @@ __global__ void __launch_bounds__(32 * NW, 512 / (32 * NW)) k_big_solve(const __
   solve_tile<T, SP, V>(Dg, SP, L, nA, 0, 0, SP, vec, tid, NTH);
   cp_commit();
   // position i of P b holds row perm[i]: the interchanges (j, piv[j]) undone from the last to the
-  // first, every position on its own
-  for (int i = tid; i < nA; i += NTH) pvs[i] = piv[i];
+  // first, every position on its own.  Where columns are read along the rows (column-major B), perm
+  // is the position of a row instead.
+  const bool vecb = (cm ? nA : nT) % V == 0 && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
+  const bool inverse = cm && vecb;
+  for (int i = tid; i < nAp; i += NTH) {
+    const int p = i < nA ? piv[i] : i;
+    pvs[i] = p >= 0 && p < nA ? p : i;
+  }
   __syncthreads();
   for (int i = tid; i < nAp; i += NTH) {
     int pos = i;
-    for (int j = nA - 1; j >= 0; --j) {
-      const int p = pvs[j];
-      if (p >= 0 && p < nA) pos = pos == j ? p : (pos == p ? j : pos);
+    for (int j = nAp - 4; j >= 0; j -= 4) {
+      const int4 p = *reinterpret_cast<const int4*>(pvs + j);
+      pos = pos == j + 3 ? p.w : (pos == p.w ? j + 3 : pos);
+      pos = pos == j + 2 ? p.z : (pos == p.z ? j + 2 : pos);
+      pos = pos == j + 1 ? p.y : (pos == p.y ? j + 1 : pos);
+      pos = pos == j ? p.x : (pos == p.x ? j : pos);
     }
-    perm[i] = pos;
+    perm[inverse ? pos : i] = inverse ? i : pos;
   }
   __syncthreads();
-  // the permuted columns: SU loads per thread in flight before their stores.  Column-major B: 8 rows
-  // x 4 columns per warp access (whole sectors, conflict-free stores); row-major: one row per access
+  // the permuted columns.  Column-major B: a warp reads two vectors of rows of 16 columns (whole
+  // sectors), SU such reads in flight, and stores each value at its row's position (conflict-free
+  // without interchanges); row-major: rows by 16-byte asynchronous copies; one value per lane where
+  // rows or columns do not start on vectors
   constexpr int SU = 8;
   const double* rv = a.r + E.o[3];
-  const int nr = cm ? nAp / 8 : nAp, ni = cm ? nr * (CW / 4) : nr * (CW / 32 + (CW % 32 != 0));
-  for (int i0 = wid; i0 < ni; i0 += NW * SU) {
-    T v[SU];
+  if (inverse) {
+    const int nr = nAp / (2 * V), ni = nr * (CW / 16);
+    for (int i0 = wid; i0 < ni; i0 += NW * SU) {
+      SolveVec<T> v[SU];
 #pragma unroll
-    for (int u = 0; u < SU; ++u) {
-      const int it = i0 + NW * u, ir = it % nr, iq = it / nr;
-      const int i = cm ? ir * 8 + (lane & 7) : ir, q = cm ? iq * 4 + (lane >> 3) : iq * 32 + lane;
-      const int c = c0 + q;
-      v[u] = T(0);
-      if (it < ni && i < nA && q < CW) {
-        const int src = perm[i];
-        v[u] = c < nT ? B[cm ? (size_t)c * nA + src : (size_t)src * nT + c] : (c == nT ? T(rv[src]) : T(0));
+      for (int u = 0; u < SU; ++u) {
+        const int it = i0 + NW * u, iq = it / nr, row = (2 * (it - iq * nr) + (lane >> 4)) * V;
+        const int c = c0 + iq * 16 + (lane & 15);
+#pragma unroll
+        for (int e = 0; e < V; ++e) v[u].v[e] = T(0);
+        if (it < ni && row < nA) {
+          if (c < nT) {
+            v[u] = *reinterpret_cast<const SolveVec<T>*>(B + (size_t)c * nA + row);
+          } else if (c == nT) {
+#pragma unroll
+            for (int e = 0; e < V; ++e) v[u].v[e] = T(rv[row + e]);
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < SU; ++u) {
+        const int it = i0 + NW * u, iq = it / nr, row = (2 * (it - iq * nr) + (lane >> 4)) * V;
+        if (it < ni)
+#pragma unroll
+          for (int e = 0; e < V; ++e) Xs[(size_t)perm[row + e] * XST + iq * 16 + (lane & 15)] = v[u].v[e];
       }
     }
+  } else if (vecb) {
+    constexpr int LV = CW / V, RW = 32 / LV;  // lanes per row, rows per warp
+    const int q = lane % LV * V, c = c0 + q;
+    for (int i = wid * RW + lane / LV; i < nAp; i += NW * RW) {
+      T* dst = Xs + (size_t)i * XST + q;
+      if (i < nA && c < nT) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                     "l"(B + (size_t)perm[i] * nT + c)
+                     : "memory");
+      } else {
+        SolveVec<T> z;
 #pragma unroll
-    for (int u = 0; u < SU; ++u) {
-      const int it = i0 + NW * u, ir = it % nr, iq = it / nr;
+        for (int e = 0; e < V; ++e) z.v[e] = T(0);
+        if (i < nA && c == nT) z.v[0] = T(rv[perm[i]]);
+        *reinterpret_cast<SolveVec<T>*>(dst) = z;
+      }
+    }
+    cp_commit();
+  } else {
+    const int nr = cm ? nAp / 8 : nAp, ni = cm ? nr * (CW / 4) : nr * (CW / 32 + (CW % 32 != 0));
+    for (int it = wid; it < ni; it += NW) {
+      const int ir = it % nr, iq = it / nr;
       const int i = cm ? ir * 8 + (lane & 7) : ir, q = cm ? iq * 4 + (lane >> 3) : iq * 32 + lane;
-      if (it < ni && q < CW) Xs[(size_t)i * XST + q] = v[u];
+      const int c = c0 + q;
+      if (q >= CW) continue;
+      T v = T(0);
+      if (i < nA) {
+        const int src = perm[i];
+        v = c < nT ? B[cm ? (size_t)c * nA + src : (size_t)src * nT + c] : (c == nT ? T(rv[src]) : T(0));
+      }
+      Xs[(size_t)i * XST + q] = v;
     }
   }
   // rows [ra, ra + rows) of X -= (factor rows, columns p0 ..) x (solved rows p0 ..); the first tile is
@@ -409,15 +463,24 @@ __global__ void __launch_bounds__(32 * NW, 512 / (32 * NW)) k_big_solve(const __
       T x[SP];
 #pragma unroll
       for (int r = 0; r < SP; ++r) x[r] = Xs[(size_t)(p0 + r) * XST + tid];
+      // four rows at a time: their sums over the solved rows are independent chains
 #pragma unroll
-      for (int r = 1; r < SP; ++r)
+      for (int rb = 0; rb < SP; rb += 4) {
 #pragma unroll
-        for (int c = 0; c < r; c += V) {
-          const SolveVec<T> l = *reinterpret_cast<const SolveVec<T>*>(D + r * SP + c);
+        for (int c = 0; c < rb; c += V) {
+          SolveVec<T> l[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) l[i] = *reinterpret_cast<const SolveVec<T>*>(D + (rb + i) * SP + c);
 #pragma unroll
           for (int s = 0; s < V; ++s)
-            if (c + s < r) x[r] = fma(-l.v[s], x[c + s], x[r]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) x[rb + i] = fma(-l[i].v[s], x[c + s], x[rb + i]);
         }
+#pragma unroll
+        for (int i = 1; i < 4; ++i)
+#pragma unroll
+          for (int c = 0; c < i; ++c) x[rb + i] = fma(-D[(rb + i) * SP + rb + c], x[rb + c], x[rb + i]);
+      }
 #pragma unroll
       for (int r = 0; r < SP; ++r) Xs[(size_t)(p0 + r) * XST + tid] = x[r];
     }
@@ -434,25 +497,43 @@ __global__ void __launch_bounds__(32 * NW, 512 / (32 * NW)) k_big_solve(const __
     first_tile(0, p0, p0);
     cp_wait<1>();
     __syncthreads();
-    if (32 * wid < live) {  // whole warps: lane r holds the reciprocal of pivot r
+    if (32 * wid < live) {  // whole warps
       const int q = min(tid, CW - 1);
-      const T dl = lane < SP && p0 + lane < nA ? D[lane * SP + lane] : T(1);
-      const T il = T(1) / dl;
+      if (lane < SP) dinv[lane] = T(1) / (p0 + lane < nA ? D[lane * SP + lane] : T(1));
       T x[SP];
 #pragma unroll
       for (int r = 0; r < SP; ++r) x[r] = Xs[(size_t)(p0 + r) * XST + q];
+      __syncwarp();
+      bool fin = true;
 #pragma unroll
-      for (int r = SP - 1; r >= 0; --r) {
+      for (int rb = SP - 4; rb >= 0; rb -= 4) {
 #pragma unroll
-        for (int c = SP - V; c + V > r + 1; c -= V) {
-          const SolveVec<T> l = *reinterpret_cast<const SolveVec<T>*>(D + r * SP + c);
+        for (int c = SP - V; c >= rb + 4; c -= V) {
+          SolveVec<T> l[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) l[i] = *reinterpret_cast<const SolveVec<T>*>(D + (rb + i) * SP + c);
 #pragma unroll
           for (int s = V - 1; s >= 0; --s)
-            if (c + s > r) x[r] = fma(-l.v[s], x[c + s], x[r]);
+#pragma unroll
+            for (int i = 3; i >= 0; --i) x[rb + i] = fma(-l[i].v[s], x[c + s], x[rb + i]);
         }
-        x[r] = solve_div<T>(x[r], __shfl_sync(0xffffffffu, dl, r), __shfl_sync(0xffffffffu, il, r));
+#pragma unroll
+        for (int i = 3; i >= 0; --i) {
+#pragma unroll
+          for (int c = 3; c > i; --c) x[rb + i] = fma(-D[(rb + i) * SP + rb + c], x[rb + c], x[rb + i]);
+          x[rb + i] = solve_div<T>(x[rb + i], D[(rb + i) * SP + rb + i], dinv[rb + i]);
+          fin = fin && isfinite(x[rb + i]);
+        }
       }
-      if (tid < CW) {
+      if (__any_sync(0xffffffffu, !fin)) {  // out of range somewhere: the columns again, by divisions
+        if (tid < CW)
+          for (int r = SP - 1; r >= 0; --r) {
+            T* xr = Xs + (size_t)(p0 + r) * XST + tid;
+            T v = *xr;
+            for (int c = SP - 1; c > r; --c) v = fma(-D[r * SP + c], xr[(size_t)(c - r) * XST], v);
+            *xr = p0 + r < nA ? v / D[r * SP + r] : v;
+          }
+      } else if (tid < CW) {
 #pragma unroll
         for (int r = 0; r < SP; ++r) Xs[(size_t)(p0 + r) * XST + tid] = x[r];
       }
