@@ -1197,111 +1197,174 @@ __global__ void k_gen_precond_build_node(size_t nnode, int nv, const long long* 
     for (int c = 0; c < nv; ++c) P[r * nv + c] = T(W[r][nv + c]);
 }
 
-// face-block Jacobi: P_t = sum over the sides of the face's diagonal block of S_k, inverted in
-// place in shared memory by Gauss-Jordan elimination with partial pivoting (row interchanges,
-// undone at the end as column interchanges in reverse order), in the block precision T; one CTA
-// of GP_THREADS per trace face, bs x bs values plus bs multipliers and bs pivot rows of shared memory
-constexpr int GP_THREADS = 128;
-template <typename T>
-size_t precond_smem_bytes(int bsmax) {
-  return ((size_t)bsmax * bsmax + bsmax) * sizeof(T) + (size_t)bsmax * sizeof(int);
+// face-block Jacobi: P_t = sum over the sides of the face's diagonal block of S_k, inverted in the
+// block precision T by Gauss-Jordan elimination with partial pivoting.
+//
+// A thread holds a row in registers (BS of them: the largest face block, rounded up; columns beyond
+// the face's bs stay zero).  Columns rotate by one register per step, so that the pivot column is
+// register 0 and the finished column comes in at the end: every index is known at compile time and
+// a step is one multiply-add per value, with the pivot row broadcast from shared memory 16 bytes at a
+// time.  Pivot rows stay unscaled until the end (scaling commutes with the steps).  Rows are not exchanged: with row p_c the pivot of column c, entry (p_c, k) of the
+// result is entry (c, p_k) of the inverse, placed when the block goes out through shared memory.
+// Faces of up to 32 rows take a warp each, larger ones a CTA of one warp per 32 rows.
+//
+// Bound by the chain of a step (pivot search, one reciprocal, pivot row through shared memory), so
+// what counts is how many faces an SM holds.
+// Measured, the whole condensation it ends (the block in shared memory, three accesses per multiply-add
+// and five barriers per step, against this): 4608 hexahedra of p = 3 (80 x 80) FP32 46.5 -> 42.9 ms,
+// p = 2 (45 x 45) 12.9 -> 12.1 ms, 10 000 wall elements of p = 2..5 7.34 -> 7.08 ms; FP64, bound by the
+// rest, 1129 -> 1129, 152.8 -> 152.2 and 47.0 -> 46.5 ms.
+template <typename T, int BS>
+struct PrecondBuild {
+  static constexpr int WPF = (BS + 31) / 32;       // warps of a face
+  static constexpr int FPC = WPF == 1 ? 4 : 1;     // faces of a CTA
+  static constexpr int LD = BS + 1;                // odd: rows of the staged block start on all banks
+  static constexpr int VALUES = BS + BS * LD;      // pivot row, block
+  static constexpr size_t SMEM = (size_t)FPC * VALUES * sizeof(T);
+  static_assert(BS % 4 == 0 && VALUES % 4 == 0, "pivot rows are read as 16-byte vectors");
+};
+// |x| as an integer that orders as |x| does; 0 for NaN (never a pivot)
+__device__ __forceinline__ unsigned long long pivot_key(float x) {
+  return x == x ? (unsigned long long)(__float_as_uint(x) & 0x7fffffffu) : 0ull;
+}
+__device__ __forceinline__ unsigned long long pivot_key(double x) {
+  return x == x ? (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull : 0ull;
 }
 template <typename T>
-__global__ void __launch_bounds__(GP_THREADS) k_gen_precond_build(int ntrace, int nv, const int* __restrict__ tpts,
-                                                                const long long* __restrict__ poff,
-                                                                const int* __restrict__ pside,
-                                                                const int* __restrict__ nTk,
-                                                                const long long* __restrict__ offD,
-                                                                const T* __restrict__ S, T* __restrict__ Pinv,
-                                                                int* status) {
+__device__ __forceinline__ unsigned long long pivot_warp_max(unsigned long long k) {
+  const unsigned lo = __reduce_max_sync(0xffffffffu, sizeof(T) == 4 ? (unsigned)k : (unsigned)(k >> 32));
+  if (sizeof(T) == 4) return lo;
+  return ((unsigned long long)lo << 32) | __reduce_max_sync(0xffffffffu, (unsigned)(k >> 32) == lo ? (unsigned)k : 0u);
+}
+
+template <typename T, int BS>
+__global__ void __launch_bounds__(32 * PrecondBuild<T, BS>::WPF * PrecondBuild<T, BS>::FPC)
+    k_gen_precond_build(int ntrace, int nv, const int* __restrict__ tpts, const long long* __restrict__ poff,
+                        const int* __restrict__ pside, const int* __restrict__ nTk,
+                        const long long* __restrict__ offD, const T* __restrict__ S, T* __restrict__ Pinv, int* status) {
+  using B = PrecondBuild<T, BS>;
+  constexpr int WPF = B::WPF, LD = B::LD, VW = 16 / (int)sizeof(T), GT = 32 * WPF;
+  struct alignas(16) Vec {
+    T v[VW];
+  };
   extern __shared__ __align__(16) unsigned char gp_smem[];
-  __shared__ int s_piv, s_bad;
-  const int t = blockIdx.x, tid = threadIdx.x;
-  if (t >= ntrace) return;
+  __shared__ int s_perm[B::FPC][BS], s_row[WPF];
+  __shared__ unsigned long long s_key[WPF];
+  __shared__ T s_inv[B::FPC];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = warp / WPF, wi = warp % WPF;
+  const int row = 32 * wi + lane;
+  const int t = blockIdx.x * B::FPC + grp;
+  if (t >= ntrace) return;  // a whole warp of a one-warp group; larger groups are a CTA each
+  auto sync = [&]() {
+    if constexpr (WPF == 1) __syncwarp();
+    else __syncthreads();
+  };
   const int bs = tpts[t] * nv;
-  T* W = reinterpret_cast<T*>(gp_smem);  // bs x bs, row-major
-  T* L = W + (size_t)bs * bs;             // multipliers of the current column
-  int* perm = reinterpret_cast<int*>(L + bs);
-  for (int i = tid; i < bs * bs; i += GP_THREADS) {
+  T* prow = reinterpret_cast<T*>(gp_smem) + (size_t)grp * B::VALUES;
+  T* W = prow + BS;
+  int* perm = s_perm[grp];
+  const int k0 = pside[4 * t], l0 = pside[4 * t + 1], k1 = pside[4 * t + 2], l1 = pside[4 * t + 3];
+  const int n0 = k0 >= 0 ? nTk[k0] : 0, n1 = k1 >= 0 ? nTk[k1] : 0;
+  const T* S0 = k0 >= 0 ? S + offD[k0] + (size_t)l0 * n0 + l0 : S;
+  const T* S1 = k1 >= 0 ? S + offD[k1] + (size_t)l1 * n1 + l1 : S;
+#pragma unroll 4
+  for (int i = row; i < bs * bs; i += GT) {
     const int r = i / bs, c = i % bs;
     T v = T(0);
-    for (int sd = 0; sd < 2; ++sd) {
-      const int kk = pside[4 * t + 2 * sd], lo = pside[4 * t + 2 * sd + 1];
-      if (kk < 0) continue;
-      const int nT = nTk[kk];
-      v += S[offD[kk] + (size_t)(lo + r) * nT + lo + c];
-    }
-    W[i] = v;
+    if (k0 >= 0) v += S0[(size_t)r * n0 + c];
+    if (k1 >= 0) v += S1[(size_t)r * n1 + c];
+    W[r * LD + c] = v;
   }
-  if (tid == 0) s_bad = 0;
-  __syncthreads();
-  for (int c = 0; c < bs; ++c) {
-    if (tid < 32) {
-      T bv = T(-1);
-      int bi = bs;
-      for (int r = c + tid; r < bs; r += 32) {
-        const T v = fabs(W[r * bs + c]);
-        if (v > bv || (v == bv && r < bi)) {
-          bv = v;
-          bi = r;
-        }
-      }
+  sync();
+  T x[BS];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const T ov = __shfl_xor_sync(0xffffffffu, bv, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ov > bv || (ov == bv && oi < bi)) {
-          bv = ov;
-          bi = oi;
+  for (int k = 0; k < BS; ++k) x[k] = row < bs && k < bs ? W[row * LD + k] : T(0);
+  int step = row < bs ? -1 : bs;  // the column this row is the pivot of
+  T inv = T(0);                   // its pivot's reciprocal
+  bool bad = false;
+  for (int c = 0; c < bs; ++c) {
+    const unsigned long long key = step < 0 ? pivot_key(x[0]) : 0ull;
+    unsigned long long best = pivot_warp_max<T>(key);
+    int pr = 32 * wi + __ffs(__ballot_sync(0xffffffffu, key == best)) - 1;
+    if constexpr (WPF == 1) {
+      __syncwarp();  // the pivot row of the step before has been read
+    } else {
+      if (lane == 0) {
+        s_key[wi] = best;
+        s_row[wi] = pr;
+      }
+      __syncthreads();
+      best = s_key[0];
+      pr = s_row[0];
+#pragma unroll
+      for (int w = 1; w < WPF; ++w)
+        if (s_key[w] > best) {
+          best = s_key[w];
+          pr = s_row[w];
         }
-      }
-      if (tid == 0) {
-        s_piv = bi;
-        perm[c] = bi;
-        if (!(bv > T(0))) s_bad = 1;
-      }
     }
-    __syncthreads();
-    if (s_bad) break;
-    const int pv = s_piv;
-    if (pv != c)
-      for (int x = tid; x < bs; x += GP_THREADS) {
-        const T u = W[c * bs + x];
-        W[c * bs + x] = W[pv * bs + x];
-        W[pv * bs + x] = u;
-      }
-    __syncthreads();
-    const T inv = T(1) / W[c * bs + c];
-    for (int r = tid; r < bs; r += GP_THREADS) L[r] = r == c ? T(0) : W[r * bs + c];
-    __syncthreads();
-    for (int x = tid; x < bs; x += GP_THREADS) W[c * bs + x] = (x == c ? T(1) : W[c * bs + x]) * inv;
-    __syncthreads();
-    for (int r = tid >> 5; r < bs; r += GP_THREADS / 32) {  // one warp per row, lanes along it
-      if (r == c) continue;
-      const T l = L[r];
-      for (int x = tid & 31; x < bs; x += 32) W[r * bs + x] = (x == c ? T(0) : W[r * bs + x]) - l * W[c * bs + x];
+    if (best == 0ull) {  // the same in every thread of the face
+      bad = true;
+      break;
     }
-    __syncthreads();
+    if (row == pr) {  // the rest of the row and the 1 of its finished column, unscaled
+#pragma unroll
+      for (int k = 0; k < BS; k += VW) {
+        Vec o;
+#pragma unroll
+        for (int u = 0; u < VW; ++u) o.v[u] = k + u + 1 < BS ? x[k + u + 1] : T(1);
+        *reinterpret_cast<Vec*>(prow + k) = o;
+      }
+      inv = T(1) / x[0];
+      s_inv[grp] = inv;
+      step = c;
+      perm[c] = row;
+    }
+    sync();
+    const T l = row == pr ? T(0) : x[0] * s_inv[grp];
+#pragma unroll
+    for (int k = 0; k < BS; k += VW) {
+      const Vec p = *reinterpret_cast<const Vec*>(prow + k);
+#pragma unroll
+      for (int u = 0; u < VW; ++u)
+        x[k + u] = (k + u + 1 < BS ? x[k + u + 1] : (row == pr ? T(1) : T(0))) - l * p.v[u];
+    }
   }
-  if (s_bad) {
-    if (tid == 0) {
+  if (bad) {
+    if (row == 0) {
       atomicOr(status, DEV_ERR_SINGULAR);
       atomicMin(status + 1, -1 - t);
     }
     return;
   }
-  for (int c = bs - 1; c >= 0; --c) {
-    const int pv = perm[c];
-    if (pv != c)
-      for (int r = tid; r < bs; r += GP_THREADS) {
-        const T u = W[r * bs + c];
-        W[r * bs + c] = W[r * bs + pv];
-        W[r * bs + pv] = u;
-      }
-    __syncthreads();
+  sync();
+  if (row < bs) {
+#pragma unroll
+    for (int k = 0; k < BS; ++k)
+      if (k >= BS - bs) W[step * LD + perm[k - (BS - bs)]] = x[k] * inv;
   }
+  sync();
   T* P = Pinv + poff[t];
-  for (int i = tid; i < bs * bs; i += GP_THREADS) P[i] = W[i];
+  for (int i = row; i < bs * bs; i += GT) P[i] = W[i / bs * LD + i % bs];
+}
+
+// the smallest row length that holds the mesh's largest face block: 24 (quadrilaterals, hexahedra of
+// p = 1), 48 (p = 2), 80 (p = 3)
+template <typename T, int BS>
+static cudaError_t precond_build_launch(const GenCtx* g, bool prepare) {
+  using B = PrecondBuild<T, BS>;
+  auto kern = k_gen_precond_build<T, BS>;
+  if (prepare) return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B::SMEM);
+  (count_launch(), kern<<<(g->ntrace + B::FPC - 1) / B::FPC, 32 * B::WPF * B::FPC, B::SMEM, g->st>>>(
+       g->ntrace, g->nv, g->tpts, g->poff, g->pside, g->nTk, g->offD, (const T*)g->S, (T*)g->Pinv, g->status));
+  return cudaGetLastError();
+}
+template <typename T>
+static cudaError_t precond_build(const GenCtx* g, bool prepare) {
+  if (g->bsmax <= 24) return precond_build_launch<T, 24>(g, prepare);
+  if (g->bsmax <= 48) return precond_build_launch<T, 48>(g, prepare);
+  if (g->bsmax <= 80) return precond_build_launch<T, 80>(g, prepare);
+  return cudaErrorInvalidValue;
 }
 
 // z_t = Pinv_t v_t (v first normalised in place by *inv_h when given); one warp per trace face
@@ -1860,11 +1923,7 @@ int create(const fr_mesh_desc* mesh, const fr_config* cfg, cudaStream_t st, cons
   g->bsmax = 0;
   for (int t = 0; t < nt; ++t) g->bsmax = std::max(g->bsmax, tpts[t] * nv);
   if (!efr && nt > 0) {
-    const size_t sm = g->pb == 8 ? precond_smem_bytes<double>(g->bsmax) : precond_smem_bytes<float>(g->bsmax);
-    const cudaError_t ea = g->pb == 8 ? cudaFuncSetAttribute(k_gen_precond_build<double>,
-                                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)
-                                   : cudaFuncSetAttribute(k_gen_precond_build<float>,
-                                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const cudaError_t ea = g->pb == 8 ? precond_build<double>(g, true) : precond_build<float>(g, true);
     if (ea != cudaSuccess) {
       destroy(g);
       return FR_ERR_UNSUPPORTED;
@@ -2412,16 +2471,8 @@ static int condense_impl(GenCtx* g) {
       (count_launch(), k_gen_precond_build_node<float><<<nb256(g->npts), 256, 0, g->st>>>(
            g->npts, g->nv, g->nptr, g->nent_k, g->nent_l, g->nTk, g->offD, (const float*)g->S, (float*)g->Pinv,
            g->status));
-    else if (g->pb == 8)
-      (count_launch(), k_gen_precond_build<double><<<g->ntrace, GP_THREADS, precond_smem_bytes<double>(g->bsmax),
-                                                      g->st>>>(g->ntrace, g->nv, g->tpts, g->poff, g->pside, g->nTk,
-                                                               g->offD, (const double*)g->S, (double*)g->Pinv,
-                                                               g->status));
     else
-      (count_launch(), k_gen_precond_build<float><<<g->ntrace, GP_THREADS, precond_smem_bytes<float>(g->bsmax),
-                                                     g->st>>>(g->ntrace, g->nv, g->tpts, g->poff, g->pside, g->nTk,
-                                                              g->offD, (const float*)g->S, (float*)g->Pinv,
-                                                              g->status));
+      GCK(g->pb == 8 ? precond_build<double>(g, false) : precond_build<float>(g, false));
     GCK(cudaGetLastError());
   }
   pend(g, ph);
