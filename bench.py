@@ -485,7 +485,7 @@ def general_leg(pkg, torch, dev, l2buf, name, steps=(3, 2), warmup=(2, 1), peaks
             "condense": {"kernel": cond_kernel, "bound": "alu", "achieved": cond_a, "peak": fp32,
                          "unit": "TFLOP/s", "frac": cond_a / fp32, "avg_launch_ms": ms / max(cnt, 1),
                          "algorithmic_flop": flop},
-            "gmres": {"kernel": "multi-kernel GMRES cycle (k_gen_matvec_elem, k_gen_gather_sum, k_gen_precond_apply, k_cgs)",
+            "gmres": {"kernel": "k_gmres_cycle_any (one launch per restart cycle)",
                       "bound": "hbm", "achieved": g_a, "peak": hbm, "unit": "GB/s", "frac": g_a / hbm,
                       "avg_solve_ms": gms / max(gcnt, 1), "iterations_per_solve": k_its, "algorithmic_bytes": alg},
         },
