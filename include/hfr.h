@@ -238,15 +238,17 @@ int imex_refresh_jacobian(fr_ctx* ctx);
  * solution update -- is one cooperative launch with one CTA per SM that meets at grid barriers;
  * available for trace blocks (nT, n nv) = (64,16), (80,20), (48,12) on devices with cooperative
  * launch.  Each barrier wait is bounded (about 2 s); a wait that runs out ends the launch and
- * hfr_trace_gmres returns FR_ERR_TIMEOUT.  FR_GMRES_MULTI: one short kernel per step with the
- * Krylov state on the device (any shape).  Contexts without the fixed-shape cycle (other trace
- * blocks, general meshes) report FR_GMRES_MULTI and until it is set explicitly run each restart
- * cycle as one launch as well (FP64 basis; bounded barriers, or one thread-block cluster for
- * systems of a few thousand values); setting it gives the short kernels.  Both compute the same iteration (classical
- * Gram-Schmidt with a conditional second pass); their results agree to rounding.
+ * hfr_trace_gmres returns FR_ERR_TIMEOUT.  FR_GMRES_MULTI: the cycle without a fixed shape: one short
+ * kernel per step with the Krylov state on the device where FR_GMRES_FUSED is available too; the
+ * default of contexts without it (other trace blocks, general meshes), which run each restart cycle
+ * as one launch as well where the device allows it (FP64 basis; bounded barriers, or one thread-block
+ * cluster for systems of a few thousand values).  FR_GMRES_SHORT: the short kernels on every
+ * context, until another mode is set.  All compute the same iteration (classical Gram-Schmidt with
+ * a second pass); their results agree to rounding.
  * set: FR_ERR_UNSUPPORTED if FR_GMRES_FUSED is not available for the context.
- * get: the mode in effect, -1 for a null context.  This switch has no counterpart in the paper. */
-enum fr_gmres_mode { FR_GMRES_MULTI = 0, FR_GMRES_FUSED = 1 };
+ * get: the mode set last (the default before), so that setting what get returned changes nothing;
+ * -1 for a null context.  This switch has no counterpart in the paper. */
+enum fr_gmres_mode { FR_GMRES_MULTI = 0, FR_GMRES_FUSED = 1, FR_GMRES_SHORT = 2 };
 int hfr_gmres_set_mode(fr_ctx* ctx, int mode);
 int hfr_gmres_get_mode(const fr_ctx* ctx);
 

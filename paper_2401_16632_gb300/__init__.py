@@ -31,7 +31,7 @@ LIB_CHECKED_PATH = os.path.join(HERE, "libhfr_checked.so")
 FR_PREC_FP64, FR_PREC_FP32, FR_PREC_TF32, FR_PREC_BF16 = 0, 1, 2, 3
 FR_TAB_BE, FR_TAB_SDIRK2 = 0, 1
 FR_PHYS_ADVDIFF, FR_PHYS_NAVIER_STOKES, FR_PHYS_EDAC = 0, 1, 2
-FR_GMRES_MULTI, FR_GMRES_FUSED = 0, 1
+FR_GMRES_MULTI, FR_GMRES_FUSED, FR_GMRES_SHORT = 0, 1, 2
 FR_BC_WALL, FR_BC_FARFIELD = 1, 2
 FR_TRACE_HFR, FR_TRACE_EFR = 0, 1
 FR_ELEM_QUAD, FR_ELEM_HEX = 0, 1

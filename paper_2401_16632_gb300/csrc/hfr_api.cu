@@ -91,7 +91,7 @@ struct fr_ctx {
   GmresBuffers gm;
   int gm_mode = 0;          // 0: multi-kernel cycle, 1: one cooperative launch per cycle
   CyclePlan plan;           // shapes without a compiled cycle: the single launch of any layout (grid 0: none)
-  int short_kernels = 0;    // FR_GMRES_MULTI asked for: one kernel per step on those shapes too
+  int short_kernels = 0;    // FR_GMRES_SHORT: one kernel per step on those shapes and meshes too
   double* yv = nullptr;     // its element view
   int jac_policy = 0;       // fr_jacobian_policy
   // condensation held for FR_JAC_KEEP: valid, for which a_ii dt, refresh asked by the caller
@@ -1163,21 +1163,24 @@ extern "C" int imex_refresh_jacobian(fr_ctx* ctx) {
 }
 
 extern "C" int hfr_gmres_set_mode(fr_ctx* ctx, int mode) {
-  if (ctx && ctx->gen && mode == FR_GMRES_MULTI) {
-    hfr::gen::set_short_kernels(ctx->gen);
+  if (ctx && ctx->gen && (mode == FR_GMRES_MULTI || mode == FR_GMRES_SHORT)) {
+    ctx->short_kernels = mode == FR_GMRES_SHORT;
+    hfr::gen::set_short_kernels(ctx->gen, ctx->short_kernels);
     return FR_OK;
   }
   NOT_GENERAL(ctx, "hfr_gmres_set_mode (single-launch cycle)");
-  if (!ctx || (mode != FR_GMRES_MULTI && mode != FR_GMRES_FUSED))
+  if (!ctx || (mode != FR_GMRES_MULTI && mode != FR_GMRES_FUSED && mode != FR_GMRES_SHORT))
     return set_err(ctx, FR_ERR_INVALID_ARG, "hfr_gmres_set_mode: bad argument");
   if (mode == FR_GMRES_FUSED && ctx->gm_fused_grid <= 0)
     return set_err(ctx, FR_ERR_UNSUPPORTED, "hfr_gmres_set_mode: no single-launch cycle for this shape or device");
-  ctx->gm_mode = mode;
-  if (mode == FR_GMRES_MULTI) ctx->short_kernels = 1;
+  ctx->gm_mode = mode == FR_GMRES_FUSED ? 1 : 0;
+  ctx->short_kernels = mode == FR_GMRES_SHORT;
   return FR_OK;
 }
 
-extern "C" int hfr_gmres_get_mode(const fr_ctx* ctx) { return ctx ? ctx->gm_mode : -1; }
+extern "C" int hfr_gmres_get_mode(const fr_ctx* ctx) {
+  return ctx ? (ctx->short_kernels ? FR_GMRES_SHORT : ctx->gm_mode) : -1;
+}
 
 extern "C" int hfr_condense_set_mode(fr_ctx* ctx, int mode) {
   NOT_GENERAL(ctx, "hfr_condense_set_mode");
@@ -1267,6 +1270,7 @@ static int autotune_uniform(fr_ctx* ctx, const double* u, const double* uhat, co
   ctx->inv_ctas = best_ctas;
   // GMRES cycle form (same iteration either way): on the condensed system of the chosen mode
   int best_gm = ctx->gm_mode;
+  ctx->short_kernels = 0;
   if (!rc && ctx->ntrace > 0) rc = condense();
   if (!rc && ctx->ntrace > 0) {
     double bg = 1e30;

@@ -2738,9 +2738,10 @@ __global__ void k_gs_gmres_done(GStageDev* sd, const GmresGraphDev* gd) {
   if (gd->timeout) sd->err |= 4;
 }
 
-void set_short_kernels(GenCtx* g) {
-  g->short_kernels = 1;
-  g->gvalid = false;
+void set_short_kernels(GenCtx* g, int on) {
+  if (g->short_kernels == on) return;
+  g->short_kernels = on;
+  g->gvalid = false;  // a captured stage holds the other form
 }
 
 int set_graph(GenCtx* g, int on) {

@@ -38,8 +38,8 @@ int stage(GenCtx* g, int stage, double dt, const double* u_n, double* u_stage, d
           double newton_tol, int newton_maxit, double gmres_rtol, int gmres_maxit, int refine, fr_stage_stats* st);
 // the implicit stages as one CUDA graph each (captured on the first call with a new key)
 int set_graph(GenCtx* g, int on);
-// GMRES as one kernel per step from now on (hfr_gmres_set_mode(FR_GMRES_MULTI))
-void set_short_kernels(GenCtx* g);
+// GMRES as one kernel per step (on = 1: FR_GMRES_SHORT) or one launch per restart cycle
+void set_short_kernels(GenCtx* g, int on);
 int nstages(const GenCtx* g);
 size_t state_values(const GenCtx* g);
 

@@ -132,7 +132,7 @@ struct GenCtx {
   int ccap = 0;
   GmresBuffers gm;
   CyclePlan plan;            // the single-launch GMRES cycle (grid 0: one kernel per step)
-  int short_kernels = 0;     // hfr_gmres_set_mode(FR_GMRES_MULTI): one kernel per step
+  int short_kernels = 0;     // hfr_gmres_set_mode(FR_GMRES_SHORT): one kernel per step
   unsigned* gm_bar = nullptr;
   bool lin_valid = false;
   void* jscratch = nullptr;  // hexahedra: pointwise Jacobians, one slab per CTA of the block kernel

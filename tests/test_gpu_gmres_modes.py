@@ -1,0 +1,86 @@
+"""hfr_gmres_set_mode / hfr_gmres_get_mode on contexts without a compiled cycle: setting the mode that
+get returned changes nothing, FR_GMRES_SHORT gives the short kernels and FR_GMRES_MULTI the default
+again; both forms of the cycle agree on the same condensed system.
+
+Tolerance: both solves end at a relative residual of 1e-11 (FP64) or 1e-6 (FP32 blocks, whose
+mat-vec carries about 1e-7), and the condition numbers of these systems are below 1e3: the
+solutions agree to 1e-8 and 1e-3."""
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need CUDA")
+    from paper_2401_16632_gb300.build import build
+
+    build()
+    torch.cuda.set_device(0)
+
+
+import paper_2401_16632_gb300 as pkg  # noqa: E402
+from workloads import make_config  # noqa: E402
+
+CASES = {
+    "advdiff_p1": lambda: make_config("advdiff", n=3, p=1),
+    "advdiff_p2": lambda: make_config("advdiff8"),
+    "advdiff_p3_large": lambda: make_config("advdiff", n=37, p=3, jitter=0.1, seed=2),
+    "edac_p2": lambda: make_config("edac", n=9, p=2),
+    "edac_p4": lambda: make_config("edac", n=12, p=4, jitter=0.1),
+    "vortex_p5": lambda: make_config("vortex", n=6, p=5, re=500.0),
+    "wall_small": lambda: make_config("boundary_layer", nx=5, ny=60),
+    "wall_large": lambda: make_config("boundary_layer", nx=60, ny=60),
+    "hex_p2": lambda: make_config("channel3d", n=(4, 7, 3), p=2, layers=2),
+    "hex_p3": lambda: make_config("channel3d", n=(3, 6, 4), p=3, layers=2),
+    "efr_p3": lambda: make_config("vortex", n=11, p=3),
+}
+
+
+def condensed(name, prec, restart, scale=0.3):
+    w = CASES[name]()
+    trace = pkg.FR_TRACE_EFR if name.startswith("efr") else pkg.FR_TRACE_HFR
+    ctx = pkg.Context(w.mesh, w.physics, precision=prec, gmres_restart=restart, trace_kind=trace)
+    u0 = ctx.pack_state(w.u0) if isinstance(w.u0, list) else np.asarray(w.u0)
+    u = torch.tensor(u0, device="cuda").reshape(ctx.state_shape).contiguous()
+    uh = ctx.hfr_initial_trace(u)
+    ctx.hfr_local_jacobian(u, uh * 1.001, u * 0.999, scale * w.dt)
+    ctx.hfr_condense()
+    return ctx
+
+
+def solve(ctx, rtol):
+    n0 = ctx.kernel_launches()
+    x, its, rel = ctx.hfr_trace_gmres(rtol=rtol, maxit=3000)
+    return x.clone(), its, rel, ctx.kernel_launches() - n0
+
+
+@pytest.mark.parametrize("name", list(CASES))
+@pytest.mark.parametrize("prec", [pkg.FR_PREC_FP64, pkg.FR_PREC_FP32])
+@pytest.mark.parametrize("restart", [30, 7])
+def test_modes_round_trip_and_both_forms_agree(name, prec, restart):
+    ctx = condensed(name, prec, restart)
+    rtol, tol = (1e-11, 1e-8) if prec == pkg.FR_PREC_FP64 else (1e-6, 1e-3)
+    a, ia, ra, la = solve(ctx, rtol)
+    assert ctx.hfr_gmres_get_mode() == pkg.FR_GMRES_MULTI
+    ctx.hfr_gmres_set_mode(ctx.hfr_gmres_get_mode())
+    b, ib, _, lb = solve(ctx, rtol)
+    assert (ib, lb) == (ia, la) and torch.equal(a, b)
+    with pytest.raises(pkg.HfrError) as ei:
+        ctx.hfr_gmres_set_mode(pkg.FR_GMRES_FUSED)
+    assert ei.value.code == pkg.FR_ERR_UNSUPPORTED
+    ctx.hfr_gmres_set_mode(pkg.FR_GMRES_SHORT)
+    assert ctx.hfr_gmres_get_mode() == pkg.FR_GMRES_SHORT
+    c, ic, rc, lc = solve(ctx, rtol)
+    assert lc >= 6 * ic  # a step: preconditioner, mat-vec, four Gram-Schmidt kernels at least
+    assert abs(ia - ic) <= 2 + ic // 10, (ia, ic)
+    assert float((a - c).norm()) <= tol * float(c.norm())
+    assert ra <= max(10 * rtol, 3 * rc)
+    ctx.hfr_gmres_set_mode(pkg.FR_GMRES_MULTI)
+    d, i_d, _, ld = solve(ctx, rtol)
+    assert (i_d, ld) == (ia, la) and torch.equal(a, d)
