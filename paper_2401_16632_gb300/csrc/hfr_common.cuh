@@ -329,11 +329,12 @@ enum { DEV_ERR_SINGULAR = 1, DEV_ERR_NAN = 2, DEV_ERR_INDEX = 4, DEV_ERR_TIMEOUT
 // Bounds-checked build (compile flag FR_CHECKED): every mesh-derived gather / scatter index of
 // the general path (trace point of an element face point, neighbour element and face, element
 // face point of a trace point, element-view entry of a trace value, trace value of an
-// element-view entry) and of the uniform path's residual and blocks (trace face, neighbour) goes
-// through FR_IDX(i, n, site): an index outside [0, n) is recorded in this translation unit's
-// device word (the first one: site and index; and a count) and replaced by 0, so the access
-// stays in bounds and the kernel goes on (never a trap).  fr_checked_status reads and clears the
-// words of every unit.  Without the flag FR_IDX is the index itself.
+// element-view entry), of the uniform path's residual and blocks (trace face, neighbour), and the
+// basis rows of the single-launch GMRES cycle of any layout go through FR_IDX(i, n, site): an index
+// outside [0, n) is recorded in this translation unit's device word (the first one: site and index;
+// and a count) and replaced by 0, so the access stays in bounds and the kernel goes on (never a
+// trap).  fr_checked_status reads and clears the words of every unit.  Without the flag FR_IDX is
+// the index itself.
 #ifdef FR_CHECKED
 namespace fr_chk {
 static __device__ unsigned long long g_first;  // (site << 48) | (index & (2^48 - 1)), 0 = none

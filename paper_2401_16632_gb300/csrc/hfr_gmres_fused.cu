@@ -1348,6 +1348,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_gmres_cycle_any(const __grid_
   const size_t pstride = (size_t)PG_ND * gridDim.x;
   double *V = a.V, *partial = a.partial;
   T* Z = reinterpret_cast<T*>(a.Z);
+  auto zrow = [&](int j) { return Z + (size_t)FR_IDX(j, GM_MAXM, 30) * n; };
   auto sync = [&]() -> bool {
     if constexpr (CLUSTER) {
       __syncthreads();
@@ -1398,18 +1399,19 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_gmres_cycle_any(const __grid_
     for (int j = 0;; ++j) {
       double* vj = V + (size_t)j * n;
       double* w = V + (size_t)(j + 1) * n;
-      // (A) lane 0 of warp 0: Givens rotation of column j-1; warps 1..: finish v_j, z_j = P^-1 v_j
+      // (A) lane 0 of warp 0: Givens rotation of column j-1; warps 1..: finish v_j, z_j = P^-1 v_j.
+      // Pass mm only ends the cycle: v_mm and z_mm are not needed, and Z has GM_MAXM rows.
       if (j > 0 && tid == 0) pg_givens(sh, j - 1, a.rtol, mm);
-      if (tid >= 32) {
+      if (tid >= 32 && j < mm) {
         pg_finish(V, n, sh.cf, sh.corr ? j : 0, sh.invT, vj, x0, x1);
         pg_sync_workers();
-        any_precond<T>(a, vj, Z + (size_t)j * n, t0, t1, tid - 32, PG_THREADS - 32);
+        any_precond<T>(a, vj, zrow(j), t0, t1, tid - 32, PG_THREADS - 32);
       }
       if (!sync()) return;
       __syncthreads();
       if (sh.done) break;
       // (B) y_k = S_k z_k
-      any_matvec<T, T>(a, Z + (size_t)j * n, xs);
+      any_matvec<T, T>(a, zrow(j), xs);
       if (!sync()) return;
       // (C) w = L z and h = V^T w
       any_gather<T>(a, nullptr, w, x0, x1);
@@ -1800,3 +1802,5 @@ int barrier_selftest(int nblocks, int absent, int rounds, double timeout_s, int*
 }
 
 }  // namespace hfr
+
+#include "hfr_checked_unit.inc"

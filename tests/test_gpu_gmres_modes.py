@@ -84,3 +84,25 @@ def test_modes_round_trip_and_both_forms_agree(name, prec, restart):
     ctx.hfr_gmres_set_mode(pkg.FR_GMRES_MULTI)
     d, i_d, _, ld = solve(ctx, rtol)
     assert (i_d, ld) == (ia, la) and torch.equal(a, d)
+
+
+# a scale of the time step at which the solve takes more than 64 iterations: whole cycles of the
+# longest restart length (and of one that is clamped to it).  The larger step raises the condition
+# numbers to some 1e4: with both residuals at 1e-11 the solutions agree to 1e-6.
+FULL = {"advdiff_p2": 30.0, "advdiff_p3_large": 3.0, "edac_p2": 3.0, "edac_p4": 3.0, "vortex_p5": 3.0, "wall_small": 0.3,
+        "wall_large": 0.3, "hex_p2": 3.0, "hex_p3": 3.0, "efr_p3": 3.0}
+
+
+@pytest.mark.parametrize("name", list(FULL))
+def test_cycles_of_the_longest_restart_length(name):
+    out = []
+    for restart in (64, 100):
+        ctx = condensed(name, pkg.FR_PREC_FP64, restart, FULL[name])
+        out.append(solve(ctx, 1e-11))
+    (a, ia, ra, la), (b, ib, _, lb) = out
+    assert ia > 64 and (ia, la) == (ib, lb) and torch.equal(a, b)
+    ctx.hfr_gmres_set_mode(pkg.FR_GMRES_SHORT)
+    c, ic, rc, _ = solve(ctx, 1e-11)
+    assert abs(ia - ic) <= 2 + ic // 10, (ia, ic)
+    assert ra <= 1e-10 and rc <= 1e-10
+    assert float((a - c).norm()) <= 1e-6 * float(c.norm())
