@@ -8,7 +8,8 @@
 //   2-3. X = A^{-1} P [B | r]: one CTA per block of columns of one element, the block whole in shared
 //      memory (permuted columns in, forward and back substitution by factor panels, X out once);
 //   4. S = D - C X_B, in FP32 on the tensor cores, in FP64 by the same batched GEMM;
-//   5. t = s - C x_r with FP64 accumulation (one CTA per element).
+//   5. t = s - C x_r with FP64 accumulation (one CTA per element); x_r is the right-hand side's column
+//      of step 2-3, in batches with FP32 blocks of more than XR32_MAX rows a substitution in FP64.
 // The batched GEMM is a register-tiled CUDA-core kernel: 128 x 128 output tiles in FP32 (32 x 32 in
 // FP64), 256 threads with 8 x 8 (2 x 2) outputs each, K staged through two shared-memory buffers 8
 // at a time; arithmetic in the block precision T.  Included by hfr_condense.cu (uses UnevenArgs and DEV_ERR_*).
@@ -897,22 +898,83 @@ __global__ void __launch_bounds__(btc::THREADS, 2) k_big_s_tc(const __grid_const
   if (w == 0) tmem_dealloc(tmem, TM);
 }
 
-// 5. t = s - C x_r (x_r came with X, the right-hand side's column of the column-block solve)
+// rows of FP32 blocks up to which x_r comes in FP32 with X: the accumulated rounding of a substitution
+// grows with the rows, and above this r stays in FP64 throughout (24 blocks of 1024 rows: error of x_r
+// 4.2e-7 of the largest value, rms 3.8e-8; 894 rows, in FP32: 5.7e-7, rms 6.5e-8)
+constexpr int XR32_MAX = 894;
+
+// y = U^{-1} L^{-1} P r in FP64 with the stored factors (row-major, unit lower L), y and pvs in shared
+// memory, one CTA: by panels of 32 rows, the products with the solved rows a row per warp (lanes along
+// it), then the panel's own triangle by one warp, a row per lane
 template <typename T>
+__device__ void xr_solve(const T* L, const int* piv, const double* r, int nA, double* y, int* pvs) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int i = threadIdx.x; i < nA; i += BT) {
+    const int p = piv[i];
+    pvs[i] = p >= 0 && p < nA ? p : i;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < nA; i += BT) {  // position i of P r: the interchanges from the last to the first
+    int pos = i;
+    for (int j = nA - 1; j >= 0; --j) {
+      const int p = pvs[j];
+      pos = pos == j ? p : (pos == p ? j : pos);
+    }
+    y[i] = r[pos];
+  }
+  __syncthreads();
+  const int np = (nA + 31) / 32;
+  for (int dir = 0; dir < 2; ++dir) {
+    for (int q = 0; q < np; ++q) {
+      const int p0 = 32 * (dir == 0 ? q : np - 1 - q), c0 = dir == 0 ? 0 : p0 + 32, c1 = dir == 0 ? p0 : nA;
+      for (int row = p0 + wid; row < min(p0 + 32, nA); row += BT / 32) {
+        double s = 0.0;
+        for (int c = c0 + lane; c < c1; c += 32) s = fma((double)L[(size_t)row * nA + c], y[c], s);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) y[row] -= s;
+      }
+      __syncthreads();
+      if (wid == 0) {
+        const int row = p0 + lane, n = min(32, nA - p0);
+        const T* Lr = L + (size_t)(row < nA ? row : p0) * nA + p0;
+        double v = row < nA ? y[row] : 0.0;
+        for (int k = 0; k < n; ++k) {
+          const int c = dir == 0 ? k : n - 1 - k;
+          if (dir == 1 && lane == c) v /= (double)Lr[c];
+          const double yc = __shfl_sync(0xffffffffu, v, c);
+          if (row < nA && (dir == 0 ? lane > c : lane < c)) v -= (double)Lr[c] * yc;
+        }
+        if (row < nA) y[row] = v;
+      }
+      __syncthreads();
+    }
+  }
+}
+
+// 5. t = s - C x_r.  XR: x_r by the FP64 substitution above, else as it came with X (the right-hand
+// side's column of the column-block solve)
+template <typename T, bool XR>
 __global__ void __launch_bounds__(BT) k_big_t(const __grid_constant__ UnevenArgs a, const int* __restrict__ list,
                                               int nlist, int uni_nA, int uni_nT) {
   __shared__ double y[1024];
+  __shared__ int pvs[XR ? 1024 : 1];
   for (int li = blockIdx.x; li < nlist; li += gridDim.x) {
     const Elem E = elem_of(a, list, li, uni_nA, uni_nT);
     const int nA = E.nA, nT = E.nT;
     const T* Cm = reinterpret_cast<const T*>(a.C) + E.o[1];
-    const double* xr = a.xr + E.o[3];
+    double* xr = a.xr + E.o[3];
     const double* sv = a.s + E.o[4];
     double* t = a.t + E.o[4];
     const bool cm = a.colmajor != 0;
     __syncthreads();
-    for (int i = threadIdx.x; i < nA; i += BT) y[i] = xr[i];
-    __syncthreads();
+    if constexpr (XR) {
+      xr_solve<T>(reinterpret_cast<const T*>(a.LU) + E.o[0], a.piv + E.o[3], a.r + E.o[3], nA, y, pvs);
+      for (int i = threadIdx.x; i < nA; i += BT) xr[i] = y[i];
+    } else {
+      for (int i = threadIdx.x; i < nA; i += BT) y[i] = xr[i];
+      __syncthreads();
+    }
     for (int row = threadIdx.x; row < nT; row += BT) {
       double acc = 0.0;
       for (int c = 0; c < nA; ++c) acc += (double)(cm ? Cm[(size_t)c * nT + row] : Cm[(size_t)row * nA + c]) * y[c];
@@ -1013,7 +1075,10 @@ cudaError_t condense_big(const UnevenArgs& a, const int* list, int nlist, int un
     }
     if (e != cudaSuccess) return e;
   }
-  (hfr::count_launch(), k_big_t<T><<<grid1, BT, 0, st>>>(a, list, nlist, uni_nA, uni_nT));
+  auto t_kern = k_big_t<T, false>;
+  if constexpr (sizeof(T) == 4)
+    if (max_nA > XR32_MAX) t_kern = k_big_t<T, true>;
+  (hfr::count_launch(), t_kern<<<grid1, BT, 0, st>>>(a, list, nlist, uni_nA, uni_nT));
   return cudaGetLastError();
 }
 
