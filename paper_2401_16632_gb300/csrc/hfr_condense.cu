@@ -1865,8 +1865,6 @@ __device__ void condense_smem_elem(const CondElem<T>& e, unsigned char* smem_raw
   int* sflag = lpiv + nA;  // [0] pivot row of the step, [1] zero pivot seen
   unsigned char* used = reinterpret_cast<unsigned char*>(sflag + 2);
   const int lane = tid & 31, wid = tid >> 5, nw = nth >> 5;
-  __shared__ T s_invs[1 + 8];  // the step's reciprocal pivot, one per thread group (its barrier id)
-  T& s_inv = s_invs[bar];
   using Key = decltype(abs_key(T(0)));
   int& s_p = sflag[0];
   int& s_bad = sflag[1];
@@ -1900,15 +1898,17 @@ __device__ void condense_smem_elem(const CondElem<T>& e, unsigned char* smem_raw
         lpiv[c] = bi;
         e.piv[c] = bi;
         if (!(best > 0)) s_bad = 1;
-        // once per step: a division by every warp took a third of the FP64 pipe at nA = 100
+        // the reciprocal once per step (a division by every warp took a third of the FP64 pipe at nA =
+        // 100), at the place where the scaled pivot row holds it: no memory beyond smem_elem_bytes
         const T pv = M[(size_t)bi * nc + c];
-        s_inv = pv != T(0) ? T(1) / pv : T(0);
+        pr[c] = pv != T(0) ? T(1) / pv : T(0);
       }
     }
     grp_sync(bar, nth);
     const int p = s_p;
-    const T inv = s_inv;
-    for (int j = tid; j < nc; j += nth) pr[j] = j == c ? inv : M[(size_t)p * nc + j] * inv;
+    const T inv = pr[c];
+    for (int j = tid; j < nc; j += nth)
+      if (j != c) pr[j] = M[(size_t)p * nc + j] * inv;
     for (int r = tid; r < nA; r += nth) cb[r] = M[(size_t)r * nc + c];
     grp_sync(bar, nth);
     // one warp per row, lanes along the row
@@ -2489,12 +2489,12 @@ __global__ void __launch_bounds__(LU_THREADS) k_condense_lu(const __grid_constan
   const int k = blockIdx.x;
   const int tid = threadIdx.x;
   const int rows2 = nA > nT ? nA : nT;
-  T* sA = reinterpret_cast<T*>(smem_raw);  // rows2 x nA (A, later C)
+  int& s_piv = *reinterpret_cast<int*>(smem_raw);
+  T* sA = reinterpret_cast<T*>(smem_raw + 16);  // rows2 x nA (A, later C)
   T* sX = sA + (size_t)rows2 * nA;          // nA x (nT + 1)
   T* sI = sX + (size_t)nA * ldx;            // nA reciprocal pivots
   using Key = decltype(abs_key(T(0)));
-  __shared__ int s_piv;
-  __shared__ int s_bad;
+  bool bad = false;                         // thread 0
   const T* gA = reinterpret_cast<const T*>(a.A) + (size_t)k * nA * nA;
   const T* gB = reinterpret_cast<const T*>(a.B) + (size_t)k * nA * nT;
   const T* gC = reinterpret_cast<const T*>(a.C) + (size_t)k * nT * nA;
@@ -2504,7 +2504,6 @@ __global__ void __launch_bounds__(LU_THREADS) k_condense_lu(const __grid_constan
     const int r = i / ldx, c = i % ldx;
     sX[i] = c < nT ? gB[(size_t)r * nT + c] : T(a.r[(size_t)k * nA + r]);
   }
-  if (tid == 0) s_bad = 0;
   __syncthreads();
   int* piv = a.piv + (size_t)k * nA;
   for (int c = 0; c < nA; ++c) {
@@ -2524,7 +2523,7 @@ __global__ void __launch_bounds__(LU_THREADS) k_condense_lu(const __grid_constan
       if (tid == 0) {
         s_piv = bi;
         piv[c] = bi;
-        if (!(best > 0)) s_bad = 1;
+        if (!(best > 0)) bad = true;
         const T pv = sA[bi * nA + c];
         sI[c] = pv != T(0) ? T(1) / pv : T(0);
       }
@@ -2575,7 +2574,7 @@ __global__ void __launch_bounds__(LU_THREADS) k_condense_lu(const __grid_constan
     }
     __syncthreads();
   }
-  if (tid == 0 && s_bad) {
+  if (tid == 0 && bad) {
     atomicOr(a.status, DEV_ERR_SINGULAR);
     atomicMin(a.status + 1, k);
   }
@@ -2731,10 +2730,16 @@ static cudaError_t cond_dispatch(const CondArgs& a, cudaStream_t st, int part) {
   return cond_smem<T>(a, st);
 }
 
+// all of the LU kernel's shared memory: the pivot row, A or C, [X_B | x_r], the reciprocals.  Nothing is
+// declared statically: any static variable takes 1 KB of the 227 that the limits below count on.
+static size_t lu_smem_bytes(size_t tb, int nA, int nT) {
+  const int rows2 = nA > nT ? nA : nT;
+  return tb * ((size_t)rows2 * nA + (size_t)nA * (nT + 1) + nA) + 16;
+}
+
 template <typename T>
 static cudaError_t cond_lu(const CondArgs& a, cudaStream_t st) {
-  const int rows2 = a.nA > a.nT ? a.nA : a.nT;
-  size_t smem = sizeof(T) * ((size_t)rows2 * a.nA + (size_t)a.nA * (a.nT + 1) + a.nA);
+  const size_t smem = lu_smem_bytes(sizeof(T), a.nA, a.nT);
   if (smem > 227 * 1024) return cond_dispatch<T>(a, st, 0);
   cudaError_t err = cudaFuncSetAttribute(k_condense_lu<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
@@ -2749,8 +2754,7 @@ int condense_tc_available(int prec_bytes, int nA, int nT) {
 }
 
 static bool lu_fits_smem(int prec_bytes, int nA, int nT) {
-  const int rows2 = nA > nT ? nA : nT;
-  return prec_bytes == 8 && sizeof(double) * ((size_t)rows2 * nA + (size_t)nA * (nT + 1) + nA) <= 227 * 1024;
+  return prec_bytes == 8 && lu_smem_bytes(8, nA, nT) <= 227 * 1024;
 }
 static bool reg_shape(int nA, int nT) {
   return (nA == 9 && nT == 12) || (nA == 16 && nT == 16) || (nA == 36 && nT == 48) || (nA == 64 && nT == 64) ||
