@@ -1122,7 +1122,7 @@ static int gmres_impl(fr_ctx* ctx, double* duhat, double rtol, int maxit, int* i
     grc = run_gmres_fused(fa, ctx->prec_bytes, ctx->gm_fused_grid, rtol, ctx->restart, maxit, &res, &timed_out,
                           ctx->stream, cond_status ? ctx->status : nullptr, cond_status);
   } else {
-    if (ctx->plan.grid > 0 && !ctx->short_kernels) {
+    if (ctx->plan.grid > 0 && !ctx->short_kernels && maxit >= 1) {
       CycleArgs a = cycle_args(ctx);
       a.x = duhat;
       grc = run_gmres_any(a, ctx->prec_bytes, ctx->plan, rtol, ctx->restart, maxit, true_res, &res, &timed_out,

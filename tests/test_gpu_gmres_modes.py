@@ -106,3 +106,25 @@ def test_cycles_of_the_longest_restart_length(name):
     assert abs(ia - ic) <= 2 + ic // 10, (ia, ic)
     assert ra <= 1e-10 and rc <= 1e-10
     assert float((a - c).norm()) <= 1e-6 * float(c.norm())
+
+
+@pytest.mark.parametrize("name", ["advdiff_p2", "edac_p2", "wall_small"])
+def test_no_krylov_iteration_is_run_where_none_is_allowed(name):
+    """imex_stage with gmres_maxit = 0: trace updates stay zero in both forms of the cycle."""
+    w = CASES[name]()
+    out = []
+    for mode in (pkg.FR_GMRES_MULTI, pkg.FR_GMRES_SHORT):
+        ctx = pkg.Context(w.mesh, w.physics, tableau=pkg.FR_TAB_SDIRK2)
+        ctx.hfr_gmres_set_mode(mode)
+        u0 = ctx.pack_state(w.u0) if isinstance(w.u0, list) else np.asarray(w.u0)
+        u = torch.tensor(u0, device="cuda").reshape(ctx.state_shape).contiguous()
+        uh = ctx.hfr_initial_trace(u)
+        uh0 = uh.clone()
+        R_hist, us = ctx.empty(3, *ctx.state_shape), ctx.empty(*ctx.state_shape)
+        ctx.imex_stage(0, w.dt, u, us, uh, R_hist)
+        with pytest.raises(pkg.HfrError) as ei:  # the trace equations are never solved
+            ctx.imex_stage(1, w.dt, u, us, uh, R_hist, newton_tol=1e-12, newton_maxit=3, gmres_maxit=0)
+        assert ei.value.code == pkg.FR_ERR_NOT_CONVERGED and ei.value.info.iteration == 3
+        assert torch.equal(uh, uh0)
+        out.append(us.clone())
+    assert torch.equal(*out)
