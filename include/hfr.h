@@ -298,7 +298,9 @@ int hfr_export(fr_ctx* ctx, int which, void* dst, size_t bytes);
  * context array with `bytes` (exactly its size) from the caller device buffer src, e.g. to condense
  * blocks formed elsewhere or to plant a defective block in a test.  A condensation held for
  * FR_JAC_KEEP is dropped.  In a bounds-checked build (FR_CHECKED) a general-mesh context also takes
- * array 64 (the face-point trace map), to plant a corrupted index that the device checks must catch.
+ * array 64 (the face-point trace map), 65 (the trace value of every element trace unknown, int32) and
+ * 66 (the element trace unknowns of every trace value, int64), and exports the latter two, to plant a
+ * corrupted index that the device checks must catch.
  * FR_ERR_INVALID_ARG for another array or size. */
 int hfr_import(fr_ctx* ctx, int which, const void* src, size_t bytes);
 

@@ -1506,7 +1506,7 @@ extern "C" int hfr_import(fr_ctx* ctx, int which, const void* src, size_t bytes)
   if (!ctx || !src) return FR_ERR_INVALID_ARG;
   if (ctx->gen) {
 #ifdef FR_CHECKED
-    const bool map = which == 64;  // the face-point trace map, a planted defect in checked builds
+    const bool map = which >= 64 && which <= 66;  // index tables, a planted defect in checked builds
 #else
     const bool map = false;
 #endif

@@ -1637,6 +1637,7 @@ static CycleArgs cycle_args(GenCtx* g) {
   a.gmap = g->gmap;
   a.vptr = g->vptr;
   a.vidx = g->vidx;
+  a.nview = (long long)g->sumT;
   a.tpts = g->tpts;
   a.toff = g->toff;
   a.poff = g->poff;
@@ -1894,7 +1895,8 @@ int create(const fr_mesh_desc* mesh, const fr_config* cfg, cudaStream_t st, cons
     }
   }
   for (size_t d = 0; d < g->nh; ++d) vptr[d + 1] += vptr[d];
-  std::vector<long long> vidx(std::max((size_t)vptr[g->nh], (size_t)1), 0);
+  g->nvidx = (size_t)vptr[g->nh];
+  std::vector<long long> vidx(std::max(g->nvidx, (size_t)1), 0);
   {
     std::vector<long long> fill(vptr.begin(), vptr.end() - 1);
     for (size_t l = 0; l < g->sumT; ++l)
@@ -2639,6 +2641,10 @@ int export_array(GenCtx* g, int which, void* buf, size_t bytes, bool import) {
       arr = g->fnode;
       need = (size_t)g->nface * g->E * g->fs * sizeof(int);
       break;
+#ifdef FR_CHECKED
+    case 65: arr = g->gmap; need = g->sumT * sizeof(int); break;        // element-view entry -> trace value
+    case 66: arr = g->vidx; need = g->nvidx * sizeof(long long); break;  // trace value -> element-view entries
+#endif
   }
   if (!arr) return err(g, FR_ERR_INVALID_ARG, "hfr_export / hfr_import: unknown array");
   if (import ? bytes != need : bytes < need)

@@ -106,6 +106,7 @@ struct GenCtx {
   unsigned char* fset = nullptr;   // per element face: 1 = GLL points (EFR)
   long long *gptr = nullptr, *gidx = nullptr;  // trace point <- element face points (CSR)
   long long *vptr = nullptr, *vidx = nullptr;  // trace value <- element-view entries (CSR)
+  size_t nvidx = 0;                            // entries of vidx
   long long* nptr = nullptr;       // EFR node blocks: entries (implicit element, local row) per node
   int *nent_k = nullptr, *nent_l = nullptr;
   double *Uf_all = nullptr, *qf_all = nullptr, *Rw = nullptr, *gview = nullptr, *gw = nullptr, *Ustar = nullptr;

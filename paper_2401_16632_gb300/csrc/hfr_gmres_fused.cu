@@ -1008,9 +1008,12 @@ struct AnyShape {  // the layout of one element or trace unit, from the tables o
   }
   // trace value of local unknown l of element k (its entries start at o), -1 off traces
   __device__ __forceinline__ long long gmap(int k, long long o, int l) const {
-    if (!a.uni_nT) return __ldg(a.gmap + o + l);
+    if (!a.uni_nT) {
+      const int g = __ldg(a.gmap + o + l);
+      return g < 0 ? -1 : (long long)FR_IDX(g, a.n, 31);
+    }
     const int f = l / a.uni_bs, t = __ldg(a.tr_of_c + 4 * k + f);
-    return t < 0 ? -1 : (long long)t * a.uni_bs + (l - f * a.uni_bs);
+    return t < 0 ? -1 : (long long)FR_IDX(t, a.ntrace, 32) * a.uni_bs + (l - f * a.uni_bs);
   }
   __device__ __forceinline__ int bs(int t) const { return a.uni_nT ? a.uni_bs : __ldg(a.tpts + t) * a.nv; }
   __device__ __forceinline__ long long toff(int t) const {
@@ -1046,7 +1049,8 @@ __device__ void any_gather(const CycleArgs& a, const double* base, double* out, 
 #pragma unroll
         for (int sd = 0; sd < 2; ++sd) {
           const int e = __ldg(a.sides + 4 * t + 2 * sd), f = __ldg(a.sides + 4 * t + 2 * sd + 1);
-          if (e >= 0) s[u] += any_widen(__ldcg(yv + (size_t)e * a.uni_nT + f * a.uni_bs + b));
+          if (e >= 0)
+            s[u] += any_widen(__ldcg(yv + (size_t)FR_IDX(e, a.Eim, 33) * a.uni_nT + FR_IDX(f, 4, 34) * a.uni_bs + b));
         }
       }
     } else {
@@ -1065,7 +1069,7 @@ __device__ void any_gather(const CycleArgs& a, const double* base, double* out, 
 #pragma unroll
         for (int u = 0; u < 4; ++u) ix[u] = c[u] + i < c1[u] ? __ldg(a.vidx + c[u] + i) : -1;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = ix[u] >= 0 ? __ldcg(yv + ix[u]) : T(0);
+        for (int u = 0; u < 4; ++u) v[u] = ix[u] >= 0 ? __ldcg(yv + FR_IDX(ix[u], a.nview, 35)) : T(0);
 #pragma unroll
         for (int u = 0; u < 4; ++u)
           if (ix[u] >= 0) s[u] += any_widen(v[u]);

@@ -101,7 +101,8 @@ struct CycleArgs {
   const int* nTk;                       // trace unknowns of each implicit element
   const long long *offD, *offs;         // their S blocks and element-view entries (Eim + 1)
   const int* gmap;                      // element-view entry -> trace value, -1 off traces
-  const long long *vptr, *vidx;         // trace value <- element-view entries (CSR)
+  const long long *vptr, *vidx;         // trace value <- element-view entries (CSR), nview entries
+  long long nview = 0;
   const int* tpts;                      // points of each trace unit
   const long long *toff, *poff;         // its values and its face-block inverse (ntrace + 1)
   int uni_nT = 0, uni_bs = 0;           // uniform mesh: nT, values per trace face
