@@ -418,6 +418,7 @@ static CycleArgs cycle_args(fr_ctx* ctx) {
   a.tr_of_c = ctx->tr_of_c;
   a.sides = ctx->sides_c;
   a.sumTT = (long long)ctx->Eim * ctx->nT * ctx->nT;
+  a.nTmax = ctx->nT;
   a.bsmax = a.uni_bs;
   a.S = ctx->S;
   a.Pinv = ctx->Pinv;

@@ -1642,6 +1642,7 @@ static CycleArgs cycle_args(GenCtx* g) {
   a.toff = g->toff;
   a.poff = g->poff;
   a.sumTT = (long long)g->sumTT;
+  a.nTmax = g->maxT;
   a.bsmax = g->bsmax;
   a.S = g->S;
   a.Pinv = g->Pinv;

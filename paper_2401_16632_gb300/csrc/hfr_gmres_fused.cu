@@ -1317,7 +1317,6 @@ __device__ void any_update_x(const T* Z, size_t n, const double* y, int k, doubl
   }
 }
 
-constexpr int ANY_MAXT = 512;    // trace unknowns of an element
 constexpr int ANY_CLUSTER = 8;
 template <typename T>
 constexpr size_t any_smem() {
@@ -1617,16 +1616,12 @@ cudaError_t launch_gmres_cycle(const FusedArgs& a, int prec_bytes, int grid, cud
 }
 
 template <typename T, bool CLUSTER>
-static cudaError_t launch_any(const CycleArgs& a, const CyclePlan& p, cudaStream_t s) {
-  auto kern = k_gmres_cycle_any<T, CLUSTER>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)any_smem<T>());
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(p.grid);
+static cudaError_t any_config(int grid, cudaStream_t s, cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&at)[1]) {
+  cfg = {};
+  cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(PG_THREADS);
   cfg.dynamicSmemBytes = any_smem<T>();
   cfg.stream = s;
-  cudaLaunchAttribute at[1];
   if (CLUSTER) {
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = ANY_CLUSTER;
@@ -1638,8 +1633,28 @@ static cudaError_t launch_any(const CycleArgs& a, const CyclePlan& p, cudaStream
   }
   cfg.attrs = at;
   cfg.numAttrs = 1;
+  return cudaFuncSetAttribute(k_gmres_cycle_any<T, CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)any_smem<T>());
+}
+
+template <typename T, bool CLUSTER>
+static cudaError_t launch_any(const CycleArgs& a, const CyclePlan& p, cudaStream_t s) {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at[1];
+  const cudaError_t e = any_config<T, CLUSTER>(p.grid, s, cfg, at);
+  if (e != cudaSuccess) return e;
   hfr::count_launch();
-  return cudaLaunchKernelEx(&cfg, kern, a);
+  return cudaLaunchKernelEx(&cfg, k_gmres_cycle_any<T, CLUSTER>, a);
+}
+
+// one cluster of the cycle can be resident on the device
+template <typename T>
+static bool cluster_fits() {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at[1];
+  int n = 0;
+  return any_config<T, true>(ANY_CLUSTER, nullptr, cfg, at) == cudaSuccess &&
+         cudaOccupancyMaxActiveClusters(&n, k_gmres_cycle_any<T, true>, &cfg) == cudaSuccess && n >= 1;
 }
 
 cudaError_t launch_cycle_any(const CycleArgs& a, int prec_bytes, const CyclePlan& p, cudaStream_t s) {
@@ -1654,12 +1669,17 @@ cudaError_t launch_cycle_any(const CycleArgs& a, int prec_bytes, const CyclePlan
 CyclePlan cycle_plan(int prec_bytes, const CycleArgs& a) {
   CyclePlan p;
   int dev = 0, coop = 0, nsm = 0, occ = 0;
-  if (a.ntrace <= 0 || a.Eim <= 0 || a.bsmax > 128) return p;
+  // what the kernel holds of an element (a warp's shared memory) and of a trace unit (registers)
+  if (a.ntrace <= 0 || a.Eim <= 0 || a.bsmax > 128 || a.nTmax > ANY_MAXT) return p;
   if (cudaGetDevice(&dev) != cudaSuccess) return p;
   if (a.sumTT + 40 * (long long)a.n <= 200000) {
-    p.grid = ANY_CLUSTER;
-    p.cluster = 1;
-    return p;
+    const bool ok = prec_bytes == 4 ? cluster_fits<float>() : cluster_fits<double>();
+    if (ok) {
+      p.grid = ANY_CLUSTER;
+      p.cluster = 1;
+      return p;
+    }
+    cudaGetLastError();
   }
   if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) return p;
   if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return p;

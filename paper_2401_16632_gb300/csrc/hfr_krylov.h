@@ -93,6 +93,7 @@ int run_gmres_fused(const FusedArgs& a, int prec_bytes, int grid, double rtol, i
 // one restart cycle (enqueue only; a.bar must be zeroed before it): cudaErrorInvalidValue when
 // the shape has no single-launch cycle
 cudaError_t launch_gmres_cycle(const FusedArgs& a, int prec_bytes, int grid, cudaStream_t s);
+constexpr int ANY_MAXT = 512;  // trace unknowns of an element that a warp stages
 // One restart cycle per launch for any trace layout (hfr_gmres_fused.cu, k_gmres_cycle_any), FP64
 // Krylov basis, the operator in the element view: y_k = S_k x_k, then the sum of the element entries
 // of every trace value.  General meshes give the tables; a uniform mesh (uni_nT > 0) its sizes.
@@ -108,6 +109,7 @@ struct CycleArgs {
   int uni_nT = 0, uni_bs = 0;           // uniform mesh: nT, values per trace face
   const int *tr_of_c = nullptr, *sides = nullptr;
   long long sumTT = 0;                  // values of all S blocks
+  int nTmax = 0;                        // trace unknowns of the largest element (at most ANY_MAXT)
   int bsmax = 0;                        // values of the largest trace unit (at most 128)
   const void *S, *Pinv;                 // block precision
   const double* t;                      // right-hand side
