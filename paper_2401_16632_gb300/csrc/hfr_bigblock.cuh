@@ -269,14 +269,30 @@ struct alignas(16) SolveVec {
   T v[16 / sizeof(T)];
 };
 
-// x / d with the reciprocal known: one Newton correction of the quotient (the division's own
-// rounding, without its long instruction sequence on the substitution's serial chain).  Not finite
-// where the reciprocal or a product leaves the range: the caller divides then.
+// x / d with inv = 1 / d (rounded) known: the product, then one correction by its remainder, the
+// quotient step of P. W. Markstein, "Computation of elementary functions on the IBM RISC System/6000
+// processor", IBM J. Res. Dev. 34 (1990).  It takes the division's instruction sequence off the
+// substitution's serial chain.  With unit roundoff u the product is within 2 u of x / d (at most two
+// units in the last place, not the one that would make the corrected quotient correctly rounded
+// always); the remainder leaves the fused multiply-add with a relative error of u and the correction
+// adds another, so that the result is within half a unit plus a few u of one.  Outside the
+// following the caller divides:
+//   * the result is not finite (the reciprocal or a product left the range);
+//   * 0 < |x| < 2^8 times the smallest normal number, where the remainder would lose bits to underflow
+//     (2^-8 of a unit at the bound, whole units below).
 template <typename T>
 __device__ __forceinline__ T solve_div(T x, T d, T inv) {
   const T q = x * inv;
   return fma(fma(-q, d, x), inv, q);
 }
+// that range of x as one integer comparison of a minimum over the values: key(x) < SOLVE_TINY (zero has
+// the largest key)
+__device__ __forceinline__ unsigned solve_key(float x) { return 2u * __float_as_uint(x) - 1u; }
+__device__ __forceinline__ unsigned solve_key(double x) {
+  return (2u * (unsigned)__double2hiint(x) | (__double2loint(x) != 0 ? 1u : 0u)) - 1u;
+}
+template <typename T>
+constexpr unsigned SOLVE_TINY = sizeof(T) == 4 ? (9u << 24) - 1u : (9u << 21) - 1u;
 
 template <typename T, int LC, int CW, int NW, int H>
 __global__ void __launch_bounds__(32 * NW, 512 / (32 * NW)) k_big_solve(const __grid_constant__ UnevenArgs a, const int* __restrict__ list,
@@ -506,6 +522,7 @@ __global__ void __launch_bounds__(32 * NW, 512 / (32 * NW)) k_big_solve(const __
       for (int r = 0; r < SP; ++r) x[r] = Xs[(size_t)(p0 + r) * XST + q];
       __syncwarp();
       bool fin = true;
+      unsigned least = ~0u;
 #pragma unroll
       for (int rb = SP - 4; rb >= 0; rb -= 4) {
 #pragma unroll
@@ -522,11 +539,12 @@ __global__ void __launch_bounds__(32 * NW, 512 / (32 * NW)) k_big_solve(const __
         for (int i = 3; i >= 0; --i) {
 #pragma unroll
           for (int c = 3; c > i; --c) x[rb + i] = fma(-D[(rb + i) * SP + rb + c], x[rb + c], x[rb + i]);
+          least = min(least, solve_key(x[rb + i]));
           x[rb + i] = solve_div<T>(x[rb + i], D[(rb + i) * SP + rb + i], dinv[rb + i]);
           fin = fin && isfinite(x[rb + i]);
         }
       }
-      if (__any_sync(0xffffffffu, !fin)) {  // out of range somewhere: the columns again, by divisions
+      if (__any_sync(0xffffffffu, !fin || least < SOLVE_TINY<T>)) {  // out of range somewhere: the columns again, by divisions
         if (tid < CW)
           for (int r = SP - 1; r >= 0; --r) {
             T* xr = Xs + (size_t)(p0 + r) * XST + tid;
