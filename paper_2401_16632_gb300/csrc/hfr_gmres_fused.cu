@@ -1416,18 +1416,35 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_gmres_cycle_any(const __grid_
       // (B) y_k = S_k z_k
       any_matvec<T, T>(a, zrow(j), xs);
       if (!sync()) return;
-      // (C) w = L z and h = V^T w
+      // (C) w = L z, h = V^T w and ||w||^2
       any_gather<T>(a, nullptr, w, x0, x1);
       double* part = partial + par * pstride;
-      pg_block_dots<double>(sh, V, n, j + 1, w, x0, x1, part);
+      pg_block_dots<double>(sh, V, n, j + 2, w, x0, x1, part);
       if (!sync()) return;
-      pg_reduce(sh, j + 1, part);
+      pg_reduce(sh, j + 2, part);
       par ^= 1;
-      for (int i = tid; i <= j; i += PG_THREADS) {
-        sh.hc[i] = sh.dot[i];
-        sh.cf[i] = sh.dot[i];
+      if (tid < 32) {
+        double hh = 0.0;
+        for (int i = tid; i <= j; i += 32) {
+          const double h = sh.dot[i];
+          hh += h * h;
+          sh.hc[i] = h;
+          sh.cf[i] = h;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) hh += __shfl_xor_sync(0xffffffffu, hh, o);
+        if (tid == 0) {
+          const double n0 = sh.dot[j + 1];
+          sh.corr = hh <= 0.5 * n0 ? 1 : 0;
+          if (sh.corr) sh.hc[j + 1] = sqrt(n0 - hh);
+        }
       }
       __syncthreads();
+      if (sh.corr) {  // little cancellation (the test of the short kernels): one pass, w' formed with v_{j+1}
+        if (tid == 0) sh.invT = sh.hc[j + 1] != 0.0 ? 1.0 / sh.hc[j + 1] : 0.0;
+        __syncthreads();
+        continue;
+      }
       // (D) w' = w - V h, then d = V^T w' and ||w'||^2
       pg_subtract(V, n, sh.cf, j, w, x0, x1);
       part = partial + par * pstride;
