@@ -1688,6 +1688,12 @@ CyclePlan cycle_plan(int prec_bytes, const CycleArgs& a) {
   int dev = 0, coop = 0, nsm = 0, occ = 0;
   // what the kernel holds of an element (a warp's shared memory) and of a trace unit (registers)
   if (a.ntrace <= 0 || a.Eim <= 0 || a.bsmax > 128 || a.nTmax > ANY_MAXT) return p;
+  // Large uniform systems of FP64 blocks with faces of more than 16 values (Navier-Stokes, p = 5): the
+  // short kernels' uniform mat-vec and preconditioner spend fewer FP64 instructions on lane sums and
+  // idle lanes, which outweighs the launches above some 10^8 values of S.  Time per iteration, single
+  // launch against short kernels: 96 x 96 elements (0.85 10^8) 416 / 448 us, 128 x 128 (1.5 10^8)
+  // 703 / 679 us, where the second Gram-Schmidt pass is not needed 380 / 385 and 637 / 586 us.
+  if (prec_bytes == 8 && a.uni_nT > 0 && a.uni_bs > 16 && a.sumTT > 100000000LL) return p;
   if (cudaGetDevice(&dev) != cudaSuccess) return p;
   if (a.sumTT + 40 * (long long)a.n <= 200000) {
     const bool ok = prec_bytes == 4 ? cluster_fits<float>() : cluster_fits<double>();

@@ -128,3 +128,25 @@ def test_no_krylov_iteration_is_run_where_none_is_allowed(name):
         assert torch.equal(uh, uh0)
         out.append(us.clone())
     assert torch.equal(*out)
+
+
+def test_large_uniform_fp64_systems_keep_the_short_kernels():
+    """More than 10^8 values of S with faces of 24: the default is the short kernels' solve, bit for bit;
+    one row of elements fewer and it is the single launch."""
+    for n, short in ((105, True), (104, False)):  # 1.016 and 0.997 10^8 values
+        w = make_config("vortex", n=n, p=5)
+        ctx = pkg.Context(w.mesh, w.physics, precision=pkg.FR_PREC_FP64)
+        u = torch.tensor(w.u0, device="cuda")
+        uh = ctx.hfr_initial_trace(u)
+        ctx.hfr_local_jacobian(u, uh * 1.001, u * 0.999, 0.3 * w.dt)
+        ctx.hfr_condense()
+        a, ia, _, la = solve(ctx, 1e-8)
+        assert ctx.hfr_gmres_get_mode() == pkg.FR_GMRES_MULTI
+        ctx.hfr_gmres_set_mode(pkg.FR_GMRES_SHORT)
+        b, ib, _, lb = solve(ctx, 1e-8)
+        assert (la == lb) == short
+        if short:
+            assert ia == ib and torch.equal(a, b)
+        else:
+            assert float((a - b).norm()) <= 1e-5 * float(b.norm())
+        ctx.close()
