@@ -21,10 +21,11 @@
 
 namespace hfr {
 
-template <typename T>
-__device__ __forceinline__ T tabs(T x) { return x < T(0) ? -x : x; }
 // |x| as an integer that orders as |x| does, -1 for NaN: pivot searches compare these on the integer
-// pipes (an FP64 comparison occupies the FP64 pipe as long as a multiply-add of a whole warp)
+// pipes (an FP64 comparison occupies the FP64 pipe as long as a multiply-add of a whole warp).  A search
+// that starts from key -1 and takes the lower row on equal keys finds an unused row in a column of NaN
+// too, so that every row is the pivot of one step whatever the values are; the kernels that leave rows
+// in place index by that step.
 __device__ __forceinline__ long long abs_key(double x) {
   const long long k = __double_as_longlong(x) & 0x7fffffffffffffffll;
   return k > 0x7ff0000000000000ll ? -1 : k;
@@ -97,7 +98,9 @@ __global__ void __launch_bounds__(GJ_THREADS) k_condense_reg(const __grid_consta
     T* pr = pivrow + buf * NC;
     T* cb = colbuf + buf * NA;
     const int qc = c / GJ_CG;
-    T best = T(-1), val = T(0);
+    using Key = decltype(abs_key(T(0)));
+    Key best = -1;
+    T val = T(0);
     int bi = 0x7fffffff;
 #pragma unroll
     for (int s = 0; s < RT; ++s) {
@@ -109,24 +112,23 @@ __global__ void __launch_bounds__(GJ_THREADS) k_condense_reg(const __grid_consta
           if (q == qc) v = m[s][q];
         cb[r] = v;
         if (!(used >> s & 1u)) {
-          const T av = tabs(v);
+          const Key av = abs_key(v);
           if (av > best || (av == best && r < bi)) { best = av; bi = r; val = v; }
         }
       }
     }
 #pragma unroll
     for (int o = 8; o > 0; o >>= 1) {
-      const T ob = __shfl_xor_sync(0x0000ffffu << (tid & 16), best, o);
+      const Key ob = __shfl_xor_sync(0x0000ffffu << (tid & 16), best, o);
       const int oi = __shfl_xor_sync(0x0000ffffu << (tid & 16), bi, o);
       const T ov = __shfl_xor_sync(0x0000ffffu << (tid & 16), val, o);
       if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; val = ov; }
     }
-    if (bi >= NA) bi = c;  // no candidate compared (NaN column): any row, flagged singular below
     if (rg == 0) {
       s_piv[buf] = bi;
       s_ipiv[bi] = c;
       a.piv[(size_t)k * NA + c] = bi;
-      if (!(best > T(0))) s_bad = 1;
+      if (!(best > 0)) s_bad = 1;  // zeros or NaN only
       pr[c] = T(1) + (val != T(0) ? T(1) / val : T(0));
     }
   };
@@ -328,8 +330,8 @@ __global__ void __launch_bounds__(InvShape<NA>::THREADS, NA <= 64 ? 8 : 3) k_inv
     if (h == 0) {
 #pragma unroll
       for (int s = 0; s < 4; ++s) {
-        const float v = fabsf(m[s][0]);
-        if (!(used >> s & 1u) && (v > best)) {
+        const float a0 = fabsf(m[s][0]), v = a0 == a0 ? a0 : -1.f;  // NaN below every value
+        if (!(used >> s & 1u) && (v > best || bi == 0x7fffffff)) {
           best = v;
           bi = 4 * g + s;
         }
@@ -370,7 +372,6 @@ __global__ void __launch_bounds__(InvShape<NA>::THREADS, NA <= 64 ? 8 : 3) k_inv
       b = __shfl_sync(0xffffffffu, b, 0);
       p = __shfl_sync(0xffffffffu, p, 0);
     }
-    if (p >= NA) p = c;  // no candidate compared (NaN column): any row, flagged singular below
     const int sp = p & 3;
     if (g == (p >> 2)) {
 #pragma unroll
@@ -1882,7 +1883,7 @@ __device__ void condense_smem_elem(const CondElem<T>& e, unsigned char* smem_raw
       for (int r = tid; r < nA; r += 32) {
         if (used[r]) continue;
         const Key v = abs_key(M[(size_t)r * nc + c]);
-        if (v > best || (v == best && v >= 0 && r < bi)) { best = v; bi = r; }
+        if (v > best || (v == best && r < bi)) { best = v; bi = r; }
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
@@ -1890,14 +1891,13 @@ __device__ void condense_smem_elem(const CondElem<T>& e, unsigned char* smem_raw
         const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
         if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
       }
-      if (bi >= nA) bi = c;  // no candidate compared (NaN column): any row, flagged singular
       if (tid == 0) {
         s_p = bi;
         used[bi] = 1;
         ipiv[bi] = c;
         lpiv[c] = bi;
         e.piv[c] = bi;
-        if (!(best > 0)) s_bad = 1;
+        if (!(best > 0)) s_bad = 1;  // zeros or NaN only
         // the reciprocal once per step (a division by every warp took a third of the FP64 pipe at nA =
         // 100), at the place where the scaled pivot row holds it: no memory beyond smem_elem_bytes
         const T pv = M[(size_t)bi * nc + c];

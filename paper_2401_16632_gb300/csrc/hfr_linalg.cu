@@ -170,7 +170,7 @@ __global__ void k_precond_build(const __grid_constant__ TraceArgs a, T* __restri
     int p = 0x7fffffff;
     if (lane < bs && !used) {
       const T v = M[lane * bs + c];
-      best = v < T(0) ? -v : v;
+      best = v != v ? T(-1) : (v < T(0) ? -v : v);  // NaN below every value
       p = lane;
     }
 #pragma unroll
@@ -179,8 +179,8 @@ __global__ void k_precond_build(const __grid_constant__ TraceArgs a, T* __restri
       const int op = __shfl_xor_sync(0xffffffffu, p, o);
       if (ob > best || (ob == best && op < p)) { best = ob; p = op; }
     }
-    if (p >= bs) p = c;  // no candidate compared (NaN column): any row, flagged singular
-    if (!(best > T(0))) bad = true;
+    if (!(best > T(0))) bad = true;  // zeros or NaN only; p is an unused row all the same
+
     if (lane == p) used = true;
     if (lane == 0) {
       ipiv[p] = c;
