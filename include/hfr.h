@@ -242,7 +242,7 @@ int imex_refresh_jacobian(fr_ctx* ctx);
  * kernel per step with the Krylov state on the device where FR_GMRES_FUSED is available too; the
  * default of contexts without it (other trace blocks, general meshes), which run each restart cycle
  * as one launch as well where the device allows it (FP64 basis; bounded barriers, or one thread-block
- * cluster for systems of a few thousand values).  FR_GMRES_SHORT: the short kernels on every
+ * cluster for small systems).  FR_GMRES_SHORT: the short kernels on every
  * context, until another mode is set.  All compute the same iteration (classical Gram-Schmidt with
  * a second pass); their results agree to rounding.
  * set: FR_ERR_UNSUPPORTED if FR_GMRES_FUSED is not available for the context.

@@ -995,7 +995,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_gmres_cycle(const __grid_cons
 // the rotations from global memory) an iteration cost 280 us on EFR nodes (128 x 128, p = 4), 290 us
 // on a wall mesh of 10 000 implicit elements and 70 us on 64 scalar elements; it takes 230, 155
 // and 22 us.
-// Systems of a few thousand values run on one cluster of eight CTAs, whose barrier is hardware.
+// Systems of some hundred values run on one cluster of eight CTAs, whose barrier is hardware.
 
 struct AnyShape {  // the layout of one element or trace unit, from the tables or the uniform sizes
   const CycleArgs& a;
@@ -1680,9 +1680,15 @@ cudaError_t launch_cycle_any(const CycleArgs& a, int prec_bytes, const CyclePlan
   return p.cluster ? launch_any<double, true>(a, p, s) : launch_any<double, false>(a, p, s);
 }
 
-// The cluster form up to about 200 000 multiply-adds per iteration (S once, the FP64 vectors some
-// forty times): above that, eight SMs' FP64 pipes take longer than the grid barriers of the whole
-// device cost (four per iteration, about 2 us each).
+// The cluster form for small systems, by the multiply-adds of an iteration (S once, the FP64 vectors some
+// forty times): above the line, eight SMs take longer for them than the grid barriers of the whole
+// device cost (four per iteration), sooner in FP64, whose pipe is the narrow one.  Time per iteration of
+// a cycle of 20, cluster / grid / short kernels, in us:
+//   FP32  25 000: 26.6 / 29.6 / 63   98 000: 29.3 / 30.5 / 65   154 000: 35.9 / 31.0 / 66   229 000: 48 / 31 / 66
+//   FP64  25 000: 28.0 / 30.2 / 67   37 000: 28.6 / 30.4 / 68   90 000: 35.4 / 31.8 / 67   187 000: 52 / 43 / 109
+// (scalar elements of 8 x 8 to 32 x 32, p = 1 to 3; the last of FP64: wall elements).  The lines are where
+// the scalar elements cross; shapes of several variables in FP64 cross below it (EDAC, p = 2, 18 000: 36.7 / 32.5
+// / 70) and FP32 faces of two values sooner (p = 1, 90 000: 33.5 / 30.7 / 64).
 CyclePlan cycle_plan(int prec_bytes, const CycleArgs& a) {
   CyclePlan p;
   int dev = 0, coop = 0, nsm = 0, occ = 0;
@@ -1695,7 +1701,7 @@ CyclePlan cycle_plan(int prec_bytes, const CycleArgs& a) {
   // 703 / 679 us, where the second Gram-Schmidt pass is not needed 380 / 385 and 637 / 586 us.
   if (prec_bytes == 8 && a.uni_nT > 0 && a.uni_bs > 16 && a.sumTT > 100000000LL) return p;
   if (cudaGetDevice(&dev) != cudaSuccess) return p;
-  if (a.sumTT + 40 * (long long)a.n <= 200000) {
+  if (a.sumTT + 40 * (long long)a.n <= (prec_bytes == 4 ? 100000 : 40000)) {
     const bool ok = prec_bytes == 4 ? cluster_fits<float>() : cluster_fits<double>();
     if (ok) {
       p.grid = ANY_CLUSTER;
