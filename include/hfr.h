@@ -397,9 +397,10 @@ int hfr_autotune(fr_ctx* ctx, const double* u, const double* uhat, const double*
  * instantiates the graph; later calls with the same arguments replay it.  Results equal the
  * stream path's.  Uniform meshes: requires implicit elements, FR_JAC_EVERY_NEWTON and (with a
  * trace) FR_GMRES_FUSED.  General meshes (mixed degree, boundary faces, hexahedra, EFR): requires
- * implicit elements; the GMRES restart cycle is the multi-kernel one, its m iterations enqueued
- * in the graph and skipped on the device once the cycle has ended, its restart decision taken on
- * the device, and the iteration limit checked per cycle.  FR_ERR_UNSUPPORTED otherwise.
+ * implicit elements; a GMRES restart cycle is one launch, its restart decision and the iteration limit
+ * taken on the device.  With FR_GMRES_SHORT, or where the device does not allow that launch, it is
+ * the cycle of short kernels: its m iterations enqueued in the graph and skipped on the device once
+ * the cycle has ended, the iteration limit checked per cycle.  FR_ERR_UNSUPPORTED otherwise.
  * Per-phase profiling (fr_profile_*) sees no phases of a graph stage. */
 int imex_stage_set_graph(fr_ctx* ctx, int on);
 int imex_stage_get_graph(const fr_ctx* ctx);
@@ -412,7 +413,7 @@ int hfr_initial_trace(fr_ctx* ctx, const double* u, double* uhat);
  * factorisation kernel (the whole condensation where it is a single kernel), 3 trace right-hand
  * side + preconditioner build, 4 trace GMRES solve, 5 back-substitution and refinement, 6 Newton
  * bookkeeping (right-hand sides, norms, updates), 7 FP64 refinement of x_r, 8 one trace mat-vec
- * kernel (multi-kernel GMRES: the restart / final-residual products), 9 condensation: the
+ * kernel (short-kernel GMRES: the restart / final-residual products), 9 condensation: the
  * products X = A^{-1}[B | r], S = D - C X_B of the two-kernel FP32 path. */
 typedef struct {
   double ms[10];

@@ -27,10 +27,10 @@
 //                    and columns of faces without a trace are zero), trace unknown
 //                    l = lto[f] + q nv + v
 // Kernels: one warp per element for the residual passes, one CTA of 256 threads per implicit
-// element for the blocks (dense tangents of the element operator, one warp per seed point), the
-// uneven-shape condensation (shared-memory Gauss-Jordan, or the global-memory LU for blocks too
-// large for shared memory), and warp-per-element / warp-per-face trace operators under the
-// multi-kernel GMRES driver.
+// element for the blocks (tangents along the grid lines of a seed point, one warp per seed point), the
+// uneven-shape condensation (shared-memory Gauss-Jordan, or the blocked LU for blocks too large for
+// shared memory), and the trace operator inside the single launch of a GMRES cycle (hfr_gmres_fused.cu)
+// or as warp-per-element / warp-per-face kernels under the driver of short kernels.
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
@@ -2702,7 +2702,7 @@ static TabG tableau_g(int which) {
 // ------------------------------------------------------------------ whole-stage CUDA graph
 // The implicit stage as one executable graph, as on the uniform path: the Newton loop a WHILE
 // node, its linear solve an IF node, the GMRES restart cycles a nested WHILE node
-// (capture_gmres); small kernels take on the device the decisions the stream path takes on the
+// (capture_gmres_any, or capture_gmres with the short kernels); small kernels take on the device the decisions the stream path takes on the
 // host (same tests, same order), and the host reads the counters once after the launch.
 struct GStageDev {
   double norm0, norm;

@@ -992,9 +992,9 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_gmres_cycle(const __grid_cons
 // pass (4 (j + 1) n multiply-adds per iteration).  The S values are cut into equal runs of rows, one
 // per warp of the grid, whatever the element shapes.  As one kernel per step (seven launches per
 // iteration, two of them reductions that ended in one block reading every partial sum and updating
-// the rotations from global memory) an iteration cost 280 us on EFR nodes (128 x 128, p = 4), 290 us
-// on a wall mesh of 10 000 implicit elements and 70 us on 64 scalar elements; it takes 230, 155
-// and 22 us.
+// the rotations from global memory) an iteration of a stage costs 284 us on EFR nodes (128 x 128, p = 4),
+// 297 us on a wall mesh of 10 000 implicit elements and 70 us on 64 scalar elements; it takes 245, 203
+// and 26 us here.
 // Systems of some hundred values run on one cluster of eight CTAs, whose barrier is hardware.
 
 struct AnyShape {  // the layout of one element or trace unit, from the tables or the uniform sizes

@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(JAC_THREADS, jac_blocks<T>(P)) k_jacobian(cons
   // Bound by the stores of the blocks, 130 KB per element at p = 4.  One seed point per warp with
   // the tangents of its two lines, six vector reads of shared memory per output vector, kept the
   // shared-memory pipe at 89 %: 368 us for 4096 elements, p = 4, FP32 (the blocks alone take 79 us
-  // at the copy rate); 194 us by the tables.  FP64, p = 3: 1.65 ms, 1.0 ms now.
+  // at the copy rate); 195 us by the tables.  FP64, p = 3: 1.65 ms, 1.0 ms now.
   constexpr int CI = N * NV * (2 * N + 2);
   for (int it = tid; it < 4 * CI; it += JAC_THREADS) {
     const int f = it / CI, s2 = it % (2 * N + 2), v = it / (2 * N + 2) % NV, m = it / ((2 * N + 2) * NV) % N;
