@@ -322,6 +322,33 @@ __device__ __forceinline__ int line_pt(int r, int m, int c) {
   return r == 0 ? (c + N * m) : (m + N * c);
 }
 
+// NV consecutive values, 16-byte accesses where the layout allows them
+template <typename T, int NV>
+__device__ __forceinline__ void ldv(const T* p, T (&x)[NV]) {
+  if constexpr (NV == 4 && sizeof(T) == 4) {
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
+  } else if constexpr (NV == 4 && sizeof(T) == 8) {
+    const double2 q0 = reinterpret_cast<const double2*>(p)[0], q1 = reinterpret_cast<const double2*>(p)[1];
+    x[0] = q0.x; x[1] = q0.y; x[2] = q1.x; x[3] = q1.y;
+  } else {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) x[v] = p[v];
+  }
+}
+template <typename T, int NV>
+__device__ __forceinline__ void stv(T* p, const T (&x)[NV]) {
+  if constexpr (NV == 4 && sizeof(T) == 4) {
+    *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
+  } else if constexpr (NV == 4 && sizeof(T) == 8) {
+    reinterpret_cast<double2*>(p)[0] = make_double2(x[0], x[1]);
+    reinterpret_cast<double2*>(p)[1] = make_double2(x[2], x[3]);
+  } else {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) p[v] = x[v];
+  }
+}
+
 // status word bits written by kernels (never trap)
 enum { DEV_ERR_SINGULAR = 1, DEV_ERR_NAN = 2, DEV_ERR_INDEX = 4, DEV_ERR_TIMEOUT = 8 };
 

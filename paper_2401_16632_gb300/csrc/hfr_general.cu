@@ -534,36 +534,11 @@ struct JWork {
 static_assert(sizeof(JWork<GN, 4, double>) <= 227 * 1024, "block kernel workspace exceeds shared memory");
 static_assert(sizeof(GWork<4>) * GEPB <= 227 * 1024, "residual workspace exceeds shared memory");
 
-template <typename T, int NV>
-__device__ __forceinline__ void gldv(const T* p, T (&x)[NV]) {
-  if constexpr (NV == 4 && sizeof(T) == 4) {
-    const float4 q = *reinterpret_cast<const float4*>(p);
-    x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
-  } else if constexpr (NV == 4 && sizeof(T) == 8) {
-    const double2 q0 = reinterpret_cast<const double2*>(p)[0], q1 = reinterpret_cast<const double2*>(p)[1];
-    x[0] = q0.x; x[1] = q0.y; x[2] = q1.x; x[3] = q1.y;
-  } else {
-#pragma unroll
-    for (int v = 0; v < NV; ++v) x[v] = p[v];
-  }
-}
-template <typename T, int NV>
-__device__ __forceinline__ void gstv(T* p, const T (&x)[NV]) {
-  if constexpr (NV == 4 && sizeof(T) == 4) {
-    *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
-  } else if constexpr (NV == 4 && sizeof(T) == 8) {
-    reinterpret_cast<double2*>(p)[0] = make_double2(x[0], x[1]);
-    reinterpret_cast<double2*>(p)[1] = make_double2(x[2], x[3]);
-  } else {
-#pragma unroll
-    for (int v = 0; v < NV; ++v) p[v] = x[v];
-  }
-}
 // o += c * p[0 .. NV)
 template <typename T, int NV>
 __device__ __forceinline__ void gfma(T c, const T* p, T (&o)[NV]) {
   T t[NV];
-  gldv<T, NV>(p, t);
+  ldv<T, NV>(p, t);
 #pragma unroll
   for (int x = 0; x < NV; ++x) o[x] += c * t[x];
 }
@@ -954,7 +929,7 @@ __global__ void __launch_bounds__(JT, sizeof(T) == 4 ? (N <= 5 ? 3 : 2) : 1) k_g
           gfma<T, NV>(d0, &w.KQ[pt][r][0][vv][0], o);
           gfma<T, NV>(d1, &w.KQ[pt][r][1][vv][0], o);
           if (vol && pt == sp) gfma<T, NV>(T(1), &w.KU[pt][r][vv][0], o);
-          gstv<T, NV>(&cw.LN[line][c][(r * NV + vv) * NV], o);
+          stv<T, NV>(&cw.LN[line][c][(r * NV + vv) * NV], o);
         }
       } else {
         const int jj = w.pt[it - 2 * N];
@@ -965,7 +940,7 @@ __global__ void __launch_bounds__(JT, sizeof(T) == 4 ? (N <= 5 ? 3 : 2) : 1) k_g
         gfma<T, NV>(cw.qp[jj][1], &w.GQ[jj][1][vv][0], o);
         if (vol) gfma<T, NV>(cw.du[jj], &w.GU[jj][vv][0], o);
         if (jj == j0) gfma<T, NV>(T(1), &w.GH[jj][vv][0], o);
-        gstv<T, NV>(&cw.FP[jj][vv * NV], o);
+        stv<T, NV>(&cw.FP[jj][vv * NV], o);
       }
     }
     __syncwarp();
@@ -979,12 +954,12 @@ __global__ void __launch_bounds__(JT, sizeof(T) == 4 ? (N <= 5 ? 3 : 2) : 1) k_g
         if (!(line == 0 ? has_row : has_col)) continue;
 #pragma unroll
         for (int c = 0; c < N; ++c) gfma<T, NV>(w.M[i][c], &cw.LN[line][c][(line * NV + vv) * NV], o);
-        gstv<T, NV>(&cw.RC[line][i][vv * NV], o);
+        stv<T, NV>(&cw.RC[line][i][vv * NV], o);
       } else {
         const int jn = it - 2 * N, f = jn / N, b = jn % N;
         if (w.own[f]) continue;
         for (int q = 0; q < w.nf[f]; ++q) gfma<T, NV>(w.Pf[f][b][q], &cw.FP[f * GN + q][vv * NV], o);
-        gstv<T, NV>(&cw.FN[jn][vv * NV], o);
+        stv<T, NV>(&cw.FN[jn][vv * NV], o);
       }
     }
     __syncwarp();
@@ -1027,7 +1002,7 @@ __global__ void __launch_bounds__(JT, sizeof(T) == 4 ? (N <= 5 ? 3 : 2) : 1) k_g
           for (int x = 0; x < NV; ++x)
             if (x == vv) o[x] += T(1);
         }
-        gstv<T, NV>(top + (size_t)(it * NV + vv) * ncol + col0, o);
+        stv<T, NV>(top + (size_t)(it * NV + vv) * ncol + col0, o);
       } else {
         // C / D rows: w_q times the trace row's tangent, zero off traces.  Interior rows are the
         // face flux; a wall keeps it in mass and energy and has rows of the trace alone in momentum;
@@ -1049,7 +1024,7 @@ __global__ void __launch_bounds__(JT, sizeof(T) == 4 ? (N <= 5 ? 3 : 2) : 1) k_g
 #pragma unroll
           for (int x = 0; x < NV; ++x) o[x] *= wm;
         }
-        gstv<T, NV>(bot + (size_t)(w.lto[f] + q * NV + vv) * ncol + col0, o);
+        stv<T, NV>(bot + (size_t)(w.lto[f] + q * NV + vv) * ncol + col0, o);
       }
     }
     __syncwarp();  // the next seed point rewrites this warp's buffers
