@@ -101,6 +101,7 @@ struct fr_ctx {
   long long jac_refreshes = 0;  // element-block linearisations made by imex_stage
   int cond_mode = 0;        // fr_condense_mode of the FP32 condensation
   int inv_ctas = 0;         // CTAs per SM of the tensor-core inverse (0: default)
+  int nsm = 1;              // multiprocessors of the device
   double* filt = nullptr;   // ns x ns modal filter operator (fr_modal_filter)
   // whole-stage CUDA graph
   int use_graph = 0;
@@ -639,6 +640,7 @@ extern "C" int fr_ctx_create(const fr_mesh_desc* mesh, const fr_config* cfg, voi
     int dev = 0, nsm = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    ctx->nsm = nsm;
     ctx->gm_fused_grid = fused_gmres_grid(ctx->prec_bytes, nT, n * nv);
     ctx->gm_mode = ctx->gm_fused_grid > 0 ? 1 : 0;
     ctx->cond_mode = condense_tc_available(ctx->prec_bytes, nA, nT);
@@ -782,6 +784,7 @@ static ResArgs res_args(fr_ctx* ctx, const double* u, const double* uhat) {
   a.qf_out = ctx->qf_all;
   a.q_out = ctx->q_all;
   a.ntrace = ctx->ntrace;
+  a.nsm = ctx->nsm;
   return a;
 }
 

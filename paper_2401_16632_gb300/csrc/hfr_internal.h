@@ -69,6 +69,7 @@ struct ResArgs {
   double* gview;         // nullable: w_q J_f F^.n on trace faces
   double* dgview;        // nullable (JVP)
   int ntrace;            // trace faces (bounds of tr_of in the checked build)
+  int nsm;               // multiprocessors of the device
 };
 
 cudaError_t launch_residual(int p, const RefOps& ref, const PhysParams& pp, const ResArgs& a, bool need_nbr,

@@ -332,11 +332,7 @@ static cudaError_t launch_elem_n(const RefOps& ref, const PhysParams& pp, const 
 template <int P, int PHYS, typename S, int MODE>
 static cudaError_t launch_elem(const RefOps& ref, const PhysParams& pp, const ResArgs& a, cudaStream_t st) {
   constexpr int EPB = P <= 2 ? 16 : 8, NT = P <= 3 ? 128 : 256;
-  int dev = 0, nsm = 0;
-  cudaError_t err = cudaGetDevice(&dev);
-  if (err == cudaSuccess) err = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (err != cudaSuccess) return err;
-  if (a.E >= 2 * nsm * EPB) return launch_elem_n<P, PHYS, S, MODE, EPB, NT>(ref, pp, a, st);
+  if (a.E >= 2 * a.nsm * EPB) return launch_elem_n<P, PHYS, S, MODE, EPB, NT>(ref, pp, a, st);
   return launch_elem_n<P, PHYS, S, MODE, 4, 128>(ref, pp, a, st);
 }
 
