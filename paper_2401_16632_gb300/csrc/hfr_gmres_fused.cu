@@ -1323,9 +1323,12 @@ constexpr size_t any_smem() {
   return (sizeof(PGShared<double>) + 15) / 16 * 16 + (size_t)PG_WARPS * ANY_MAXT * sizeof(T);
 }
 
-// CLUSTER: one cluster of ANY_CLUSTER CTAs instead of a cooperative grid
-template <typename T, bool CLUSTER>
+// forms: a cooperative grid, where cancellation asks for the second Gram-Schmidt pass; one cluster of
+// ANY_CLUSTER CTAs, and a grid for small systems, which make it always
+enum { ANY_GRID = 0, ANY_ONE_CLUSTER = 1, ANY_GRID_SMALL = 2 };
+template <typename T, int FORM>
 __global__ void __launch_bounds__(PG_THREADS, 1) k_gmres_cycle_any(const __grid_constant__ CycleArgs a) {
+  constexpr bool CLUSTER = FORM == ANY_ONE_CLUSTER, TEST = FORM == ANY_GRID;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   PGShared<double>& sh = *reinterpret_cast<PGShared<double>*>(smem_raw);
   T* xs = reinterpret_cast<T*>(smem_raw + (sizeof(PGShared<double>) + 15) / 16 * 16) + (threadIdx.x >> 5) * ANY_MAXT;
@@ -1416,10 +1419,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_gmres_cycle_any(const __grid_
       // (B) y_k = S_k z_k
       any_matvec<T, T>(a, zrow(j), xs);
       if (!sync()) return;
-      // (C) w = L z, h = V^T w (and ||w||^2).  The cluster makes the second pass always: its dots are of a
-      // few hundred values, no dearer than the test for leaving them out (64 scalar elements, FP64, 1 / 10 /
-      // 100 times the step: 26.5 / 28.0 / 29.5 us per iteration without the test, 27.8 / 28.7 / 30.1 with it)
-      constexpr bool TEST = !CLUSTER;
+      // (C) w = L z, h = V^T w (and ||w||^2)
       any_gather<T>(a, nullptr, w, x0, x1);
       double* part = partial + par * pstride;
       pg_block_dots<double>(sh, V, n, j + (TEST ? 2 : 1), w, x0, x1, part);
@@ -1643,14 +1643,14 @@ cudaError_t launch_gmres_cycle(const FusedArgs& a, int prec_bytes, int grid, cud
   return fn(a, grid, s);
 }
 
-template <typename T, bool CLUSTER>
+template <typename T, int FORM>
 static cudaError_t any_config(int grid, cudaStream_t s, cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&at)[1]) {
   cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(PG_THREADS);
   cfg.dynamicSmemBytes = any_smem<T>();
   cfg.stream = s;
-  if (CLUSTER) {
+  if (FORM == ANY_ONE_CLUSTER) {
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = ANY_CLUSTER;
     at[0].val.clusterDim.y = 1;
@@ -1661,18 +1661,24 @@ static cudaError_t any_config(int grid, cudaStream_t s, cudaLaunchConfig_t& cfg,
   }
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaFuncSetAttribute(k_gmres_cycle_any<T, CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  return cudaFuncSetAttribute(k_gmres_cycle_any<T, FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)any_smem<T>());
 }
 
-template <typename T, bool CLUSTER>
+template <typename T, int FORM>
 static cudaError_t launch_any(const CycleArgs& a, const CyclePlan& p, cudaStream_t s) {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at[1];
-  const cudaError_t e = any_config<T, CLUSTER>(p.grid, s, cfg, at);
+  const cudaError_t e = any_config<T, FORM>(p.grid, s, cfg, at);
   if (e != cudaSuccess) return e;
   hfr::count_launch();
-  return cudaLaunchKernelEx(&cfg, k_gmres_cycle_any<T, CLUSTER>, a);
+  return cudaLaunchKernelEx(&cfg, k_gmres_cycle_any<T, FORM>, a);
+}
+template <typename T>
+static cudaError_t launch_form(const CycleArgs& a, const CyclePlan& p, cudaStream_t s) {
+  if (p.form == ANY_ONE_CLUSTER) return launch_any<T, ANY_ONE_CLUSTER>(a, p, s);
+  if (p.form == ANY_GRID_SMALL) return launch_any<T, ANY_GRID_SMALL>(a, p, s);
+  return launch_any<T, ANY_GRID>(a, p, s);
 }
 
 // one cluster of the cycle can be resident on the device
@@ -1681,14 +1687,13 @@ static bool cluster_fits() {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at[1];
   int n = 0;
-  return any_config<T, true>(ANY_CLUSTER, nullptr, cfg, at) == cudaSuccess &&
-         cudaOccupancyMaxActiveClusters(&n, k_gmres_cycle_any<T, true>, &cfg) == cudaSuccess && n >= 1;
+  return any_config<T, ANY_ONE_CLUSTER>(ANY_CLUSTER, nullptr, cfg, at) == cudaSuccess &&
+         cudaOccupancyMaxActiveClusters(&n, k_gmres_cycle_any<T, ANY_ONE_CLUSTER>, &cfg) == cudaSuccess && n >= 1;
 }
 
 cudaError_t launch_cycle_any(const CycleArgs& a, int prec_bytes, const CyclePlan& p, cudaStream_t s) {
   if (p.grid < 1) return cudaErrorInvalidValue;
-  if (prec_bytes == 4) return p.cluster ? launch_any<float, true>(a, p, s) : launch_any<float, false>(a, p, s);
-  return p.cluster ? launch_any<double, true>(a, p, s) : launch_any<double, false>(a, p, s);
+  return prec_bytes == 4 ? launch_form<float>(a, p, s) : launch_form<double>(a, p, s);
 }
 
 // The cluster form for small systems, by the multiply-adds of an iteration (S once, the FP64 vectors some
@@ -1716,7 +1721,7 @@ CyclePlan cycle_plan(int prec_bytes, const CycleArgs& a) {
     const bool ok = prec_bytes == 4 ? cluster_fits<float>() : cluster_fits<double>();
     if (ok) {
       p.grid = ANY_CLUSTER;
-      p.cluster = 1;
+      p.form = ANY_ONE_CLUSTER;
       return p;
     }
     cudaGetLastError();
@@ -1727,9 +1732,22 @@ CyclePlan cycle_plan(int prec_bytes, const CycleArgs& a) {
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, PG_THREADS, smem) == cudaSuccess && occ >= 1;
   };
-  const bool ok = prec_bytes == 4 ? fits(k_gmres_cycle_any<float, false>, any_smem<float>())
-                                  : fits(k_gmres_cycle_any<double, false>, any_smem<double>());
-  if (ok) p.grid = nsm;  // one CTA per SM
+  // The test for the second Gram-Schmidt pass sits on the chain of every iteration (0.5 us).  Systems of
+  // fewer than some 25 000 trace values make the pass always: where the test never lets them off they
+  // lose up to 1.3 % by it, where it does the single launch is ahead of the short kernels by 40 % either way.
+  // Per iteration with the test / without, in us, ten times the explicit step and 300 times: EFR p = 4,
+  // 15 000 values 47.9 / 47.5 and 40.0 / 47.3, 64 500 values 59.9 / 60.5 and 49.0 / 60.4, 459 000 values
+  // 244.7 / 244.9 and 220.2 / 245.9 (short kernels 236.3); scalar, p = 2, FP64, 14 000 values 35.7 / 35.4; one
+  // cluster, 64 scalar elements 27.8 / 26.5.
+  const bool small = a.n < 25000;
+  const bool ok = prec_bytes == 4 ? (small ? fits(k_gmres_cycle_any<float, ANY_GRID_SMALL>, any_smem<float>())
+                                           : fits(k_gmres_cycle_any<float, ANY_GRID>, any_smem<float>()))
+                                  : (small ? fits(k_gmres_cycle_any<double, ANY_GRID_SMALL>, any_smem<double>())
+                                           : fits(k_gmres_cycle_any<double, ANY_GRID>, any_smem<double>()));
+  if (ok) {
+    p.grid = nsm;  // one CTA per SM
+    p.form = small ? ANY_GRID_SMALL : ANY_GRID;
+  }
   return p;
 }
 

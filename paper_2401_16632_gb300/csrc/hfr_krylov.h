@@ -126,7 +126,7 @@ struct CycleArgs {
 // how the cycle is launched: grid 0 not available; cluster 1 = one cluster of 8 CTAs (small systems:
 // its hardware barrier), else a cooperative launch of one CTA per SM
 struct CyclePlan {
-  int grid = 0, cluster = 0;
+  int grid = 0, form = 0;  // form: the template argument of k_gmres_cycle_any
 };
 CyclePlan cycle_plan(int prec_bytes, const CycleArgs& a);
 cudaError_t launch_cycle_any(const CycleArgs& a, int prec_bytes, const CyclePlan& p, cudaStream_t s);
